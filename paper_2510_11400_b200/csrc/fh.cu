@@ -13,15 +13,27 @@
 #include <utility>
 #include <vector>
 
-#include "fh_channel.cuh"
-#include "fh_compress.cuh"
-#include "fh_decompress.cuh"
+#include "fh_launch.cuh"
+
+namespace fh {
+
+int sm_count() {
+  static int count[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!count[dev]) cudaDeviceGetAttribute(&count[dev], cudaDevAttrMultiProcessorCount, dev);
+  return count[dev];
+}
+
+}  // namespace fh
 
 namespace {
 
+using fh::A16;
+using fh::kSmemLimit;
 using fh::Plan;
+using fh::Variant;
 
-constexpr size_t kSmemLimit = 227 * 1024 - 4096;  // dynamic shared memory a CTA may ask for
 constexpr size_t kTileTarget = 32 * 1024;         // dense bytes a tile of the generic kernel aims for
 constexpr size_t kStageTarget = 72 * 1024;        // shared memory the stages of the CTA-team kernel aim for
 constexpr size_t kWarpStageTarget = 72 * 1024;    // ... and those of the warp-team kernel (two CTAs per SM)
@@ -29,7 +41,6 @@ constexpr uint32_t kMaxPpt = 2048;
 
 std::atomic<uint64_t> g_launches{0};
 
-inline size_t A16(size_t x) { return (x + 15) & ~(size_t)15; }
 inline size_t A256(size_t x) { return (x + 255) & ~(size_t)255; }
 inline size_t esize_of(int dtype) { return dtype == FH_F32 ? 4 : 2; }
 
@@ -64,13 +75,6 @@ uint32_t pow2_ceil(uint32_t x) {
   while (r < x) r *= 2;
   return r;
 }
-
-// Which kernel a plan runs on.
-struct Variant {
-  bool fast = false;  // compress_warp / compress_cta (bulk-copy pipeline) instead of compress_generic
-  bool cta = false;   // fast: compress_cta (one plane per CTA) instead of compress_warp (one plane per team of lanes)
-  int G = 0;          // fast: groups per thread
-};
 
 // Tiling and shared-memory layout.  `compress` selects the compress kernels' layout; the decompress
 // kernel only needs the block-wise scratch.
@@ -113,23 +117,23 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   const long double worst = 64.0L + (long double)pl.P * (16.0L + (long double)A16(pl.plane_bytes));
   if (worst / 16.0L >= 4294967295.0L) return FH_ERR_UNSUPPORTED;
   if (pl.P > 0x7FFFFFFFull) return FH_ERR_UNSUPPORTED;
-  // measuring scratch of the block-wise path: row pointers and three words per block; with the Huffman stage two
-  // more words per block and the encoder's tables.  Decompress: two words per block and the decoder's tables.
-  const size_t sal_words = compress ? (size_t)(pl.H + 1 + 3 * pl.nblk) + (pl.entropy ? 2 * (size_t)pl.nblk + sizeof(fh::HufEncode) / 4 + 4 : 0)
+  // block-wise path: blocks per step side by side, rows of steps (see fh_blocks.cuh)
+  pl.qs = pl.nbx >= 3 ? 2u : pl.nbx - 1u;
+  pl.nsr = (pl.nby + (4u >> pl.qs) - 1u) / (4u >> pl.qs);
+  // its measuring scratch: row pointers, two sums per step row, the bitmap; with the Huffman stage one more sum and the
+  // encoder's tables.  Decompress: two words per block and the decoder's tables.
+  const size_t sal_words = compress ? (size_t)pl.H + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
+                                          (pl.entropy ? (size_t)pl.nsr + 1 + sizeof(fh::HufEncode) / 4 : 0)
                                     : 2 * (size_t)pl.nblk + sizeof(fh::HufDecode) / 4 + 4;
-  pl.sal_words = (uint32_t)sal_words;
   const uint32_t sal_bytes = (uint32_t)A16(4 * sal_words + 16);  // one measuring area of the block-wise path
   const bool blockwise = compress && pl.mode != FH_SALIENT_OFF;
 
   Variant v;
   // ---- fast compress kernels: planes of whole 16-byte chunks whose groups fit the register budget
   const bool whole16 = pl.HW % 4 == 0 && pl.plane_bytes % 16 == 0;
-  // (the Huffman stage runs on the generic kernel; random rounding on the warp-team kernels in the plane-wise
-  // three-sigma mode, on the generic kernel otherwise)
-  // (a warp-team kernel keeps one measuring area per warp: planes whose area is large -- very tall, narrow
-  // ones -- go to the general-purpose kernel)
+  // (random rounding runs on the warp-team kernels in the plane-wise three-sigma mode, on the generic kernel otherwise)
   const bool rounding_ok = pl.rounding == 0 || (pl.groups <= 256 && pl.mode == FH_SALIENT_AUTO);
-  if (compress && rounding_ok && pl.entropy == 0 && ((pl.groups <= 256 && (!blockwise || sal_bytes <= 1024)) || (pl.groups > 256 && whole16))) {
+  if (compress && rounding_ok && (pl.groups <= 256 || whole16)) {
     v.fast = true;
     if (pl.groups <= 256) {
       uint32_t t = pow2_ceil((pl.groups + 7) / 8);
@@ -247,7 +251,6 @@ inline size_t scan_words(size_t tile_cap) { return tile_cap + 3 * (tile_cap / 32
 
 std::mutex g_mu;
 std::map<std::pair<int, cudaStream_t>, StreamScratch> g_scratch;
-int g_sm_count[64] = {0};
 
 // Fault injection for the time-out test (see fh_debug_set in the header): limit of the device-side waits
 // of the placement scan, and a tile that never publishes.
@@ -326,8 +329,6 @@ int next_call(uint32_t* calls, unsigned long long* scan, size_t tile_cap, Stream
   return FH_OK;
 }
 
-int sm_count();
-
 // Scratch of the channel-wide three-sigma mode (grown on demand like the per-stream scratch).
 int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels) {
   if (planes > s->pn_cap) {
@@ -357,263 +358,13 @@ int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels) {
   return FH_OK;
 }
 
-template <int DT>
-int launch_channel_passes(const Plan& pl, const fh::ChannelArgs& ca, cudaStream_t stream) {
-  const int sms = sm_count();
-  if (sms < 1) return FH_ERR_CUDA;
-  const uint64_t want = (pl.P + fh::kWarps - 1) / fh::kWarps, most = (uint64_t)sms * 8;
-  const int grid = (int)(want < most ? want : most);
-  if (cudaMemsetAsync(ca.chan, 0, pl.C * sizeof(fh::ChanStat), stream) != cudaSuccess) return FH_ERR_CUDA;
-  fh::channel_pass<DT, 0><<<grid, fh::kThreads, 0, stream>>>(pl, ca);
-  fh::channel_pass<DT, 1><<<grid, fh::kThreads, 0, stream>>>(pl, ca);
-  fh::channel_pass<DT, 2><<<grid, fh::kThreads, 0, stream>>>(pl, ca);
-  if (cudaGetLastError() != cudaSuccess) return FH_ERR_CUDA;
-  g_launches.fetch_add(3);
-  return FH_OK;
-}
-
-int sm_count() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!g_sm_count[dev]) cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
-  return g_sm_count[dev];
-}
-
-template <typename K>
-int grid_for(K kernel, size_t smem, uint32_t ntiles, int* grid, int threads = fh::kThreads) {
-  static std::map<std::tuple<int, const void*, size_t>, int> cache;  // guarded by g_mu; per device: the attribute is
-  int dev = 0;                                                        // set once for every device that runs the kernel
-  if (cudaGetDevice(&dev) != cudaSuccess) return FH_ERR_CUDA;
-  const auto key = std::make_tuple(dev, (const void*)kernel, (smem << 12) | (size_t)threads);
-  auto it = cache.find(key);
-  int per_sm;
-  if (it == cache.end()) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess)
-      return FH_ERR_CUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess)
-      return FH_ERR_CUDA;
-    if (per_sm < 1) return FH_ERR_UNSUPPORTED;
-    cache[key] = per_sm;
-  } else {
-    per_sm = it->second;
-  }
-  const int sms = sm_count();
-  if (sms < 1) return FH_ERR_CUDA;
-  const uint64_t g = (uint64_t)per_sm * sms;
-  *grid = (int)(ntiles < g ? ntiles : g);
-  return FH_OK;
-}
-
-template <typename K>
-int launch_on(K kernel, const Plan& pl, cudaStream_t stream, int* grid) {
-  return grid_for(kernel, pl.sm_total, pl.ntiles, grid);
-}
-
-// Launch that may overlap the tail of the previous kernel on the stream: every kernel of this library
-// passes dep_wait() before it touches global memory, so stream order is kept.
-// Tiles a CTA requests at once when it starts: all its stages when every CTA of the grid gets that many, fewer
-// when the tensor is small, so that the tiles spread over all CTAs before any CTA takes a second one.
-Plan with_first_request(const Plan& pl, int grid, uint32_t least) {
-  Plan q = pl;
-  const uint32_t each = pl.ntiles / (uint32_t)(grid > 0 ? grid : 1);
-  q.nstage = each < least ? least : (each > pl.nstage ? pl.nstage : each);
-  return q;
-}
-
-template <typename K, typename A>
-cudaError_t launch_dependent(K kernel, int grid, int threads, size_t smem, cudaStream_t stream, const Plan& pl,
-                             const A& a) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, pl, a);
-}
-
-template <int DT, int BITS>
-int launch_generic_t(const Plan& pl, const fh::CompressArgs& a, cudaStream_t stream) {
-  int grid = 0;
-  int rc = grid_for(fh::compress_generic<DT, BITS>, pl.sm_total, pl.ntiles, &grid);
-  if (rc != FH_OK) return rc;
-  return launch_dependent(fh::compress_generic<DT, BITS>, grid, fh::kThreads, pl.sm_total, stream, pl, a) == cudaSuccess
-             ? FH_OK : FH_ERR_CUDA;
-}
-
-template <int DT, bool SIGMA, int NT>
-int launch_cta_t(const Plan& pl, const fh::CompressArgs& a, cudaStream_t stream) {
-  int grid = 0;
-  int rc = grid_for(fh::compress_cta<DT, SIGMA, NT>, pl.sm_total, pl.ntiles, &grid, NT);
-  if (rc != FH_OK) return rc;
-  return launch_dependent(fh::compress_cta<DT, SIGMA, NT>, grid, NT, pl.sm_total, stream, with_first_request(pl, grid, 2), a) == cudaSuccess
-             ? FH_OK : FH_ERR_CUDA;
-}
-
-template <int DT, bool SIGMA, int NT, int G>
-int launch_cta_regs_t(const Plan& pl, const fh::CompressArgs& a, cudaStream_t stream) {
-  int grid = 0;
-  if (pl.groups == (uint32_t)(NT * G)) {
-    int rc = grid_for(fh::compress_cta_regs<DT, SIGMA, NT, G, true>, pl.sm_total, pl.ntiles, &grid, NT);
-    if (rc != FH_OK) return rc;
-    return launch_dependent(fh::compress_cta_regs<DT, SIGMA, NT, G, true>, grid, NT, pl.sm_total, stream,
-                            with_first_request(pl, grid, 2), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
-  }
-  int rc = grid_for(fh::compress_cta_regs<DT, SIGMA, NT, G, false>, pl.sm_total, pl.ntiles, &grid, NT);
-  if (rc != FH_OK) return rc;
-  return launch_dependent(fh::compress_cta_regs<DT, SIGMA, NT, G, false>, grid, NT, pl.sm_total, stream,
-                          with_first_request(pl, grid, 2), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
-}
-
-template <int DT, int SIGMA, int TT, bool FULLVEC>
-int launch_warp_t(const Plan& pl, const fh::CompressArgs& a, cudaStream_t stream) {
-  int grid = 0;
-  int rc = grid_for(fh::compress_warp<DT, SIGMA, TT, FULLVEC>, pl.sm_total, pl.ntiles, &grid, fh::kWarpKernelThreads);
-  if (rc != FH_OK) return rc;
-  return launch_dependent(fh::compress_warp<DT, SIGMA, TT, FULLVEC>, grid, fh::kWarpKernelThreads, pl.sm_total, stream,
-                          with_first_request(pl, grid, 1), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
-}
-
-template <int DT, int SIGMA, bool FULLVEC>
-int launch_warp_tt(const Plan& pl, const fh::CompressArgs& a, cudaStream_t stream) {
-  switch (pl.team) {
-    case 1: return launch_warp_t<DT, SIGMA, 1, FULLVEC>(pl, a, stream);
-    case 2: return launch_warp_t<DT, SIGMA, 2, FULLVEC>(pl, a, stream);
-    case 4: return launch_warp_t<DT, SIGMA, 4, FULLVEC>(pl, a, stream);
-    case 8: return launch_warp_t<DT, SIGMA, 8, FULLVEC>(pl, a, stream);
-    case 16: return launch_warp_t<DT, SIGMA, 16, FULLVEC>(pl, a, stream);
-    case 32: return launch_warp_t<DT, SIGMA, 32, FULLVEC>(pl, a, stream);
-  }
-  return FH_ERR_UNSUPPORTED;
-}
-
-template <int DT, bool SIGMA>
-int launch_cta_g(const Plan& pl, const Variant& v, const fh::CompressArgs& a, cudaStream_t stream);
-
-template <int DT, int SIGMA>
-int launch_fast_g(const Plan& pl, const Variant& v, const fh::CompressArgs& a, cudaStream_t stream) {
-  if (!v.cta) {
-    const bool fullvec = pl.plane_bytes % 16 == 0 && pl.HW % 4 == 0 && pl.groups == 8u * pl.team;
-    return fullvec ? launch_warp_tt<DT, SIGMA, true>(pl, a, stream) : launch_warp_tt<DT, SIGMA, false>(pl, a, stream);
-  }
-  if constexpr (SIGMA == 2) return FH_ERR_UNSUPPORTED;  // (make_plan sends random rounding on large planes elsewhere)
-  else return launch_cta_g<DT, SIGMA != 0>(pl, v, a, stream);
-}
-
-template <int DT, bool SIGMA>
-int launch_cta_g(const Plan& pl, const Variant& v, const fh::CompressArgs& a, cudaStream_t stream) {
-  if (v.G) {
-    switch (pl.team * 16 + v.G) {
-      case 128 * 16 + 7: return launch_cta_regs_t<DT, SIGMA, 128, 7>(pl, a, stream);
-      case 128 * 16 + 8: return launch_cta_regs_t<DT, SIGMA, 128, 8>(pl, a, stream);
-      case 256 * 16 + 7: return launch_cta_regs_t<DT, SIGMA, 256, 7>(pl, a, stream);
-      case 256 * 16 + 8: return launch_cta_regs_t<DT, SIGMA, 256, 8>(pl, a, stream);
-      case 448 * 16 + 7: return launch_cta_regs_t<DT, SIGMA, 448, 7>(pl, a, stream);
-      case 512 * 16 + 8: return launch_cta_regs_t<DT, SIGMA, 512, 8>(pl, a, stream);
-    }
-    return FH_ERR_UNSUPPORTED;
-  }
-  switch (pl.team) {
-    case 128: return launch_cta_t<DT, SIGMA, 128>(pl, a, stream);
-    case 256: return launch_cta_t<DT, SIGMA, 256>(pl, a, stream);
-    case 512: return launch_cta_t<DT, SIGMA, 512>(pl, a, stream);
-  }
-  return FH_ERR_UNSUPPORTED;
-}
-
 int launch_compress(const Plan& pl, const Variant& v, const fh::CompressArgs& a, cudaStream_t stream) {
-  int rc;
-  if (v.fast) {
-    const int sigma = pl.mode == FH_SALIENT_AUTO ? (pl.rounding ? 2 : 1) : 0;
-    if (pl.dtype == FH_F32)
-      rc = sigma == 2 ? launch_fast_g<fh::kF32, 2>(pl, v, a, stream)
-           : sigma    ? launch_fast_g<fh::kF32, 1>(pl, v, a, stream) : launch_fast_g<fh::kF32, 0>(pl, v, a, stream);
-    else
-      rc = sigma == 2 ? launch_fast_g<fh::kBF16, 2>(pl, v, a, stream)
-           : sigma    ? launch_fast_g<fh::kBF16, 1>(pl, v, a, stream) : launch_fast_g<fh::kBF16, 0>(pl, v, a, stream);
-  } else if (pl.dtype == FH_F32) {
-    rc = pl.bits == 2   ? launch_generic_t<fh::kF32, 2>(pl, a, stream)
-         : pl.bits == 4 ? launch_generic_t<fh::kF32, 4>(pl, a, stream)
-                        : launch_generic_t<fh::kF32, 8>(pl, a, stream);
-  } else {
-    rc = pl.bits == 2   ? launch_generic_t<fh::kBF16, 2>(pl, a, stream)
-         : pl.bits == 4 ? launch_generic_t<fh::kBF16, 4>(pl, a, stream)
-                        : launch_generic_t<fh::kBF16, 8>(pl, a, stream);
-  }
-  if (rc != FH_OK) return rc;
-  g_launches.fetch_add(1);
-  return FH_OK;
-}
-
-// Largest prime <= n (n >= 2), or 1.
-uint64_t prime_at_most(uint64_t n) {
-  static std::map<uint64_t, uint64_t> cache;  // guarded by g_mu
-  auto it = cache.find(n);
-  if (it != cache.end()) return it->second;
-  for (uint64_t c = n; c >= 2; --c) {
-    bool prime = true;
-    for (uint64_t f = 2; f * f <= c; ++f)
-      if (c % f == 0) {
-        prime = false;
-        break;
-      }
-    if (prime) return cache[n] = c;
-  }
-  return cache[n] = 1;
-}
-
-template <int DT, int TT, bool DEFER = false>
-int launch_decompress_t(const Plan& pl, const fh::DecompressArgs& a, cudaStream_t stream) {
-  if (TT == 32 && !DEFER && pl.nblk >= fh::kDeferBlocks) return launch_decompress_t<DT, TT, TT == 32>(pl, a, stream);
-  int grid = 0;
-  int rc = grid_for(fh::decompress_kernel<DT, TT, DEFER>, pl.sm_total, pl.ntiles, &grid);
-  if (rc != FH_OK) return rc;
-  fh::DecompressArgs b = a;
-  b.team_stride = prime_at_most((uint64_t)grid * (fh::kThreads / TT));
-  if (launch_dependent(fh::decompress_kernel<DT, TT, DEFER>, grid, fh::kThreads, pl.sm_total, stream, pl, b) != cudaSuccess)
-    return FH_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return FH_OK;
-}
-
-// Planes of at most 128 groups: tiles of 256 / team planes restored in shared memory, one bulk store per tile.
-template <int DT>
-int launch_decompress_small(const Plan& pl0, const fh::DecompressArgs& a, cudaStream_t stream) {
-  Plan pl = pl0;
-  pl.ppt = fh::kThreads / pl.team;
-  if (pl.ppt > pl.P) pl.ppt = (uint32_t)pl.P;
-  pl.stage_bytes = (uint32_t)((pl.ppt * pl.plane_bytes + 127) & ~(uint64_t)127);
-  pl.ntiles = (uint32_t)((pl.P + pl.ppt - 1) / pl.ppt);
-  // two tile buffers, then per warp: scratch for a small plane's payload, or the general path's scratch
-  const uint32_t pay = (uint32_t)A16(pl.plane_bytes) + 16u;
-  if (pl.sal_stride < pay) pl.sal_stride = pay;
-  pl.sm_total = 2u * pl.stage_bytes + (uint32_t)fh::kWarps * pl.sal_stride;
-  if (pl.sm_total > kSmemLimit) return FH_ERR_UNSUPPORTED;
-  int grid = 0;
-  int rc = grid_for(fh::decompress_small<DT>, pl.sm_total, pl.ntiles, &grid);
-  if (rc != FH_OK) return rc;
-  if (launch_dependent(fh::decompress_small<DT>, grid, fh::kThreads, pl.sm_total, stream, pl, a) != cudaSuccess)
-    return FH_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return FH_OK;
-}
-
-template <int DT>
-int launch_decompress(const Plan& pl, const fh::DecompressArgs& a, cudaStream_t stream) {
-  if (pl.groups <= 128 && pl.P <= 0x7FFFFFFFull) return launch_decompress_small<DT>(pl, a, stream);
-  switch (pl.team) {
-    case 1: return launch_decompress_t<DT, 1>(pl, a, stream);
-    case 2: return launch_decompress_t<DT, 2>(pl, a, stream);
-    case 4: return launch_decompress_t<DT, 4>(pl, a, stream);
-    case 8: return launch_decompress_t<DT, 8>(pl, a, stream);
-    case 16: return launch_decompress_t<DT, 16>(pl, a, stream);
-    case 32: return launch_decompress_t<DT, 32>(pl, a, stream);
-  }
-  return FH_ERR_UNSUPPORTED;
+  const bool f32 = pl.dtype == FH_F32;
+  const int rc = !v.fast ? fh::launch_compress_generic(pl, a, stream)
+                 : v.cta ? (f32 ? fh::launch_compress_cta_f32(pl, v, a, stream) : fh::launch_compress_cta_bf16(pl, v, a, stream))
+                         : (f32 ? fh::launch_compress_warp_f32(pl, a, stream) : fh::launch_compress_warp_bf16(pl, a, stream));
+  if (rc == FH_OK) g_launches.fetch_add(1);
+  return rc;
 }
 
 int enqueue_compress(const fh_tensor_desc* desc, const fh_params* params, const void* d_src, void* d_dst,
@@ -648,8 +399,9 @@ int enqueue_compress(const fh_tensor_desc* desc, const fh_params* params, const 
     ca.chan = s->chan;
     ca.plane_nout = s->plane_nout;
     ca.inv_nhw = 1.0 / ((double)(pl.mode == fh::kModeTensor ? pl.P : pl.N) * (double)pl.HW);
-    rc = pl.dtype == FH_F32 ? launch_channel_passes<fh::kF32>(pl, ca, stream) : launch_channel_passes<fh::kBF16>(pl, ca, stream);
+    rc = fh::launch_channel_passes(pl, ca, stream);
     if (rc != FH_OK) return rc;
+    g_launches.fetch_add(3);
     a.chan_nout = reinterpret_cast<const unsigned long long*>(s->chan) + 3;
     a.plane_nout = s->plane_nout;
   }
@@ -672,8 +424,9 @@ int enqueue_decompress(const void* d_src, size_t src_bytes, const fh_tensor_desc
   a.dst = (uint8_t*)d_dst;
   a.d_status = d_status;
   a.sc = s->sc;
-  if (pl.dtype == FH_F32) return launch_decompress<fh::kF32>(pl, a, stream);
-  return launch_decompress<fh::kBF16>(pl, a, stream);
+  rc = fh::launch_decompress(pl, a, stream);
+  if (rc == FH_OK) g_launches.fetch_add(1);
+  return rc;
 }
 
 bool misaligned(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) != 0; }

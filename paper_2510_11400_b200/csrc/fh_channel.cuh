@@ -15,14 +15,6 @@
 
 namespace fh {
 
-struct ChanStat {
-  unsigned int lo_inv;       // ~key(minimum): atomicMax
-  unsigned int hi_key;       // key(maximum): atomicMax
-  unsigned long long Is, Iq;  // fixed-point moment sums (two's complement)
-  unsigned long long nout;    // three-sigma outliers of the channel
-};
-static_assert(sizeof(ChanStat) == 32, "ChanStat layout");
-
 // Order-preserving map float -> unsigned (finite values; -0.0 sorts below +0.0, and a distance from either is
 // the same number).
 __device__ __forceinline__ unsigned int float_key(float f) {
@@ -32,13 +24,6 @@ __device__ __forceinline__ unsigned int float_key(float f) {
 __device__ __forceinline__ float key_float(unsigned int k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
-
-struct ChannelArgs {
-  const uint8_t* src;
-  ChanStat* chan;        // C entries (one in the tensor-wide mode), zeroed before pass 0
-  uint32_t* plane_nout;  // P entries, written by pass 2
-  double inv_nhw;        // 1 / (N * HW); tensor-wide: 1 / (N * C * HW)
-};
 
 template <int DT>
 __device__ __forceinline__ void load_group_global(const uint8_t* plane, uint32_t g, uint32_t HW, float v[4]) {

@@ -18,31 +18,9 @@
 // The kernel's last CTA writes the header and the result words and returns the scratch to its idle state.
 #pragma once
 
-#include "fh_device.cuh"
+#include "fh_blocks.cuh"
 
 namespace fh {
-
-struct SalientInfo {
-  uint32_t nnz_s, n_dense, n_out_d, size;
-  uint32_t coded;  // bytes of the Huffman-coded section that replaces the dense blocks' code bytes; 0: plain codes
-};
-
-struct CompressArgs {
-  const uint8_t* src;
-  uint8_t* dst_base;
-  unsigned long long capacity;          // bytes available at dst_base (minus the offset below)
-  const unsigned long long* d_off_in;   // optional: byte offset of the container in dst_base
-  unsigned long long* d_off_out;        // optional: offset for the next container
-  unsigned long long* out2;             // optional: {total bytes, status}
-  Scratch* sc;
-  Scan scan;                            // placement of overflow parts (unused with salient_mode OFF)
-  uint32_t* defer_next;                 // one word per tile: links the tiles a CTA has put off (see BlockCtl)
-  uint32_t parity;                      // which of the two ticket counters this call uses
-  uint32_t early_ticket;                // 1: tiles may be requested before the previous kernel on the stream has completed
-  // channel-wide three-sigma mode: per-channel outlier counts and per-plane counts from the statistics passes
-  const unsigned long long* chan_nout;  // stride: 4 words (see ChanStat)
-  const uint32_t* plane_nout;
-};
 
 // Class and outlier count of plane gp when mu and sigma are taken per channel over the batch (the class is
 // the channel's) or over the whole tensor (the class follows from the plane's own count).
@@ -65,18 +43,6 @@ __device__ __forceinline__ void report_error(const CompressArgs& a, uint32_t cod
   *cta_dirty() = 1u;
   atomicMax(&a.sc->status, (unsigned long long)code);
 }
-
-// Where the bytes of a salient / raw payload go: offsets below npay land in the plane's slot, the
-// rest in its overflow part.  Offsets and npay are multiples of the access size.
-struct SplitOut {
-  uint8_t* slot;
-  uint8_t* ovf;
-  uint32_t npay;
-  __device__ __forceinline__ uint8_t* at(uint32_t o) const { return o < npay ? slot + o : ovf + (o - npay); }
-  __device__ __forceinline__ void st32(uint32_t o, uint32_t v) const { *reinterpret_cast<uint32_t*>(at(o)) = v; }
-  __device__ __forceinline__ void st16(uint32_t o, uint32_t v) const { *reinterpret_cast<uint16_t*>(at(o)) = (uint16_t)v; }
-  __device__ __forceinline__ void st8(uint32_t o, uint32_t v) const { *at(o) = (uint8_t)v; }
-};
 
 // One 8x8 block in the registers of a warp: lane l holds the elements (l >> 3, l & 7) and
 // ((l >> 3) + 4, l & 7) of the block, i.e. raster positions l and l + 32.  Positions outside the
@@ -130,242 +96,8 @@ __device__ __forceinline__ void block_codes(const BlockRegs& r, float inv2e, uin
   m1 = __ballot_sync(full, v1);
 }
 
-// Block-wise path, measuring part (Section 4.4.1): one pass over the plane's 8x8 blocks, a warp per
-// block.  The non-zero mask of a block is two ballots; its pooled density against tau says dense or
-// sparse; a sparse block adds its row counts to the CSR row counters, a dense block is coded once to
-// count its verbatim elements.  The team is a whole warp or a whole CTA.  Leaves in shared scratch:
-// rowp[0..H] = CSR row pointers, blk_a[b] = 1 for dense blocks, blk_b[b] = rank of block b among the
-// dense blocks, blk_c[b] = index of the block's first verbatim value.
-template <int DT>
-__device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
-  uint32_t* rowp = sal;
-  uint32_t* blk_a = sal + pl.H + 1;
-  uint32_t* blk_b = blk_a + pl.nblk;
-  uint32_t* blk_c = blk_b + pl.nblk;
-  const int H = pl.H, W = pl.W;
-  const uint32_t nblk = pl.nblk, nbx = pl.nbx;
-  const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane32 = threadIdx.x & 31u;
-  const float inv2e = __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps));
-  for (uint32_t y = t.lane; y <= (uint32_t)H; y += t.size) rowp[y] = 0;
-  team_sync(t);
-  for (uint32_t b = wid; b < nblk; b += nw) {
-    const uint32_t by = b / nbx, bx = b - by * nbx;
-    const BlockRegs r = block_load<DT>(plane, H, W, (int)by, (int)bx, lane32);
-    const uint32_t z0 = __ballot_sync(0xFFFFFFFFu, r.x0 != 0.0f), z1 = __ballot_sync(0xFFFFFFFFu, r.x1 != 0.0f);
-    const uint32_t nnz = __popc(z0) + __popc(z1);
-    const bool dense = (uint64_t)nnz * pl.tau_den >= (uint64_t)pl.tau_num * 64u;
-    uint32_t n_out = 0;
-    if (dense) {
-      uint32_t c0, c1, m0, m1;
-      block_codes(r, inv2e, lane32, c0, c1, m0, m1);
-      n_out = __popc(m0) + __popc(m1);
-    } else if (lane32 < 8u) {  // lane r: non-zeros of row r of the block
-      const uint32_t cnt = __popc(((lane32 < 4u ? z0 : z1) >> ((lane32 & 3u) * 8u)) & 0xFFu);
-      if (cnt) atomicAdd(&rowp[by * 8u + lane32], cnt);
-    }
-    if (lane32 == 0) {
-      blk_a[b] = dense;
-      blk_b[b] = dense;
-      blk_c[b] = n_out;
-    }
-  }
-  team_sync(t);
-  SalientInfo info;
-  info.n_dense = team_excl_scan(t, blk_b, nblk);
-  info.nnz_s = team_excl_scan(t, rowp, (uint32_t)H + 1u);
-  info.n_out_d = team_excl_scan(t, blk_c, nblk);
-  info.coded = 0;
-  if (pl.entropy && info.n_dense) {
-    // Huffman stage (Section 4.4.1): histogram of the plane's code bytes, the code, the size of every chunk
-    uint32_t* blk_d = blk_c + nblk;   // bytes of a dense block's chunk
-    uint32_t* blk_e = blk_d + nblk;   // ... and where it starts
-    HufEncode* h = reinterpret_cast<HufEncode*>(blk_e + nblk);
-    for (uint32_t i = t.lane; i < 256u; i += t.size) h->hist[i] = 0;
-    team_sync(t);
-    for (uint32_t b = wid; b < nblk; b += nw) {
-      if (!blk_a[b]) continue;
-      const uint32_t by = b / nbx, bx = b - by * nbx;
-      const BlockRegs r = block_load<DT>(plane, H, W, (int)by, (int)bx, lane32);
-      uint32_t c0, c1, m0, m1;
-      block_codes(r, inv2e, lane32, c0, c1, m0, m1);
-      atomicAdd(&h->hist[c0], 1u);
-      atomicAdd(&h->hist[c1], 1u);
-    }
-    team_sync(t);
-    if (t.lane == 0) huffman_build(h);
-    team_sync(t);
-    if (h->maxlen <= kHufMaxLen) {
-      for (uint32_t b = wid; b < nblk; b += nw) {
-        uint32_t bits = 0;
-        if (blk_a[b]) {
-          const uint32_t by = b / nbx, bx = b - by * nbx;
-          const BlockRegs r = block_load<DT>(plane, H, W, (int)by, (int)bx, lane32);
-          uint32_t c0, c1, m0, m1;
-          block_codes(r, inv2e, lane32, c0, c1, m0, m1);
-          bits = (uint32_t)h->len[c0] + (uint32_t)h->len[c1];
-          asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(bits) : "r"(0xFFFFFFFFu));
-        }
-        if (lane32 == 0) blk_d[b] = blk_e[b] = (bits + 7u) >> 3;
-      }
-      team_sync(t);
-      const uint32_t chunks = team_excl_scan(t, blk_e, nblk);
-      const uint32_t section = a4(4u + a4(h->nlens) + a4(info.n_dense) + chunks);
-      if (section < 64u * info.n_dense) info.coded = section;
-    }
-  }
-  const uint32_t e = (uint32_t)pl.esize;
-  info.size = 16u + 4u * pl.nbm + 4u * ((uint32_t)H + 1u) + a4(2u * info.nnz_s) + a4(e * info.nnz_s) +
-              (info.coded ? info.coded : 64u * info.n_dense) + a4(e * info.n_out_d);
-  return info;
-}
-
-// Block-wise path, writing part; `sal` holds what salient_measure left.
-template <int DT>
-__device__ __noinline__ void salient_write(const Team& t, const Plan& pl, const uint8_t* plane, const SalientInfo& info,
-                                           const uint32_t* sal, const SplitOut& out) {
-  const uint32_t* rowp = sal;
-  const uint32_t* blk_a = sal + pl.H + 1;
-  const uint32_t* blk_b = blk_a + pl.nblk;
-  const uint32_t* blk_c = blk_b + pl.nblk;
-  const int H = pl.H, W = pl.W;
-  const uint32_t nblk = pl.nblk, nbx = pl.nbx, e = (uint32_t)pl.esize;
-  const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane32 = threadIdx.x & 31u;
-  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * pl.nbm, o_col = o_rp + 4u * ((uint32_t)H + 1u);
-  const uint32_t o_val = o_col + a4(2u * info.nnz_s), o_codes = o_val + a4(e * info.nnz_s);
-  const uint32_t o_outl = o_codes + (info.coded ? info.coded : 64u * info.n_dense);
-  if (t.lane == 0) {
-    out.st32(0, info.nnz_s);
-    out.st32(4, info.n_dense);
-    out.st32(8, info.n_out_d);
-    out.st32(12, info.coded);
-    // pads the section writers leave: col (2 bytes), val / verbatim values (bf16: 2 bytes)
-    if (info.nnz_s & 1u) out.st16(o_col + 2u * info.nnz_s, 0);
-    if (DT == kBF16 && (info.nnz_s & 1u)) out.st16(o_val + 2u * info.nnz_s, 0);
-    if (DT == kBF16 && (info.n_out_d & 1u)) out.st16(o_outl + 2u * info.n_out_d, 0);
-  }
-  // zero padding up to the end of the slot / of the 16-byte padded overflow part
-  const uint32_t end = max(pl.npay, a16(info.size));
-  for (uint32_t o = info.size + 4u * t.lane; o < end; o += 4u * t.size) out.st32(o, 0);
-  for (uint32_t w = t.lane; w < pl.nbm; w += t.size) {
-    uint32_t word = 0;
-    const uint32_t hi = min(nblk, w * 32u + 32u);
-    for (uint32_t b = w * 32u; b < hi; ++b) word |= blk_a[b] << (b & 31u);
-    out.st32(o_bm + 4u * w, word);
-  }
-  for (uint32_t y = t.lane; y <= (uint32_t)H; y += t.size) out.st32(o_rp + 4u * y, rowp[y]);
-  // CSR entries: one warp per row, columns in chunks of 32, positions by ballot
-  if (info.nnz_s) {
-    for (int y = (int)wid; y < H; y += (int)nw) {
-      uint32_t o = rowp[y];
-      if (o == rowp[y + 1]) continue;
-      const uint32_t* brow = blk_a + (uint32_t)(y >> 3) * nbx;
-      for (int x0 = 0; x0 < W; x0 += 32) {
-        const int x = x0 + (int)lane32;
-        const uint32_t idx = (uint32_t)y * W + (uint32_t)x;
-        const bool take = x < W && load_elem<DT>(plane, idx) != 0.0f && !brow[x >> 3];
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, take);
-        if (take) {
-          const uint32_t pos = o + __popc(m & ((1u << lane32) - 1u));
-          out.st16(o_col + 2u * pos, (uint32_t)x);
-          if (DT == kF32) out.st32(o_val + 4u * pos, reinterpret_cast<const uint32_t*>(plane)[idx]);
-          else out.st16(o_val + 2u * pos, reinterpret_cast<const uint16_t*>(plane)[idx]);
-        }
-        o += __popc(m);
-      }
-    }
-  }
-  // dense blocks: 64 code bytes each (or their Huffman-coded chunk), verbatim values in raster order
-  const float inv2e = __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps));
-  const uint32_t lt = (1u << lane32) - 1u;
-  const uint32_t* blk_d = blk_c + nblk;
-  const uint32_t* blk_e = blk_d + nblk;
-  HufEncode* h = reinterpret_cast<HufEncode*>(const_cast<uint32_t*>(blk_e + nblk));  // (only looked at when info.coded)
-  uint32_t o_chunks = 0;
-  if (info.coded) {  // the section's head: code lengths, then the bytes of every chunk; pads are zero
-    const uint32_t nl = h->nlens, o_cb = o_codes + 4u + a4(nl);
-    o_chunks = o_cb + a4(info.n_dense);
-    if (t.lane == 0) {
-      out.st8(o_codes, h->len[0]);
-      out.st8(o_codes + 1u, h->smin);
-      out.st8(o_codes + 2u, h->smax);
-      out.st8(o_codes + 3u, 0);
-      for (uint32_t o = o_codes + 4u + nl; o < o_cb; ++o) out.st8(o, 0);
-      for (uint32_t o = o_cb + info.n_dense; o < o_chunks; ++o) out.st8(o, 0);
-      uint32_t last_end = 0;  // end of the chunks: the last dense block's start + bytes
-      for (uint32_t b = nblk; b-- > 0;)
-        if (blk_a[b]) {
-          last_end = blk_e[b] + blk_d[b];
-          break;
-        }
-      for (uint32_t o = o_chunks + last_end; o < o_codes + info.coded; ++o) out.st8(o, 0);
-    }
-    for (uint32_t i = t.lane; i < nl; i += t.size) out.st8(o_codes + 4u + i, h->len[h->smin + i]);
-    for (uint32_t b = t.lane; b < nblk; b += t.size)
-      if (blk_a[b]) out.st8(o_cb + blk_b[b], blk_d[b]);
-  }
-  for (uint32_t b = wid; b < nblk; b += nw) {
-    if (!blk_a[b]) continue;
-    const uint32_t by = b / nbx, bx = b - by * nbx;
-    const BlockRegs r = block_load<DT>(plane, H, W, (int)by, (int)bx, lane32);
-    uint32_t c0, c1, m0, m1;
-    block_codes(r, inv2e, lane32, c0, c1, m0, m1);
-    const uint32_t oc = o_codes + 64u * blk_b[b], oo = o_outl + e * blk_c[b];
-    if ((m0 >> lane32) & 1u) {
-      const uint32_t rank = __popc(m0 & lt);
-      if (DT == kF32) out.st32(oo + 4u * rank, reinterpret_cast<const uint32_t*>(plane)[r.idx0]);
-      else out.st16(oo + 2u * rank, reinterpret_cast<const uint16_t*>(plane)[r.idx0]);
-    }
-    if ((m1 >> lane32) & 1u) {
-      const uint32_t rank = __popc(m0) + __popc(m1 & lt), idx1 = r.idx0 + 4u * (uint32_t)W;
-      if (DT == kF32) out.st32(oo + 4u * rank, reinterpret_cast<const uint32_t*>(plane)[idx1]);
-      else out.st16(oo + 2u * rank, reinterpret_cast<const uint16_t*>(plane)[idx1]);
-    }
-    if (info.coded) {
-      // the chunk's bits are assembled in shared memory (a code goes in most significant bit first, the words
-      // hold the stream big-endian) and leave byte by byte
-      uint32_t* stg = h->stage[wid];
-      for (uint32_t i = lane32; i < kHufStageWords; i += 32u) stg[i] = 0;
-      __syncwarp();
-      const uint32_t l0 = h->len[c0], l1 = h->len[c1];
-      uint32_t i0 = l0, i1 = l1;  // inclusive prefix sums of the lengths, raster positions l and l + 32
-      for (uint32_t o = 1; o < 32u; o <<= 1) {
-        const uint32_t u0 = __shfl_up_sync(0xFFFFFFFFu, i0, o), u1 = __shfl_up_sync(0xFFFFFFFFu, i1, o);
-        if (lane32 >= o) {
-          i0 += u0;
-          i1 += u1;
-        }
-      }
-      const uint32_t first_half = __shfl_sync(0xFFFFFFFFu, i0, 31);
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const uint32_t len = half ? l1 : l0, at = half ? first_half + i1 - l1 : i0 - l0, cv = h->code[half ? c1 : c0];
-        const uint32_t wi = at >> 5;
-        const int shift = 32 - (int)(at & 31u) - (int)len;
-        if (shift >= 0) {
-          atomicOr(&stg[wi], cv << shift);
-        } else {
-          atomicOr(&stg[wi], cv >> (-shift));
-          atomicOr(&stg[wi + 1u], cv << (32 + shift));
-        }
-      }
-      __syncwarp();
-      for (uint32_t j = lane32; j < blk_d[b]; j += 32u) out.st8(o_chunks + blk_e[b] + j, (stg[j >> 2] >> (24u - 8u * (j & 3u))) & 0xFFu);
-      __syncwarp();
-      continue;
-    }
-    uint32_t w0 = c0 | (__shfl_down_sync(0xFFFFFFFFu, c0, 1) << 8);
-    w0 |= __shfl_down_sync(0xFFFFFFFFu, w0, 2) << 16;
-    uint32_t w1 = c1 | (__shfl_down_sync(0xFFFFFFFFu, c1, 1) << 8);
-    w1 |= __shfl_down_sync(0xFFFFFFFFu, w1, 2) << 16;
-    if ((lane32 & 3u) == 0u) {
-      out.st32(oc + lane32, w0);
-      out.st32(oc + 32u + lane32, w1);
-    }
-  }
-}
-
 // Raw plane: verbatim copy through the slot into the overflow part, zero padded.
-__device__ __noinline__ void raw_write(const Team& t, const Plan& pl, const uint8_t* plane, const SplitOut& out) {
+static __device__ __noinline__ void raw_write(const Team& t, const Plan& pl, const uint8_t* plane, const SplitOut& out) {
   const uint32_t n = (uint32_t)pl.plane_bytes, end = max(pl.npay, a16(n));
   for (uint32_t o = 2u * t.lane; o < end; o += 2u * t.size)
     out.st16(o, o < n ? (uint32_t)*reinterpret_cast<const uint16_t*>(plane + o) : 0u);
@@ -377,7 +109,7 @@ __device__ __noinline__ void raw_write(const Team& t, const Plan& pl, const uint
 // results are those of salient_measure / salient_write.
 // -------------------------------------------------------------------------------------------------
 constexpr uint32_t kSmallBlocks = 4;
-__device__ __forceinline__ bool is_small_plane(const Plan& pl) { return pl.nblk <= kSmallBlocks && pl.H < 32; }
+__device__ __forceinline__ bool is_small_plane(const Plan& pl) { return pl.nblk <= kSmallBlocks && pl.H < 32 && !pl.entropy; }
 
 struct SmallBlocks {
   uint32_t z0[kSmallBlocks], z1[kSmallBlocks];  // non-zero masks of the block's two halves (ballots)
@@ -571,7 +303,7 @@ __device__ __forceinline__ void count_blockwise(const CompressArgs& a, uint32_t 
 // salient_measure) with its overflow part `at` units into the overflow region, and its table entry.
 template <int DT>
 __device__ __forceinline__ void write_blockwise(const Team& t, const Plan& pl, const Dest& d, uint64_t gp,
-                                                const uint8_t* plane, const SalientInfo& info, const uint32_t* sal,
+                                                const uint8_t* plane, const SalientInfo& info, uint32_t* sal,
                                                 uint32_t n_out, uint32_t at) {
   bool raw;
   const uint32_t my_units = plane_units(pl, info, raw);
@@ -1230,7 +962,7 @@ __device__ __noinline__ void warp_tile_measure(BlockCtl* c, const uint8_t* tbuf,
 }
 
 // Phase 1, the last of a tile's eight warps (one thread): the tile's sums are complete.
-__device__ __noinline__ void warp_tile_publish(BlockCtl* c, uint32_t s, uint32_t tile) {
+static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, uint32_t s, uint32_t tile) {
   __threadfence_block();  // the other warps' sums after their arrivals
   const uint32_t U = c->U[s], C = c->C[s];
   c->U[s] = 0;

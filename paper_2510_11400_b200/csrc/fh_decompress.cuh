@@ -15,16 +15,6 @@
 
 namespace fh {
 
-struct DecompressArgs {
-  const uint8_t* src_base;
-  unsigned long long src_bytes;
-  const unsigned long long* d_off_in;  // optional: byte offset of the container in src_base
-  uint8_t* dst;
-  unsigned long long* d_status;        // optional
-  Scratch* sc;
-  unsigned long long team_stride;      // a prime, at most the number of teams of the grid (see the kernel)
-};
-
 // Reads of a salient / raw payload: offsets below npay come from the plane's slot, the rest from its
 // overflow part.
 struct SplitIn {

@@ -46,6 +46,7 @@ struct Plan {
   uint64_t slots_off;    // 64 + 16 P
   uint64_t ovf_off;      // slots_off + P * npay: start of the overflow region
   uint32_t nbx, nby, nblk, nbm;  // 8x8 blocks per row / column / plane, bitmap words
+  uint32_t qs, nsr;              // block-wise path: log2 of the blocks side by side in a step of four, rows of steps
   // tiling
   uint32_t ppt;          // planes per tile
   uint32_t ntiles;
@@ -55,7 +56,6 @@ struct Plan {
   // shared-memory layout (byte offsets into dynamic shared memory)
   uint32_t sm_tile, sm_out, sm_rec, sm_total;
   // block-wise path (outlier-rich planes): measuring scratch of one unit (a warp, or the whole CTA)
-  uint32_t sal_words;       // words of measuring scratch per plane: H + 1 + 3 * nblk
   uint32_t sm_sal;          // byte offset of the first measuring area in dynamic shared memory
   uint32_t sal_stride;      // bytes between the areas of consecutive units
 };
@@ -587,77 +587,106 @@ constexpr uint32_t kHufStageWords = 48;  // a chunk has at most 64 * 24 / 8 = 19
 // Encoder scratch of one unit (shared memory).
 struct HufEncode {
   uint32_t hist[256];
-  uint32_t code[256];
-  uint32_t w[512];        // node weights: 0..255 leaves by symbol, 256.. merged nodes
-  uint16_t parent[512];
-  uint16_t leaf[256];     // symbols that occur, sorted by (weight, symbol)
-  uint8_t len[256];
+  uint32_t code[256];                // by symbol: length << 24 | code value; 0: does not occur
+  uint32_t key[256 + 2];             // symbols that occur, weight << 8 | symbol, sorted; two sentinels behind them
+  uint32_t mw[256];                  // weights of the merged nodes, in order of creation
+  uint16_t lpar[256], mpar[256];     // parent (a merged node) of a sorted leaf, of a merged node
+  uint32_t cnt[32], first[32];       // symbols of a length, then running rank; a length's first code value
   uint32_t smin, smax, maxlen, nlens;
-  uint32_t stage[kMaxWarps][kHufStageWords];  // a chunk's bits while a warp assembles them
+  uint32_t stage[kMaxWarps][4 * kHufStageWords];  // chunks' bits while a warp assembles four of them
 };
 
-// One thread: code lengths and canonical codes from h->hist.
-__device__ __noinline__ void huffman_build(HufEncode* h) {
+// A whole warp: code lengths and canonical codes from h->hist.  Symbols are ranked by comparison with all others (a few
+// dozen occur); one lane merges the two queues with the heads of both in registers, the next elements already on
+// their way from shared memory; depths are walks up the tree, a lane per leaf; code values are first-of-length plus
+// rank among the length's symbols.  About 3 us for 60 symbols; one thread doing all of it took 220 us.
+static __device__ __noinline__ void huffman_build(HufEncode* h) {
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, lt = (1u << lane) - 1u;
   uint32_t n = 0;
-  for (uint32_t sym = 0; sym < 256u; ++sym) {
-    h->len[sym] = 0;
+  for (uint32_t i = 0; i < 8u; ++i) {
+    const uint32_t sym = i * 32u + lane, w = h->hist[sym], m = __ballot_sync(full, w != 0u);
+    if (w) h->mw[n + __popc(m & lt)] = w << 8 | sym;  // (weights stay below 2^24; mw serves as a buffer here)
+    n += __popc(m);
     h->code[sym] = 0;
-    h->w[sym] = h->hist[sym];
-    if (h->hist[sym]) h->leaf[n++] = (uint16_t)sym;
   }
-  if (n == 1) h->len[h->leaf[0]] = 1;
-  if (n > 1) {
-    for (uint32_t i = 1; i < n; ++i) {  // insertion sort: equal weights stay in symbol order
-      const uint16_t v = h->leaf[i];
-      uint32_t j = i;
-      while (j > 0 && h->hist[h->leaf[j - 1]] > h->hist[v]) {
-        h->leaf[j] = h->leaf[j - 1];
-        --j;
-      }
-      h->leaf[j] = v;
-    }
-    uint32_t li = 0, mi = 256, mn = 256;  // head of the leaf queue, head and end of the queue of merged nodes
-    while ((n - li) + (mn - mi) > 1u) {
-      uint32_t pick[2];
+  h->cnt[lane] = 0;
+  __syncwarp();
+  for (uint32_t i = lane; i < n; i += 32u) {
+    const uint32_t k = h->mw[i];
+    uint32_t rank = 0;
+#pragma unroll 4
+    for (uint32_t j = 0; j < n; ++j) rank += h->mw[j] < k;
+    h->key[rank] = k;
+  }
+  if (lane < 2u) h->key[n + lane] = 0xFFFFFFFFu;
+  __syncwarp();
+  if (lane == 0 && n > 1u) {
+    constexpr uint32_t kNone = 0xFFFFFFu;
+    uint32_t li = 0, mi = 0, a0 = h->key[0] >> 8, a1 = h->key[1] >> 8, b0 = kNone, b1 = kNone;
+    for (uint32_t mn = 0; mn + 1u < n; ++mn) {
+      uint32_t sum = 0;
+#pragma unroll
       for (int k = 0; k < 2; ++k) {
-        bool take_leaf;
-        if (li >= n) take_leaf = false;
-        else if (mi >= mn) take_leaf = true;
-        else take_leaf = h->w[h->leaf[li]] <= h->w[mi];  // equal weights: the leaf has the smaller id
-        pick[k] = take_leaf ? h->leaf[li++] : mi++;
+        if (a0 <= b0) {  // equal weights: the leaf has the smaller id
+          sum += a0;
+          h->lpar[li] = (uint16_t)mn;
+          ++li;
+          a0 = a1;
+          a1 = h->key[li + 1u] >> 8;
+        } else {
+          sum += b0;
+          h->mpar[mi] = (uint16_t)mn;
+          ++mi;
+          b0 = b1;
+          b1 = mi + 1u < mn ? h->mw[mi + 1u] : kNone;
+        }
       }
-      h->w[mn] = h->w[pick[0]] + h->w[pick[1]];
-      h->parent[pick[0]] = h->parent[pick[1]] = (uint16_t)mn;
-      ++mn;
-    }
-    const uint32_t root = mn - 1u;
-    for (uint32_t i = 0; i < n; ++i) {
-      uint32_t d = 0;
-      for (uint32_t v = h->leaf[i]; v != root; v = h->parent[v]) ++d;
-      h->len[h->leaf[i]] = (uint8_t)min(d, 255u);
+      h->mw[mn] = sum;
+      if (mi == mn) b0 = sum;
+      else if (mi + 1u == mn) b1 = sum;
     }
   }
-  uint32_t next = 0, prev = 0, maxlen = 0, smin = 1, smax = 1;
-  bool any = false;
-  for (uint32_t l = 1; l <= 32u; ++l)
-    for (uint32_t sym = 0; sym < 256u; ++sym)
-      if (h->len[sym] == l) {
-        next <<= (l - prev);
-        prev = l;
-        h->code[sym] = next++;
-      }
-  for (uint32_t sym = 0; sym < 256u; ++sym) {
-    maxlen = max(maxlen, (uint32_t)h->len[sym]);
-    if (sym && h->len[sym]) {
-      if (!any) smin = sym;
-      smax = sym;
-      any = true;
+  __syncwarp();
+  uint32_t deepest = 0;
+  for (uint32_t i = lane; i < n; i += 32u) {
+    uint32_t d = 1;
+    if (n > 1u)
+      for (uint32_t v = h->lpar[i]; v + 2u != n; v = h->mpar[v]) ++d;  // (the root is merged node n - 2)
+    d = min(d, 31u);
+    h->code[h->key[i] & 255u] = d << 24;
+    atomicAdd(&h->cnt[d], 1u);
+    deepest = max(deepest, d);
+  }
+  asm volatile("redux.sync.max.u32 %0, %0, %1;" : "+r"(deepest) : "r"(full));
+  __syncwarp();
+  uint32_t first = 0;
+  for (uint32_t k = 1; k < lane; ++k) first += h->cnt[k] << (lane - k);
+  __syncwarp();
+  h->first[lane] = first;
+  h->cnt[lane] = 0;
+  __syncwarp();
+  uint32_t smin = 256, smax = 0;
+  for (uint32_t i = 0; i < 8u; ++i) {
+    const uint32_t sym = i * 32u + lane, len = h->code[sym] >> 24;
+    const uint32_t same = __match_any_sync(full, len), used = h->cnt[len];
+    __syncwarp();
+    if (len) h->code[sym] = len << 24 | ((h->first[len] + used + __popc(same & lt)) & 0xFFFFFFu);
+    if ((same & lt) == 0u) h->cnt[len] = used + __popc(same);
+    __syncwarp();
+    const uint32_t m = __ballot_sync(full, len != 0u && sym != 0u);
+    if (m) {
+      smin = min(smin, i * 32u + (uint32_t)__ffs((int)m) - 1u);
+      smax = i * 32u + 31u - (uint32_t)__clz((int)m);
     }
   }
-  h->smin = smin;
-  h->smax = smax;
-  h->maxlen = maxlen;
-  h->nlens = smax - smin + 1u;
+  if (smin > 255u) smin = smax = 1u;
+  if (lane == 0) {
+    h->smin = smin;
+    h->smax = smax;
+    h->maxlen = deepest;
+    h->nlens = smax - smin + 1u;
+  }
+  __syncwarp();
 }
 
 // Decoder tables of one unit (shared memory), from the lengths stored in a section.
@@ -670,7 +699,7 @@ struct HufDecode {
   uint32_t ok;
 };
 // One thread: tables from t->len; t->ok = 0 unless the lengths form a complete prefix code (or a single code of any length).
-__device__ __noinline__ void huffman_tables(HufDecode* t) {
+static __device__ __noinline__ void huffman_tables(HufDecode* t) {
   for (uint32_t l = 0; l <= kHufMaxLen; ++l) t->count[l] = 0;
   unsigned long long kraft = 0;  // in units of 2^-32
   uint32_t nsym = 0;
@@ -742,7 +771,7 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
 }
 
 // A whole warp: sum of U over the tiles before t.  False when a wait ran out.
-__device__ __noinline__ bool scan_prefix(const Scan& s, uint32_t t, uint32_t& prefix) {
+static __device__ __noinline__ bool scan_prefix(const Scan& s, uint32_t t, uint32_t& prefix) {
   const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu;
   const uint32_t g = t >> 5, within = t & 31u;
   // tiles of the own group before t
@@ -804,5 +833,50 @@ __device__ __noinline__ bool scan_prefix(const Scan& s, uint32_t t, uint32_t& pr
   prefix = (uint32_t)(gsum + acc);
   return true;
 }
+
+// ------------------------------------------------------------------------------------------------
+// Arguments of the kernels beside the plan
+// ------------------------------------------------------------------------------------------------
+struct CompressArgs {
+  const uint8_t* src;
+  uint8_t* dst_base;
+  unsigned long long capacity;          // bytes available at dst_base (minus the offset below)
+  const unsigned long long* d_off_in;   // optional: byte offset of the container in dst_base
+  unsigned long long* d_off_out;        // optional: offset for the next container
+  unsigned long long* out2;             // optional: {total bytes, status}
+  Scratch* sc;
+  Scan scan;                            // placement of overflow parts (unused with salient_mode OFF)
+  uint32_t* defer_next;                 // one word per tile: links the tiles a CTA has put off (see BlockCtl)
+  uint32_t parity;                      // which of the two ticket counters this call uses
+  uint32_t early_ticket;                // 1: tiles may be requested before the previous kernel on the stream has completed
+  // channel-wide three-sigma mode: per-channel outlier counts and per-plane counts from the statistics passes
+  const unsigned long long* chan_nout;  // stride: 4 words (see ChanStat)
+  const uint32_t* plane_nout;
+};
+
+struct DecompressArgs {
+  const uint8_t* src_base;
+  unsigned long long src_bytes;
+  const unsigned long long* d_off_in;  // optional: byte offset of the container in src_base
+  uint8_t* dst;
+  unsigned long long* d_status;        // optional
+  Scratch* sc;
+  unsigned long long team_stride;      // a prime, at most the number of teams of the grid (see the kernel)
+};
+
+struct ChanStat {
+  unsigned int lo_inv;       // ~key(minimum): atomicMax
+  unsigned int hi_key;       // key(maximum): atomicMax
+  unsigned long long Is, Iq;  // fixed-point moment sums (two's complement)
+  unsigned long long nout;    // three-sigma outliers of the channel
+};
+static_assert(sizeof(ChanStat) == 32, "ChanStat layout");
+
+struct ChannelArgs {
+  const uint8_t* src;
+  ChanStat* chan;        // C entries (one in the tensor-wide mode), zeroed before pass 0
+  uint32_t* plane_nout;  // P entries, written by pass 2
+  double inv_nhw;        // 1 / (N * HW); tensor-wide: 1 / (N * C * HW)
+};
 
 }  // namespace fh
