@@ -25,6 +25,24 @@ int sm_count() {
   return count[dev];
 }
 
+
+// Largest prime <= n (n >= 2), or 1.
+uint64_t prime_at_most(uint64_t n) {
+  static std::map<uint64_t, uint64_t> cache;  // guarded by the library's mutex
+  auto it = cache.find(n);
+  if (it != cache.end()) return it->second;
+  for (uint64_t c = n; c >= 2; --c) {
+    bool prime = true;
+    for (uint64_t f = 2; f * f <= c; ++f)
+      if (c % f == 0) {
+        prime = false;
+        break;
+      }
+    if (prime) return cache[n] = c;
+  }
+  return cache[n] = 1;
+}
+
 }  // namespace fh
 
 namespace {
@@ -70,14 +88,8 @@ uint32_t pow2_floor(uint32_t x) {
   return r;
 }
 
-uint32_t pow2_ceil(uint32_t x) {
-  uint32_t r = 1;
-  while (r < x) r *= 2;
-  return r;
-}
-
 // Tiling and shared-memory layout.  `compress` selects the compress kernels' layout; the decompress
-// kernel only needs the block-wise scratch.
+// kernels' plan is completed where they are launched.
 int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* out, Variant* var) {
   Plan pl;
   std::memset(&pl, 0, sizeof(pl));
@@ -121,10 +133,9 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   pl.qs = pl.nbx >= 3 ? 2u : pl.nbx - 1u;
   pl.nsr = (pl.nby + (4u >> pl.qs) - 1u) / (4u >> pl.qs);
   // its measuring scratch: row pointers, two sums per step row, the bitmap; with the Huffman stage one more sum and the
-  // encoder's tables.  Decompress: two words per block and the decoder's tables.
-  const size_t sal_words = compress ? (size_t)pl.H + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
-                                          (pl.entropy ? (size_t)pl.nsr + 1 + sizeof(fh::HufEncode) / 4 : 0)
-                                    : 2 * (size_t)pl.nblk + sizeof(fh::HufDecode) / 4 + 4;
+  // encoder's tables
+  const size_t sal_words = (size_t)pl.H + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
+                           (pl.entropy ? (size_t)pl.nsr + 1 + sizeof(fh::HufEncode) / 4 : 0);
   const uint32_t sal_bytes = (uint32_t)A16(4 * sal_words + 16);  // one measuring area of the block-wise path
   const bool blockwise = compress && pl.mode != FH_SALIENT_OFF;
 
@@ -136,8 +147,7 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   if (compress && rounding_ok && (pl.groups <= 256 || whole16)) {
     v.fast = true;
     if (pl.groups <= 256) {
-      uint32_t t = pow2_ceil((pl.groups + 7) / 8);
-      pl.team = t > 32 ? 32 : t;
+      pl.team = fh::team_of_groups(pl.groups);
       v.G = 8;  // the warp-team kernels keep eight groups per thread
       pl.ppt = fh::kThreads / pl.team;
     } else {
@@ -179,17 +189,22 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     }
   }
   if (!compress) {
-    // decompress: sub-warp teams, planes assigned round-robin (ntiles only bounds the grid)
-    uint32_t t = pow2_ceil((pl.groups + 7) / 8);
-    pl.team = t > 32 ? 32 : t;
-    const uint32_t nteams = fh::kThreads / pl.team;
-    pl.sal_stride = sal_bytes;
-    pl.sm_total = nteams * sal_bytes + 16;
+    // Units of the block-wise path: a warp for planes of up to a lane per block, the CTA otherwise.  Scratch of a unit:
+    // the bitmap and its prefix sums, a word per warp, the blocks by rank and, since planes may be Huffman-coded (the
+    // host cannot know), chunk offsets and tables.
+    pl.team = pl.nblk <= 32 ? 32u : (uint32_t)fh::kThreads;
+    const uint32_t units = pl.team == 32u ? (uint32_t)fh::kWarps : 1u;
+    const size_t base = A16(4 * (2 * (size_t)pl.nbm + 1 + fh::kMaxWarps + pl.nblk + 1) + sizeof(fh::HufDecode) + 2 * (size_t)pl.nblk);
+    // ... and a payload: as much as leaves room for four CTAs on an SM (a payload is shorter than its plane; one that
+    // does not fit is read where it lies)
+    size_t room = 48 * 1024 / units;
+    room = room > base ? room - base : 0;
+    pl.pay_bytes = (uint32_t)(A16(pl.plane_bytes) <= room ? A16(pl.plane_bytes) : room & ~(size_t)15);
+    pl.sal_stride = (uint32_t)base + pl.pay_bytes;
+    pl.sm_total = units * pl.sal_stride;
     if (pl.sm_total > kSmemLimit) return FH_ERR_UNSUPPORTED;
-    pl.ppt = nteams;
     {
-      const uint64_t chunks = (pl.groups + 8 * pl.team - 1) / (8 * pl.team);
-      const uint64_t ctas = (pl.P * chunks + nteams - 1) / nteams;
+      const uint64_t ctas = (pl.P * ((pl.HW + 7 + 1023) / 1024) + fh::kWarps - 1) / fh::kWarps;
       pl.ntiles = (uint32_t)(ctas > 0x7FFFFFFFull ? 0x7FFFFFFFull : ctas);
     }
     *out = pl;

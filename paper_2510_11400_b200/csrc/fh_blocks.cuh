@@ -33,20 +33,29 @@ struct SplitOut {
   __device__ __forceinline__ void st8(uint32_t o, uint32_t v) const { *at(o) = (uint8_t)v; }
 };
 
+// What the block-wise path needs to know of the plan, in registers: the outlined functions get the plan by address, and
+// a field read through it would be read again after every store.
+struct Geometry {
+  uint32_t H, W, HW, nbx, nby, nblk, nbm, nsr, qs, esize;
+  __device__ __forceinline__ explicit Geometry(const Plan& pl)
+      : H((uint32_t)pl.H), W((uint32_t)pl.W), HW(pl.HW), nbx(pl.nbx), nby(pl.nby), nblk(pl.nblk), nbm(pl.nbm), nsr(pl.nsr),
+        qs(pl.qs), esize((uint32_t)pl.esize) {}
+};
+
 // Shared scratch of one measured plane: words of rowp[H + 1], dense[nsr + 1], outl[nsr + 1], bitmap[nbm] and, with the
 // Huffman stage, chunks[nsr + 1] and a HufEncode.
 struct SalScratch {
   uint32_t *rowp, *dense, *outl, *bitmap, *chunks;
   HufEncode* huf;
 };
-__device__ __forceinline__ SalScratch sal_scratch(const Plan& pl, uint32_t* sal) {
+__device__ __forceinline__ SalScratch sal_scratch(const Geometry& pl, uint32_t* sal) {
   SalScratch s;
   s.rowp = sal;
-  s.dense = s.rowp + pl.H + 1;
-  s.outl = s.dense + pl.nsr + 1;
-  s.bitmap = s.outl + pl.nsr + 1;
+  s.dense = s.rowp + pl.H + 1u;
+  s.outl = s.dense + pl.nsr + 1u;
+  s.bitmap = s.outl + pl.nsr + 1u;
   s.chunks = s.bitmap + pl.nbm;
-  s.huf = reinterpret_cast<HufEncode*>(s.chunks + pl.nsr + 1);
+  s.huf = reinterpret_cast<HufEncode*>(s.chunks + pl.nsr + 1u);
   return s;
 }
 
@@ -56,7 +65,7 @@ struct StepLane {
   uint32_t qm;      // blocks side by side in a step, less one
   uint32_t qrow;    // the block's row of blocks within the step
 };
-__device__ __forceinline__ StepLane step_lane(const Plan& pl) {
+__device__ __forceinline__ StepLane step_lane(const Geometry& pl) {
   StepLane s;
   const uint32_t lane = threadIdx.x & 31u;
   s.r = lane >> 2;
@@ -98,8 +107,8 @@ __device__ __forceinline__ bool seg_vec(const uint8_t* plane, uint32_t W) {
   return (W & 3u) == 0u && ((uint32_t)(uintptr_t)plane & (DT == kF32 ? 15u : 7u)) == 0u;
 }
 // Elements of the segment that lie inside the plane.
-__device__ __forceinline__ uint32_t seg_in(const Plan& pl, bool valid, uint32_t y, uint32_t x0) {
-  return valid && y < (uint32_t)pl.H ? min(8u, (uint32_t)pl.W - x0) : 0u;
+__device__ __forceinline__ uint32_t seg_in(const Geometry& g, bool valid, uint32_t y, uint32_t x0) {
+  return valid && y < g.H ? min(8u, g.W - x0) : 0u;
 }
 __device__ __forceinline__ uint32_t nonzero_mask(const float (&v)[8]) {
   uint32_t m = 0;
@@ -180,42 +189,44 @@ __device__ __forceinline__ void warp_excl_scan(uint32_t* arr, uint32_t n) {
 // Measuring part: block classes, CSR row lengths, sizes.  The team is a whole warp or a whole CTA.  Leaves rowp, dense
 // and outl (and chunks) as exclusive prefix sums with the total behind the last entry, the bitmap and the code.
 template <int DT>
-__device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
-  const SalScratch sc = sal_scratch(pl, sal);
-  const uint32_t H = (uint32_t)pl.H, W = (uint32_t)pl.W, nsr = pl.nsr, full = 0xFFFFFFFFu;
+__device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
+  const Geometry g(pl);
+  const SalScratch sc = sal_scratch(g, sal);
+  const uint32_t H = g.H, W = g.W, nsr = g.nsr, tau_den = pl.tau_den, full = 0xFFFFFFFFu;
+  const bool entropy = pl.entropy != 0;
   const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane = threadIdx.x & 31u;
   const float inv2e = __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps));
-  const StepLane sl = step_lane(pl);
+  const StepLane sl = step_lane(g);
   const bool vec = seg_vec<DT>(plane, W);
   const uint32_t least = pl.tau_num * 64u;  // (at most 2^22)
-  for (uint32_t i = t.lane; i < pl.nbm; i += t.size) sc.bitmap[i] = 0;
-  if (pl.entropy)
+  for (uint32_t i = t.lane; i < g.nbm; i += t.size) sc.bitmap[i] = 0;
+  if (entropy)
     for (uint32_t i = t.lane; i < 256u; i += t.size) sc.huf->hist[i] = 0;
   if (t.lane == 0) sc.rowp[H] = sc.dense[nsr] = sc.outl[nsr] = 0;
   team_sync(t);
   for (uint32_t sr = wid; sr < nsr; sr += nw) {
-    const uint32_t by = sr * (4u >> pl.qs) + sl.qrow, y = by * 8u + sl.r;
+    const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
     uint32_t row = 0, n_dense = 0, n_out = 0;
-    for (uint32_t bx0 = 0; bx0 < pl.nbx; bx0 += sl.qm + 1u) {
+    for (uint32_t bx0 = 0; bx0 < g.nbx; bx0 += sl.qm + 1u) {
       const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u;
-      const bool valid = by < pl.nby && bx < pl.nbx;
-      const uint32_t nin = seg_in(pl, valid, y, x0);
+      const bool valid = by < g.nby && bx < g.nbx;
+      const uint32_t nin = seg_in(g, valid, y, x0);
       float v[8];
       load_seg<DT>(plane, W, y, x0, nin, vec, v);
       const uint32_t cnt = __popc(nonzero_mask(v));
-      const bool dense = block_sum(cnt) * pl.tau_den >= least && valid;
+      const bool dense = block_sum(cnt) * tau_den >= least && valid;
       const uint32_t dm = __ballot_sync(full, dense) & 15u;  // (row 0 of every block)
       if (dm) {
         uint32_t ca, cb, vm;
         seg_codes(v, nin, inv2e, ca, cb, vm);
         if (dense) {
           n_out += __popc(vm);
-          if (pl.entropy) {
+          if (entropy) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) atomicAdd(&sc.huf->hist[((j < 4 ? ca : cb) >> (8 * (j & 3))) & 255u], 1u);
           }
           if (sl.r == 0) {
-            const uint32_t b = by * pl.nbx + bx;
+            const uint32_t b = by * g.nbx + bx;
             atomicOr(&sc.bitmap[b >> 5], 1u << (b & 31u));
           }
         }
@@ -223,8 +234,8 @@ __device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& p
       }
       if (!dense) row += cnt;
     }
-    if (pl.qs > 0) row += __shfl_xor_sync(full, row, 1);
-    if (pl.qs > 1) row += __shfl_xor_sync(full, row, 2);
+    if (g.qs > 0) row += __shfl_xor_sync(full, row, 1);
+    if (g.qs > 1) row += __shfl_xor_sync(full, row, 2);
     if ((sl.q & sl.qm) == 0u && y < H) sc.rowp[y] = row;
     asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_out) : "r"(full));
     if (lane == 0) {
@@ -244,7 +255,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& p
   info.nnz_s = sc.rowp[H];
   info.n_out_d = sc.outl[nsr];
   info.coded = 0;
-  if (pl.entropy && info.n_dense) {
+  if (entropy && info.n_dense) {
     // Huffman stage (Section 4.4.1): the code from the histogram, then the size of every dense block's chunk
     HufEncode* h = sc.huf;
     if (wid == 0) huffman_build(h);
@@ -252,14 +263,14 @@ __device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& p
     team_sync(t);
     if (h->maxlen <= kHufMaxLen) {
       for (uint32_t sr = wid; sr < nsr; sr += nw) {
-        const uint32_t by = sr * (4u >> pl.qs) + sl.qrow, y = by * 8u + sl.r;
+        const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
         uint32_t bytes = 0;
-        for (uint32_t bx0 = 0; bx0 < pl.nbx; bx0 += sl.qm + 1u) {
-          const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u, b = by * pl.nbx + bx;
-          const bool valid = by < pl.nby && bx < pl.nbx;
+        for (uint32_t bx0 = 0; bx0 < g.nbx; bx0 += sl.qm + 1u) {
+          const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u, b = by * g.nbx + bx;
+          const bool valid = by < g.nby && bx < g.nbx;
           const bool dense = valid && ((sc.bitmap[b >> 5] >> (b & 31u)) & 1u);
           if (!__any_sync(full, dense)) continue;
-          const uint32_t nin = seg_in(pl, valid, y, x0);
+          const uint32_t nin = seg_in(g, valid, y, x0);
           float v[8];
           load_seg<DT>(plane, W, y, x0, nin, vec, v);
           uint32_t ca, cb, vm, bits = 0;
@@ -279,8 +290,8 @@ __device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& p
       if (section < 64u * info.n_dense) info.coded = section;
     }
   }
-  const uint32_t e = (uint32_t)pl.esize;
-  info.size = 16u + 4u * pl.nbm + 4u * (H + 1u) + a4(2u * info.nnz_s) + a4(e * info.nnz_s) +
+  const uint32_t e = g.esize;
+  info.size = 16u + 4u * g.nbm + 4u * (H + 1u) + a4(2u * info.nnz_s) + a4(e * info.nnz_s) +
               (info.coded ? info.coded : 64u * info.n_dense) + a4(e * info.n_out_d);
   return info;
 }
@@ -288,12 +299,13 @@ __device__ __noinline__ SalientInfo salient_measure(const Team& t, const Plan& p
 // Writing part; `sal` holds what salient_measure left.  Every lane recomputes the codes of its block rows and stores
 // them (and the CSR entries and verbatim values) straight to their places.
 template <int DT>
-__device__ __noinline__ void salient_write(const Team& t, const Plan& pl, const uint8_t* plane, const SalientInfo& info,
-                                           uint32_t* sal, const SplitOut& out) {
-  const SalScratch sc = sal_scratch(pl, sal);
-  const uint32_t H = (uint32_t)pl.H, W = (uint32_t)pl.W, nsr = pl.nsr, e = (uint32_t)pl.esize, full = 0xFFFFFFFFu;
+__device__ __noinline__ void salient_write(const Team t, const Plan& pl, const uint8_t* plane, const SalientInfo info,
+                                           uint32_t* sal, const SplitOut out) {
+  const Geometry g(pl);
+  const SalScratch sc = sal_scratch(g, sal);
+  const uint32_t H = g.H, W = g.W, nsr = g.nsr, e = g.esize, full = 0xFFFFFFFFu;
   const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane = threadIdx.x & 31u;
-  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * pl.nbm, o_col = o_rp + 4u * (H + 1u);
+  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * g.nbm, o_col = o_rp + 4u * (H + 1u);
   const uint32_t o_val = o_col + a4(2u * info.nnz_s), o_codes = o_val + a4(e * info.nnz_s);
   const uint32_t o_outl = o_codes + (info.coded ? info.coded : 64u * info.n_dense);
   if (t.lane == 0) {
@@ -307,9 +319,9 @@ __device__ __noinline__ void salient_write(const Team& t, const Plan& pl, const 
     if (DT == kBF16 && (info.n_out_d & 1u)) out.st16(o_outl + 2u * info.n_out_d, 0);
   }
   // zero padding up to the end of the slot / of the 16-byte padded overflow part
-  const uint32_t end = max(pl.npay, a16(info.size));
+  const uint32_t end = max(out.npay, a16(info.size));
   for (uint32_t o = info.size + 4u * t.lane; o < end; o += 4u * t.size) out.st32(o, 0);
-  for (uint32_t w = t.lane; w < pl.nbm; w += t.size) out.st32(o_bm + 4u * w, sc.bitmap[w]);
+  for (uint32_t w = t.lane; w < g.nbm; w += t.size) out.st32(o_bm + 4u * w, sc.bitmap[w]);
   for (uint32_t y = t.lane; y <= H; y += t.size) out.st32(o_rp + 4u * y, sc.rowp[y]);
   const HufEncode* h = sc.huf;  // (only looked at when info.coded)
   uint32_t o_cb = 0, o_chunks = 0;
@@ -329,16 +341,16 @@ __device__ __noinline__ void salient_write(const Team& t, const Plan& pl, const 
     for (uint32_t i = t.lane; i < nl; i += t.size) out.st8(o_codes + 4u + i, h->code[h->smin + i] >> 24);
   }
   const float inv2e = __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps));
-  const StepLane sl = step_lane(pl);
+  const StepLane sl = step_lane(g);
   const bool vec = seg_vec<DT>(plane, W);
   for (uint32_t sr = wid; sr < nsr; sr += nw) {
-    const uint32_t by = sr * (4u >> pl.qs) + sl.qrow, y = by * 8u + sl.r;
+    const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
     uint32_t rank0 = sc.dense[sr], outl0 = sc.outl[sr], chunk0 = info.coded ? sc.chunks[sr] : 0u;
     uint32_t csr = y < H ? sc.rowp[y] : 0u;
-    for (uint32_t bx0 = 0; bx0 < pl.nbx; bx0 += sl.qm + 1u) {
-      const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u, b = by * pl.nbx + bx;
-      const bool valid = by < pl.nby && bx < pl.nbx;
-      const uint32_t nin = seg_in(pl, valid, y, x0);
+    for (uint32_t bx0 = 0; bx0 < g.nbx; bx0 += sl.qm + 1u) {
+      const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u, b = by * g.nbx + bx;
+      const bool valid = by < g.nby && bx < g.nbx;
+      const uint32_t nin = seg_in(g, valid, y, x0);
       float v[8];
       load_seg<DT>(plane, W, y, x0, nin, vec, v);
       const bool dense = valid && ((sc.bitmap[b >> 5] >> (b & 31u)) & 1u);
@@ -414,11 +426,11 @@ __device__ __noinline__ void salient_write(const Team& t, const Plan& pl, const 
       if (info.nnz_s) {  // CSR entries of the sparse blocks
         const uint32_t nz = dense ? 0u : nonzero_mask(v), c = __popc(nz);
         uint32_t incl = c;
-        if (pl.qs > 0) {
+        if (g.qs > 0) {
           const uint32_t up = __shfl_up_sync(full, incl, 1);
           if ((sl.q & sl.qm) >= 1u) incl += up;
         }
-        if (pl.qs > 1) {
+        if (g.qs > 1) {
           const uint32_t up = __shfl_up_sync(full, incl, 2);
           if (sl.q >= 2u) incl += up;
         }

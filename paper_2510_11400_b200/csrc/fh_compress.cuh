@@ -97,8 +97,8 @@ __device__ __forceinline__ void block_codes(const BlockRegs& r, float inv2e, uin
 }
 
 // Raw plane: verbatim copy through the slot into the overflow part, zero padded.
-static __device__ __noinline__ void raw_write(const Team& t, const Plan& pl, const uint8_t* plane, const SplitOut& out) {
-  const uint32_t n = (uint32_t)pl.plane_bytes, end = max(pl.npay, a16(n));
+static __device__ __noinline__ void raw_write(const Team t, const Plan& pl, const uint8_t* plane, const SplitOut out) {
+  const uint32_t n = (uint32_t)pl.plane_bytes, end = max(out.npay, a16(n));
   for (uint32_t o = 2u * t.lane; o < end; o += 2u * t.size)
     out.st16(o, o < n ? (uint32_t)*reinterpret_cast<const uint16_t*>(plane + o) : 0u);
 }

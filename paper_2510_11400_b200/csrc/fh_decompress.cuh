@@ -1,17 +1,13 @@
 // Decompress kernel: container -> dense tensor, one pass.
 //
-// Planes are independent and their slots sit at closed-form offsets, so the kernel needs no
-// hand-out and no barrier: team t of the grid restores planes t, t + teams, ...  A team is a
-// power-of-two slice of a warp (a whole warp for planes of 256 groups and more).  Normal planes are
-// the fused unpack-and-dequantise: code bytes are read straight from the slot (they are 1/16 to 1/4
-// of the output), four values per thread and step go out as one 16-byte (fp32) or 8-byte (bf16)
-// store.  Raw planes are copied; outlier-rich planes take zero fill + CSR scatter + inverse Lorenzo
-// walk of the dense blocks.  Every read of the container is bounds-checked against src_bytes; a
-// plane whose table entry or payload is inconsistent is left unwritten and the call reports
-// FH_ERR_CORRUPT.
+// Planes are independent and their slots sit at closed-form offsets, so the kernels need no hand-out.  Normal planes
+// are the fused unpack-and-dequantise: codes are read straight from the slot (they are 1/16 to 1/4 of the output) and
+// leave as 16-byte stores.  Raw planes are copied; outlier-rich planes are restored four blocks per warp and step
+// (decode_salient).  Every read of the container is bounds-checked against src_bytes; a plane whose table entry or
+// payload is inconsistent reports FH_ERR_CORRUPT.
 #pragma once
 
-#include "fh_device.cuh"
+#include "fh_blocks.cuh"
 
 namespace fh {
 
@@ -27,31 +23,64 @@ struct SplitIn {
   __device__ __forceinline__ uint32_t ld8(uint32_t o) const { return __ldg(at(o)); }
 };
 
+// A payload copied to shared memory as one piece.
+struct FlatIn {
+  const uint8_t* p;
+  uint32_t npay;  // (kept for the size check: bytes of the payload that came from the slot)
+  __device__ __forceinline__ uint32_t ld32(uint32_t o) const { return *reinterpret_cast<const uint32_t*>(p + o); }
+  __device__ __forceinline__ uint32_t ld16(uint32_t o) const { return *reinterpret_cast<const uint16_t*>(p + o); }
+  __device__ __forceinline__ uint32_t ld8(uint32_t o) const { return p[o]; }
+};
+
 // One thread decodes a dense block's chunk of the Huffman-coded section (`nbytes` bytes at payload offset
-// `o_chunk`) into the block's 64 code bytes, four to a word.  False when the chunk is inconsistent.
+// `o_chunk`; `end`: bytes of the payload) into the block's 64 code bytes, four to a word.  False when the chunk is
+// inconsistent.  The chain of a symbol is a table look-up and a shift; the 64-bit window on the stream is fetched anew
+// for every group of symbols that surely fits it (four of at most 16 bits, two otherwise), without a branch, so that
+// the lanes' chunks stay in step.
 template <typename In>
-__device__ __noinline__ bool huffman_decode_chunk(const In& in, uint32_t o_chunk, uint32_t nbytes, const HufDecode* hd,
-                                                  uint32_t* codes) {
-  const uint32_t nbits = nbytes * 8u;
-  uint32_t pos = 0, cur = 0;
-  for (uint32_t i = 0; i < 16u; ++i) codes[i] = 0;
-  for (uint32_t i = 0; i < 64u; ++i) {
-    uint32_t acc = 0, sym = 256;
-    for (uint32_t l = 1; l <= kHufMaxLen; ++l) {
-      if (pos >= nbits) return false;
-      if ((pos & 7u) == 0u) cur = in.ld8(o_chunk + (pos >> 3));
-      acc = (acc << 1) | ((cur >> (7u - (pos & 7u))) & 1u);
-      ++pos;
-      const uint32_t k = acc - hd->first[l];
-      if (k < (uint32_t)hd->count[l]) {
-        sym = hd->sorted[hd->base[l] + k];
-        break;
-      }
+__device__ __forceinline__ bool huffman_decode_chunk(const In& in, uint32_t o_chunk, uint32_t nbytes, uint32_t end,
+                                                     const HufDecode* hd, uint32_t (&codes)[16]) {
+  uint32_t pos = o_chunk * 8u;  // in bits from the start of the payload
+  bool ok = true;
+  const uint32_t longest = hd->maxlen;
+  const bool four = longest <= 16u;
+  auto symbol = [&](uint32_t& hi, uint32_t& lo) -> uint32_t {
+    uint32_t en = hd->lut[hi >> (32 - kHufLutBits)];
+    if (en == 0u) {  // a longer code: the first length whose codes, left-aligned, reach beyond the window
+      uint32_t l = kHufLutBits + 1;
+      while (l < longest && hi >= hd->limit[l]) ++l;
+      const uint32_t at = (hi >> (32u - l)) + hd->base[l];
+      if (l > longest) ok = false;  // (a lone symbol's code leaves half of the windows without a meaning)
+      en = l << 8 | hd->sorted[at & 255u];
     }
-    if (sym > 255u) return false;
-    codes[i >> 2] |= sym << (8u * (i & 3u));
+    const uint32_t l = en >> 8;
+    pos += l;
+    hi = __funnelshift_l(lo, hi, l);
+    lo <<= l;
+    return en & 255u;
+  };
+  auto window = [&](uint32_t& hi, uint32_t& lo) {
+    const uint32_t o = (pos >> 5) << 2;
+    const uint32_t w0 = o + 4u <= end ? in.ld32(o) : 0u, w1 = o + 8u <= end ? in.ld32(o + 4u) : 0u, w2 = o + 12u <= end ? in.ld32(o + 8u) : 0u;
+    const uint32_t b0 = __byte_perm(w0, 0u, 0x0123), b1 = __byte_perm(w1, 0u, 0x0123), b2 = __byte_perm(w2, 0u, 0x0123);
+    hi = __funnelshift_l(b1, b0, pos & 31u);
+    lo = __funnelshift_l(b2, b1, pos & 31u);
+  };
+#pragma unroll 1
+  for (uint32_t i = 0; i < 16u; ++i) {
+    uint32_t hi, lo;
+    window(hi, lo);
+    uint32_t word = symbol(hi, lo);
+    word |= symbol(hi, lo) << 8;
+    if (!four) window(hi, lo);
+    word |= symbol(hi, lo) << 16;
+    word |= symbol(hi, lo) << 24;
+    // (the words move up by one and the new one comes in last: registers need static indexes)
+#pragma unroll
+    for (int k = 0; k < 15; ++k) codes[k] = codes[k + 1];
+    codes[15] = word;
   }
-  return true;
+  return ok && pos <= (o_chunk + nbytes) * 8u;
 }
 
 template <int DT>
@@ -66,29 +95,186 @@ __device__ __forceinline__ float dequant(uint32_t q, float scale, float lo) {
   return __fmaf_rn(qf, scale, lo);
 }
 
-// Outlier-rich plane.  `scr` is the team's shared scratch: 2 * nblk words, followed by a HufDecode.  `ovf_avail`
-// is the number of readable bytes behind in.ovf; `version` the container's (2: the dense blocks' codes may be
-// Huffman-coded, Section 4.4.1 "Decompression involves Huffman decoding").
+// Eight restored values of row y from column x0 on, `nin` of them inside the plane.  `vec`: rows are whole aligned
+// groups of four.
 template <int DT>
-__device__ __noinline__ bool decode_salient(const Team& t, const Plan& pl, const SplitIn& in, uint64_t ovf_avail, float eps,
-                               uint8_t* out, uint32_t* scr, uint32_t version) {
-  const int H = pl.H, W = pl.W;
-  const uint32_t nblk = pl.nblk, nbx = pl.nbx, nbm = pl.nbm, e = (uint32_t)pl.esize, HW = pl.HW;
+__device__ __forceinline__ void store_seg(uint8_t* out, uint32_t W, uint32_t y, uint32_t x0, uint32_t nin, bool vec,
+                                          const float (&v)[8]) {
+  const uint32_t i = y * W + x0;
+  if (vec) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (nin > 4u * h) {
+        if (DT == kF32)
+          *reinterpret_cast<float4*>(out + 4ull * (i + 4u * h)) = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+        else
+          *reinterpret_cast<uint2*>(out + 2ull * (i + 4u * h)) =
+              make_uint2(f32x2_to_bf16x2(v[4 * h], v[4 * h + 1]), f32x2_to_bf16x2(v[4 * h + 2], v[4 * h + 3]));
+      }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if ((uint32_t)j < nin) store_elem<DT>(out, i + j, v[j]);
+  }
+}
+
+// Zero bytes of a word, as one bit (0x80) each.
+__device__ __forceinline__ uint32_t zero_bytes(uint32_t w) { return ~(((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w | 0x7F7F7F7Fu); }
+
+// A dense block by one lane, in raster order: k = pred + residual (Eq. 7-9), x = k * 2 eps; a verbatim element's k
+// follows from its stored value.  Row by row, with the differences e[j] = k[j] - k[j-1] of the row above in registers;
+// all that does not depend on the left neighbour -- the row's verbatim values and their k -- is worked out for the eight
+// columns side by side and without branches (a column without a verbatim value reads the one that comes next), which
+// leaves an addition and a selection per element as the serial chain.  `codes`: the block's 64 code bytes; oi: index of
+// its first verbatim value (all of them are there, the caller has counted); o_outl, last: where the values are and the
+// last one's index.  A warp restores 32 blocks in about 1,200 instructions; a lane per block row, in a wavefront over
+// the columns, took 1,000 for four.
+template <int DT, typename In>
+__device__ __forceinline__ void restore_block(const In& in, uint32_t o_outl, uint32_t last, uint32_t oi, uint32_t (&codes)[16],
+                                              float two_eps, float inv2e, uint8_t* out, uint32_t H, uint32_t W, uint32_t y0,
+                                              uint32_t x0, bool vec) {
+  const uint32_t nin = min(8u, W - x0), rows = min(8u, H - y0);
+  int32_t e[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) e[j] = 0;
+#pragma unroll 1
+  for (uint32_t i = 0; i < rows; ++i) {
+    const uint32_t a = codes[0], c = codes[1];
+#pragma unroll
+    for (int k = 0; k < 14; ++k) codes[k] = codes[k + 2];
+    float v[8];
+    int32_t kv[8];
+    bool is[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t code = __byte_perm(a, c, 0x4440u + j) & 255u;
+      e[j] += (int32_t)code - 128;
+      is[j] = code == 0u && (uint32_t)j < nin;
+      const uint32_t at = min(oi, last);
+      v[j] = DT == kF32 ? __uint_as_float(in.ld32(o_outl + 4u * at)) : bf16_bits_to_f32(in.ld16(o_outl + 2u * at));
+      oi += is[j] ? 1u : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) kv[j] = max(min(__float2int_rn(__fmul_rn(v[j], inv2e)), 1 << 24), -(1 << 24));
+    int32_t left = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int32_t k = is[j] ? kv[j] : left + e[j];
+      v[j] = is[j] ? v[j] : __fmul_rn((float)k, two_eps);
+      e[j] = k - left;
+      left = k;
+    }
+    store_seg<DT>(out, W, y0 + i, x0, nin, vec, v);
+  }
+}
+
+// Zero bytes of a block's codes: its verbatim elements.
+__device__ __forceinline__ uint32_t count_verbatim(const uint32_t (&codes)[16]) {
+  uint32_t n = 0;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) n += __popc(zero_bytes(codes[k]));
+  return n;
+}
+
+// Four dense blocks by one warp: lane 8 q + j has column j of block q.  Within a row, k[j] = k[j-1] + e[j] + residual[j]
+// is a scan over the block's eight lanes that starts anew at every verbatim element, so a row is four shuffles and the
+// block eight such rows in series; the verbatim values and their k are worked out for all rows beforehand.  About 330
+// instructions for four blocks: twice those of a lane per block (restore_block), but a quarter of its latency, which is
+// what counts for planes of few blocks (14 x 14, fp32, 67 outlier-rich planes of 16,384: 22.6 -> 13.7 us a call).
+//   code_at(i)  the lane's code byte of row i;  dense  the lane's block is one (the others take part with codes of 128)
+//   out, y0, x0 where the block's elements go
+// `locate` is told the number of verbatim elements of the lane's block (all lanes call it) and returns the payload offset
+// of the first.
+template <int DT, typename In, typename CodeAt, typename Locate>
+__device__ __forceinline__ void restore_columns(const In& in, CodeAt code_at, Locate locate, bool dense, float two_eps, float inv2e,
+                                                uint8_t* out, uint32_t H, uint32_t W, uint32_t y0, uint32_t x0) {
+  const uint32_t full = 0xFFFFFFFFu, lane = threadIdx.x & 31u, j = lane & 7u, q = lane >> 3;
+  int32_t res[8];
+  uint32_t mask[8];  // verbatim elements of row i: this lane's block's byte
+  uint32_t any = 0, n = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t code = dense ? code_at(i) : 128u;
+    res[i] = (int32_t)code - 128;
+    const uint32_t m = __ballot_sync(full, code == 0u);
+    mask[i] = (m >> (8u * q)) & 255u;
+    any |= m;
+    n += __popc(mask[i]);
+  }
+  float raw[8];
+  int32_t kv[8];
+  if (any) {
+    uint32_t o = locate(n);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t at = o + (DT == kF32 ? 4u : 2u) * __popc(mask[i] & ((1u << j) - 1u));
+      raw[i] = 0.0f;
+      if ((mask[i] >> j) & 1u) raw[i] = DT == kF32 ? __uint_as_float(in.ld32(at)) : bf16_bits_to_f32(in.ld16(at));
+      o += (DT == kF32 ? 4u : 2u) * __popc(mask[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) kv[i] = max(min(__float2int_rn(__fmul_rn(raw[i], inv2e)), 1 << 24), -(1 << 24));
+  } else {
+    locate(0u);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) raw[i] = 0.0f, kv[i] = 0;
+  }
+  int32_t e = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t upto = mask[i] & ((2u << j) - 1u);                            // verbatim elements at or before the column
+    const uint32_t reach = upto ? j - (31u - (uint32_t)__clz((int)upto)) : j;   // lanes the sum may reach back
+    const bool is = (mask[i] >> j) & 1u;
+    int32_t k = is ? kv[i] : e + res[i];
+#pragma unroll
+    for (uint32_t o = 1; o < 8u; o <<= 1) {
+      const int32_t t = __shfl_up_sync(full, k, o);
+      if (reach >= o) k += t;
+    }
+    const int32_t left = __shfl_up_sync(full, k, 1);
+    e = j == 0u ? k : k - left;
+    if (dense && y0 + i < H && x0 + j < W) store_elem<DT>(out, (y0 + i) * W + x0 + j, is ? raw[i] : __fmul_rn((float)k, two_eps));
+  }
+}
+
+// Outlier-rich plane: the inverse of salient_write.  Dense blocks a lane each, by rank (so that all lanes have one);
+// where a block's verbatim values start is a scan over the zero bytes of the codes.  Sparse blocks are
+// zeroed first, a lane per block row, and take their values entry by entry, eight lanes to a CSR row.  `scr` is the team's shared scratch, laid out by
+// make_plan; `ovf_avail` the number of readable bytes behind in.ovf; `version` the container's (2: the dense blocks'
+// codes may be Huffman-coded, Section 4.4.1 "Decompression involves Huffman decoding").  Returns false in the threads
+// that found the payload inconsistent.
+template <int DT, typename In>
+__device__ __noinline__ bool decode_salient(const Team t, const Plan& pl, const In in, uint64_t ovf_avail, float eps, uint8_t* out,
+                                            uint32_t* scr, uint32_t version) {
+  const Geometry g(pl);
+  const uint32_t H = g.H, W = g.W, nblk = g.nblk, nbx = g.nbx, nbm = g.nbm, e = g.esize, HW = g.HW;
+  const uint32_t full = 0xFFFFFFFFu;
   const uint32_t nnz_s = in.ld32(0), n_dense = in.ld32(4), n_out_d = in.ld32(8), coded = in.ld32(12);
   if (nnz_s > HW || n_dense > nblk || n_out_d > HW) return false;
   if (coded && (version != 2u || (coded & 3u) || coded >= 64u * n_dense)) return false;
   const uint64_t size = 16ull + 4ull * nbm + 4ull * ((uint64_t)H + 1) + a4(2u * nnz_s) + a4(e * nnz_s) +
                         (coded ? (uint64_t)coded : 64ull * n_dense) + a4(e * n_out_d);
   if (size > in.npay && size - in.npay > ovf_avail) return false;
-  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * nbm, o_col = o_rp + 4u * ((uint32_t)H + 1u);
+  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * nbm, o_col = o_rp + 4u * (H + 1u);
   const uint32_t o_val = o_col + a4(2u * nnz_s), o_codes = o_val + a4(e * nnz_s);
   const uint32_t o_outl = o_codes + (coded ? coded : 64u * n_dense);
+  const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane = threadIdx.x & 31u;
+  uint32_t* bm = scr;              // the bitmap
+  uint32_t* wp = bm + nbm;         // dense blocks before each of its words
+  uint32_t* wsum = wp + nbm + 1u;  // one word per warp
+  uint32_t* cho = wsum + kMaxWarps;  // (Huffman) start of every chunk
+  HufDecode* hd = reinterpret_cast<HufDecode*>(cho + nblk + 1u);
+  uint16_t* block_of = reinterpret_cast<uint16_t*>(hd + 1);  // by rank
   bool ok = true;
-  // Huffman-coded section: decoding tables from the stored lengths, start of every chunk from the chunks' sizes
-  uint32_t* cho = scr + nblk;  // by rank among the dense blocks
-  HufDecode* hd = reinterpret_cast<HufDecode*>(scr + 2u * nblk);
+  for (uint32_t w = t.lane; w < nbm; w += t.size) {
+    uint32_t m = in.ld32(o_bm + 4u * w);
+    if (w == nblk >> 5) m &= (1u << (nblk & 31u)) - 1u;
+    bm[w] = m;
+    wp[w] = __popc(m);
+  }
+  if (t.lane == 0) wp[nbm] = 0;
   uint32_t o_chunks = 0, o_cb = 0;
-  if (coded) {
+  if (coded) {  // Huffman-coded section: the stored lengths and the chunks' sizes
     const uint32_t smin = in.ld8(o_codes + 1u), smax = in.ld8(o_codes + 2u);
     if (smin < 1u || smax < smin) return false;
     const uint32_t nl = smax - smin + 1u;
@@ -97,116 +283,176 @@ __device__ __noinline__ bool decode_salient(const Team& t, const Plan& pl, const
     if (o_chunks - o_codes > coded) return false;
     for (uint32_t sym = t.lane; sym < 256u; sym += t.size)
       hd->len[sym] = sym == 0u ? (uint8_t)in.ld8(o_codes) : ((sym >= smin && sym <= smax) ? (uint8_t)in.ld8(o_codes + 4u + sym - smin) : (uint8_t)0);
-    for (uint32_t r = t.lane; r < nblk; r += t.size) cho[r] = r < n_dense ? in.ld8(o_cb + r) : 0u;
-    team_sync(t);
-    if (t.lane == 0) huffman_tables(hd);
-    const uint32_t chunks = team_excl_scan(t, cho, nblk);
-    if (!hd->ok || o_chunks - o_codes + chunks > coded) return false;  // (the same for every thread)
-  }
-  // zero fill (16-bit units cover both element sizes)
-  for (uint32_t i = t.lane; i < (uint32_t)(pl.plane_bytes >> 1); i += t.size) reinterpret_cast<uint16_t*>(out)[i] = 0;
-  // verbatim counts of the dense blocks -> first verbatim index of each block
-  for (uint32_t b = t.lane; b < nblk; b += t.size) {
-    uint32_t cnt = 0;
-    if ((in.ld32(o_bm + 4u * (b >> 5)) >> (b & 31u)) & 1u) {
-      uint32_t rank = 0;
-      for (uint32_t w = 0; w < (b >> 5); ++w) rank += __popc(in.ld32(o_bm + 4u * w));
-      rank += __popc(in.ld32(o_bm + 4u * (b >> 5)) & ((1u << (b & 31u)) - 1u));
-      if (rank < n_dense) {
-        uint32_t cw[16];
-        if (coded && !huffman_decode_chunk(in, o_chunks + cho[rank], in.ld8(o_cb + rank), hd, cw)) ok = false;
-        for (uint32_t k = 0; k < 16; ++k) {
-          const uint32_t w = coded ? cw[k] : in.ld32(o_codes + 64u * rank + 4u * k);
-          cnt += ((w & 0xFFu) == 0) + ((w & 0xFF00u) == 0) + ((w & 0xFF0000u) == 0) + ((w & 0xFF000000u) == 0);
-        }
-      } else {
-        ok = false;
-      }
-    }
-    scr[b] = cnt;
+    for (uint32_t r = t.lane; r <= n_dense; r += t.size) cho[r] = r < n_dense ? in.ld8(o_cb + r) : 0u;
   }
   team_sync(t);
-  const uint32_t tot_out = team_excl_scan(t, scr, nblk);
-  if (tot_out > n_out_d) ok = false;
-  // CSR scatter
-  for (int y = (int)t.lane; y < H; y += (int)t.size) {
-    const uint32_t r0 = in.ld32(o_rp + 4u * y), r1 = in.ld32(o_rp + 4u * (y + 1));
-    if (r0 > r1 || r1 > nnz_s) { ok = false; continue; }
-    for (uint32_t k = r0; k < r1; ++k) {
-      const uint32_t col = in.ld16(o_col + 2u * k);
-      if (col >= (uint32_t)W) { ok = false; continue; }
-      const uint32_t idx = (uint32_t)y * W + col;
-      if (DT == kF32) reinterpret_cast<uint32_t*>(out)[idx] = in.ld32(o_val + 4u * k);
-      else reinterpret_cast<uint16_t*>(out)[idx] = (uint16_t)in.ld16(o_val + 2u * k);
+  if (wid == 0) warp_excl_scan(wp, nbm + 1u);
+  if (coded) {
+    if (wid == min(1u, nw - 1u)) huffman_tables(hd);
+    if (wid == nw - 1u) warp_excl_scan(cho, n_dense + 1u);
+  }
+  team_sync(t);
+  if (wp[nbm] != n_dense) return false;  // (the same for every thread, and so is the next)
+  if (coded) {
+    if (!hd->ok || o_chunks - o_codes + cho[n_dense] > coded) return false;
+    huffman_lut(hd, t.lane, t.size);
+  }
+  for (uint32_t b = t.lane; b < nblk; b += t.size)
+    if ((bm[b >> 5] >> (b & 31u)) & 1u) block_of[wp[b >> 5] + __popc(bm[b >> 5] & ((1u << (b & 31u)) - 1u))] = (uint16_t)b;
+  const bool vec = (W & 3u) == 0u && ((uint32_t)(uintptr_t)out & (DT == kF32 ? 15u : 7u)) == 0u;
+  if (n_dense < nblk) {  // sparse blocks are zero but for the CSR entries
+    const StepLane sl = step_lane(g);
+    const float zero[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    for (uint32_t sr = wid; sr < g.nsr; sr += nw) {
+      const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
+      for (uint32_t bx = sl.q & sl.qm; by < g.nby && y < H && bx < nbx; bx += sl.qm + 1u) {
+        const uint32_t b = by * nbx + bx;
+        if (!((bm[b >> 5] >> (b & 31u)) & 1u)) store_seg<DT>(out, W, y, bx * 8u, min(8u, W - bx * 8u), vec, zero);
+      }
     }
   }
-  // dense blocks: raster walk, k = pred + residual (Eq. 7-9), x = k * 2 eps
-  const float two_eps = __fmul_rn(2.0f, eps);
-  const float inv2e = __fdiv_rn(1.0f, two_eps);
-  if (ok && tot_out <= n_out_d) {
-    for (uint32_t b = t.lane; b < nblk; b += t.size) {
-      if (!((in.ld32(o_bm + 4u * (b >> 5)) >> (b & 31u)) & 1u)) continue;
-      uint32_t rank = 0;
-      for (uint32_t w = 0; w < (b >> 5); ++w) rank += __popc(in.ld32(o_bm + 4u * w));
-      rank += __popc(in.ld32(o_bm + 4u * (b >> 5)) & ((1u << (b & 31u)) - 1u));
-      const uint32_t oc = o_codes + 64u * rank;
-      uint32_t cw[16];
-      if (coded && !huffman_decode_chunk(in, o_chunks + cho[rank], in.ld8(o_cb + rank), hd, cw)) {
+  team_sync(t);
+  const float two_eps = __fmul_rn(2.0f, eps), inv2e = __fdiv_rn(1.0f, two_eps);
+  uint32_t outl0 = 0;
+  for (uint32_t base = 0; base < n_dense; base += t.size) {
+    const uint32_t rank = base + t.lane;
+    uint32_t codes[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) codes[k] = 0x80808080u;
+    if (rank < n_dense) {
+      if (coded) {
+        ok &= huffman_decode_chunk(in, o_chunks + cho[rank], cho[rank + 1u] - cho[rank], (uint32_t)size, hd, codes);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) codes[k] = in.ld32(o_codes + 64u * rank + 4u * k);
+      }
+    }
+    const uint32_t n = count_verbatim(codes);
+    uint32_t incl = n;
+#pragma unroll
+    for (uint32_t o = 1; o < 32u; o <<= 1) {
+      const uint32_t up = __shfl_up_sync(full, incl, o);
+      if (lane >= o) incl += up;
+    }
+    uint32_t first = outl0 + incl - n, all = __shfl_sync(full, incl, 31);
+    if (t.block) {
+      if (lane == 31u) wsum[wid] = incl;
+      __syncthreads();
+      all = 0;
+      for (uint32_t k = 0; k < nw; ++k) {
+        first += k < wid ? wsum[k] : 0u;
+        all += wsum[k];
+      }
+      __syncthreads();
+    }
+    outl0 += all;
+    if (rank < n_dense) {
+      const uint32_t b = block_of[rank], by = b / nbx, bx = b - by * nbx;
+      if (first + n > n_out_d) {
         ok = false;
-        continue;
+      } else {
+        restore_block<DT>(in, n_out_d ? o_outl : 0u, n_out_d ? n_out_d - 1u : 0u, first, codes, two_eps, inv2e, out, H, W, by * 8u, bx * 8u, vec);
       }
-      uint32_t oi = scr[b];
-      const int by = (int)(b / nbx), bx = (int)(b % nbx);
-      int32_t prev[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) prev[j] = 0;
-#pragma unroll 1
-      for (int i = 0; i < 8; ++i) {
-        const int y = by * 8 + i;
-        const uint32_t w0 = coded ? cw[2 * i] : in.ld32(oc + 8u * i), w1 = coded ? cw[2 * i + 1] : in.ld32(oc + 8u * i + 4u);
-        int32_t left = 0, ul = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int x = bx * 8 + j;
-          const uint32_t code = ((j < 4 ? w0 : w1) >> (8 * (j & 3))) & 0xFFu;
-          const int32_t up = prev[j];
-          const int32_t pred = up + left - ul;
-          int32_t k = pred;
-          if (y < H && x < W) {
-            const uint32_t idx = (uint32_t)y * W + x;
-            if (code == 0u) {
-              float v;
-              if (DT == kF32) {
-                const uint32_t raw = in.ld32(o_outl + 4u * oi);
-                reinterpret_cast<uint32_t*>(out)[idx] = raw;
-                v = __uint_as_float(raw);
-              } else {
-                const uint32_t raw = in.ld16(o_outl + 2u * oi);
-                reinterpret_cast<uint16_t*>(out)[idx] = (uint16_t)raw;
-                v = bf16_bits_to_f32(raw);
-              }
-              bool big;
-              k = dense_k(v, inv2e, &big);
-              ++oi;
-            } else {
-              k = pred + (int32_t)code - 128;
-              store_elem<DT>(out, idx, __fmul_rn((float)k, two_eps));
-            }
-          }
-          ul = up;
-          left = k;
-          prev[j] = k;
-        }
-      }
+    }
+  }
+  if (n_dense == nblk) return ok && nnz_s == 0u;
+  for (uint32_t y = t.lane >> 3; y < H && nnz_s; y += t.size >> 3) {
+    const uint32_t r0 = in.ld32(o_rp + 4u * y), r1 = in.ld32(o_rp + 4u * y + 4u);
+    if (r0 > r1 || r1 > nnz_s) {
+      ok = false;
+      continue;
+    }
+    for (uint32_t k = r0 + (lane & 7u); k < r1; k += 8u) {
+      const uint32_t col = in.ld16(o_col + 2u * k), b = (y >> 3) * nbx + (col >> 3);
+      if (col >= W || ((bm[b >> 5] >> (b & 31u)) & 1u)) ok = false;
+      else if (DT == kF32) reinterpret_cast<uint32_t*>(out)[y * W + col] = in.ld32(o_val + 4u * k);
+      else reinterpret_cast<uint16_t*>(out)[y * W + col] = (uint16_t)in.ld16(o_val + 2u * k);
     }
   }
   return ok;
 }
 
+// Outlier-rich planes of at most four blocks (plain codes) by one warp, all their dense blocks in one step: one plane, or
+// four of one block each (FOUR: the eight lanes 8 q ... of plane q pass its payload `in` -- `avail` bytes of it --, its
+// destination and whether it is there).  Destinations are shared memory.
+template <int DT, bool FOUR>
+__device__ __noinline__ bool decode_few(const Plan& pl, const FlatIn in, uint32_t avail, bool there, float eps, uint8_t* out) {
+  const Geometry g(pl);
+  const uint32_t H = g.H, W = g.W, e = g.esize, full = 0xFFFFFFFFu, lane = threadIdx.x & 31u, q = lane >> 3, j = lane & 7u;
+  uint32_t nnz_s = 0, n_dense = 0, n_out_d = 0, bitmap = 0;
+  bool ok = true;
+  if (there) {
+    nnz_s = in.ld32(0);
+    n_dense = in.ld32(4);
+    n_out_d = in.ld32(8);
+    bitmap = in.ld32(16) & ((1u << g.nblk) - 1u);
+    ok = nnz_s <= g.HW && n_dense == (uint32_t)__popc(bitmap) && n_out_d <= g.HW && in.ld32(12) == 0u &&
+         20u + 4u * (H + 1u) + a4(2u * nnz_s) + a4(e * nnz_s) + 64u * n_dense + a4(e * n_out_d) <= avail;
+  }
+  there = there && ok;
+  const uint32_t o_rp = 20u, o_col = o_rp + 4u * (H + 1u), o_val = o_col + a4(2u * nnz_s), o_codes = o_val + a4(e * nnz_s);
+  const uint32_t o_outl = o_codes + 64u * n_dense;
+  const bool some_sparse = there && n_dense < g.nblk;
+  if (some_sparse) {
+    if (FOUR) {
+      for (uint32_t i = j; i < g.HW; i += 8u) store_elem<DT>(out, i, 0.0f);
+    } else {
+      for (uint32_t i = lane; i < g.HW; i += 32u) store_elem<DT>(out, i, 0.0f);
+    }
+  }
+  __syncwarp();
+  const uint32_t rank = FOUR ? 0u : q;
+  const bool dense = there && rank < n_dense;
+  if (__any_sync(full, dense)) {
+    uint32_t b = 0;
+    if (!FOUR) {  // the rank-th dense block
+      uint32_t m = bitmap;
+      for (uint32_t k = 0; k < rank; ++k) m &= m - 1u;
+      b = m ? (uint32_t)__ffs((int)m) - 1u : 0u;
+    }
+    const uint32_t by = b / g.nbx, bx = b - by * g.nbx;
+    const float two_eps = __fmul_rn(2.0f, eps);
+    restore_columns<DT>(
+        in, [&](int i) { return in.ld8(o_codes + 64u * rank + 8u * i + j); },
+        [&](uint32_t n) {
+          uint32_t first = 0;
+          if (!FOUR) {
+            const uint32_t n0 = __shfl_sync(full, n, 0), n1 = __shfl_sync(full, n, 8), n2 = __shfl_sync(full, n, 16);
+            first = (q > 0u ? n0 : 0u) + (q > 1u ? n1 : 0u) + (q > 2u ? n2 : 0u);
+          }
+          if (dense && first + n > n_out_d) {  // (reads stay within the payload)
+            ok = false;
+            return 0u;
+          }
+          return o_outl + e * first;
+        },
+        dense, two_eps, __fdiv_rn(1.0f, two_eps), out, H, W, by * 8u, bx * 8u);
+  }
+  __syncwarp();
+  if (some_sparse && nnz_s) {  // CSR entries: eight lanes to a row, or a lane to a row of its plane
+    for (uint32_t y = FOUR ? j : q; y < H; y += FOUR ? 8u : 4u) {
+      const uint32_t r0 = in.ld32(o_rp + 4u * y), r1 = in.ld32(o_rp + 4u * y + 4u);
+      if (r0 > r1 || r1 > nnz_s) {
+        ok = false;
+        continue;
+      }
+      for (uint32_t k = r0 + (FOUR ? 0u : j); k < r1; k += FOUR ? 1u : 8u) {
+        const uint32_t col = in.ld16(o_col + 2u * k);
+        if (col >= W || ((bitmap >> ((y >> 3) * g.nbx + (col >> 3))) & 1u)) ok = false;
+        else if (DT == kF32) reinterpret_cast<uint32_t*>(out)[y * W + col] = in.ld32(o_val + 4u * k);
+        else reinterpret_cast<uint16_t*>(out)[y * W + col] = (uint16_t)in.ld16(o_val + 2u * k);
+      }
+    }
+  } else if (there && nnz_s) {
+    ok = false;
+  }
+  return ok;
+}
+
 // Header of a container against what the caller expects: 0 if it does not fit, the container's version (1, 2)
-// otherwise; also returns code width, eps and total size.
+// otherwise; also returns code width, eps, total size and the number of outlier-rich planes.
 __device__ __forceinline__ uint32_t check_header(const Plan& pl, const uint8_t* src, unsigned long long src_bytes, uint32_t& bits,
-                                                 float& eps, unsigned long long& total) {
+                                                 float& eps, unsigned long long& total, uint32_t& nsal) {
   if (src_bytes < 64ull + 16ull * pl.P) return 0u;
   const uint32_t* h = reinterpret_cast<const uint32_t*>(src);
   bits = __ldg(h + 1) >> 24;
@@ -216,6 +462,7 @@ __device__ __forceinline__ uint32_t check_header(const Plan& pl, const uint8_t* 
             __ldg(h + 4) == (uint32_t)pl.H && __ldg(h + 5) == (uint32_t)pl.W && (__ldg(h + 6) & 0xFFFFu) == (8u | (8u << 8));
   total = (unsigned long long)__ldg(h + 14) | ((unsigned long long)__ldg(h + 15) << 32);
   eps = __uint_as_float(__ldg(h + 9));
+  nsal = __ldg(h + 10);
   const unsigned long long npay = a16(4u * ((pl.HW * (bits & 15u) + 31u) / 32u));
   ok = ok && total <= src_bytes && total >= 64ull + 16ull * pl.P + pl.P * npay && eps >= 1e-30f && eps <= 1e30f;
   return ok ? version : 0u;
@@ -323,36 +570,62 @@ __device__ __forceinline__ void decode_chunk32_bf16_pairs(const uint32_t (&w)[8]
   }
 }
 
-// Normal plane, sub-warp team of TT lanes (planes of at most 8 * TT groups, one chunk).  cw[k] holds the
-// code word of group lane + k * TT, requested before the table entry was known.  Whole groups of planes
-// that start on a vector boundary leave as one store; everything else (planes that do not, the ragged
-// last group) as element stores.
-template <int DT, int BITS, int TT>
-__device__ __forceinline__ void decode_small(const uint32_t (&cw)[8], uint32_t lane, uint32_t groups, uint32_t nfull,
-                                             uint32_t HW, float scale, float lo, uint8_t* out) {
+// Normal plane that does not start on a 16-byte boundary of the tensor (or whose last vector is shared with the next
+// plane): lanes own aligned 16-byte vectors of the OUTPUT, and since decoding is element by element, each picks its
+// elements' codes out of the bit stream with a funnel shift.  The plane's first and last vectors, which it may share
+// with its neighbours, leave as element stores.  `v0`: first vector of the chunk, counted from the one that holds the
+// plane's first element; `shift`: elements of that vector that belong to the plane before.
+template <int DT, int BITS>
+__device__ __forceinline__ void decode_chunk_shifted(const uint8_t* slot, uint32_t nwords, uint32_t lane, uint32_t v0, uint32_t HW,
+                                                     uint32_t shift, float scale, float lo, uint8_t* out) {
+  constexpr int VE = DT == kF32 ? 4 : 8, K = DT == kF32 ? 8 : 4;  // elements of a vector, vectors per lane
   constexpr uint32_t L = (1u << BITS) - 1u;
+  constexpr int NW = VE * BITS > 32 ? 2 : 1;                      // words of codes of a vector
+  const uint32_t* s32 = reinterpret_cast<const uint32_t*>(slot);
+  uint32_t cw[K][NW];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint32_t g = lane + (uint32_t)k * TT, word = cw[k];
-    if (g >= groups) break;
-    const float v0 = dequant(word & L, scale, lo), v1 = dequant((word >> BITS) & L, scale, lo);
-    const float v2 = dequant((word >> (2 * BITS)) & L, scale, lo), v3 = dequant((word >> (3 * BITS)) & L, scale, lo);
-    if (g < nfull) {
-      store_group<DT>(out, g, v0, v1, v2, v3);
+  for (int k = 0; k < K; ++k) {
+    const int32_t i0 = (int32_t)((v0 + k * 32u + lane) * VE) - (int32_t)shift;
+    const int32_t bit = i0 * BITS, w0 = bit >> 5;
+    uint32_t w[NW + 1];
+#pragma unroll
+    for (int n = 0; n <= NW; ++n) w[n] = (i0 < (int32_t)HW && (uint32_t)(w0 + n) < nwords) ? __ldg(s32 + w0 + n) : 0u;
+#pragma unroll
+    for (int n = 0; n < NW; ++n) cw[k][n] = __funnelshift_r(w[n], w[n + 1], (uint32_t)bit & 31u);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int32_t i0 = (int32_t)((v0 + k * 32u + lane) * VE) - (int32_t)shift;
+    float v[VE];
+#pragma unroll
+    for (int j = 0; j < VE; ++j) v[j] = dequant((cw[k][(j * BITS) >> 5] >> ((j * BITS) & 31)) & L, scale, lo);
+    if (i0 >= 0 && i0 + VE <= (int32_t)HW) {
+      if (DT == kF32) {
+        *reinterpret_cast<float4*>(out + 4ll * i0) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+        uint4 q;
+        q.x = f32x2_to_bf16x2(v[0], v[1]);
+        q.y = f32x2_to_bf16x2(v[2], v[3]);
+        q.z = f32x2_to_bf16x2(v[VE - 4], v[VE - 3]);
+        q.w = f32x2_to_bf16x2(v[VE - 2], v[VE - 1]);
+        *reinterpret_cast<uint4*>(out + 2ll * i0) = q;
+      }
     } else {
-      const uint32_t i = 4u * g;
-      store_elem<DT>(out, i, v0);
-      if (i + 1u < HW) store_elem<DT>(out, i + 1u, v1);
-      if (i + 2u < HW) store_elem<DT>(out, i + 2u, v2);
-      if (i + 3u < HW) store_elem<DT>(out, i + 3u, v3);
+#pragma unroll
+      for (int j = 0; j < VE; ++j)
+        if (i0 + j >= 0 && i0 + j < (int32_t)HW) store_elem<DT>(out, (uint32_t)(i0 + j), v[j]);
     }
   }
 }
 
-constexpr uint32_t kDeferBlocks = 128;  // planes of at least this many 8x8 blocks: outlier-rich ones go to the whole CTA
-
-// DEFER: instantiated for whole-warp teams on planes of at least kDeferBlocks blocks.
-template <int DT, int TT, bool DEFER>
+// Planes of more than 128 groups.  Work items are (plane, chunk of 1024 elements) pairs, a warp each, so that large
+// planes spread over many warps; no barrier in the streaming part.  Warp w takes items w, w + stride, ...; the stride is
+// a prime (warps beyond it stay idle), so that a periodic pattern of expensive planes -- every eighth channel
+// outlier-rich, say -- spreads over all warps instead of landing on the few whose index shares a factor with the period.
+// Outlier-rich planes are left for the end (when the header says that there are any): CTA c then looks at the table
+// entries of planes c, c + stride, ... -- the stride a prime again -- gathers those that are outlier-rich and restores
+// them, a warp each (pl.team = 32) or, when they have many blocks, the whole CTA one after the other.
+template <int DT>
 __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, const DecompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 5];
@@ -360,32 +633,26 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
   __shared__ float s_eps;
   __shared__ unsigned long long s_total;
   __shared__ Plan s_pl;  // copy for the outlined slow path, which takes it by address
-  // Outlier-rich planes of many blocks are not restored by the warp that meets them (one lane per block:
-  // nblk / 32 rounds of a long serial walk while the CTA's other warps wait at the exit) but put on this list
-  // and restored afterwards by the whole CTA, one lane per block.
-  constexpr uint32_t kDeferCap = 64;
-  __shared__ uint32_t s_defer[kDeferCap];
-  __shared__ uint32_t s_ndefer;
-  const uint32_t tid = threadIdx.x;
+  __shared__ uint32_t s_nsal, s_list[kThreads], s_nlist;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   if (tid == 0) {
     s_pl = pl;
-    s_ndefer = 0;
+    s_nlist = 0;
   }
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
   dep_wait();     // the previous kernel on the stream (the one that wrote the container) has completed
   const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
   const uint8_t* src = a.src_base + off_in;
   const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;
-  const Team team = make_team(TT, s_red);
-  constexpr uint32_t kTeams = kThreads / TT;
-  const uint32_t my_team = tid / TT, lane = team.lane;
 
   // header check (every CTA, it is 64 bytes)
   if (tid == 0) {
     uint32_t bits = 0;
     float eps = 0.0f;
     unsigned long long total = 0;
-    s_hdr_ok = check_header(pl, src, src_bytes, bits, eps, total);
+    uint32_t nsal = 0;
+    s_hdr_ok = check_header(pl, src, src_bytes, bits, eps, total, nsal);
+    s_nsal = nsal;
     s_bits = bits;
     s_eps = eps;
     s_total = total;
@@ -395,131 +662,120 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
   bool bad = !hdr_ok;
   if (hdr_ok) {
     const uint32_t bits = s_bits;
-    const float eps = s_eps;
     const unsigned long long total = s_total;
     const uint32_t npay = a16(4u * ((pl.HW * bits + 31u) / 32u));
     const unsigned long long slots_off = 64ull + 16ull * pl.P, ovf_off = slots_off + pl.P * (unsigned long long)npay;
-    const bool vec = (pl.plane_bytes & (DT == kF32 ? 15u : 7u)) == 0u;  // dst base is 16-byte aligned
-    const uint32_t nfull = vec ? pl.HW >> 2 : 0u;                       // groups restored with vector stores
-    // Work items are (plane, chunk of 8 * TT groups) pairs so that large planes spread over many
-    // teams; a salient or raw plane is restored as a whole by the team that draws its first chunk.
-    const uint32_t chunk_groups = 8u * TT;
-    const uint32_t chunks = (pl.groups + chunk_groups - 1u) / chunk_groups;
-    // Team t takes items t, t + stride, ...  The stride is a prime (teams beyond it stay idle), so that a
-    // periodic pattern of expensive planes -- every eighth channel outlier-rich, say -- spreads over all
-    // teams instead of landing on the few whose index shares a factor with the period.
-    const uint64_t items = pl.P * chunks, stride = a.team_stride;
-    const uint64_t first = (uint64_t)blockIdx.x * kTeams + my_team;
-    for (uint64_t item = first < stride ? first : items; item < items; item += stride) {
-      const uint64_t gp = item / chunks;
-      const uint32_t ch = (uint32_t)(item - gp * chunks);
-      const uint32_t g0 = ch * chunk_groups, g1 = min(nfull, g0 + chunk_groups);
-      // whole-warp teams: the chunk's code words are requested before the table entry is known (the slot
-      // sits at a closed-form offset; what a salient plane keeps there is read and dropped)
+    constexpr uint32_t VE = DT == kF32 ? 4u : 8u;
+    const bool aligned = (pl.plane_bytes & 15u) == 0u;  // (dst is 16-byte aligned)
+    const uint32_t chunks = (pl.HW + (aligned ? 0u : VE - 1u) + 1023u) >> 10;
+    const uint32_t items = (uint32_t)pl.P * chunks, stride = (uint32_t)a.team_stride;
+    const uint32_t first = blockIdx.x * kWarps + warp;
+    for (uint32_t item = first < stride ? first : items; item < items; item += stride) {
+      const uint32_t gp = item / chunks, ch = item - gp * chunks;
+      const uint32_t g0 = ch * 256u, g1 = min(pl.groups, g0 + 256u);
+      const uint8_t* slot = src + slots_off + (uint64_t)gp * npay;
+      // the chunk's code words are requested before the table entry is known (the slot sits at a closed-form offset;
+      // what a salient plane keeps there is read and dropped)
       uint32_t cw[8];
-      if (TT == 32) {
-        const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src + slots_off + gp * npay);
+      if (aligned) {
+        const uint32_t* s32 = reinterpret_cast<const uint32_t*>(slot);
         const uint32_t nwords = npay >> 2, w0 = (g0 * bits) >> 3, per = bits;  // words per lane: 2, 4 or 8
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const uint32_t i = w0 + (uint32_t)j * 32u + lane;
           cw[j] = ((uint32_t)j < per && i < nwords) ? __ldg(s32 + i) : 0u;
         }
-      } else {  // sub-warp teams: one code word (1, 2 or 4 bytes) per group, the plane is one chunk
-        const uint8_t* sl = src + slots_off + gp * npay;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint32_t g = lane + (uint32_t)k * TT;
-          uint32_t w = 0;
-          if (g < pl.groups)
-            w = bits == 2u ? (uint32_t)__ldg(sl + g)
-                           : (bits == 4u ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(sl) + g)
-                                         : __ldg(reinterpret_cast<const uint32_t*>(sl) + g));
-          cw[k] = w;
-        }
       }
       const uint4 e = __ldg(reinterpret_cast<const uint4*>(src + 64) + gp);
       const unsigned long long off = (unsigned long long)e.x * 16ull;
       const uint32_t cls = e.y & 3u;
       uint8_t* out = a.dst + gp * pl.plane_bytes;
-      const uint8_t* slot = src + slots_off + gp * npay;
       if (cls == kClsNormal) {
-        if (off != slots_off + gp * npay) { bad = true; continue; }
+        if (off != slots_off + (uint64_t)gp * npay) {
+          bad = true;
+          continue;
+        }
         const float lo = __uint_as_float(e.z), scale = __uint_as_float(e.w);
-        if (TT == 32 && DT == kBF16 && (pl.plane_bytes & 15u) == 0u) {
+        if (!aligned) {
+          const uint32_t shift = ((uint32_t)(gp * pl.plane_bytes) & 15u) / (DT == kF32 ? 4u : 2u), v0 = ch * (1024u / VE);
+          if (bits == 2u) decode_chunk_shifted<DT, 2>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
+          else if (bits == 4u) decode_chunk_shifted<DT, 4>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
+          else decode_chunk_shifted<DT, 8>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
+        } else if (DT == kBF16) {
           if (bits == 2u) decode_chunk32_bf16_pairs<2>(cw, lane, g0, g1, scale, lo, out);
           else if (bits == 4u) decode_chunk32_bf16_pairs<4>(cw, lane, g0, g1, scale, lo, out);
           else decode_chunk32_bf16_pairs<8>(cw, lane, g0, g1, scale, lo, out);
-        } else if (TT == 32) {
+        } else {
           if (bits == 2u) decode_chunk32<DT, 2>(cw, lane, g0, g1, scale, lo, out);
           else if (bits == 4u) decode_chunk32<DT, 4>(cw, lane, g0, g1, scale, lo, out);
           else decode_chunk32<DT, 8>(cw, lane, g0, g1, scale, lo, out);
-        } else if (bits == 2u) decode_small<DT, 2, TT>(cw, lane, pl.groups, nfull, pl.HW, scale, lo, out);
-        else if (bits == 4u) decode_small<DT, 4, TT>(cw, lane, pl.groups, nfull, pl.HW, scale, lo, out);
-        else decode_small<DT, 8, TT>(cw, lane, pl.groups, nfull, pl.HW, scale, lo, out);
-        if (TT == 32 && ch == chunks - 1u && nfull * 4u < pl.HW) {  // ragged or unaligned rest: element stores
-          const uint32_t L = (1u << bits) - 1u;
-          for (uint32_t i = nfull * 4u + lane; i < pl.HW; i += TT) {
-            const uint32_t bit = i * bits;
-            const uint32_t q = (__ldg(reinterpret_cast<const uint32_t*>(slot) + (bit >> 5)) >> (bit & 31u)) & L;
-            store_elem<DT>(out, i, dequant(q, scale, lo));
-          }
         }
-      } else if (cls == kClsRaw || cls == kClsSalient) {
-        if (ch != 0) continue;
+      } else if (cls == kClsRaw) {
         // the continuation, when there is one, lies in the overflow region
-        if (off != 0 && (off < ovf_off || off > total)) { bad = true; continue; }
+        const unsigned long long ovf_avail = off ? total - off : 0ull;
+        if ((off != 0 && (off < ovf_off || off > total)) || (pl.plane_bytes > npay && pl.plane_bytes - npay > ovf_avail)) {
+          bad = true;
+          continue;
+        }
         SplitIn in;
         in.slot = slot;
         in.ovf = src + off;
         in.npay = npay;
-        const unsigned long long ovf_avail = off ? total - off : 0ull;
-        if (cls == kClsRaw) {
-          if (pl.plane_bytes > npay && pl.plane_bytes - npay > ovf_avail) { bad = true; continue; }
-          for (uint32_t i = lane; i < (uint32_t)(pl.plane_bytes >> 1); i += TT)
-            reinterpret_cast<uint16_t*>(out)[i] = (uint16_t)in.ld16(2u * i);
-        } else {
-          if (DEFER) {
-            uint32_t at = 0;
-            if (lane == 0) at = atomicAdd(&s_ndefer, 1u);
-            at = __shfl_sync(0xFFFFFFFFu, at, 0);
-            if (at < kDeferCap) {
-              if (lane == 0) s_defer[at] = (uint32_t)gp;
-              continue;
-            }
-          }
-          uint32_t* scr = reinterpret_cast<uint32_t*>(smem + (uint64_t)my_team * pl.sal_stride);
-          if (!decode_salient<DT>(team, s_pl, in, ovf_avail, eps, out, scr, s_hdr_ok)) bad = true;
-        }
-      } else {
+        const uint32_t i1 = min(pl.HW * (DT == kF32 ? 2u : 1u), (ch + 1u) * (DT == kF32 ? 2048u : 1024u));
+        for (uint32_t i = ch * (DT == kF32 ? 2048u : 1024u) + lane; i < i1; i += 32u)
+          reinterpret_cast<uint16_t*>(out)[i] = (uint16_t)in.ld16(2u * i);
+      } else if (cls != kClsSalient || s_nsal == 0u) {
         bad = true;
       }
     }
-  }
-  if (DEFER && hdr_ok) {  // (uniform over the CTA)
-    __syncthreads();
-    const uint32_t n = min(s_ndefer, kDeferCap);
-    const Team cta = make_team(kThreads, s_red);
-    const uint32_t bits = s_bits;
-    const uint32_t npay = a16(4u * ((pl.HW * bits + 31u) / 32u));
-    const unsigned long long total = s_total;
-    const unsigned long long slots_off = 64ull + 16ull * pl.P, ovf_off = slots_off + pl.P * (unsigned long long)npay;
-    for (uint32_t q = 0; q < n; ++q) {
-      const uint64_t gp = s_defer[q];
-      const uint4 e = __ldg(reinterpret_cast<const uint4*>(src + 64) + gp);
-      const unsigned long long off = (unsigned long long)e.x * 16ull;
-      if (off != 0 && (off < ovf_off || off > total)) {  // (the same for every thread)
-        bad = true;
-        continue;
+    // the outlier-rich planes, from up to 256 table entries at a time
+    if (s_nsal) {
+      const uint32_t hop = (uint32_t)a.cta_stride, most = blockIdx.x < hop ? ((uint32_t)pl.P + hop - 1u) / hop : 0u;
+      const Team unit = pl.team == 32u ? make_warp_team(s_red) : make_team(kThreads, s_red);
+      uint32_t* scr = reinterpret_cast<uint32_t*>(smem + (pl.team == 32u ? (uint64_t)warp * pl.sal_stride : 0ull));
+      for (uint32_t base = 0; base < most; base += kThreads) {
+        const uint64_t gp = blockIdx.x + (uint64_t)(base + tid) * hop;
+        if (gp < pl.P && (__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp) + 1) & 3u) == kClsSalient)
+          s_list[atomicAdd(&s_nlist, 1u)] = (uint32_t)gp;
+        __syncthreads();
+        const uint32_t n = s_nlist;
+        for (uint32_t q = pl.team == 32u ? warp : 0u; q < n; q += pl.team == 32u ? (uint32_t)kWarps : 1u) {
+          const uint32_t gp = s_list[q];
+          const unsigned long long off = (unsigned long long)__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp)) * 16ull;
+          if (off != 0 && (off < ovf_off || off > total)) {  // (the same for every thread of the unit)
+            bad = true;
+            continue;
+          }
+          SplitIn in;
+          in.slot = src + slots_off + (uint64_t)gp * npay;
+          in.ovf = src + off;
+          in.npay = npay;
+          // the payload comes to shared memory first when it fits there
+          const unsigned long long ovf_avail = off ? total - off : 0ull;
+          const uint32_t got = (uint32_t)min((unsigned long long)pl.pay_bytes, npay + (ovf_avail & ~15ull));
+          const uint32_t nnz_s = in.ld32(0), n_dense = in.ld32(4), n_out_d = in.ld32(8), coded = in.ld32(12), es = (uint32_t)pl.esize;
+          const uint64_t size = 16ull + 4ull * pl.nbm + 4ull * ((uint64_t)pl.H + 1) + a4(2u * nnz_s) + a4(es * nnz_s) +
+                                (coded ? (uint64_t)coded : 64ull * n_dense) + a4(es * n_out_d);
+          uint8_t* pay = reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes;
+          bool good;
+          if (nnz_s <= pl.HW && n_dense <= pl.nblk && n_out_d <= pl.HW && size <= got) {
+            for (uint32_t o = 16u * unit.lane; o < (uint32_t)size; o += 16u * unit.size)
+              *reinterpret_cast<uint4*>(pay + o) = __ldg(reinterpret_cast<const uint4*>(in.at(o)));
+            team_sync(unit);
+            FlatIn flat;
+            flat.p = pay;
+            flat.npay = got;
+            good = decode_salient<DT>(unit, s_pl, flat, 0ull, s_eps, a.dst + gp * pl.plane_bytes, scr, s_hdr_ok);
+          } else {
+            good = decode_salient<DT>(unit, s_pl, in, ovf_avail, s_eps, a.dst + gp * pl.plane_bytes, scr, s_hdr_ok);
+          }
+          if (!good) bad = true;
+          team_sync(unit);  // the scratch is reused
+        }
+        __syncthreads();
+        if (tid == 0) s_nlist = 0;
+        __syncthreads();
       }
-      SplitIn in;
-      in.slot = src + slots_off + gp * npay;
-      in.ovf = src + off;
-      in.npay = npay;
-      if (!decode_salient<DT>(cta, s_pl, in, off ? total - off : 0ull, s_eps, a.dst + gp * pl.plane_bytes,
-                              reinterpret_cast<uint32_t*>(smem), s_hdr_ok))
-        bad = true;
-      __syncthreads();  // the scratch is reused
     }
   }
   decompress_exit(a, bad);
@@ -532,137 +788,6 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
 // normal plane, the whole warp for an outlier-rich one -- and the tile leaves as one bulk (TMA) store.
 // Tiles (256 / team planes) start on 16-byte boundaries; two buffers alternate.
 // -------------------------------------------------------------------------------------------------
-
-// Outlier-rich plane of at most four blocks and fewer than 32 rows, restored by one warp: CSR scatter, then per
-// dense block the inverse of the Lorenzo prediction as a two-dimensional prefix sum of the residuals over the
-// warp's lanes (lane l holds raster positions l and l + 32), corrected in raster order for every verbatim
-// element, whose k follows from its stored value.  The result is that of the raster walk in decode_salient.
-// A payload copied to shared memory as one piece.
-struct FlatIn {
-  const uint8_t* p;
-  uint32_t npay;  // (kept for the size check: bytes of the payload that came from the slot)
-  __device__ __forceinline__ uint32_t ld32(uint32_t o) const { return *reinterpret_cast<const uint32_t*>(p + o); }
-  __device__ __forceinline__ uint32_t ld16(uint32_t o) const { return *reinterpret_cast<const uint16_t*>(p + o); }
-};
-
-template <int DT, typename In>
-__device__ __forceinline__ bool small_decode(const Plan& pl, const In& in, uint64_t ovf_avail, float eps, uint8_t* out) {
-  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu;
-  const uint32_t H = (uint32_t)pl.H, W = (uint32_t)pl.W, nblk = pl.nblk, nbx = pl.nbx, e = (uint32_t)pl.esize, HW = pl.HW;
-  const uint32_t nnz_s = in.ld32(0), n_dense = in.ld32(4), n_out_d = in.ld32(8);
-  if (nnz_s > HW || n_dense > nblk || n_out_d > HW) return false;
-  const uint64_t size = 16ull + 4ull * pl.nbm + 4ull * ((uint64_t)H + 1) + a4(2u * nnz_s) + a4(e * nnz_s) +
-                        64ull * n_dense + a4(e * n_out_d);
-  if (size > in.npay && size - in.npay > ovf_avail) return false;
-  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * pl.nbm, o_col = o_rp + 4u * (H + 1u);
-  const uint32_t o_val = o_col + a4(2u * nnz_s), o_codes = o_val + a4(e * nnz_s), o_outl = o_codes + 64u * n_dense;
-  const uint32_t bitmap = in.ld32(o_bm) & ((1u << nblk) - 1u);
-  if ((uint32_t)__popc(bitmap) != n_dense) return false;
-  bool ok = true;
-  for (uint32_t i = lane; i < (uint32_t)(pl.plane_bytes >> 1); i += 32u) reinterpret_cast<uint16_t*>(out)[i] = 0;
-  __syncwarp();
-  if (lane < H) {  // CSR scatter, a lane per row
-    const uint32_t r0 = in.ld32(o_rp + 4u * lane), r1 = in.ld32(o_rp + 4u * lane + 4u);
-    if (r0 > r1 || r1 > nnz_s) {
-      ok = false;
-    } else {
-      for (uint32_t k = r0; k < r1; ++k) {
-        const uint32_t col = in.ld16(o_col + 2u * k);
-        if (col >= W) {
-          ok = false;
-          continue;
-        }
-        const uint32_t idx = lane * W + col;
-        if (DT == kF32) reinterpret_cast<uint32_t*>(out)[idx] = in.ld32(o_val + 4u * k);
-        else reinterpret_cast<uint16_t*>(out)[idx] = (uint16_t)in.ld16(o_val + 2u * k);
-      }
-    }
-  }
-  const float two_eps = __fmul_rn(2.0f, eps), inv2e = __fdiv_rn(1.0f, two_eps);
-  const uint32_t c = lane & 7u, r0 = lane >> 3, lt = (1u << lane) - 1u;
-  uint32_t oi = 0, rank = 0;
-#pragma unroll 1
-  for (uint32_t b = 0; b < nblk; ++b) {
-    if (!((bitmap >> b) & 1u)) continue;
-    const uint32_t oc = o_codes + 64u * rank;
-    const uint32_t code0 = (in.ld32(oc + (lane & ~3u)) >> (8u * (lane & 3u))) & 0xFFu;
-    const uint32_t code1 = (in.ld32(oc + 32u + (lane & ~3u)) >> (8u * (lane & 3u))) & 0xFFu;
-    const uint32_t by = b / nbx, bx = b - by * nbx;
-    const uint32_t y0 = by * 8u + r0, x = bx * 8u + c;
-    const bool in0 = y0 < H && x < W, in1 = y0 + 4u < H && x < W;
-    const bool v0 = in0 && code0 == 0u, v1 = in1 && code1 == 0u;
-    int32_t k0 = (in0 && !v0) ? (int32_t)code0 - 128 : 0, k1 = (in1 && !v1) ? (int32_t)code1 - 128 : 0;
-#pragma unroll
-    for (uint32_t o = 1; o < 8u; o <<= 1) {  // along the rows
-      const int32_t t0 = __shfl_up_sync(full, k0, o), t1 = __shfl_up_sync(full, k1, o);
-      if (c >= o) {
-        k0 += t0;
-        k1 += t1;
-      }
-    }
-#pragma unroll
-    for (uint32_t o = 8; o < 32u; o <<= 1) {  // down the columns, within each half
-      const int32_t t0 = __shfl_up_sync(full, k0, o), t1 = __shfl_up_sync(full, k1, o);
-      if (lane >= o) {
-        k0 += t0;
-        k1 += t1;
-      }
-    }
-    k1 += __shfl_sync(full, k0, 24 + (int)c);  // rows 4-7 continue below row 3
-    const uint32_t m0 = __ballot_sync(full, v0), m1 = __ballot_sync(full, v1);
-    const uint32_t nv = (uint32_t)(__popc(m0) + __popc(m1));
-    if (oi + nv > n_out_d) return false;  // (the same for every lane)
-    uint32_t raw0 = 0, raw1 = 0;
-    int32_t kv0 = 0, kv1 = 0;
-    if (v0) {
-      const uint32_t at = oi + (uint32_t)__popc(m0 & lt);
-      raw0 = DT == kF32 ? in.ld32(o_outl + 4u * at) : in.ld16(o_outl + 2u * at);
-      bool big;
-      kv0 = dense_k(DT == kF32 ? __uint_as_float(raw0) : bf16_bits_to_f32(raw0), inv2e, &big);
-    }
-    if (v1) {
-      const uint32_t at = oi + (uint32_t)__popc(m0) + (uint32_t)__popc(m1 & lt);
-      raw1 = DT == kF32 ? in.ld32(o_outl + 4u * at) : in.ld16(o_outl + 2u * at);
-      bool big;
-      kv1 = dense_k(DT == kF32 ? __uint_as_float(raw1) : bf16_bits_to_f32(raw1), inv2e, &big);
-    }
-    // a verbatim element replaces its k: the difference moves every k below and to the right of it
-    for (uint32_t mm = m0; mm; mm &= mm - 1u) {
-      const uint32_t src = (uint32_t)__ffs((int)mm) - 1u, i = src >> 3, j = src & 7u;
-      const int32_t diff = __shfl_sync(full, kv0 - k0, (int)src);
-      if (c >= j) {
-        if (r0 >= i) k0 += diff;
-        k1 += diff;
-      }
-    }
-    for (uint32_t mm = m1; mm; mm &= mm - 1u) {
-      const uint32_t src = (uint32_t)__ffs((int)mm) - 1u, i = src >> 3, j = src & 7u;
-      const int32_t diff = __shfl_sync(full, kv1 - k1, (int)src);
-      if (c >= j && r0 >= i) k1 += diff;
-    }
-    if (in0) {
-      const uint32_t idx = y0 * W + x;
-      if (v0) {
-        if (DT == kF32) reinterpret_cast<uint32_t*>(out)[idx] = raw0;
-        else reinterpret_cast<uint16_t*>(out)[idx] = (uint16_t)raw0;
-      } else {
-        store_elem<DT>(out, idx, __fmul_rn((float)k0, two_eps));
-      }
-    }
-    if (in1) {
-      const uint32_t idx = (y0 + 4u) * W + x;
-      if (v1) {
-        if (DT == kF32) reinterpret_cast<uint32_t*>(out)[idx] = raw1;
-        else reinterpret_cast<uint16_t*>(out)[idx] = (uint16_t)raw1;
-      } else {
-        store_elem<DT>(out, idx, __fmul_rn((float)k1, two_eps));
-      }
-    }
-    oi += nv;
-    ++rank;
-  }
-  return __all_sync(full, ok);
-}
 
 template <int DT>
 __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, const DecompressArgs a) {
@@ -683,7 +808,8 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
     uint32_t bits = 0;
     float eps = 0.0f;
     unsigned long long total = 0;
-    s_hdr_ok = check_header(pl, src, src_bytes, bits, eps, total);
+    uint32_t nsal = 0;
+    s_hdr_ok = check_header(pl, src, src_bytes, bits, eps, total, nsal);
     s_bits = bits;
     s_eps = eps;
     s_total = total;
@@ -700,7 +826,6 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
     const Team warp_team = make_warp_team(s_red);
     const bool vec = (pl.plane_bytes & (DT == kF32 ? 15u : 7u)) == 0u;  // planes start on vector boundaries in the tile buffer
     const uint32_t tile_bytes_max = pl.stage_bytes;
-    const uint32_t pay_stride = pl.sal_stride;  // per-warp scratch: a small plane's payload, or the general path's tables
     uint32_t buf = 0;
     for (uint32_t tile = blockIdx.x; tile < pl.ntiles; tile += gridDim.x, buf ^= 1u) {
       uint8_t* tbuf = smem + (uint64_t)buf * tile_bytes_max;
@@ -709,10 +834,12 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
       const uint64_t p0 = (uint64_t)tile * pl.ppt;
       const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
       const uint32_t lp = my_team;
-      bool salient = false;
+      bool salient = false, raw = false;
+      uint32_t my_off16 = 0;
       if (lp < np) {
         const uint64_t gp = p0 + lp;
         const uint4 en = __ldg(reinterpret_cast<const uint4*>(src + 64) + gp);
+        my_off16 = en.x;
         const unsigned long long off = (unsigned long long)en.x * 16ull;
         const uint32_t cls = en.y & 3u;
         uint8_t* out = tbuf + (uint64_t)lp * pl.plane_bytes;
@@ -738,65 +865,78 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
             }
           }
         } else if (cls == kClsRaw) {
-          if (off != 0 && (off < ovf_off || off > total)) {
-            bad = true;
-          } else {
-            SplitIn in;
-            in.slot = slot;
-            in.ovf = src + off;
-            in.npay = npay;
-            const unsigned long long ovf_avail = off ? total - off : 0ull;
-            if (pl.plane_bytes > npay && pl.plane_bytes - npay > ovf_avail) bad = true;
-            else
-              for (uint32_t i = lane; i < (uint32_t)(pl.plane_bytes >> 1); i += tt)
-                reinterpret_cast<uint16_t*>(out)[i] = (uint16_t)in.ld16(2u * i);
-          }
+          const unsigned long long ovf_avail = off ? total - off : 0ull;
+          raw = !((off != 0 && (off < ovf_off || off > total)) || (pl.plane_bytes > npay && pl.plane_bytes - npay > ovf_avail));
+          if (!raw) bad = true;
         } else if (cls == kClsSalient) {
           salient = true;
         } else {
           bad = true;
         }
       }
-      // outlier-rich planes of the warp's slice: the whole warp restores them one after the other
-      for (uint32_t m = __ballot_sync(0xFFFFFFFFu, salient && lane == 0); m; m &= m - 1u) {
-        const uint32_t slp = (tid & ~31u) / tt + ((uint32_t)__ffs((int)m) - 1u) / tt;
-        const uint64_t gp = p0 + slp;
-        const unsigned long long off = (unsigned long long)__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp)) * 16ull;
-        if (off != 0 && (off < ovf_off || off > total)) {
-          bad = true;
-          continue;
+      // raw planes of the warp's slice, one after the other by the whole warp, a word per lane
+      for (uint32_t m = __ballot_sync(0xFFFFFFFFu, raw && lane == 0); m; m &= m - 1u) {
+        const uint32_t first = (uint32_t)__ffs((int)m) - 1u, rlp = (tid & ~31u) / tt + first / tt;
+        SplitIn in;
+        in.slot = src + slots_off + (p0 + rlp) * npay;
+        in.ovf = src + (unsigned long long)__shfl_sync(0xFFFFFFFFu, my_off16, (int)first) * 16ull;
+        in.npay = npay;
+        uint8_t* out = tbuf + (uint64_t)rlp * pl.plane_bytes;
+        for (uint32_t o = 4u * wlane; o < (uint32_t)pl.plane_bytes; o += 128u) {  // (payloads are padded to 16 bytes)
+          const uint32_t w = in.ld32(o);
+          if (DT == kF32) {
+            *reinterpret_cast<uint32_t*>(out + o) = w;
+          } else {
+            *reinterpret_cast<uint16_t*>(out + o) = (uint16_t)w;
+            if (o + 2u < (uint32_t)pl.plane_bytes) *reinterpret_cast<uint16_t*>(out + o + 2u) = (uint16_t)(w >> 16);
+          }
         }
+      }
+      // outlier-rich planes of the warp's slice, by the whole warp: four at a time when a plane is one block, one after
+      // the other otherwise.  A payload (shorter than its plane, or it would have been stored raw) is copied to the
+      // warp's scratch in one go, before its header is known, and decoded from there.
+      uint32_t* scr = reinterpret_cast<uint32_t*>(smem + 2ull * tile_bytes_max + (uint64_t)(tid >> 5) * pl.sal_stride);
+      const bool four = pl.nblk == 1u;
+      const uint32_t pay_max = a16((uint32_t)pl.plane_bytes), per = four ? 8u : 32u;
+      uint8_t* pay = reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes + (four ? (wlane >> 3) * (pay_max + 16u) : 0u);
+      for (uint32_t m = __ballot_sync(0xFFFFFFFFu, salient && lane == 0); m;) {
+        uint32_t mm = m;  // the lane's plane: the (lane / 8)-th or the first of those that are left
+        for (uint32_t k = 0; k < (four ? wlane >> 3 : 0u); ++k) mm &= mm - 1u;
+        for (uint32_t k = 0; k < (four ? 4u : 1u); ++k) m &= m - 1u;
+        const bool there = mm != 0u;
+        const uint32_t first = there ? (uint32_t)__ffs((int)mm) - 1u : 0u, slp = (tid & ~31u) / tt + first / tt;
+        const uint64_t gp = p0 + slp;
+        const unsigned long long off = (unsigned long long)__shfl_sync(0xFFFFFFFFu, my_off16, (int)first) * 16ull;
+        const bool use = there && !(off != 0 && (off < ovf_off || off > total));
+        if (there && !use) bad = true;
         SplitIn in;
         in.slot = src + slots_off + gp * npay;
         in.ovf = src + off;
         in.npay = npay;
-        uint8_t* out = tbuf + (uint64_t)slp * pl.plane_bytes;
         const unsigned long long ovf_avail = off ? total - off : 0ull;
+        const uint32_t avail = use ? (uint32_t)min((unsigned long long)pay_max, npay + (ovf_avail & ~15ull)) : 0u;
+        for (uint32_t o = 16u * (wlane & (per - 1u)); o < avail; o += 16u * per)
+          *reinterpret_cast<uint4*>(pay + o) = __ldg(reinterpret_cast<const uint4*>(in.at(o)));
         __syncwarp();
-        bool good;
-        if (pl.nblk <= 4u && pl.H < 32 && in.ld32(12) == 0u) {  // (a Huffman-coded plane takes the general path)
-          // the payload (shorter than the plane, or it would have been stored raw) is fetched in one go into the
-          // warp's scratch and decoded from there
-          uint8_t* pay = smem + 2ull * tile_bytes_max + (uint64_t)(tid >> 5) * pay_stride;
-          const uint32_t nnz_s = in.ld32(0), n_dense = in.ld32(4), n_out_d = in.ld32(8), es = (uint32_t)pl.esize;
-          const uint64_t size = 16ull + 4ull * pl.nbm + 4ull * ((uint64_t)pl.H + 1) + a4(2u * nnz_s) + a4(es * nnz_s) +
-                                64ull * n_dense + a4(es * n_out_d);
-          good = nnz_s <= pl.HW && n_dense <= pl.nblk && n_out_d <= pl.HW && size <= pay_stride &&
-                 !(size > npay && size - npay > ovf_avail);
-          if (good) {
-            for (uint32_t o = 4u * wlane; o < (uint32_t)size; o += 128u) *reinterpret_cast<uint32_t*>(pay + o) = in.ld32(o);
+        FlatIn flat;
+        flat.p = pay;
+        flat.npay = avail;  // (what was copied: a payload longer than that is no salient plane's)
+        uint8_t* out = tbuf + (uint64_t)slp * pl.plane_bytes;
+        const bool coded = use && flat.ld32(12) != 0u;
+        if (pl.nblk <= 4u && !__any_sync(0xFFFFFFFFu, coded)) {
+          if (!(four ? decode_few<DT, true>(s_pl, flat, avail, use, eps, out) : decode_few<DT, false>(s_pl, flat, avail, use, eps, out)))
+            bad = true;
+        } else {  // planes of more blocks, and Huffman-coded ones (one after the other)
+          for (uint32_t k = 0; k < 32u; k += per) {
+            if (!__shfl_sync(0xFFFFFFFFu, use, (int)k)) continue;
+            uint8_t* to = (uint8_t*)__shfl_sync(0xFFFFFFFFu, (unsigned long long)out, (int)k);
+            FlatIn one;
+            one.p = (const uint8_t*)__shfl_sync(0xFFFFFFFFu, (unsigned long long)flat.p, (int)k);
+            one.npay = __shfl_sync(0xFFFFFFFFu, avail, (int)k);
+            if (!decode_salient<DT>(warp_team, s_pl, one, 0ull, eps, to, scr, s_hdr_ok)) bad = true;
             __syncwarp();
-            FlatIn flat;
-            flat.p = pay;
-            flat.npay = npay;
-            good = small_decode<DT>(s_pl, flat, ovf_avail, eps, out);
           }
-        } else {
-          good = decode_salient<DT>(warp_team, s_pl, in, ovf_avail, eps, out,
-                                    reinterpret_cast<uint32_t*>(smem + 2ull * tile_bytes_max + (uint64_t)(tid >> 5) * pl.sal_stride),
-                                    s_hdr_ok);
         }
-        if (!good) bad = true;
         __syncwarp();
       }
       __syncthreads();

@@ -58,6 +58,7 @@ struct Plan {
   // block-wise path (outlier-rich planes): measuring scratch of one unit (a warp, or the whole CTA)
   uint32_t sm_sal;          // byte offset of the first measuring area in dynamic shared memory
   uint32_t sal_stride;      // bytes between the areas of consecutive units
+  uint32_t pay_bytes;       // decompress: bytes at the end of an area that hold payloads
 };
 
 // Book-keeping scratch, one per stream: a header of counters and three arrays for the plane-ordered
@@ -573,6 +574,11 @@ __device__ __forceinline__ uint32_t team_excl_scan(const Team& t, uint32_t* arr,
   return total;
 }
 
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+  for (uint32_t o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+
 // ------------------------------------------------------------------------------------------------
 // Huffman stage on the residual code bytes of an outlier-rich plane's dense blocks (entropy = 1)
 // ------------------------------------------------------------------------------------------------
@@ -582,6 +588,7 @@ __device__ __forceinline__ uint32_t team_excl_scan(const Team& t, uint32_t* arr,
 // most significant first.  Section: u8 len(0) | u8 smin | u8 smax | u8 0 | u8 len(smin..smax) (pad 4) |
 // u8 bytes of each chunk (pad 4) | chunks (pad 4).  Lengths stay below 25 (a plane has fewer than 2^17 codes).
 constexpr uint32_t kHufMaxLen = 24;
+constexpr uint32_t kHufLutBits = 10;     // decoder: with 60 symbols about one code in a hundred is longer
 constexpr uint32_t kHufStageWords = 48;  // a chunk has at most 64 * 24 / 8 = 192 bytes
 
 // Encoder scratch of one unit (shared memory).
@@ -691,42 +698,76 @@ static __device__ __noinline__ void huffman_build(HufEncode* h) {
 
 // Decoder tables of one unit (shared memory), from the lengths stored in a section.
 struct HufDecode {
-  uint32_t first[kHufMaxLen + 1];   // first code value of every length
-  uint16_t count[kHufMaxLen + 1];   // symbols of every length
-  uint16_t base[kHufMaxLen + 1];    // index of a length's first symbol in `sorted`
-  uint8_t sorted[256];              // symbols by (length, symbol)
+  uint32_t count[32];   // symbols of every length
+  uint32_t limit[32];   // end of a length's codes, left-aligned (2^32, the end of the longest's, as all ones)
+  uint32_t base[32];    // index of a length's first symbol in `sorted`, less the length's first code value
+  uint16_t lut[1 << kHufLutBits];  // by the next bits: length << 8 | symbol of a code of at most so many bits, 0 otherwise
+  uint8_t sorted[256];  // symbols by (length, symbol)
   uint8_t len[256];
-  uint32_t ok;
+  uint32_t maxlen, ok;
 };
-// One thread: tables from t->len; t->ok = 0 unless the lengths form a complete prefix code (or a single code of any length).
+// A whole warp: tables from t->len; t->ok = 0 unless the lengths form a complete prefix code (or a single code of any length).
 static __device__ __noinline__ void huffman_tables(HufDecode* t) {
-  for (uint32_t l = 0; l <= kHufMaxLen; ++l) t->count[l] = 0;
-  unsigned long long kraft = 0;  // in units of 2^-32
-  uint32_t nsym = 0;
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, lt = (1u << lane) - 1u;
   bool bad = false;
-  for (uint32_t sym = 0; sym < 256u; ++sym) {
-    const uint32_t l = t->len[sym];
-    if (l > kHufMaxLen) bad = true;
-    else if (l) {
-      ++t->count[l];
-      kraft += 1ull << (32u - l);
-      ++nsym;
+  t->count[lane] = 0;
+  __syncwarp();
+  uint32_t rank[8];  // of the lane's symbols among those of the same length
+#pragma unroll
+  for (uint32_t i = 0; i < 8u; ++i) {
+    const uint32_t l = t->len[i * 32u + lane];
+    bad |= l > kHufMaxLen;
+    const uint32_t lc = min(l, 31u), same = __match_any_sync(full, lc), used = t->count[lc];
+    rank[i] = used + __popc(same & lt);
+    __syncwarp();
+    if ((same & lt) == 0u) t->count[lc] = used + __popc(same);
+    __syncwarp();
+  }
+  bad = __any_sync(full, bad);
+  const uint32_t n = lane >= 1u && lane <= kHufMaxLen ? t->count[lane] : 0u;
+  uint32_t incl = n;
+#pragma unroll
+  for (uint32_t o = 1; o < 32u; o <<= 1) {
+    const uint32_t up = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += up;
+  }
+  const uint32_t nsym = __shfl_sync(full, incl, 31);
+  const unsigned long long kraft = warp_sum_u64((unsigned long long)n << (32u - min(lane, 32u)));  // in units of 2^-32
+  if (nsym == 0u || kraft > (1ull << 32) || (nsym > 1u && kraft != (1ull << 32))) bad = true;
+  __syncwarp();
+  if (lane == 0) {
+    t->count[0] = 0;
+    t->ok = bad ? 0u : 1u;
+  }
+  const uint32_t longest = __ballot_sync(full, n != 0u);
+  __syncwarp();
+  uint32_t first = 0;
+  for (uint32_t k = 1; k < lane && k <= kHufMaxLen; ++k) first += t->count[k] << (lane - k);
+  const uint32_t index = incl - n;
+  t->base[lane] = index - first;
+  const unsigned long long lim = (unsigned long long)(first + n) << (32u - min(max(lane, 1u), 31u));
+  t->limit[lane] = lim > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)lim;
+  if (lane == 0) t->maxlen = longest ? 31u - (uint32_t)__clz((int)longest) : 0u;
+  if (!bad) {
+#pragma unroll
+    for (uint32_t i = 0; i < 8u; ++i) {
+      const uint32_t l = t->len[i * 32u + lane];
+      const uint32_t at = __shfl_sync(full, index, (int)(l & 31u)) + rank[i];
+      if (l) t->sorted[at] = (uint8_t)(i * 32u + lane);
     }
   }
-  if (nsym == 0 || kraft > (1ull << 32) || (nsym > 1 && kraft != (1ull << 32))) bad = true;
-  uint32_t next = 0, prev = 0, idx = 0;
-  for (uint32_t l = 1; l <= kHufMaxLen; ++l) {
-    t->base[l] = (uint16_t)idx;
-    if (t->count[l]) {
-      next <<= (l - prev);
-      prev = l;
-    }
-    t->first[l] = next;
-    for (uint32_t sym = 0; sym < 256u && !bad; ++sym)
-      if (t->len[sym] == l) t->sorted[idx++] = (uint8_t)sym;
-    next += t->count[l];
+  __syncwarp();
+}
+// The look-up table, by all `n` threads of the team (this is thread `i`), once huffman_tables is through.
+__device__ __forceinline__ void huffman_lut(HufDecode* t, uint32_t i, uint32_t n) {
+  for (uint32_t bits = i; bits < (1u << kHufLutBits); bits += n) {
+    const uint32_t hi = bits << (32 - kHufLutBits);
+    uint32_t len = 1;
+#pragma unroll
+    for (uint32_t l = 1; l < kHufLutBits; ++l) len += hi >= t->limit[l] ? 1u : 0u;  // (limits ascend with the length)
+    const uint32_t at = (hi >> (32u - len)) + t->base[len];
+    t->lut[bits] = hi < t->limit[len] ? (uint16_t)(len << 8 | t->sorted[at & 255u]) : (uint16_t)0;
   }
-  t->ok = bad ? 0u : 1u;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -763,11 +804,6 @@ __device__ __forceinline__ void scan_publish(const Scan& s, uint32_t t, uint32_t
   if (t == s.skip_tile) return;
   st_relaxed(&s.tile[t], ((unsigned long long)s.epoch << 32) | U);
   atomicAdd(&s.grp[t >> 5], (1ull << 40) | (unsigned long long)U);
-}
-
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-  for (uint32_t o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  return v;
 }
 
 // A whole warp: sum of U over the tiles before t.  False when a wait ran out.
@@ -861,7 +897,8 @@ struct DecompressArgs {
   uint8_t* dst;
   unsigned long long* d_status;        // optional
   Scratch* sc;
-  unsigned long long team_stride;      // a prime, at most the number of teams of the grid (see the kernel)
+  unsigned long long team_stride;      // a prime, at most the number of warps of the grid (see decompress_kernel)
+  unsigned long long cta_stride;       // ... of CTAs
 };
 
 struct ChanStat {

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <map>
+#include <mutex>
 #include <tuple>
 
 #include "fh_device.cuh"
@@ -17,6 +18,13 @@ constexpr size_t kSmemLimit = 227 * 1024 - 4096;  // dynamic shared memory a CTA
 
 inline size_t A16(size_t x) { return (x + 15) & ~(size_t)15; }
 
+// Lanes of the team that works on a plane of so many groups, eight groups to a lane: a power of two, at most a warp.
+inline uint32_t team_of_groups(uint32_t groups) {
+  uint32_t t = 1;
+  while (t < 32u && t * 8u < groups) t *= 2u;
+  return t;
+}
+
 // Which kernel a plan runs on.
 struct Variant {
   bool fast = false;  // compress_warp / compress_cta (bulk-copy pipeline) instead of compress_generic
@@ -26,6 +34,9 @@ struct Variant {
 
 // SMs of the current device (0: none).
 int sm_count();
+
+// Largest prime <= n (n >= 2), or 1.  The caller holds the library's mutex.
+uint64_t prime_at_most(uint64_t n);
 
 // All of these enqueue on `stream` and return an fh_status; the caller holds the library's mutex.
 int launch_compress_warp_f32(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
@@ -65,6 +76,14 @@ int grid_for(K kernel, size_t smem, uint32_t ntiles, int* grid, int threads = fh
 // passes dep_wait() before it touches global memory, so stream order is kept.
 // Tiles a CTA requests at once when it starts: all its stages when every CTA of the grid gets that many, fewer
 // when the tensor is small, so that the tiles spread over all CTAs before any CTA takes a second one.
+// Grid of a compress kernel that hands out tiles in order: when every CTA gets several, a prime number of CTAs.  Equally
+// fast CTAs then take tiles c, c + grid, ..., and a periodic pattern of outlier-rich planes -- every eighth channel, say --
+// spreads over all of them instead of landing on the few whose index shares a factor with the period (with 296 CTAs and
+// period 8, 37 CTAs got every such plane of the bf16 112 x 112 tensor).
+inline int spread_grid(int grid, uint32_t ntiles) {
+  return ntiles >= 2u * (uint32_t)grid && grid >= 2 ? (int)prime_at_most((uint64_t)grid) : grid;
+}
+
 inline Plan with_first_request(const Plan& pl, int grid, uint32_t least) {
   Plan q = pl;
   const uint32_t each = pl.ntiles / (uint32_t)(grid > 0 ? grid : 1);

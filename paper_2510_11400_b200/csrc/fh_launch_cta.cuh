@@ -11,6 +11,7 @@ int launch_cta_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int grid = 0;
   int rc = grid_for(compress_cta<DT, SIGMA, NT>, pl.sm_total, pl.ntiles, &grid, NT);
   if (rc != FH_OK) return rc;
+  grid = spread_grid(grid, pl.ntiles);
   return launch_dependent(compress_cta<DT, SIGMA, NT>, grid, NT, pl.sm_total, stream, with_first_request(pl, grid, 2), a) == cudaSuccess
              ? FH_OK : FH_ERR_CUDA;
 }
@@ -21,11 +22,13 @@ int launch_cta_regs_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream
   if (pl.groups == (uint32_t)(NT * G)) {
     int rc = grid_for(compress_cta_regs<DT, SIGMA, NT, G, true>, pl.sm_total, pl.ntiles, &grid, NT);
     if (rc != FH_OK) return rc;
+    grid = spread_grid(grid, pl.ntiles);
     return launch_dependent(compress_cta_regs<DT, SIGMA, NT, G, true>, grid, NT, pl.sm_total, stream,
                             with_first_request(pl, grid, 2), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
   }
   int rc = grid_for(compress_cta_regs<DT, SIGMA, NT, G, false>, pl.sm_total, pl.ntiles, &grid, NT);
   if (rc != FH_OK) return rc;
+  grid = spread_grid(grid, pl.ntiles);
   return launch_dependent(compress_cta_regs<DT, SIGMA, NT, G, false>, grid, NT, pl.sm_total, stream,
                           with_first_request(pl, grid, 2), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }

@@ -11,6 +11,7 @@ int launch_warp_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int grid = 0;
   int rc = grid_for(compress_warp<DT, SIGMA, TT, FULLVEC>, pl.sm_total, pl.ntiles, &grid, kWarpKernelThreads);
   if (rc != FH_OK) return rc;
+  grid = spread_grid(grid, pl.ntiles);
   return launch_dependent(compress_warp<DT, SIGMA, TT, FULLVEC>, grid, kWarpKernelThreads, pl.sm_total, stream,
                           with_first_request(pl, grid, 1), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
