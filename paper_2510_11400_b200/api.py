@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from dataclasses import dataclass
 from typing import List, Optional, Sequence, Tuple
 
@@ -49,6 +50,10 @@ class fh_params(C.Structure):
 class fh_sched_entry(C.Structure):
     _fields_ = [("desc", fh_tensor_desc), ("action", C.c_int32), ("d_dense", C.c_void_p),
                 ("d_restored", C.c_void_p)]
+
+
+_SCHED_ENTRY = struct.Struct(f"={C.sizeof(fh_tensor_desc)}si4xQQ")    # fh_sched_entry, field by field
+assert _SCHED_ENTRY.size == C.sizeof(fh_sched_entry)
 
 
 class fh_sched_report(C.Structure):
@@ -150,17 +155,19 @@ def compressed_bytes(d: fh_tensor_desc, p: fh_params, which: int = 0) -> int:
 
 
 def _stream_ptr(stream) -> int:
+    """The raw stream.  Making a torch Stream object for the current one takes 3 us, asking for its pointer 0.2."""
+    if stream is not None:
+        return int(stream.cuda_stream)
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def fh_compress(d: fh_tensor_desc, p: fh_params, src, dst, out2=None, stream=None, capacity: Optional[int] = None) -> int:
     """Enqueue compression of the torch CUDA tensor `src` into the uint8 CUDA tensor `dst`.
     `out2` is an optional 2-element int64/uint64 CUDA tensor receiving (total bytes, status)."""
-    cap = dst.numel() * dst.element_size() if capacity is None else capacity
-    return int(lib().fh_compress(C.byref(d), C.byref(p), src.data_ptr(), dst.data_ptr(), cap,
-                                 out2.data_ptr() if out2 is not None else None, _stream_ptr(stream)))
+    return lib().fh_compress(C.byref(d), C.byref(p), src.data_ptr(), dst.data_ptr(),
+                             dst.nbytes if capacity is None else capacity,
+                             None if out2 is None else out2.data_ptr(), _stream_ptr(stream))
 
 
 def fh_compress_static(d: fh_tensor_desc, p: fh_params, src, dst, out2=None, stream=None,
@@ -168,14 +175,14 @@ def fh_compress_static(d: fh_tensor_desc, p: fh_params, src, dst, out2=None, str
     """fh_compress for callers that must not allocate: same arguments and bytes, book-keeping scratch in a
     fixed array inside the library (at most FH_STATIC_MAX_PLANES planes; calls sharing a device must not
     overlap)."""
-    cap = dst.numel() * dst.element_size() if capacity is None else capacity
-    return int(lib().fh_compress_static(C.byref(d), C.byref(p), src.data_ptr(), dst.data_ptr(), cap,
-                                        out2.data_ptr() if out2 is not None else None, _stream_ptr(stream)))
+    return lib().fh_compress_static(C.byref(d), C.byref(p), src.data_ptr(), dst.data_ptr(),
+                                    dst.nbytes if capacity is None else capacity,
+                                    None if out2 is None else out2.data_ptr(), _stream_ptr(stream))
 
 
 def fh_decompress(src, src_bytes: int, d: fh_tensor_desc, dst, status=None, stream=None) -> int:
-    return int(lib().fh_decompress(src.data_ptr(), src_bytes, C.byref(d), dst.data_ptr(),
-                                   status.data_ptr() if status is not None else None, _stream_ptr(stream)))
+    return lib().fh_decompress(src.data_ptr(), src_bytes, C.byref(d), dst.data_ptr(),
+                               None if status is None else status.data_ptr(), _stream_ptr(stream))
 
 
 @dataclass
@@ -187,12 +194,14 @@ class SchedItem:
 
 
 def fh_run_schedule(items: List[SchedItem], p: fh_params, arena, stream=None) -> fh_sched_report:
-    arr = (fh_sched_entry * len(items))()
-    for i, it in enumerate(items):
-        arr[i].desc = it.desc
-        arr[i].action = it.action
-        arr[i].d_dense = it.dense.data_ptr() if it.dense is not None else None
-        arr[i].d_restored = it.restored.data_ptr() if it.restored is not None else None
+    # (packed by hand: setting the fields of a ctypes array takes a microsecond per item)
+    buf, at = bytearray(_SCHED_ENTRY.size * len(items)), 0
+    for it in items:
+        dense, restored = it.dense, it.restored
+        _SCHED_ENTRY.pack_into(buf, at, bytes(it.desc), it.action, 0 if dense is None else dense.data_ptr(),
+                               0 if restored is None else restored.data_ptr())
+        at += _SCHED_ENTRY.size
+    arr = (fh_sched_entry * len(items)).from_buffer(buf)
     rep = fh_sched_report()
     rc = lib().fh_run_schedule(arr, len(items), C.byref(p), arena.data_ptr(),
                                arena.numel() * arena.element_size(), C.byref(rep), _stream_ptr(stream))

@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <tuple>
 #include <utility>
@@ -247,6 +248,35 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
 }
 
 // ---- per-stream scratch ---------------------------------------------------------------------
+// What one call of the schedule runner needs: offsets, sizes and statuses on the device, where they are read back to
+// (pinned), and its events.  A stream's scratch keeps one for the next call (allocating all of it anew took 20 us of a
+// 400 us schedule); calls that overlap on a stream get their own, freed when they end.
+struct SchedSpace {
+  unsigned long long *words = nullptr, *host = nullptr;
+  size_t cap = 0;
+  cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+  ~SchedSpace() {
+    if (words) cudaFree(words);
+    if (host) cudaFreeHost(host);
+    for (cudaEvent_t e : ev)
+      if (e) cudaEventDestroy(e);
+  }
+  bool reserve(size_t n) {
+    for (cudaEvent_t& e : ev)
+      if (!e && cudaEventCreate(&e) != cudaSuccess) return false;
+    if (n <= cap) return true;
+    if (words) cudaFree(words);
+    if (host) cudaFreeHost(host);
+    words = host = nullptr;
+    cap = 0;
+    const size_t want = n < 1024 ? 1024 : 2 * n;
+    if (cudaMalloc(&words, want * sizeof(unsigned long long)) != cudaSuccess) return false;
+    if (cudaMallocHost(&host, want * sizeof(unsigned long long)) != cudaSuccess) return false;
+    cap = want;
+    return true;
+  }
+};
+
 struct StreamScratch {
   fh::Scratch* sc = nullptr;             // counters
   unsigned long long* scan = nullptr;    // placement scan: tile words, group sums, group prefixes; then the tile links
@@ -258,8 +288,7 @@ struct StreamScratch {
   size_t pn_cap = 0;
   fh::ChanStat* chan = nullptr;          // ... and per-channel statistics
   size_t chan_cap = 0;
-  unsigned long long* sched = nullptr;   // schedule runner: offsets, sizes, statuses
-  size_t sched_cap = 0;
+  SchedSpace* sched = nullptr;           // schedule runner: the workspace that is not in use, if any
 };
 // tile words | two sets of group sums | group prefixes | tile links (32-bit)
 inline size_t scan_words(size_t tile_cap) { return tile_cap + 3 * (tile_cap / 32) + tile_cap / 2; }
@@ -530,76 +559,64 @@ int fh_run_schedule(const fh_sched_entry* entries, int32_t count, const fh_param
   }
   const size_t k = idx.size();
   if (k == 0) return FH_OK;
-  // device words: offsets[k+1] | out2[2k] | decode status[k]
+  // device words: offsets[k+1] | out2[2k] | decode status[k]; cleared, so that a call that ends early reports nothing stale
   const size_t words = (k + 1) + 2 * k + k;
-  unsigned long long* d_words = nullptr;
+  std::unique_ptr<SchedSpace> space;
   {
     std::lock_guard<std::mutex> lock(g_mu);
     StreamScratch* s = nullptr;
     rc = get_scratch(stream, 0, &s);
     if (rc != FH_OK) return rc;
-    if (s->sched_cap < words) {
-      if (s->sched) {
-        cudaDeviceSynchronize();
-        cudaFree(s->sched);
-        s->sched = nullptr;
-      }
-      size_t cap = words < 1024 ? 1024 : 2 * words;
-      if (cudaMalloc(&s->sched, cap * sizeof(unsigned long long)) != cudaSuccess) return FH_ERR_CUDA;
-      s->sched_cap = cap;
-    }
-    d_words = s->sched;
+    space.reset(s->sched);
+    s->sched = nullptr;
   }
-  unsigned long long* d_off = d_words;
-  unsigned long long* d_out2 = d_words + (k + 1);
+  if (!space) space.reset(new SchedSpace);
+  if (!space->reserve(words)) return FH_ERR_CUDA;
+  unsigned long long* d_off = space->words;
+  unsigned long long* d_out2 = d_off + (k + 1);
   unsigned long long* d_dst = d_out2 + 2 * k;
-  cudaEvent_t e0, e1, e2;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
-      cudaEventCreate(&e2) != cudaSuccess)
-    return FH_ERR_CUDA;
-  rc = FH_OK;
-  if (cudaMemsetAsync(d_words, 0, words * sizeof(unsigned long long), stream) != cudaSuccess) rc = FH_ERR_CUDA;
-  cudaEventRecord(e0, stream);
+  if (cudaMemsetAsync(space->words, 0, words * sizeof(unsigned long long), stream) != cudaSuccess) rc = FH_ERR_CUDA;
+  cudaEventRecord(space->ev[0], stream);
   for (size_t j = 0; j < k && rc == FH_OK; ++j) {  // forward order
     const fh_sched_entry& en = entries[idx[j]];
     rc = enqueue_compress(&en.desc, params, en.d_dense, d_arena, arena_bytes, d_off + j, d_off + j + 1,
                           d_out2 + 2 * j, stream);
   }
-  cudaEventRecord(e1, stream);
+  cudaEventRecord(space->ev[1], stream);
   for (size_t j = k; j-- > 0 && rc == FH_OK;) {  // reverse order
     const fh_sched_entry& en = entries[idx[j]];
     rc = enqueue_decompress(d_arena, arena_bytes, &en.desc, en.d_restored, d_off + j, d_dst + j, stream);
   }
-  cudaEventRecord(e2, stream);
+  cudaEventRecord(space->ev[2], stream);
+  // (read back behind the last kernel on the stream: one wait for everything)
+  if (rc == FH_OK && cudaMemcpyAsync(space->host, space->words, words * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                     stream) != cudaSuccess)
+    rc = FH_ERR_CUDA;
   if (cudaStreamSynchronize(stream) != cudaSuccess) rc = rc == FH_OK ? FH_ERR_CUDA : rc;
   if (rc == FH_OK) {
-    std::vector<unsigned long long> h(words);
-    if (cudaMemcpy(h.data(), d_words, words * sizeof(unsigned long long), cudaMemcpyDeviceToHost) != cudaSuccess) {
-      rc = FH_ERR_CUDA;
-    } else {
-      cudaEventElapsedTime(&report->ms_forward, e0, e1);
-      cudaEventElapsedTime(&report->ms_backward, e1, e2);
-      int status = FH_OK;
-      uint64_t peak = 0;
-      for (size_t j = 0; j < k; ++j) {
-        const int cs = (int)(long long)h[(k + 1) + 2 * j + 1];
-        if (status == FH_OK && cs != FH_OK) status = cs;
-        if (cs == FH_OK) {
-          report->total_packed_bytes += h[(k + 1) + 2 * j];
-          if (h[j + 1] > peak) peak = h[j + 1];
-        }
+    const unsigned long long* h = space->host;
+    cudaEventElapsedTime(&report->ms_forward, space->ev[0], space->ev[1]);
+    cudaEventElapsedTime(&report->ms_backward, space->ev[1], space->ev[2]);
+    int status = FH_OK;
+    uint64_t peak = 0;
+    for (size_t j = 0; j < k; ++j) {
+      const int cs = (int)(long long)h[(k + 1) + 2 * j + 1];
+      if (status == FH_OK && cs != FH_OK) status = cs;
+      if (cs == FH_OK) {
+        report->total_packed_bytes += h[(k + 1) + 2 * j];
+        if (h[j + 1] > peak) peak = h[j + 1];
       }
-      for (size_t j = 0; j < k; ++j) {
-        const int ds = (int)(long long)h[(k + 1) + 2 * k + j];
-        if (status == FH_OK && ds != FH_OK) status = ds;
-      }
-      report->peak_packed_bytes = peak;
-      report->status = status;
     }
+    for (size_t j = 0; j < k; ++j) {
+      const int ds = (int)(long long)h[(k + 1) + 2 * k + j];
+      if (status == FH_OK && ds != FH_OK) status = ds;
+    }
+    report->peak_packed_bytes = peak;
+    report->status = status;
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  cudaEventDestroy(e2);
+  std::lock_guard<std::mutex> lock(g_mu);
+  StreamScratch* s = nullptr;
+  if (get_scratch(stream, 0, &s) == FH_OK && !s->sched) s->sched = space.release();
   return rc;
 }
 
@@ -817,7 +834,7 @@ void fh_shutdown(void) {
     if (kv.second.scan) cudaFree(kv.second.scan);
     if (kv.second.plane_nout) cudaFree(kv.second.plane_nout);
     if (kv.second.chan) cudaFree(kv.second.chan);
-    if (kv.second.sched) cudaFree(kv.second.sched);
+    delete kv.second.sched;
   }
   g_scratch.clear();
   cudaSetDevice(cur);
