@@ -180,8 +180,8 @@ size_t fh_compressed_bytes(const fh_tensor_desc* desc, const fh_params* params, 
  * (i / 4, plane index, tensor_id low, tensor_id high), i the element's index within its plane.  The draw
  * thus depends on (seed, tensor id, element position) only and results are reproducible.  Dense-block codes
  * keep round-to-nearest (their error bound needs it).  One generator call per four elements makes this mode
- * about twice as slow as rounding = 0 (planes of at most 1024 elements with salient_mode AUTO; other cases run
- * on the general-purpose kernel and are slower still).
+ * about twice as slow as rounding = 0 (with salient_mode AUTO; other modes run on the general-purpose kernel and are
+ * slower still).
  *
  * entropy = 1 (Section 4.4.1: "a Huffman tree is constructed from the quantization array for encoding"): the
  * residual code bytes of an outlier-rich plane's dense blocks are Huffman-coded, one code per plane (see the

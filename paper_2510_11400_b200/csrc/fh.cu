@@ -133,54 +133,52 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   // block-wise path: blocks per step side by side, rows of steps (see fh_blocks.cuh)
   pl.qs = pl.nbx >= 3 ? 2u : pl.nbx - 1u;
   pl.nsr = (pl.nby + (4u >> pl.qs) - 1u) / (4u >> pl.qs);
-  // its measuring scratch: row pointers, two sums per step row, the bitmap; with the Huffman stage one more sum and the
-  // encoder's tables
-  const size_t sal_words = (size_t)pl.H + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
-                           (pl.entropy ? (size_t)pl.nsr + 1 + sizeof(fh::HufEncode) / 4 : 0);
-  const uint32_t sal_bytes = (uint32_t)A16(4 * sal_words + 16);  // one measuring area of the block-wise path
+  // its measuring scratch (of a team of `warps`): row pointers, two sums per step row, the bitmap; with the Huffman stage
+  // one more sum and the encoder's tables
+  auto sal_bytes_of = [&](uint32_t warps) {
+    const size_t words = (size_t)pl.H + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
+                         (pl.entropy ? (size_t)pl.nsr + 1 + sizeof(fh::HufEncode) / 4 + (warps - 1) * 4 * fh::kHufStageWords : 0);
+    return (uint32_t)A16(4 * words + 16);
+  };
   const bool blockwise = compress && pl.mode != FH_SALIENT_OFF;
 
   Variant v;
-  // ---- fast compress kernels: planes of whole 16-byte chunks whose groups fit the register budget
+  // ---- fast compress kernels.  Random rounding runs on the register kernels in the plane-wise three-sigma mode, on the
+  // generic kernel otherwise; planes beyond the register kernels' reach on the kernel that sweeps them in shared memory
+  // when they are whole 16-byte chunks.
   const bool whole16 = pl.HW % 4 == 0 && pl.plane_bytes % 16 == 0;
-  // (random rounding runs on the warp-team kernels in the plane-wise three-sigma mode, on the generic kernel otherwise)
-  const bool rounding_ok = pl.rounding == 0 || (pl.groups <= 256 && pl.mode == FH_SALIENT_AUTO);
-  if (compress && rounding_ok && (pl.groups <= 256 || whole16)) {
+  const bool warp_fits = pl.groups <= 256, regs_fit = pl.groups <= (uint32_t)(fh::kCtaMaxWarps * fh::kCtaGroups);
+  if (compress && (pl.rounding == 0 || pl.mode == FH_SALIENT_AUTO) && (warp_fits || regs_fit || (whole16 && pl.rounding == 0))) {
     v.fast = true;
-    if (pl.groups <= 256) {
+    pl.ppt = 1;
+    if (warp_fits) {
       pl.team = fh::team_of_groups(pl.groups);
-      v.G = 8;  // the warp-team kernels keep eight groups per thread
       pl.ppt = fh::kThreads / pl.team;
+      if (pl.ppt > pl.P) pl.ppt = (uint32_t)pl.P;
+      pl.stage_bytes = (uint32_t)((pl.ppt * pl.plane_bytes + 127) & ~(uint64_t)127);
+    } else if (regs_fit) {
+      v.cta = v.regs = true;
+      pl.team = 32u * ((pl.groups + fh::kCtaGroups - 1u) / fh::kCtaGroups);
+      pl.stage_bytes = (uint32_t)((pl.plane_bytes + 16 + 127) & ~(uint64_t)127);
     } else {
       v.cta = true;  // CTA size by plane size: enough work per thread between barriers
-      // (the per-plane reductions and scalar steps cost every warp the same, whatever its share of the plane:
-      // fewer, busier threads win as long as enough warps stay resident)
-      pl.team = pl.plane_bytes <= 16 * 1024 ? 128 : (pl.plane_bytes <= 64 * 1024 ? 256 : 512);
-      v.G = 0;
-      // planes of up to 4096 groups: the register variant, with the smallest (threads, groups per thread)
-      // that holds the plane
-      static const uint32_t kCombo[6][2] = {{128, 7}, {128, 8}, {256, 7}, {256, 8}, {448, 7}, {512, 8}};
-      for (int k = 0; k < 6; ++k)
-        if (kCombo[k][0] * kCombo[k][1] >= pl.groups) {
-          pl.team = kCombo[k][0];
-          v.G = (int)kCombo[k][1];
-          break;
-        }
-      pl.ppt = 1;
+      pl.team = pl.plane_bytes <= 64 * 1024 ? 256 : 512;
+      pl.stage_bytes = (uint32_t)((pl.plane_bytes + 127) & ~(uint64_t)127);
     }
-    if (pl.ppt > pl.P) pl.ppt = (uint32_t)pl.P;
-    pl.stage_bytes = (uint32_t)((pl.ppt * pl.plane_bytes + 127) & ~(uint64_t)127);
     uint32_t ns = (uint32_t)((v.cta ? kStageTarget : kWarpStageTarget) / pl.stage_bytes);
-    // (CTA-team kernel: two stages; a third buys nothing that more resident CTAs do not give)
+    // (CTA-team kernels: two stages; a third buys nothing that more resident CTAs do not give)
     const uint32_t ns_max = v.cta ? 2u : (uint32_t)fh::kMaxStages;
     ns = ns < 2 ? 2 : (ns > ns_max ? ns_max : ns);
+    const uint32_t sal_bytes = sal_bytes_of(v.cta ? pl.team / 32 : 1u);
     const uint32_t areas = blockwise ? (v.cta ? 1u : (uint32_t)fh::kWarps) : 0u;
     for (;;) {
       pl.nstage = ns;
       pl.sm_tile = 0;
       pl.sm_sal = (uint32_t)A16((size_t)ns * pl.stage_bytes);
       pl.sal_stride = sal_bytes;
-      pl.sm_total = pl.sm_sal + areas * sal_bytes;
+      // (a load of a plane's last group may read up to 16 bytes past the stage)
+      const uint32_t behind = areas * sal_bytes;
+      pl.sm_total = pl.sm_sal + (behind > 32u ? behind : 32u);
       if (pl.sm_total <= kSmemLimit) break;
       if (ns == 2) {  // the pipeline needs two stages
         v.fast = false;
@@ -222,6 +220,7 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     }
     pl.nstage = 0;
     pl.stage_bytes = 0;
+    const uint32_t sal_bytes = sal_bytes_of(fh::kWarps);
     uint64_t ppt = kTileTarget / pl.plane_bytes;
     if (ppt < 1) ppt = 1;
     if (ppt > kMaxPpt) ppt = kMaxPpt;

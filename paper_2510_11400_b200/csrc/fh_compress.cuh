@@ -10,11 +10,13 @@
 //   other planes:   measured at once while they lie in shared memory (block classes, CSR and code sizes,
 //                   salient versus raw); the tile publishes the overflow size of its planes, obtains the sum
 //                   over all earlier tiles from the placement scan (fh_device.cuh) and writes the payloads.
-// Three variants by plane size:
-//   compress_warp<DT, SIGMA, TT, FULLVEC>  planes of at most 256 groups: bulk-copy (TMA) pipeline, a sub-warp
+// Variants by plane size:
+//   compress_warp<DT, SIGMA, TT, K, EDGE>   planes of at most 256 groups: bulk-copy (TMA) pipeline, a sub-warp
 //       team per plane, groups kept in registers; a warp handles the outlier-rich planes of its slice;
-//   compress_cta<DT, SIGMA, NT>            larger planes of whole 16-byte chunks: one plane per CTA and tile;
-//   compress_generic<DT, BITS>             everything else (ragged large planes, random rounding).
+//   compress_cta_regs<DT, SIGMA, K, EDGE>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
+//   compress_cta<DT, SIGMA, NT>            still larger ones of whole 16-byte chunks: swept in shared memory;
+//   compress_generic<DT, BITS>             everything else (still larger ragged planes, random rounding outside the
+//       plane-wise three-sigma mode).
 // The kernel's last CTA writes the header and the result words and returns the scratch to its idle state.
 #pragma once
 
@@ -444,7 +446,12 @@ struct BlockCtl {
   uint32_t wcnt[kMaxWarps];                                // phase 2: outlier-rich planes per warp's slice
   uint32_t base, ok;
   uint32_t head;                                           // the tile this CTA listed last
-  uint32_t held[kMaxStages];                               // warp-team kernel: the tile each stage buffer holds
+  uint32_t held[kMaxStages];                               // the tile each stage buffer holds
+  uint32_t measured;                                       // CTA-team kernels: the plane the measuring scratch is about ...
+  SalientInfo measured_info;                               // ... and its sizes
+};
+
+struct BlockList {
   // phase 2 of the warp-team kernel: the outlier-rich planes of the tile in hand, in plane order
   uint32_t list_at[256];                                   // overflow units, then (scanned) the place within the tile's part
   uint32_t list_meta[256];
@@ -716,213 +723,314 @@ __global__ void __launch_bounds__(kThreads) compress_generic(const Plan pl, cons
 // =================================================================================================
 // Fast kernels
 // =================================================================================================
-// One plane per team.  Warp-team variant: kThreads / team planes per tile, each handled by `team` lanes of a
-// warp; thread t of a team owns groups t, t + team, ... (G of them) and keeps them in registers for every
-// pass.  FULL: groups == G * team, so no group needs a bounds check.
+// A team of TT lanes takes a run of groups, lane l groups l, l + TT, ... (K slots per lane), and keeps them in registers
+// as fp32 for all that follows: minimum and maximum, distances from the minimum, integer moments, outlier count, codes.
+// A run is a whole plane (warp-team kernel) or a warp's share of one (CTA-team kernel).
 //
-// One sweep over a plane: min/max -> distances from the minimum -> (integer moments -> thresholds -> count
-// -> class) -> codes, stored straight to the plane's slot together with its table entry.
+// K is chosen so that all slots but the last EDGE of them lie wholly inside the run for every lane; only those EDGE slots
+// are masked.  (Checking every element against the plane's end made the 7 x 7 planes cost 75 instructions per element;
+// a slot count known at run time only made the compiler spill: 56 x 56 18 -> 40 us.)  A masked position reads as another
+// element of the run for minimum and maximum and is then held as distance 0, which adds exactly nothing to the moments
+// and carries code 0; a lower threshold above 0 counts it, and it is subtracted again.
 //
-// Codes of the thread's groups, packed and stored to the plane's slot (used inside plane_sweep, on its
-// register-resident distances x[k][e]).  Four codes of a group are the sum of (magic + q_e) << (e * BITS)
-// minus the magic's contribution.
-#define FH_STORE_CODES(BITS)                                                                                  \
-  {                                                                                                           \
-    constexpr uint32_t bias = kMagicBits * (1u + (1u << (BITS)) + (1u << (2 * (BITS))) + (1u << (3 * (BITS)))); \
-    const f32x2 inv2 = pack2(inv, inv), mag2 = pack2(kMagicF, kMagicF);                                         \
-    _Pragma("unroll") for (int k = 0; k < G; ++k) {                                                           \
-      const uint32_t g = lane + (uint32_t)(k * TT);                                                           \
-      uint32_t w0, w1, w2, w3;                                                                                \
-      unpack2u(fma2(pack2(x[k][0], x[k][1]), inv2, mag2), w0, w1); /* packed pairs */                         \
-      unpack2u(fma2(pack2(x[k][2], x[k][3]), inv2, mag2), w2, w3);                                            \
-      uint32_t word = w0 + (w1 << (BITS)) + (w2 << (2 * (BITS))) + (w3 << (3 * (BITS))) - bias;               \
-      if (FULL || g < groups) {                                                                               \
-        if ((BITS) == 2) slot[g] = (uint8_t)word;                                                             \
-        else if ((BITS) == 4) reinterpret_cast<uint16_t*>(slot)[g] = (uint16_t)word;                          \
-        else reinterpret_cast<uint32_t*>(slot)[g] = word;                                                     \
-      }                                                                                                       \
-    }                                                                                                         \
+// Loads group `v` of the run at `p` (shared memory).  `grain`: the run starts on a 16-byte (2) or 8-byte (1) boundary, or
+// on an element (0).  May read up to 16 bytes past the group.  fp32: the four values; bf16: two words of two.
+template <int DT>
+__device__ __forceinline__ void group_load(const uint8_t* p, uint32_t v, uint32_t grain, uint32_t (&w)[4]) {
+  if (DT == kF32) {
+    if (grain == 2u) {
+      const uint4 t = reinterpret_cast<const uint4*>(p)[v];
+      w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+    } else if (grain == 1u) {
+      const uint2 t = reinterpret_cast<const uint2*>(p)[2u * v], u = reinterpret_cast<const uint2*>(p)[2u * v + 1u];
+      w[0] = t.x; w[1] = t.y; w[2] = u.x; w[3] = u.y;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) w[e] = reinterpret_cast<const uint32_t*>(p)[4u * v + e];
+    }
+  } else {
+    if (grain >= 1u) {
+      const uint2 t = reinterpret_cast<const uint2*>(p)[v];
+      w[0] = t.x; w[1] = t.y;
+    } else {  // three aligned words hold the four elements at either parity
+      const uint32_t odd = smem_u32(p) & 2u;
+      const uint32_t* q = reinterpret_cast<const uint32_t*>(p - odd) + 2u * v;
+      const uint32_t q0 = q[0], q1 = q[1], q2 = q[2];
+      w[0] = __funnelshift_r(q0, q1, odd * 8u);
+      w[1] = __funnelshift_r(q1, q2, odd * 8u);
+    }
+    w[2] = w[3] = 0;
   }
+}
+// Two bf16 minima / maxima per instruction; a NaN anywhere surfaces, -0 sorts below +0, as with the fp32 ones.
+__device__ __forceinline__ uint32_t min2_nan_bf16(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("min.NaN.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t max2_nan_bf16(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
 
-// TT: team size (1..32), a compile-time constant so that the strides between a thread's groups are
-// immediates.  FULL: groups == G * TT.  VEC: planes are whole 16-byte chunks (vector loads, no ragged last
-// group).  Returns class | n_out << 2; a normal plane is complete when the function returns.
-// SIGMA: 0 no three-sigma statistics, 1 the plane's own, 2 the same with random rounding of the codes.
-template <int DT, int SIGMA, int G, int TT, bool FULL, bool VEC>
-__device__ __forceinline__ uint32_t plane_sweep(const Team& team, const Plan& pl, const Dest& d, const CompressArgs& a,
-                                                const uint8_t* plane, uint64_t gp, uint32_t& rp) {
-  // A thread's G group slots that lie past the plane, and the elements past a ragged last group, are
-  // kept out of minimum and maximum with neutral values and then held as distance 0: they add exactly
-  // nothing to the moments, are subtracted from the outlier count when 0 lies outside the thresholds, and
-  // carry code 0 (a ragged last group) or are not stored at all.  The arithmetic runs unpredicated over all
-  // G slots.
-  const uint32_t groups = pl.groups, lane = team.lane;
-  const float pinf = __int_as_float(0x7F800000), ninf = __int_as_float(0xFF800000);
-  float x[G][4];
-  float lo = pinf, hi = ninf, lo1 = pinf, hi1 = ninf;
-  uint32_t npad = 0;  // padded elements among this thread's slots
+// Runs of exactly K * TT groups (EDGE 0) start on 16-byte boundaries; in bf16 a lane then takes groups in neighbouring
+// pairs, so that loads are 16 bytes wide and codes leave twice as wide (1 GiB of 32 x 32 planes: 373 -> 342 us).
+// Slot k's group within the run:
+template <int DT, int K, int TT, int EDGE>
+__device__ __forceinline__ uint32_t slot_group(uint32_t lane, int k) {
+  if (DT == kBF16 && EDGE == 0) return 2u * (lane + (uint32_t)((k >> 1) * TT)) + (uint32_t)(k & 1);
+  return lane + (uint32_t)(k * TT);
+}
+
+// Loads the run of `n` elements and takes the lane's minimum and maximum.
+template <int DT, int K, int TT, int EDGE, int GRAIN>
+__device__ __forceinline__ void run_load_as(const uint8_t* p, uint32_t lane, int32_t n, float (&x)[K][4], float& lo, float& hi) {
+  const uint32_t last = (uint32_t)(n - 1) >> 2;
+  if (DT == kF32) {
+    float lo1, hi1;
 #pragma unroll
-  for (int k = 0; k < G; ++k) {
-    const uint32_t g = lane + (uint32_t)(k * TT);
-    if (VEC) {
-      const bool act = FULL || g < groups;
-      if (DT == kF32) {
-        float4 t4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (act) t4 = (reinterpret_cast<const float4*>(plane) + lane)[k * TT];
-        x[k][0] = t4.x; x[k][1] = t4.y; x[k][2] = t4.z; x[k][3] = t4.w;
-      } else {
-        uint2 t2 = make_uint2(0u, 0u);
-        if (act) t2 = (reinterpret_cast<const uint2*>(plane) + lane)[k * TT];
-        x[k][0] = __uint_as_float(t2.x << 16); x[k][1] = __uint_as_float(t2.x & 0xFFFF0000u);
-        x[k][2] = __uint_as_float(t2.y << 16); x[k][3] = __uint_as_float(t2.y & 0xFFFF0000u);
-      }
-      // per-group partial results keep the dependency chains short
-      float gl = min_nan(min3_nan(x[k][0], x[k][1], x[k][2]), x[k][3]);
-      float gh = max_nan(max3_nan(x[k][0], x[k][1], x[k][2]), x[k][3]);
-      if (!FULL) {
-        gl = act ? gl : pinf;
-        gh = act ? gh : ninf;
-        npad += act ? 0u : 4u;
-      }
-      if (k & 1) {
-        lo1 = min_nan(lo1, gl);
-        hi1 = max_nan(hi1, gh);
-      } else {
-        lo = min_nan(lo, gl);
-        hi = max_nan(hi, gh);
-      }
-    } else {  // plane not on a 16-byte boundary, possibly with a ragged last group
+    for (int k = 0; k < K; ++k) {
+      const uint32_t v = lane + (uint32_t)(k * TT);
+      uint32_t w[4];
+      group_load<DT>(p, k >= K - EDGE ? min(v, last) : v, GRAIN, w);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t i = g * 4u + e;
-        const bool in = i < pl.HW;
-        x[k][e] = in ? load_elem<DT>(plane, i) : 0.0f;
-        if (e & 1) {
-          lo1 = min_nan(lo1, in ? x[k][e] : pinf);
-          hi1 = max_nan(hi1, in ? x[k][e] : ninf);
-        } else {
-          lo = min_nan(lo, in ? x[k][e] : pinf);
-          hi = max_nan(hi, in ? x[k][e] : ninf);
-        }
-        npad += in ? 0u : 1u;
+      for (int e = 0; e < 4; ++e) x[k][e] = __uint_as_float(w[e]);
+      if (k >= K - EDGE) {
+        const int32_t in = n - 4 * (int32_t)v;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[k][e] = e < in ? x[k][e] : (k == 0 ? __uint_as_float(w[0]) : x[0][0]);
       }
     }
+    // per-group partial results keep the dependency chains short
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const float gl = min_nan(min3_nan(x[k][0], x[k][1], x[k][2]), x[k][3]);
+      const float gh = max_nan(max3_nan(x[k][0], x[k][1], x[k][2]), x[k][3]);
+      if (k == 0) lo = gl, hi = gh;
+      else if (k == 1) lo1 = gl, hi1 = gh;
+      else if (k & 1) lo1 = min_nan(lo1, gl), hi1 = max_nan(hi1, gh);
+      else lo = min_nan(lo, gl), hi = max_nan(hi, gh);
+    }
+    lo = min_nan(lo, lo1);
+    hi = max_nan(hi, hi1);
+  } else {
+    static_assert(EDGE > 0 || K % 2 == 0, "pairs");
+    uint32_t l0 = 0, h0 = 0, l1 = 0, h1 = 0, safe = 0;
+    uint4 pair = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const uint32_t v = lane + (uint32_t)(k * TT);
+      uint32_t w[4];
+      if (EDGE == 0) {
+        if (k & 1) {
+          w[0] = pair.z; w[1] = pair.w;
+        } else {
+          pair = (reinterpret_cast<const uint4*>(p) + lane)[(k >> 1) * TT];
+          w[0] = pair.x; w[1] = pair.y;
+        }
+      } else {
+        group_load<DT>(p, k >= K - EDGE ? min(v, last) : v, GRAIN, w);
+      }
+      if (k == 0) safe = __byte_perm(w[0], 0u, 0x1010);
+      if (k >= K - EDGE) {
+        const int32_t in = n - 4 * (int32_t)v;
+        w[0] = in >= 2 ? w[0] : (in == 1 ? __byte_perm(w[0], safe, 0x5410) : safe);
+        w[1] = in >= 4 ? w[1] : (in == 3 ? __byte_perm(w[1], safe, 0x5410) : safe);
+      }
+      if (k == 0) l0 = h0 = w[0], l1 = h1 = w[1];
+      else {
+        l0 = min2_nan_bf16(l0, w[0]); l1 = min2_nan_bf16(l1, w[1]);
+        h0 = max2_nan_bf16(h0, w[0]); h1 = max2_nan_bf16(h1, w[1]);
+      }
+      x[k][0] = __uint_as_float(w[0] << 16); x[k][1] = __uint_as_float(w[0] & 0xFFFF0000u);
+      x[k][2] = __uint_as_float(w[1] << 16); x[k][3] = __uint_as_float(w[1] & 0xFFFF0000u);
+    }
+    l0 = min2_nan_bf16(l0, l1);
+    h0 = max2_nan_bf16(h0, h1);
+    lo = min_nan(__uint_as_float(l0 << 16), __uint_as_float(l0 & 0xFFFF0000u));
+    hi = max_nan(__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xFFFF0000u));
   }
-  lo = min_nan(lo, lo1);
-  hi = max_nan(hi, hi1);
+}
+template <int DT, int K, int TT, int EDGE>
+__device__ __forceinline__ void run_load(const uint8_t* p, uint32_t lane, int32_t n, uint32_t grain, float (&x)[K][4], float& lo, float& hi) {
+  if (EDGE == 0 || grain == 2u) run_load_as<DT, K, TT, EDGE, 2>(p, lane, n, x, lo, hi);
+  else if (DT == kF32 && grain == 1u) run_load_as<DT, K, TT, EDGE, 1>(p, lane, n, x, lo, hi);
+  else run_load_as<DT, K, TT, EDGE, 0>(p, lane, n, x, lo, hi);
+}
+// The grain of planes that follow one another from a 16-byte boundary on (for bf16 an 8-byte boundary is as good).
+__device__ __forceinline__ uint32_t plane_grain(const Plan& pl) {
+  return (pl.plane_bytes & 15u) == 0u ? 2u : ((pl.plane_bytes & 7u) == 0u ? (pl.esize == 2 ? 2u : 1u) : 0u);
+}
+
+// Distances from the minimum, in place (x - lo is x + (-lo): the same rounding); masked positions become distance 0.
+// With SIGMA also the raw mantissa images of the groups' fixed-point addends (see sigma_addends2), summed with
+// wrap-around: K magics beyond the addends themselves.
+template <int DT, int K, int TT, int EDGE, bool SIGMA>
+__device__ __forceinline__ void run_distances(uint32_t lane, int32_t n, float lo, const SigmaScale& sc, float (&x)[K][4], uint32_t& as,
+                                              uint32_t& aq) {
+  const float nlo = -lo;
+  const f32x2 nlo2 = pack2(nlo, nlo);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    unpack2(add2(pack2(x[k][0], x[k][1]), nlo2), x[k][0], x[k][1]);
+    unpack2(add2(pack2(x[k][2], x[k][3]), nlo2), x[k][2], x[k][3]);
+    if (k >= K - EDGE) {
+      const int32_t in = n - 4 * (int32_t)(lane + (uint32_t)(k * TT));
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[k][e] = e < in ? x[k][e] : 0.0f;
+    }
+    if (SIGMA) sigma_addends4(x[k][0], x[k][1], x[k][2], x[k][3], sc, as, aq);
+  }
+}
+
+// Outliers among the lane's distances.  (Called only when some element can lie outside.)
+template <int DT, int K, int TT, int EDGE>
+__device__ __forceinline__ uint32_t run_count(uint32_t lane, int32_t n, float dlo, float dhi, const float (&x)[K][4]) {
+  uint32_t c[4] = {0, 0, 0, 0};  // four counters: short dependency chains
+  if (!__any_sync(0xFFFFFFFFu, 0.0f < dlo)) {  // nothing below: one compare per element
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) c[e] += x[k][e] > dhi;
+    }
+    return (c[0] + c[1]) + (c[2] + c[3]);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] += (x[k][e] > dhi) || (x[k][e] < dlo);
+  }
+  uint32_t all = (c[0] + c[1]) + (c[2] + c[3]);
+#pragma unroll
+  for (int k = K - EDGE; k < K && EDGE > 0; ++k)  // masked positions (distance 0) are no elements
+    if (0.0f < dlo) all -= (uint32_t)(4 - min(max(n - 4 * (int32_t)(lane + (uint32_t)(k * TT)), 0), 4));
+  return all;
+}
+
+// Codes of the lane's groups, packed and stored to `slot` (where the run's first group goes).  Four codes of a group are
+// the sum of (magic + q_e) << (e * BITS) minus the magic's contribution.
+template <int DT, int K, int TT, int EDGE, int BITS>
+__device__ __forceinline__ void run_codes(uint32_t lane, int32_t n, float inv, uint8_t* slot, const float (&x)[K][4]) {
+  constexpr uint32_t bias = kMagicBits * (1u + (1u << BITS) + (1u << (2 * BITS)) + (1u << (3 * BITS)));
+  constexpr bool PAIR = DT == kBF16 && EDGE == 0;
+  const f32x2 inv2 = pack2(inv, inv), mag2 = pack2(kMagicF, kMagicF);
+  uint8_t* out = slot + lane * (PAIR ? BITS : BITS / 2);
+  uint32_t before = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    uint32_t w0, w1, w2, w3;
+    unpack2u(fma2(pack2(x[k][0], x[k][1]), inv2, mag2), w0, w1);
+    unpack2u(fma2(pack2(x[k][2], x[k][3]), inv2, mag2), w2, w3);
+    const uint32_t word = w0 + (w1 << BITS) + (w2 << (2 * BITS)) + (w3 << (3 * BITS)) - bias;
+    if (PAIR) {
+      const int o = (k >> 1) * TT * BITS;
+      if (!(k & 1)) before = word;
+      else if (BITS == 2) *reinterpret_cast<uint16_t*>(out + o) = (uint16_t)(before | (word << 8));
+      else if (BITS == 4) *reinterpret_cast<uint32_t*>(out + o) = before | (word << 16);
+      else *reinterpret_cast<uint2*>(out + o) = make_uint2(before, word);
+    } else if (k < K - EDGE || n > 4 * (int32_t)(lane + (uint32_t)(k * TT))) {
+      if (BITS == 2) out[k * TT] = (uint8_t)word;
+      else if (BITS == 4) *reinterpret_cast<uint16_t*>(out + 2 * k * TT) = (uint16_t)word;
+      else *reinterpret_cast<uint32_t*>(out + 4 * k * TT) = word;
+    }
+  }
+}
+// Codes under random rounding: one generator call per group, counter = (group, plane, tensor id), key = seed; positions
+// past the plane's end carry code 0 whatever the draw.  The run is read from its stage at `p` once more, in a loop: with
+// the distances held in registers the generator's rounds, unrolled over the slots, spilled and overran the instruction
+// cache (112 x 112: 150 us a call).  `g0`: the run's first group, whose codes go to `slot`.
+template <int DT>
+__device__ __forceinline__ void run_codes_random(const Plan& pl, const uint8_t* p, uint32_t grain, uint32_t lane, uint32_t step, int32_t n,
+                                                 float lo, float inv, uint32_t g0, uint64_t gp, uint8_t* slot) {
+  const uint32_t bits = (uint32_t)pl.bits, L = (1u << bits) - 1u, groups = (uint32_t)(n + 3) >> 2;
+#pragma unroll 2
+  for (uint32_t v = lane; v < groups; v += step) {
+    uint32_t w[4], rnd[4];
+    group_load<DT>(p, v, grain, w);
+    philox4x32_10(g0 + v, (uint32_t)gp, (uint32_t)pl.tensor_id, (uint32_t)(pl.tensor_id >> 32), (uint32_t)pl.seed,
+                  (uint32_t)(pl.seed >> 32), rnd);
+    float x[4];
+    if (DT == kF32) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = __uint_as_float(w[e]);
+    } else {
+      x[0] = __uint_as_float(w[0] << 16); x[1] = __uint_as_float(w[0] & 0xFFFF0000u);
+      x[2] = __uint_as_float(w[1] << 16); x[3] = __uint_as_float(w[1] & 0xFFFF0000u);
+    }
+    uint32_t word = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) word |= quant_code_random(__fsub_rn(x[e], lo), inv, L, rnd[e]) << (e * bits);
+    const int32_t in = n - 4 * (int32_t)v;
+    if (in < 4) word &= (1u << ((uint32_t)in * bits)) - 1u;
+    if (bits == 2u) slot[v] = (uint8_t)word;
+    else if (bits == 4u) reinterpret_cast<uint16_t*>(slot)[v] = (uint16_t)word;
+    else reinterpret_cast<uint32_t*>(slot)[v] = word;
+  }
+}
+// Codes of a run, however they are rounded; `slot`: the plane's.
+template <int DT, int SIGMA, int K, int TT, int EDGE>
+__device__ __forceinline__ void run_codes_any(const Plan& pl, const uint8_t* p, uint32_t grain, uint32_t lane, int32_t n, float lo,
+                                              float inv, uint32_t g0, uint64_t gp, uint8_t* slot, const float (&x)[K][4]) {
+  uint8_t* at = slot + g0 * (uint32_t)pl.bits / 2u;
+  if (SIGMA == 2) run_codes_random<DT>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+  else if (pl.bits == 2) run_codes<DT, K, TT, EDGE, 2>(lane, n, inv, at, x);
+  else if (pl.bits == 4) run_codes<DT, K, TT, EDGE, 4>(lane, n, inv, at, x);
+  else run_codes<DT, K, TT, EDGE, 8>(lane, n, inv, at, x);
+}
+// Zero padding of a slot behind the codes, by `n` threads of which this is number `i`.
+__device__ __forceinline__ void pad_slot(const Plan& pl, uint8_t* slot, uint32_t i, uint32_t n) {
+  const uint32_t end = pl.groups * (uint32_t)pl.bits / 2u;
+  if (end >= pl.npay) return;
+  for (uint32_t o = end + i; o < a4(end); o += n) slot[o] = 0;
+  for (uint32_t o = a4(end) + 4u * i; o < pl.npay; o += 4u * n) *reinterpret_cast<uint32_t*>(slot + o) = 0u;
+}
+
+// One sweep over a plane by a team of TT lanes: min/max -> distances from the minimum -> (integer moments -> thresholds
+// -> count -> class) -> codes, stored straight to the plane's slot together with its table entry.  Returns class |
+// n_out << 2; a normal plane is complete when the function returns.  All lanes of the warp run through it together
+// (`active` is false in teams without a plane of their own: they look at somebody's and store nothing); what differs
+// between teams is selected, not branched on, but for whole warps.
+// SIGMA: 0 no three-sigma statistics, 1 the plane's own, 2 the same with random rounding of the codes.
+template <int DT, int SIGMA, int K, int TT, int EDGE>
+__device__ __forceinline__ uint32_t plane_sweep(const Team& team, const Plan& pl, const Dest& d, const CompressArgs& a,
+                                                const uint8_t* plane, uint64_t gp, uint32_t grain, bool active, uint32_t& rp) {
+  const uint32_t lane = team.lane, full = 0xFFFFFFFFu;
+  const int32_t n = (int32_t)pl.HW;
+  float x[K][4], lo, hi;
+  run_load<DT, K, TT, EDGE>(plane, lane, n, grain, x, lo, hi);
   team_minmax(team, lo, hi, rp);
   const float range = __fsub_rn(hi, lo);
-  if (!(fabsf(range) <= 3.402823466e38f) && lane == 0) report_error(a, kErrNonfinite);
-
-  // distances from the minimum, in place (x - lo is x + (-lo): the same rounding)
-  {
-    const float nlo = -lo;
-    const f32x2 nlo2 = pack2(nlo, nlo);
-#pragma unroll
-    for (int k = 0; k < G; ++k) {
-      unpack2(add2(pack2(x[k][0], x[k][1]), nlo2), x[k][0], x[k][1]);
-      unpack2(add2(pack2(x[k][2], x[k][3]), nlo2), x[k][2], x[k][3]);
-      if (!(FULL && VEC)) {
-        const uint32_t g = lane + (uint32_t)(k * TT);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const bool in = VEC ? g < groups : g * 4u + e < pl.HW;
-          x[k][e] = in ? x[k][e] : 0.0f;
-        }
-      }
-    }
-  }
-
-  uint32_t cls = kClsNormal, n_out = 0;
+  if (!(fabsf(range) <= 3.402823466e38f) && lane == 0 && active) report_error(a, kErrNonfinite);
+  uint32_t cls = kClsNormal, n_out = 0, as = 0, aq = 0;
+  const SigmaScale sc = sigma_scale(range);
+  run_distances<DT, K, TT, EDGE, (SIGMA != 0)>(lane, n, lo, sc, x, as, aq);
   if (SIGMA) {
-    const SigmaScale sc = sigma_scale(range);
-    if (sc.applies) {  // (the same for every thread of the team)
-      uint32_t as = 0, aq = 0;
-#pragma unroll
-      for (int k = 0; k < G; ++k) sigma_addends4(x[k][0], x[k][1], x[k][2], x[k][3], sc, as, aq);
-      long long Is, Iq;
-      team_sum2(team, (int32_t)(as - (uint32_t)G * kMagicBits), (int32_t)(aq - (uint32_t)G * kMagicBits), Is, Iq, rp);
-      float dlo, dhi;
-      if (TT > 32) sigma_thresholds(Is, Iq, sc, pl.inv_hw, dlo, dhi);  // (a CTA team's sums may pass 32 bits)
-      else sigma_thresholds((int32_t)Is, (int32_t)Iq, sc, pl.inv_hw, dlo, dhi);
-      uint32_t cnt = 0;
-      if (range > dhi || 0.0f < dlo) {  // otherwise no element can lie outside: the count is zero
-        uint32_t c[4] = {0, 0, 0, 0};  // four counters: short dependency chains
-        if (!(0.0f < dlo)) {           // nothing below: one compare per element
-#pragma unroll
-          for (int k = 0; k < G; ++k) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) c[e] += x[k][e] > dhi;
-          }
-          cnt = (c[0] + c[1]) + (c[2] + c[3]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < G; ++k) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) c[e] += (x[k][e] > dhi) || (x[k][e] < dlo);
-          }
-          cnt = (c[0] + c[1]) + (c[2] + c[3]);
-          if (!(FULL && VEC)) cnt -= npad;  // padded positions (distance 0, below the lower threshold) are not elements
-        }
-        cnt = team_sum_u32(team, cnt, rp);
-      }
-      n_out = cnt;
-      if ((uint64_t)n_out * pl.rho_den > (uint64_t)pl.rho_num * pl.HW) cls = kClsSalient;
+    long long Is, Iq;
+    team_sum2(team, (int32_t)(as - (uint32_t)K * kMagicBits), (int32_t)(aq - (uint32_t)K * kMagicBits), Is, Iq, rp);
+    float dlo, dhi;
+    sigma_thresholds((int32_t)Is, (int32_t)Iq, sc, pl.inv_hw, dlo, dhi);
+    // outside [dlo, dhi] of a plane that the rule does not apply to, or whose extremes lie inside, there is nothing
+    const bool look = sc.applies && (range > dhi || 0.0f < dlo);
+    if (__any_sync(full, look)) {
+      const uint32_t cnt = team_sum_u32(team, run_count<DT, K, TT, EDGE>(lane, n, dlo, dhi, x), rp);
+      n_out = look ? cnt : 0u;
     }
+    if ((uint64_t)n_out * pl.rho_den > (uint64_t)pl.rho_num * pl.HW) cls = kClsSalient;
   } else if (pl.mode == kModeAll) {
     cls = kClsSalient;
   } else if (pl.mode >= kModeChannel) {
     cls = channel_class(pl, a, gp, n_out);
   }
-
   const uint32_t meta = cls | (n_out << 2);
-  if (cls != kClsNormal || !d.fits) return meta;  // (the caller sees to a plane that is not normal)
-  const uint32_t bits = (uint32_t)pl.bits;
+  if (cls != kClsNormal || !d.fits || !active) return meta;  // (the caller sees to a plane that is not normal)
   float inv, scale;
-  quant_params(range, (1u << bits) - 1u, inv, scale);
+  quant_params(range, (1u << pl.bits) - 1u, inv, scale);
   uint8_t* slot = d.dst + pl.slots_off + gp * pl.npay;
-  if (SIGMA == 2) {
-    // random rounding: one generator call per group, counter = (group, plane, tensor id), key = seed; a padded
-    // position (distance 0) gets code 0 whatever the draw
-    const uint32_t L = (1u << bits) - 1u;
-#pragma unroll
-    for (int k = 0; k < G; ++k) {
-      const uint32_t g = lane + (uint32_t)(k * TT);
-      if (FULL || g < groups) {
-        uint32_t rnd[4];
-        philox4x32_10(g, (uint32_t)gp, (uint32_t)pl.tensor_id, (uint32_t)(pl.tensor_id >> 32), (uint32_t)pl.seed,
-                      (uint32_t)(pl.seed >> 32), rnd);
-        uint32_t word = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) word |= quant_code_random(x[k][e], inv, L, rnd[e]) << (e * bits);
-        if (bits == 2u) slot[g] = (uint8_t)word;
-        else if (bits == 4u) reinterpret_cast<uint16_t*>(slot)[g] = (uint16_t)word;
-        else reinterpret_cast<uint32_t*>(slot)[g] = word;
-      }
-    }
-  } else if (bits == 2u) FH_STORE_CODES(2)
-  else if (bits == 4u) FH_STORE_CODES(4)
-  else FH_STORE_CODES(8)
-  // zero padding of the slot behind the codes
-  const uint32_t code_bytes = groups * bits / 2u;
-  if (code_bytes < pl.npay) {
-    for (uint32_t o = code_bytes + lane; o < a4(code_bytes); o += TT) slot[o] = 0;
-    for (uint32_t o = a4(code_bytes) + 4u * lane; o < pl.npay; o += 4u * TT)
-      *reinterpret_cast<uint32_t*>(slot + o) = 0u;
-  }
+  run_codes_any<DT, SIGMA, K, TT, EDGE>(pl, plane, grain, lane, n, lo, inv, 0u, gp, slot, x);
+  pad_slot(pl, slot, lane, TT);
   if (lane == 0) store_table_entry(d, gp, (uint32_t)((pl.slots_off + gp * pl.npay) >> 4), meta, lo, scale);
   return meta;
-}
-
-// Picks the specialisation of the sweep.  FULLVEC kernels are launched only for planes of exactly
-// G * TT whole groups, so they carry nothing but the lean variant; the others choose at run time.
-template <int DT, int SIGMA, int G, int TT, bool FULLVEC>
-__device__ __forceinline__ uint32_t plane_sweep_any(const Team& team, const Plan& pl, const Dest& d,
-                                                    const CompressArgs& a, const uint8_t* plane, uint64_t gp,
-                                                    bool vec, uint32_t& rp) {
-  if (FULLVEC) return plane_sweep<DT, SIGMA, G, TT, true, true>(team, pl, d, a, plane, gp, rp);
-  if (vec) return plane_sweep<DT, SIGMA, G, TT, false, true>(team, pl, d, a, plane, gp, rp);
-  return plane_sweep<DT, SIGMA, G, TT, false, false>(team, pl, d, a, plane, gp, rp);
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -974,7 +1082,7 @@ static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, uint32_t s, u
 // planes are listed in plane order (their markers carry class, count and size), placed by one scan over
 // the list, and dealt out to the warps in turn.
 template <int DT, int TT>
-__device__ __noinline__ void warp_phase2(BlockCtl* c, uint8_t* stages, uint8_t* sal_base) {
+__device__ __noinline__ void warp_phase2(BlockCtl* c, BlockList* l, uint8_t* stages, uint8_t* sal_base) {
   const Plan& pl = c->pl;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const Team team = make_warp_team(nullptr);
@@ -1012,21 +1120,21 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, uint8_t* stages, uint8_t* 
       }
       if (mine) {
         const uint32_t r = before + __popc(leaders & ((1u << lane) - 1u));
-        c->list_at[r] = mk.x;
-        c->list_meta[r] = mk.y;
-        c->list_lp[r] = (uint16_t)lp;
+        l->list_at[r] = mk.x;
+        l->list_meta[r] = mk.y;
+        l->list_lp[r] = (uint16_t)lp;
       }
       __syncthreads();
       if (warp == 0) {  // places within the tile's part of the overflow region, and the tile's place
         uint32_t run = 0;
         for (uint32_t r0 = 0; r0 < total; r0 += 32u) {
-          const uint32_t v = r0 + lane < total ? c->list_at[r0 + lane] : 0u;
+          const uint32_t v = r0 + lane < total ? l->list_at[r0 + lane] : 0u;
           uint32_t incl = v;
           for (uint32_t o = 1; o < 32u; o <<= 1) {
             const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
             if (lane >= o) incl += up;
           }
-          if (r0 + lane < total) c->list_at[r0 + lane] = run + incl - v;
+          if (r0 + lane < total) l->list_at[r0 + lane] = run + incl - v;
           run += __shfl_sync(0xFFFFFFFFu, incl, 31);
         }
         bool ok = true;
@@ -1041,9 +1149,9 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, uint8_t* stages, uint8_t* 
       __syncthreads();
       if (c->ok && warp < (uint32_t)kWarps)
         for (uint32_t r = warp; r < total; r += (uint32_t)kWarps) {
-          const uint32_t pl_lp = c->list_lp[r];
+          const uint32_t pl_lp = l->list_lp[r];
           warp_plane_write<DT>(team, pl, c->d, (uint64_t)p0 + pl_lp, tbuf + (uint64_t)pl_lp * pl.plane_bytes, sal,
-                               c->list_meta[r] >> 2, c->base + c->list_at[r]);
+                               l->list_meta[r] >> 2, c->base + l->list_at[r]);
           __syncwarp();
         }
       __syncthreads();
@@ -1052,7 +1160,7 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, uint8_t* stages, uint8_t* 
   }
 }
 
-template <int DT, int SIGMA, int TT, bool FULLVEC>
+template <int DT, int SIGMA, int TT, int K, int EDGE>
 __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 5];
@@ -1061,6 +1169,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   __shared__ volatile uint32_t s_abort;
   __shared__ uint32_t s_last;
   __shared__ BlockCtl s_ctl;
+  __shared__ BlockList s_list;
 
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t nstage = pl.nstage;
@@ -1151,13 +1260,15 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
         const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
         const uint32_t bytes = np * (uint32_t)pl.plane_bytes;
         uint8_t* stage = smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes;
-        if ((bytes & 15u) == 0u) {
+        // whole 16-byte chunks by bulk copy; what is left of the tensor's last tile by this thread, ahead of its arrival
+        const uint32_t whole = bytes & ~15u;
+        const uint8_t* from = a.src + (uint64_t)p0 * pl.plane_bytes;
+        for (uint32_t i = whole; i < bytes; i += 2u) *reinterpret_cast<uint16_t*>(stage + i) = *reinterpret_cast<const uint16_t*>(from + i);
+        if (whole) {
           fence_proxy_async();
-          mbar_expect_tx(&s_full[s], bytes);
-          bulk_g2s(stage, a.src + (uint64_t)p0 * pl.plane_bytes, bytes, &s_full[s]);
-        } else {  // ragged last tile of a tensor of ragged planes: plain loads by this thread
-          const uint16_t* g = reinterpret_cast<const uint16_t*>(a.src + (uint64_t)p0 * pl.plane_bytes);
-          for (uint32_t i = 0; i < bytes / 2u; ++i) reinterpret_cast<uint16_t*>(stage)[i] = g[i];
+          mbar_expect_tx(&s_full[s], whole);
+          bulk_g2s(stage, from, whole, &s_full[s]);
+        } else {
           mbar_arrive(&s_full[s]);
         }
       }
@@ -1176,10 +1287,9 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     }
   } else {
     // ======================= consumers =======================
-    constexpr int G = 8;  // groups per thread: a plane has at most 8 * TT groups
     const Team team = make_team(TT, s_red);
     const uint32_t my_team = tid / TT;
-    const bool vec = (pl.plane_bytes & 15u) == 0u;
+    const uint32_t grain = plane_grain(pl);
     uint32_t rp = 0, s = 0, phase = 0;
     for (;;) {
       const uint32_t par = (phase >> s) & 1u;
@@ -1194,13 +1304,11 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
       if (tile >= pl.ntiles) break;
       const uint32_t p0 = tile * pl.ppt;
       const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
-      const uint32_t lp = my_team;
+      const uint32_t lp = my_team, at = min(lp, np - 1u);
       const bool active = lp < np;
       const uint8_t* stage = smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes;
-      uint32_t meta = kClsNormal;
-      if (active)
-        meta = plane_sweep_any<DT, SIGMA, G, TT, FULLVEC>(team, pl, d, a, stage + (uint64_t)lp * pl.plane_bytes,
-                                                          (uint64_t)p0 + lp, vec, rp);
+      const uint32_t meta = plane_sweep<DT, SIGMA, K, TT, EDGE>(team, pl, d, a, stage + (uint64_t)at * pl.plane_bytes,
+                                                                (uint64_t)p0 + at, grain, active, rp);
       if (scan_on) {  // phase 1 of the block-wise path
         const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, active && (meta & 3u) != kClsNormal && team.lane == 0);
         if (leaders)
@@ -1219,7 +1327,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   }
   if (scan_on) {
     __syncthreads();
-    if (s_ctl.head != kNoTile && !s_abort) warp_phase2<DT, TT>(&s_ctl, smem + pl.sm_tile, smem + pl.sm_sal);
+    if (s_ctl.head != kNoTile && !s_abort) warp_phase2<DT, TT>(&s_ctl, &s_list, smem + pl.sm_tile, smem + pl.sm_sal);
   }
   cta_exit(pl, a, d, &s_last);
 }
@@ -1234,43 +1342,66 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
 // An outlier-rich plane is measured by the whole CTA while it lies in its stage and written in phase 2.
 // -------------------------------------------------------------------------------------------------
 // Phase 1: the plane in `plane` is measured, tile (= plane) `tile` published and put on the CTA's list.
-template <int DT, int NT>
+template <int DT>
 __device__ __noinline__ void cta_tile_measure(BlockCtl* c, double* red, const uint8_t* plane, uint32_t* sal, uint32_t tile,
                                               uint32_t meta) {
-  const Team team = make_team(NT, red);
+  const Team team = make_cta_team(blockDim.x, red);
   const SalientInfo info = salient_measure<DT>(team, c->pl, plane, sal);
   bool raw;
   const uint32_t units = plane_units(c->pl, info, raw);
   if (threadIdx.x == 0) {
+    c->measured = tile;
+    c->measured_info = info;
     if (c->d.fits) store_marker(c->d, tile, meta, units);
     publish_tile(c, tile, units, raw ? 0u : 1u, raw ? 1u : 0u);
   }
 }
 
-// Phase 2 of the CTA-team kernel: every plane the CTA has put off, newest first.
-template <int DT, int NT>
-__device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage, uint32_t* sal, uint64_t* bar, uint32_t parity) {
+// Bulk load of plane `gp` with the 16-byte chunks around it (one thread); plane_head says where the plane starts in the
+// stage.  The last bytes of a tensor that does not end on a 16-byte boundary are copied by the thread itself, ahead of
+// its arrival at the barrier.
+__device__ __forceinline__ uint32_t plane_head(const Plan& pl, uint64_t gp) { return (uint32_t)(gp * pl.plane_bytes) & 15u; }
+__device__ __forceinline__ void plane_load(const Plan& pl, const uint8_t* src, uint64_t gp, uint8_t* stage, uint64_t* bar) {
+  const uint64_t start = gp * pl.plane_bytes, a0 = start & ~15ull;
+  const uint64_t whole = min((start + pl.plane_bytes + 15ull) & ~15ull, pl.dense_bytes & ~15ull);
+  for (uint64_t i = whole; i < start + pl.plane_bytes; i += 2)
+    *reinterpret_cast<uint16_t*>(stage + (i - a0)) = *reinterpret_cast<const uint16_t*>(src + i);
+  fence_proxy_async();
+  mbar_expect_tx(bar, (uint32_t)(whole - a0));
+  bulk_g2s(stage, src + a0, (uint32_t)(whole - a0), bar);
+}
+
+// Phase 2 of the CTA-team kernels: every plane the CTA has put off, newest first.  The newest often still lies in a
+// stage (`c->held`), and what was measured of it in the scratch.
+template <int DT>
+__device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal, uint64_t* bar, uint32_t parity) {
   const Plan& pl = c->pl;
-  const Team team = make_team(NT, red);
+  const Team team = make_cta_team(blockDim.x, red);
   const uint32_t tid = threadIdx.x;
   for (uint32_t tile = c->head; tile != kNoTile;) {
     const uint32_t next = c->a.defer_next[tile];
-    if (tid == 0) {
-      fence_proxy_async();
-      mbar_expect_tx(bar, (uint32_t)pl.plane_bytes);
-      bulk_g2s(stage, c->a.src + (uint64_t)tile * pl.plane_bytes, (uint32_t)pl.plane_bytes, bar);
-    }
-    bool ready = mbar_wait(bar, parity, 1u << 20);
-    ready = __syncthreads_and(ready);
-    parity ^= 1u;
-    if (!ready) {  // the load timed out: report, wait (bounded) for the copy, give up
+    const uint32_t at = c->held[1] == tile ? 1u : 0u;
+    const uint8_t* plane = stages + (uint64_t)at * pl.stage_bytes + plane_head(pl, tile);
+    if (c->held[at] != tile) {  // (the same for every thread)
+      __syncthreads();
       if (tid == 0) {
-        report_error(c->a, kErrTimeout);
-        mbar_wait(bar, parity ^ 1u, 1u << 10);
+        c->held[0] = tile;
+        plane_load(pl, c->a.src, tile, stages, bar);
       }
-      return;
+      bool ready = mbar_wait(bar, parity, 1u << 20);
+      ready = __syncthreads_and(ready);
+      parity ^= 1u;
+      if (!ready) {  // the load timed out: report, wait (bounded) for the copy, give up
+        if (tid == 0) {
+          report_error(c->a, kErrTimeout);
+          mbar_wait(bar, parity ^ 1u, 1u << 10);
+        }
+        return;
+      }
     }
-    const SalientInfo info = salient_measure<DT>(team, pl, stage, sal);
+    SalientInfo info;
+    if (c->measured == tile) info = c->measured_info;
+    else info = salient_measure<DT>(team, pl, plane, sal);
     bool raw;
     const uint32_t units = plane_units(pl, info, raw);
     if (tid < 32u) {
@@ -1284,7 +1415,8 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
       }
     }
     __syncthreads();
-    if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, stage, info, sal, load_marker(c->d, tile).y >> 2, c->base);
+    if (tid == 0) c->measured = kNoTile;
+    if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, plane, info, sal, load_marker(c->d, tile).y >> 2, c->base);
     __syncthreads();
     tile = next;
   }
@@ -1368,7 +1500,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
   if (tid == 0 && scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
     s_ctl.pl = pl;
     s_ctl.a = a;
-    s_ctl.head = kNoTile;
+    s_ctl.head = s_ctl.measured = s_ctl.held[0] = s_ctl.held[1] = kNoTile;
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
@@ -1509,7 +1641,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
         issue(s);  // the stage is free: next load
       }
     } else {  // (the same for every thread) phase 1 of the block-wise path
-      cta_tile_measure<DT, NT>(&s_ctl, s_red, plane, sal, tile, cls | (n_out << 2));
+      cta_tile_measure<DT>(&s_ctl, s_red, plane, sal, tile, cls | (n_out << 2));
       __syncthreads();  // every thread is done with the stage
       if (tid == 0) issue(s);
     }
@@ -1528,46 +1660,55 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
   if (scan_on) {
     __syncthreads();
     if (s_ctl.head != kNoTile && !s_abort)
-      cta_phase2<DT, NT>(&s_ctl, s_red, smem + pl.sm_tile, sal, &s_full[0], phase & 1u);
+      cta_phase2<DT>(&s_ctl, s_red, smem + pl.sm_tile, sal, &s_full[0], phase & 1u);
   }
   cta_exit(pl, a, d, &s_last);
 }
 
 // -------------------------------------------------------------------------------------------------
-// CTA-team kernel, register variant: planes of 257 to NT * G groups (whole 16-byte chunks).  As compress_cta, but
-// every thread takes its G groups out of the stage once and keeps them in registers for the whole sweep
-// (plane_sweep with the CTA as the team): one pass over shared memory instead of three, the distances
-// computed once.  A normal plane's stage is free as soon as the sweep returns -- its last read of the stage
-// lies before the first reduction's barrier -- and takes the next load at once.
+// CTA-team kernel, register variant: planes of more than 1024 elements, up to kCtaMaxWarps * kCtaGroups groups.  One plane
+// per tile; the CTA's warps (as few as hold the plane) take equal contiguous runs of its groups and keep them in
+// registers, so the plane is read from its stage once.  Planes may start anywhere: the load takes in the 16-byte chunks
+// around them.
+//
+// What every warp repeats per plane -- reductions, scalar steps, barriers: about 200 instructions -- is spread over up to
+// 56 elements a lane, and what can wait does: the codes are computed and stored as if the plane were normal while the
+// first warp works out the three-sigma thresholds, and the count of outliers is looked at behind the NEXT plane's
+// first barrier, so that a plane costs three barriers.  A plane that turns out outlier-rich is still in its stage then;
+// it is measured at the end of that turn, and phase 2 rewrites its slot.
 // -------------------------------------------------------------------------------------------------
-template <int DT, bool SIGMA, int NT, int G, bool FULL>
-__global__ void __launch_bounds__(NT, NT > 256 ? 2 : (NT > 128 ? 3 : 6)) compress_cta_regs(const Plan pl, const CompressArgs a) {
+constexpr int kCtaThreads = kCtaMaxWarps * 32;
+
+template <int DT, int SIGMA, int K, int EDGE>
+__global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 5];
-  __shared__ __align__(8) uint64_t s_full[kMaxStages];
-  __shared__ uint32_t s_tiles[kMaxStages];
-  __shared__ uint32_t s_abort, s_last;
+  __shared__ __align__(8) uint64_t s_full[2];
+  __shared__ uint32_t s_tiles[2], s_abort, s_last, s_count[2];
+  __shared__ float2 s_thr;
   __shared__ BlockCtl s_ctl;
 
-  const uint32_t tid = threadIdx.x;
-  const Team team = make_team(NT, s_red);
-  const uint32_t nstage = pl.nstage;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const Team team = make_cta_team(blockDim.x, s_red);
   const bool scan_on = pl.mode != kModeOff;
   uint32_t* sal = reinterpret_cast<uint32_t*>(smem + pl.sm_sal);
   uint32_t rp = 0;
-  // Thread 0 requests the tiles and issues the loads: the first nstage tiles in one request, later ones one
-  // at a time, the request running one tile ahead of its use.  Tiles come in ticket order.
+  // Thread 0 requests the tiles and issues the loads: the first two in one request (one, when there are too few for every
+  // CTA to get two), later ones one at a time, the request running one tile ahead of its use.  Tiles come in ticket order.
   uint32_t next_ticket = 0, issued = 0;
+  const uint32_t early = pl.nstage;
   if (tid == 0) {
-    for (uint32_t s = 0; s < nstage; ++s) mbar_init(&s_full[s], 1);
+    mbar_init(&s_full[0], 1);
+    mbar_init(&s_full[1], 1);
     fence_mbar_init();
     s_abort = 0;
+    s_count[0] = s_count[1] = 0;
     *cta_dirty() = 0u;
-    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
+    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)early);
     if (scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
       s_ctl.pl = pl;
       s_ctl.a = a;
-      s_ctl.head = kNoTile;
+      s_ctl.head = s_ctl.measured = s_ctl.held[0] = s_ctl.held[1] = kNoTile;
     }
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
@@ -1576,17 +1717,16 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : (NT > 128 ? 3 : 6)) compres
     const uint32_t t = next_ticket;
     s_tiles[s] = t;
     if (t < pl.ntiles) {
-      fence_proxy_async();
-      mbar_expect_tx(&s_full[s], (uint32_t)pl.plane_bytes);
-      bulk_g2s(smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes, a.src + (uint64_t)t * pl.plane_bytes,
-               (uint32_t)pl.plane_bytes, &s_full[s]);
+      if (scan_on) s_ctl.held[s] = t;
+      plane_load(pl, a.src, t, smem + (uint64_t)s * pl.stage_bytes, &s_full[s]);
       ++issued;
-      next_ticket = issued < nstage ? t + 1u : (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
+      next_ticket = issued < early ? t + 1u : (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
     }
   };
   if (tid == 0) {  // the first loads before anything else
-    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
-    for (uint32_t s = 0; s < nstage; ++s) issue(s);
+    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)early);
+    issue(0);
+    issue(1);
   }
   const Dest d = make_dest(pl, a);
   if (tid == 0) {
@@ -1595,35 +1735,112 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : (NT > 128 ? 3 : 6)) compres
   }
   __syncthreads();
 
+  const uint32_t grain = plane_grain(pl);
+  const uint32_t g0 = pl.groups * warp / team.nwarps, g1 = pl.groups * (warp + 1u) / team.nwarps;
+  const int32_t n = (int32_t)(min(4u * g1, pl.HW) - 4u * g0);
+  // the plane before, whose class is still open: its tile (kNoTile: none), and for its table entry minimum, scale
+  uint32_t prev = kNoTile, prev_meta = 0;
+  float prev_lo = 0.0f, prev_scale = 0.0f;
+  // Class of the plane before, behind a barrier that all its counts precede (every thread gets the same answer): a
+  // normal plane is complete -- table entry, publication, its stage takes the next load --, another is to be measured.
+  auto settle = [&](uint32_t s) -> bool {
+    if (prev == kNoTile) return false;
+    if (SIGMA) {
+      const uint32_t n_out = s_count[s];
+      prev_meta = ((uint64_t)n_out * pl.rho_den > (uint64_t)pl.rho_num * pl.HW ? kClsSalient : kClsNormal) | (n_out << 2);
+    }
+    if ((prev_meta & 3u) != kClsNormal) return true;
+    if (tid == 0) {
+      if (d.fits) store_table_entry(d, prev, (uint32_t)((pl.slots_off + (uint64_t)prev * pl.npay) >> 4), prev_meta, prev_lo, prev_scale);
+      if (scan_on) scan_publish(a.scan, prev, 0u);
+      issue(s);
+    }
+    return false;
+  };
+  auto measure = [&](uint32_t s) {
+    cta_tile_measure<DT>(&s_ctl, s_red, smem + (uint64_t)s * pl.stage_bytes + plane_head(pl, prev), sal, prev, prev_meta);
+    __syncthreads();  // every thread is done with the stage
+    if (tid == 0) issue(s);
+  };
+
   uint32_t s = 0, phase = 0;
   for (;;) {
     const uint32_t tile = s_tiles[s];
     if (tile >= pl.ntiles) break;
-    bool ready = mbar_wait(&s_full[s], (phase >> s) & 1u, 1u << 20);
+    const bool ready = mbar_wait(&s_full[s], (phase >> s) & 1u, 1u << 20);
     phase ^= 1u << s;
-    if (!__syncthreads_and(ready)) {  // a load timed out (the same answer for every thread)
-      if (tid == 0) s_abort = 1;
-      break;
-    }
-    const uint8_t* plane = smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes;
-    const uint32_t meta = plane_sweep<DT, SIGMA, G, NT, FULL, true>(team, pl, d, a, plane, (uint64_t)tile, rp);
-    if ((meta & 3u) == kClsNormal) {  // (the same for every thread) complete; every read of the stage lies behind a barrier
-      if (tid == 0) {
-        if (scan_on) scan_publish(a.scan, tile, 0u);
-        issue(s);
+    float x[K][4], lo, hi;
+    const uint8_t* run = smem + (uint64_t)s * pl.stage_bytes + plane_head(pl, tile) + (uint64_t)g0 * (DT == kF32 ? 16u : 8u);
+    run_load<DT, K, 32, EDGE>(run, lane, n, grain, x, lo, hi);
+    if (!ready) s_abort = 1;
+    team_minmax(team, lo, hi, rp);  // the first barrier
+    if (s_abort) break;
+    const bool open = settle(s ^ 1u);
+    const float range = __fsub_rn(hi, lo);
+    if (!(fabsf(range) <= 3.402823466e38f) && tid == 0) report_error(a, kErrNonfinite);
+    const SigmaScale sc = sigma_scale(range);
+    uint32_t as = 0, aq = 0;
+    run_distances<DT, K, 32, EDGE, (SIGMA != 0)>(lane, n, lo, sc, x, as, aq);
+    const bool rule = SIGMA && sc.applies;  // (the same for every thread)
+    if (SIGMA) {
+      int32_t pa = (int32_t)(as - (uint32_t)K * kMagicBits), pb = (int32_t)(aq - (uint32_t)K * kMagicBits);
+      asm volatile("redux.sync.add.s32 %0, %0, %1;" : "+r"(pa) : "r"(0xFFFFFFFFu));
+      asm volatile("redux.sync.add.s32 %0, %0, %1;" : "+r"(pb) : "r"(0xFFFFFFFFu));
+      int2* r = reinterpret_cast<int2*>(red_half(team, rp));
+      if (lane == 0) r[warp] = make_int2(pa, pb);
+      __syncthreads();  // the second barrier
+      if (warp == 0 && rule) {  // the first warp adds up the warps' sums and works out the thresholds, for all
+        const int2 pr = lane < team.nwarps ? r[lane] : make_int2(0, 0);
+        const long long Is = warp_sum_s32_wide(pr.x), Iq = warp_sum_s32_wide(pr.y);
+        float tl, th;
+        sigma_thresholds(Is, Iq, sc, pl.inv_hw, tl, th);
+        if (lane == 0) s_thr = make_float2(tl, th);
       }
-    } else {  // phase 1 of the block-wise path
-      cta_tile_measure<DT, NT>(&s_ctl, s_red, plane, sal, tile, meta);
-      __syncthreads();  // every thread is done with the stage
-      if (tid == 0) issue(s);
+      if (tid == 0) s_count[s ^ 1u] = 0;  // (settled by every thread before the barrier just passed)
     }
-    s = s + 1 == nstage ? 0 : s + 1;
-    // s_tiles[s] for the next iteration was written at least one barrier ago (nstage >= 2)
+    float inv, scale;
+    quant_params(range, (1u << pl.bits) - 1u, inv, scale);
+    uint32_t n_out = 0, cls = kClsNormal;
+    if (!SIGMA) {
+      if (pl.mode == kModeAll) cls = kClsSalient;
+      if (pl.mode >= kModeChannel) cls = channel_class(pl, a, tile, n_out);
+    }
+    if (d.fits && cls == kClsNormal) {
+      uint8_t* slot = d.dst + pl.slots_off + (uint64_t)tile * pl.npay;
+      run_codes_any<DT, SIGMA, K, 32, EDGE>(pl, run, grain, lane, n, lo, inv, g0, tile, slot, x);
+      pad_slot(pl, slot, tid, blockDim.x);
+    }
+    if (rule) {
+      __syncthreads();  // the third barrier: the thresholds
+      const float dlo = s_thr.x, dhi = s_thr.y;
+      if (range > dhi || 0.0f < dlo) {  // otherwise no element can lie outside
+        uint32_t cnt = run_count<DT, K, 32, EDGE>(lane, n, dlo, dhi, x);
+        asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(cnt) : "r"(0xFFFFFFFFu));
+        if (lane == 0 && cnt) atomicAdd(&s_count[s], cnt);
+      }
+    }
+    if (open) {  // the plane before, which is outlier-rich
+      __syncthreads();
+      measure(s ^ 1u);
+    }
+    prev = tile;
+    prev_meta = cls | (n_out << 2);
+    prev_lo = lo;
+    prev_scale = scale;
+    s ^= 1u;
+    // (s_tiles of the next turn was written when the plane before was settled, behind the first barrier: a later one --
+    // the second, with three-sigma statistics, or this one -- makes it known)
+    if (!SIGMA || open) __syncthreads();
+  }
+  __syncthreads();
+  if (!s_abort) {
+    const bool open = settle(s ^ 1u);
+    if (open) measure(s ^ 1u);
   }
   __syncthreads();
   if (s_abort && tid == 0) {  // a load timed out: report, then wait (bounded) for copies still in flight
     report_error(a, kErrTimeout);
-    for (uint32_t k = 0; k < nstage; ++k)
+    for (uint32_t k = 0; k < 2u; ++k)
       if (s_tiles[k] < pl.ntiles) {
         mbar_wait(&s_full[k], 0u, 1u << 10);
         mbar_wait(&s_full[k], 1u, 1u << 10);
@@ -1631,8 +1848,7 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : (NT > 128 ? 3 : 6)) compres
   }
   if (scan_on) {
     __syncthreads();
-    if (s_ctl.head != kNoTile && !s_abort)
-      cta_phase2<DT, NT>(&s_ctl, s_red, smem + pl.sm_tile, sal, &s_full[0], phase & 1u);
+    if (s_ctl.head != kNoTile && !s_abort) cta_phase2<DT>(&s_ctl, s_red, smem, sal, &s_full[0], phase & 1u);
   }
   cta_exit(pl, a, d, &s_last);
 }

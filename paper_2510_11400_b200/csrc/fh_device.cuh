@@ -13,7 +13,9 @@ namespace fh {
 
 constexpr int kThreads = 256;             // CTA size of every kernel
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxWarps = 16;            // largest CTA of any kernel: 512 threads
+constexpr int kMaxWarps = 20;            // largest CTA of any kernel: 640 threads
+constexpr int kCtaMaxWarps = 20;         // CTA-team kernel, register variant: warps of a CTA at most ...
+constexpr int kCtaGroups = 14 * 32;      // ... and groups of a warp (112 x 112: seven warps exactly)
 constexpr uint32_t kMagic = 0x31434846u;  // "FHC1"
 constexpr uint32_t kClsNormal = 0, kClsSalient = 1, kClsRaw = 2;
 constexpr int kModeAuto = 0, kModeOff = 1, kModeAll = 2, kModeChannel = 3, kModeTensor = 4;
@@ -352,14 +354,18 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
   out[3] = c3;
 }
 // Code of one element (distance d = x - lo) under random rounding: t = fp32 product d * inv, n = floor(t), and the code
-// goes up iff floor(frac(t) * 2^24) + (word >> 8) reaches 2^24.
+// goes up iff floor(frac(t) * 2^24) + r reaches 2^24, r = word >> 8.  As r is an integer that says frac(t) >= 1 - r * 2^-24,
+// a number that fp32 holds exactly: it is put together from r's upper 23 bits (1 + a * 2^-23 by bit pattern) and its
+// lowest one, and floor(t) is an addition of 2^23 rounded down.  Conversions between float and integer run at an
+// eighth of the issue rate; three of them per element made this mode a third slower than its arithmetic.
 __device__ __forceinline__ uint32_t quant_code_random(float d, float inv, uint32_t L, uint32_t word) {
   const float t = __fmul_rn(d, inv);
-  const float nf = floorf(t);
-  const uint32_t fi = (uint32_t)__fmul_rn(__fsub_rn(t, nf), 16777216.0f);
-  const uint32_t up = (fi + (word >> 8)) >> 24;
-  const uint32_t n = nf >= (float)L ? L : (uint32_t)nf;
-  return min(n + up, L);
+  const float magic = __fadd_rd(t, 8388608.0f);
+  const float frac = __fsub_rn(t, __fsub_rn(magic, 8388608.0f));
+  const float upper = __fsub_rn(2.0f, __uint_as_float((word >> 9) | 0x3F800000u));        // 1 - (r >> 1) * 2^-23
+  const float least = __fsub_rn(upper, __uint_as_float((word & 0x100u) * 0x338000u));     // ... less 2^-24 when r is odd
+  const uint32_t n = __float_as_uint(magic) - 0x4B000000u;
+  return min(n + (frac >= least ? 1u : 0u), L);
 }
 
 // Pre-quantisation of dense-block elements (Eq. 9 on integers): k = rne(fp32(x * inv2e)), |k| <= 2^24.
@@ -399,6 +405,17 @@ __device__ __forceinline__ Team make_team(uint32_t team_size, double* red) {
   }
   return t;
 }
+// The whole CTA as a team, also when it is one warp (make_team would take that for a warp among others).
+__device__ __forceinline__ Team make_cta_team(uint32_t threads, double* red) {
+  Team t;
+  t.size = threads;
+  t.red = red;
+  t.nwarps = threads >> 5;
+  t.block = true;
+  t.lane = threadIdx.x;
+  t.mask = 0xFFFFFFFFu;
+  return t;
+}
 // The warp of this thread as a team (used for the block-wise path of the warp-team kernels).
 __device__ __forceinline__ Team make_warp_team(double* red) {
   Team t;
@@ -424,11 +441,19 @@ __device__ __forceinline__ double* red_half(const Team& t, uint32_t& rp) {
   return r;
 }
 
-// min / max over the team with NaN propagation (hardware warp reduction for fp32).
+// min / max over the team with NaN propagation (hardware warp reduction for fp32; teams of a few lanes by butterflies:
+// a reduction instruction whose member mask differs within the warp is executed mask by mask, and leaves the warp's
+// teams running one after the other -- 2,870 instructions for a warp's sixteen 7 x 7 planes).
 __device__ __forceinline__ void team_minmax(const Team& t, float& lo, float& hi, uint32_t& rp) {
-  if (!t.block && t.size == 1u) return;
-  asm volatile("redux.sync.min.NaN.f32 %0, %0, %1;" : "+f"(lo) : "r"(t.mask));
-  asm volatile("redux.sync.max.NaN.f32 %0, %0, %1;" : "+f"(hi) : "r"(t.mask));
+  if (!t.block && t.size < 32u) {
+    for (uint32_t o = t.size >> 1; o > 0; o >>= 1) {
+      lo = min_nan(lo, __shfl_xor_sync(t.mask, lo, o));
+      hi = max_nan(hi, __shfl_xor_sync(t.mask, hi, o));
+    }
+    return;
+  }
+  asm volatile("redux.sync.min.NaN.f32 %0, %0, %1;" : "+f"(lo) : "r"(0xFFFFFFFFu));
+  asm volatile("redux.sync.max.NaN.f32 %0, %0, %1;" : "+f"(hi) : "r"(0xFFFFFFFFu));
   if (t.block) {
     float* r = reinterpret_cast<float*>(red_half(t, rp));
     const uint32_t warp = threadIdx.x >> 5;
@@ -462,13 +487,17 @@ __device__ __forceinline__ long long warp_sum_s32_wide(int32_t v) {
 // must fit 32 bits (at most 512 groups per warp, see sigma_addends); warps are combined in 64 bits.
 __device__ __forceinline__ void team_sum2(const Team& t, int32_t a, int32_t b, long long& A, long long& B,
                                           uint32_t& rp) {
-  if (!t.block && t.size == 1u) {
+  if (!t.block && t.size < 32u) {
+    for (uint32_t o = t.size >> 1; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(t.mask, a, o);
+      b += __shfl_xor_sync(t.mask, b, o);
+    }
     A = a;
     B = b;
     return;
   }
-  asm volatile("redux.sync.add.s32 %0, %0, %1;" : "+r"(a) : "r"(t.mask));
-  asm volatile("redux.sync.add.s32 %0, %0, %1;" : "+r"(b) : "r"(t.mask));
+  asm volatile("redux.sync.add.s32 %0, %0, %1;" : "+r"(a) : "r"(0xFFFFFFFFu));
+  asm volatile("redux.sync.add.s32 %0, %0, %1;" : "+r"(b) : "r"(0xFFFFFFFFu));
   A = a;
   B = b;
   if (t.block) {
@@ -507,8 +536,11 @@ __device__ __forceinline__ void team_sum2_wide(const Team& t, long long a, long 
 }
 
 __device__ __forceinline__ uint32_t team_sum_u32(const Team& t, uint32_t v, uint32_t& rp) {
-  if (!t.block && t.size == 1u) return v;
-  asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(v) : "r"(t.mask));
+  if (!t.block && t.size < 32u) {
+    for (uint32_t o = t.size >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(t.mask, v, o);
+    return v;
+  }
+  asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(v) : "r"(0xFFFFFFFFu));
   if (t.block) {
     uint32_t* r = reinterpret_cast<uint32_t*>(red_half(t, rp));
     const uint32_t warp = threadIdx.x >> 5;
@@ -600,7 +632,7 @@ struct HufEncode {
   uint16_t lpar[256], mpar[256];     // parent (a merged node) of a sorted leaf, of a merged node
   uint32_t cnt[32], first[32];       // symbols of a length, then running rank; a length's first code value
   uint32_t smin, smax, maxlen, nlens;
-  uint32_t stage[kMaxWarps][4 * kHufStageWords];  // chunks' bits while a warp assembles four of them
+  uint32_t stage[1][4 * kHufStageWords];  // chunks' bits while a warp assembles four of them; one per warp of the team
 };
 
 // A whole warp: code lengths and canonical codes from h->hist.  Symbols are ranked by comparison with all others (a few

@@ -28,8 +28,8 @@ inline uint32_t team_of_groups(uint32_t groups) {
 // Which kernel a plan runs on.
 struct Variant {
   bool fast = false;  // compress_warp / compress_cta (bulk-copy pipeline) instead of compress_generic
-  bool cta = false;   // fast: compress_cta (one plane per CTA) instead of compress_warp (one plane per team of lanes)
-  int G = 0;          // fast: groups per thread
+  bool cta = false;   // fast: a plane per CTA instead of compress_warp (a plane per team of lanes)
+  bool regs = false;  // cta: compress_cta_regs instead of compress_cta
 };
 
 // SMs of the current device (0: none).

@@ -16,38 +16,30 @@ int launch_cta_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
              ? FH_OK : FH_ERR_CUDA;
 }
 
-template <int DT, bool SIGMA, int NT, int G>
+template <int DT, int SIGMA, int K, int EDGE>
 int launch_cta_regs_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int grid = 0;
-  if (pl.groups == (uint32_t)(NT * G)) {
-    int rc = grid_for(compress_cta_regs<DT, SIGMA, NT, G, true>, pl.sm_total, pl.ntiles, &grid, NT);
-    if (rc != FH_OK) return rc;
-    grid = spread_grid(grid, pl.ntiles);
-    return launch_dependent(compress_cta_regs<DT, SIGMA, NT, G, true>, grid, NT, pl.sm_total, stream,
-                            with_first_request(pl, grid, 2), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
-  }
-  int rc = grid_for(compress_cta_regs<DT, SIGMA, NT, G, false>, pl.sm_total, pl.ntiles, &grid, NT);
+  int rc = grid_for(compress_cta_regs<DT, SIGMA, K, EDGE>, pl.sm_total, pl.ntiles, &grid, (int)pl.team);
   if (rc != FH_OK) return rc;
   grid = spread_grid(grid, pl.ntiles);
-  return launch_dependent(compress_cta_regs<DT, SIGMA, NT, G, false>, grid, NT, pl.sm_total, stream,
-                          with_first_request(pl, grid, 2), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+  return launch_dependent(compress_cta_regs<DT, SIGMA, K, EDGE>, grid, (int)pl.team, pl.sm_total, stream,
+                          with_first_request(pl, grid, 1), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+}
+
+// Slots per lane; as the CTA has as few warps as hold the plane, a warp's share is 225 to 448 groups (8 to 14 slots).
+template <int DT, int SIGMA>
+int launch_cta_regs(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+  const uint32_t nw = pl.team / 32u, slots = ((pl.groups + nw - 1u) / nw + 31u) / 32u;
+  if (pl.HW == nw * 4u * kCtaGroups) return launch_cta_regs_t<DT, SIGMA, 14, 0>(pl, a, stream);  // (112 x 112)
+  if (slots <= 10u) return launch_cta_regs_t<DT, SIGMA, 10, 3>(pl, a, stream);
+  if (slots <= 12u) return launch_cta_regs_t<DT, SIGMA, 12, 2>(pl, a, stream);
+  if (slots <= 13u) return launch_cta_regs_t<DT, SIGMA, 13, 1>(pl, a, stream);
+  return launch_cta_regs_t<DT, SIGMA, 14, 1>(pl, a, stream);
 }
 
 template <int DT, bool SIGMA>
-int launch_cta_g(const Plan& pl, const Variant& v, const CompressArgs& a, cudaStream_t stream) {
-  if (v.G) {
-    switch (pl.team * 16 + v.G) {
-      case 128 * 16 + 7: return launch_cta_regs_t<DT, SIGMA, 128, 7>(pl, a, stream);
-      case 128 * 16 + 8: return launch_cta_regs_t<DT, SIGMA, 128, 8>(pl, a, stream);
-      case 256 * 16 + 7: return launch_cta_regs_t<DT, SIGMA, 256, 7>(pl, a, stream);
-      case 256 * 16 + 8: return launch_cta_regs_t<DT, SIGMA, 256, 8>(pl, a, stream);
-      case 448 * 16 + 7: return launch_cta_regs_t<DT, SIGMA, 448, 7>(pl, a, stream);
-      case 512 * 16 + 8: return launch_cta_regs_t<DT, SIGMA, 512, 8>(pl, a, stream);
-    }
-    return FH_ERR_UNSUPPORTED;
-  }
+int launch_cta_g(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   switch (pl.team) {
-    case 128: return launch_cta_t<DT, SIGMA, 128>(pl, a, stream);
     case 256: return launch_cta_t<DT, SIGMA, 256>(pl, a, stream);
     case 512: return launch_cta_t<DT, SIGMA, 512>(pl, a, stream);
   }
@@ -56,7 +48,10 @@ int launch_cta_g(const Plan& pl, const Variant& v, const CompressArgs& a, cudaSt
 
 template <int DT>
 int launch_compress_cta(const Plan& pl, const Variant& v, const CompressArgs& a, cudaStream_t stream) {
-  return pl.mode == FH_SALIENT_AUTO ? launch_cta_g<DT, true>(pl, v, a, stream) : launch_cta_g<DT, false>(pl, v, a, stream);
+  const bool sigma = pl.mode == FH_SALIENT_AUTO;
+  if (!v.regs) return sigma ? launch_cta_g<DT, true>(pl, a, stream) : launch_cta_g<DT, false>(pl, a, stream);
+  if (!sigma) return launch_cta_regs<DT, 0>(pl, a, stream);
+  return pl.rounding ? launch_cta_regs<DT, 2>(pl, a, stream) : launch_cta_regs<DT, 1>(pl, a, stream);
 }
 
 }  // namespace fh
