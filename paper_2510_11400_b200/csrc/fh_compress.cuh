@@ -34,68 +34,18 @@ __device__ __forceinline__ uint32_t channel_class(const Plan& pl, const Compress
   return total * pl.rho_den > (unsigned long long)pl.rho_num * pl.N * pl.HW ? kClsSalient : kClsNormal;
 }
 
-// A CTA whose threads change one of the call's counters (error code, overflow size, plane counts) notes it in
-// this flag; cta_exit passes it on through the exit counter, so that the last CTA of a call in which nobody did
-// -- every plane normal, no error: the usual case -- neither fences nor reads the counters back.
-__device__ __forceinline__ volatile uint32_t* cta_dirty() {
-  __shared__ uint32_t flag;
-  return &flag;
+// What a CTA adds to the call's sums: the overflow units and numbers of its outlier-rich planes, and whether it has
+// reported an error.  They stay with the CTA until it leaves (cta_exit).
+struct CtaTotals {
+  uint32_t units, nsal, nraw, err;
+};
+__device__ __forceinline__ CtaTotals* cta_totals() {
+  __shared__ CtaTotals t;
+  return &t;
 }
 __device__ __forceinline__ void report_error(const CompressArgs& a, uint32_t code) {
-  *cta_dirty() = 1u;
+  *(volatile uint32_t*)&cta_totals()->err = 1u;
   atomicMax(&a.sc->status, (unsigned long long)code);
-}
-
-// One 8x8 block in the registers of a warp: lane l holds the elements (l >> 3, l & 7) and
-// ((l >> 3) + 4, l & 7) of the block, i.e. raster positions l and l + 32.  Positions outside the
-// plane count as value 0.
-struct BlockRegs {
-  float x0, x1;    // values (rows 0-3, rows 4-7)
-  bool in0, in1;   // the positions lie inside the plane
-  uint32_t idx0;   // plane index of the first position; the second is idx0 + 4 W
-};
-template <int DT>
-__device__ __forceinline__ BlockRegs block_load(const uint8_t* plane, int H, int W, int by, int bx, uint32_t lane) {
-  BlockRegs r;
-  const int y0 = by * 8 + (int)(lane >> 3), x = bx * 8 + (int)(lane & 7u);
-  r.in0 = y0 < H && x < W;
-  r.in1 = y0 + 4 < H && x < W;
-  r.idx0 = (uint32_t)y0 * (uint32_t)W + (uint32_t)x;
-  r.x0 = r.in0 ? load_elem<DT>(plane, r.idx0) : 0.0f;
-  r.x1 = r.in1 ? load_elem<DT>(plane, r.idx0 + 4u * (uint32_t)W) : 0.0f;
-  return r;
-}
-
-// Residual codes of a dense block (Eq. 7-9): first-order Lorenzo prediction on the pre-quantised
-// integers k, neighbours outside the block count as 0.  Every element is independent because
-// prediction runs on k, which follows from the input alone; the neighbours' k come from the other
-// lanes by shuffle.  code0/code1: the lane's two code bytes; m0/m1: ballots of the verbatim elements.
-__device__ __forceinline__ void block_codes(const BlockRegs& r, float inv2e, uint32_t lane, uint32_t& code0,
-                                            uint32_t& code1, uint32_t& m0, uint32_t& m1) {
-  const uint32_t full = 0xFFFFFFFFu, c = lane & 7u, r0 = lane >> 3;
-  bool big0, big1;
-  const int32_t k0 = dense_k(r.x0, inv2e, &big0), k1 = dense_k(r.x1, inv2e, &big1);
-  int32_t left0 = __shfl_up_sync(full, k0, 1), up0 = __shfl_up_sync(full, k0, 8), ul0 = __shfl_up_sync(full, k0, 9);
-  int32_t left1 = __shfl_up_sync(full, k1, 1), up1 = __shfl_up_sync(full, k1, 8), ul1 = __shfl_up_sync(full, k1, 9);
-  const int32_t up1r = __shfl_sync(full, k0, 24 + (int)c), ul1r = __shfl_sync(full, k0, 23 + (int)c);  // row 3 feeds row 4
-  if (r0 == 0) {
-    up0 = 0;
-    ul0 = 0;
-    up1 = up1r;
-    ul1 = ul1r;
-  }
-  if (c == 0) {
-    left0 = 0;
-    ul0 = 0;
-    left1 = 0;
-    ul1 = 0;
-  }
-  const int32_t d0 = k0 - (up0 + left0 - ul0), d1 = k1 - (up1 + left1 - ul1);
-  const bool v0 = r.in0 && (big0 || d0 > 127 || d0 < -127), v1 = r.in1 && (big1 || d1 > 127 || d1 < -127);
-  code0 = !r.in0 ? 128u : (v0 ? 0u : (uint32_t)(d0 + 128));
-  code1 = !r.in1 ? 128u : (v1 ? 0u : (uint32_t)(d1 + 128));
-  m0 = __ballot_sync(full, v0);
-  m1 = __ballot_sync(full, v1);
 }
 
 // Raw plane: verbatim copy through the slot into the overflow part, zero padded.
@@ -106,162 +56,135 @@ static __device__ __noinline__ void raw_write(const Team t, const Plan& pl, cons
 }
 
 // -------------------------------------------------------------------------------------------------
-// Small planes (at most kSmallBlocks blocks and fewer than 32 rows: 7x7, 8x8, 14x14, 16x16, ...) take the
-// block-wise path in the registers of one warp: no measuring scratch, no second look at the plane.  The
-// results are those of salient_measure / salient_write.
+// Small planes (at most four blocks: 7x7, 8x8, 14x14, 16x16, ...) are encoded by one warp in one step, a lane per block
+// row as in salient_measure: the blocks of one plane, or (FOUR) the single blocks of four planes, plane q = lane & 3.
+// The elements are in registers, so the payload -- shorter than the plane, or the plane would be stored raw -- is put
+// together in shared memory over the plane itself; what is left to do once its place is known is a copy.
+// With a lane per two elements and a second encoding when the place was known, a plane took 1.6 us and 1.8 us of a warp's
+// latency; the four of a step now take about the first together, and 0.5 us for the copy.
 // -------------------------------------------------------------------------------------------------
 constexpr uint32_t kSmallBlocks = 4;
-__device__ __forceinline__ bool is_small_plane(const Plan& pl) { return pl.nblk <= kSmallBlocks && pl.H < 32 && !pl.entropy; }
+__device__ __forceinline__ bool is_small_plane(const Plan& pl) { return pl.nblk <= kSmallBlocks && !pl.entropy; }
+// Where a small plane's payload begins: its first word boundary (a bf16 plane may start between two).
+__device__ __forceinline__ uint8_t* small_payload(uint8_t* plane) { return plane + (smem_u32(plane) & 2u); }
 
-struct SmallBlocks {
-  uint32_t z0[kSmallBlocks], z1[kSmallBlocks];  // non-zero masks of the block's two halves (ballots)
-  uint32_t m0[kSmallBlocks], m1[kSmallBlocks];  // verbatim elements of a dense block (ballots)
-  uint32_t c0[kSmallBlocks], c1[kSmallBlocks];  // this lane's two residual codes
-  uint32_t w0[kSmallBlocks], w1[kSmallBlocks];  // this lane's two elements, verbatim bits
-  uint32_t dense;                               // bit b: block b is dense
-  uint32_t rowp;                                // lane y: CSR row pointer of row y; lane H: nnz_s
-  SalientInfo info;
-};
-// Non-zero bits of row rr (0..7) of a block.
-__device__ __forceinline__ uint32_t block_row_bits(uint32_t z0, uint32_t z1, uint32_t rr) {
-  return ((rr < 4u ? z0 : z1) >> ((rr & 3u) * 8u)) & 0xFFu;
-}
-
-template <int DT>
-__device__ __forceinline__ void small_blocks(const Plan& pl, const uint8_t* plane, SmallBlocks& sb) {
-  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu;
-  const float inv2e = __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps));
-  sb.dense = 0;
-  uint32_t n_dense = 0, n_out_d = 0;
-#pragma unroll
-  for (uint32_t b = 0; b < kSmallBlocks; ++b) {
-    sb.z0[b] = sb.z1[b] = sb.m0[b] = sb.m1[b] = 0;
-    sb.c0[b] = sb.c1[b] = 128u;
-    sb.w0[b] = sb.w1[b] = 0;
-    if (b < pl.nblk) {
-      const uint32_t by = b / pl.nbx, bx = b - by * pl.nbx;
-      const BlockRegs r = block_load<DT>(plane, pl.H, pl.W, (int)by, (int)bx, lane);
-      sb.w0[b] = DT == kF32 ? __float_as_uint(r.x0) : __float_as_uint(r.x0) >> 16;
-      sb.w1[b] = DT == kF32 ? __float_as_uint(r.x1) : __float_as_uint(r.x1) >> 16;
-      sb.z0[b] = __ballot_sync(full, r.x0 != 0.0f);
-      sb.z1[b] = __ballot_sync(full, r.x1 != 0.0f);
-      const uint32_t nnz = __popc(sb.z0[b]) + __popc(sb.z1[b]);
-      if ((uint64_t)nnz * pl.tau_den >= (uint64_t)pl.tau_num * 64u) {  // (the same for every lane)
-        sb.dense |= 1u << b;
-        ++n_dense;
-        block_codes(r, inv2e, lane, sb.c0[b], sb.c1[b], sb.m0[b], sb.m1[b]);
-        n_out_d += __popc(sb.m0[b]) + __popc(sb.m1[b]);
-      }
-    }
+// `there`: the lane's plane is one to encode.  size: bytes of its payload; raw: it is left as it is and stored verbatim.
+template <int DT, bool FOUR>
+__device__ __noinline__ void encode_few(const Plan& pl, uint8_t* plane, bool there, uint32_t& size, bool& raw) {
+  const uint32_t lane = threadIdx.x & 31u, r = lane >> 2, q = lane & 3u, full = 0xFFFFFFFFu;
+  const uint32_t H = (uint32_t)pl.H, W = (uint32_t)pl.W, e = (uint32_t)pl.esize;
+  const uint32_t qs = FOUR ? 0u : pl.qs, qm = (1u << qs) - 1u;
+  const uint32_t by = FOUR ? 0u : q >> qs, bx = q & qm, y = by * 8u + r, x0 = bx * 8u;
+  const bool valid = there && by < pl.nby && bx < pl.nbx;
+  const uint32_t nin = valid && y < H ? min(8u, W - x0) : 0u;
+  float v[8];
+  load_seg<DT>(plane, W, y, x0, nin, seg_vec<DT>(plane, W), v);
+  uint32_t nz = nonzero_mask(v), cnt = __popc(nz);
+  const bool dense = block_sum(cnt) * pl.tau_den >= pl.tau_num * 64u && valid;
+  const uint32_t dm = __ballot_sync(full, dense) & 15u;  // (row 0 of every block)
+  uint32_t ca = 0, cb = 0, vm = 0;
+  if (dm) {
+    seg_codes(v, nin, __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps)), ca, cb, vm);
+    if (!dense) vm = 0;
   }
-  // CSR row pointers: lane y counts the non-zeros of row y that lie in sparse blocks
-  uint32_t cnt = 0;
-  {
-    const uint32_t by = lane >> 3, rr = lane & 7u;
-#pragma unroll
-    for (uint32_t b = 0; b < kSmallBlocks; ++b)
-      if (b < pl.nblk && !((sb.dense >> b) & 1u) && b / pl.nbx == by && lane < (uint32_t)pl.H)
-        cnt += __popc(block_row_bits(sb.z0[b], sb.z1[b], rr));
+  if (dense) nz = cnt = 0;
+  // CSR: entries of the plane's row and of the rows before it; entries of the row in the blocks to the left
+  uint32_t left = cnt;
+  if (qs > 0) {
+    const uint32_t up = __shfl_up_sync(full, left, 1);
+    if (bx >= 1u) left += up;
   }
-  uint32_t incl = cnt;
-  for (uint32_t o = 1; o < 32u; o <<= 1) {
-    const uint32_t up = __shfl_up_sync(full, incl, o);
-    if (lane >= o) incl += up;
+  if (qs > 1) {
+    const uint32_t up = __shfl_up_sync(full, left, 2);
+    if (bx >= 2u) left += up;
   }
-  sb.rowp = incl - cnt;
-  const uint32_t nnz_s = __shfl_sync(full, incl, 31), e = (uint32_t)pl.esize;
-  sb.info.nnz_s = nnz_s;
-  sb.info.n_dense = n_dense;
-  sb.info.n_out_d = n_out_d;
-  sb.info.coded = 0;
-  sb.info.size = 16u + 4u * pl.nbm + 4u * ((uint32_t)pl.H + 1u) + a4(2u * nnz_s) + a4(e * nnz_s) + 64u * n_dense +
-                 a4(e * n_out_d);
-}
-
-template <int DT>
-__device__ __forceinline__ void small_write(const Plan& pl, const SmallBlocks& sb, const SplitOut& out) {
-  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, e = (uint32_t)pl.esize, H = (uint32_t)pl.H;
-  const SalientInfo& info = sb.info;
-  const uint32_t o_bm = 16u, o_rp = o_bm + 4u * pl.nbm, o_col = o_rp + 4u * (H + 1u);
-  const uint32_t o_val = o_col + a4(2u * info.nnz_s), o_codes = o_val + a4(e * info.nnz_s);
-  const uint32_t o_outl = o_codes + 64u * info.n_dense;
-  if (lane == 0) {
-    out.st32(0, info.nnz_s);
-    out.st32(4, info.n_dense);
-    out.st32(8, info.n_out_d);
-    out.st32(12, 0);
-    out.st32(o_bm, sb.dense);  // (at most kSmallBlocks blocks: one bitmap word)
+  const uint32_t row = __shfl_sync(full, left, (int)(lane | qm));
+  const uint32_t rincl = block_prefix(row);
+  const uint32_t r0 = __shfl_sync(full, rincl, 28), r1 = __shfl_sync(full, rincl, 29), r2 = __shfl_sync(full, rincl, 30),
+                 r3 = __shfl_sync(full, rincl, 31);
+  uint32_t rbefore = 0, nnz = 0;
+  if (FOUR) {
+    nnz = q < 2u ? (q ? r1 : r0) : (q == 2u ? r2 : r3);
+  } else if (qs == 0u) {
+    rbefore = (q > 0u ? r0 : 0u) + (q > 1u ? r1 : 0u) + (q > 2u ? r2 : 0u);
+    nnz = r0 + r1 + r2 + r3;
+  } else {
+    rbefore = qs == 1u && q >= 2u ? r0 : 0u;
+    nnz = qs == 1u ? r0 + r2 : r0;
+  }
+  const uint32_t rowp = rbefore + rincl - row;
+  uint32_t pos = rowp + left - cnt;
+  // verbatim elements, in raster order within a block
+  const uint32_t c = __popc(vm), vincl = block_prefix(c);
+  uint32_t vbefore = 0, n_out = 0;
+  if (FOUR) n_out = __shfl_sync(full, vincl, (int)(28u + q));
+  else across_blocks(vincl, q, vbefore, n_out);
+  const uint32_t n_dense = FOUR ? (dense ? 1u : 0u) : __popc(dm), rank = FOUR ? 0u : __popc(dm & ((1u << q) - 1u));
+  const uint32_t o_rp = 20u, o_col = o_rp + 4u * (H + 1u), o_val = o_col + a4(2u * nnz), o_codes = o_val + a4(e * nnz);
+  const uint32_t o_outl = o_codes + 64u * n_dense;
+  size = o_outl + a4(e * n_out);
+  raw = a16(size) >= a16((uint32_t)pl.plane_bytes);
+  __syncwarp();  // every element has been read
+  if (!there || raw) return;
+  uint8_t* const pay = small_payload(plane);
+  auto st32 = [&](uint32_t o, uint32_t w) { *reinterpret_cast<uint32_t*>(pay + o) = w; };
+  auto st16 = [&](uint32_t o, uint32_t w) { *reinterpret_cast<uint16_t*>(pay + o) = (uint16_t)w; };
+  auto value = [&](uint32_t o, float f) {
+    if (DT == kF32) st32(o, __float_as_uint(f));
+    else st16(o, __float_as_uint(f) >> 16);
+  };
+  if (r == 0u && (FOUR || q == 0u)) {
+    st32(0, nnz);
+    st32(4, n_dense);
+    st32(8, n_out);
+    st32(12, 0);
+    st32(16, FOUR ? n_dense : dm);
+    st32(o_rp + 4u * H, nnz);
     // pads the section writers leave: col (2 bytes), val / verbatim values (bf16: 2 bytes)
-    if (info.nnz_s & 1u) out.st16(o_col + 2u * info.nnz_s, 0);
-    if (DT == kBF16 && (info.nnz_s & 1u)) out.st16(o_val + 2u * info.nnz_s, 0);
-    if (DT == kBF16 && (info.n_out_d & 1u)) out.st16(o_outl + 2u * info.n_out_d, 0);
+    if (nnz & 1u) st16(o_col + 2u * nnz, 0);
+    if (DT == kBF16 && (nnz & 1u)) st16(o_val + 2u * nnz, 0);
+    if (DT == kBF16 && (n_out & 1u)) st16(o_outl + 2u * n_out, 0);
   }
-  // zero padding up to the end of the slot / of the 16-byte padded overflow part
-  const uint32_t end = max(pl.npay, a16(info.size));
-  for (uint32_t o = info.size + 4u * lane; o < end; o += 128u) out.st32(o, 0);
-  if (lane <= H) out.st32(o_rp + 4u * lane, sb.rowp);
-  const uint32_t lt = (1u << lane) - 1u, c = lane & 7u, r0 = lane >> 3;
-  uint32_t dense_rank = 0, outl_at = 0;
+  if (valid && bx == 0u && y < H) st32(o_rp + 4u * y, rowp);
 #pragma unroll
-  for (uint32_t b = 0; b < kSmallBlocks; ++b) {
-    if (b >= pl.nblk) continue;
-    const uint32_t by = b / pl.nbx, bx = b - by * pl.nbx;
-    if ((sb.dense >> b) & 1u) {
-      const uint32_t oc = o_codes + 64u * dense_rank, oo = o_outl + e * outl_at;
-      if ((sb.m0[b] >> lane) & 1u) {
-        const uint32_t rank = __popc(sb.m0[b] & lt);
-        if (DT == kF32) out.st32(oo + 4u * rank, sb.w0[b]);
-        else out.st16(oo + 2u * rank, sb.w0[b]);
-      }
-      if ((sb.m1[b] >> lane) & 1u) {
-        const uint32_t rank = __popc(sb.m0[b]) + __popc(sb.m1[b] & lt);
-        if (DT == kF32) out.st32(oo + 4u * rank, sb.w1[b]);
-        else out.st16(oo + 2u * rank, sb.w1[b]);
-      }
-      uint32_t v0 = sb.c0[b] | (__shfl_down_sync(full, sb.c0[b], 1) << 8);
-      v0 |= __shfl_down_sync(full, v0, 2) << 16;
-      uint32_t v1 = sb.c1[b] | (__shfl_down_sync(full, sb.c1[b], 1) << 8);
-      v1 |= __shfl_down_sync(full, v1, 2) << 16;
-      if ((lane & 3u) == 0u) {
-        out.st32(oc + lane, v0);
-        out.st32(oc + 32u + lane, v1);
-      }
-      ++dense_rank;
-      outl_at += __popc(sb.m0[b]) + __popc(sb.m1[b]);
-    } else {
-      // CSR entries of the block's two halves: row pointer of the element's row, plus the non-zeros of that
-      // row in sparse blocks to the left, plus those before it in the block's row
-#pragma unroll
-      for (uint32_t half = 0; half < 2u; ++half) {
-        const uint32_t rr = r0 + 4u * half, y = by * 8u + rr;
-        uint32_t pos = __shfl_sync(full, sb.rowp, (int)(y & 31u));
-#pragma unroll
-        for (uint32_t bl = 0; bl < kSmallBlocks; ++bl)
-          if (bl < b && bl / pl.nbx == by && !((sb.dense >> bl) & 1u)) pos += __popc(block_row_bits(sb.z0[bl], sb.z1[bl], rr));
-        const uint32_t bits = block_row_bits(sb.z0[b], sb.z1[b], rr);
-        pos += __popc(bits & ((1u << c) - 1u));
-        if ((bits >> c) & 1u) {
-          out.st16(o_col + 2u * pos, bx * 8u + c);
-          const uint32_t w = half ? sb.w1[b] : sb.w0[b];
-          if (DT == kF32) out.st32(o_val + 4u * pos, w);
-          else out.st16(o_val + 2u * pos, w);
-        }
-      }
+  for (uint32_t j = 0; j < 8u; ++j)
+    if ((nz >> j) & 1u) {
+      st16(o_col + 2u * pos, x0 + j);
+      value(o_val + e * pos, v[j]);
+      ++pos;
     }
+  if (dense) {
+    st32(o_codes + 64u * rank + 8u * r, ca);
+    st32(o_codes + 64u * rank + 8u * r + 4u, cb);
+    uint32_t o = o_outl + e * (vbefore + vincl - c);
+#pragma unroll
+    for (uint32_t j = 0; j < 8u; ++j)
+      if ((vm >> j) & 1u) {
+        value(o, v[j]);
+        o += e;
+      }
   }
 }
 
-// A warp measures an outlier-rich plane that lies in shared memory: small planes in registers, others through
-// the measuring scratch `sal`.
-template <int DT>
-__device__ __forceinline__ SalientInfo warp_plane_measure(const Team& warp_team, const Plan& pl, const uint8_t* plane,
-                                                          uint32_t* sal) {
-  if (is_small_plane(pl)) {
-    SmallBlocks sb;
-    small_blocks<DT>(pl, plane, sb);
-    return sb.info;
+// `lanes` lanes (this is number j of them) store `n` bytes of a payload or a raw plane from shared memory through slot and
+// overflow part, zero padded.  A bf16 plane may start between two words.
+__device__ __forceinline__ void payload_copy(const uint8_t* from, uint32_t n, const SplitOut& out, uint32_t j, uint32_t lanes) {
+  const uint32_t end = max(out.npay, a16(n));
+  const bool half = (smem_u32(from) & 2u) != 0u;
+  for (uint32_t o = 16u * j; o < end; o += 16u * lanes) {
+    uint32_t w[4];
+#pragma unroll
+    for (uint32_t k = 0; k < 4u; ++k) {
+      const uint32_t i = o + 4u * k;
+      w[k] = 0;
+      if (i + 4u <= n && !half) w[k] = *reinterpret_cast<const uint32_t*>(from + i);
+      else if (i + 2u <= n) {
+        w[k] = *reinterpret_cast<const uint16_t*>(from + i);
+        if (i + 4u <= n) w[k] |= (uint32_t)*reinterpret_cast<const uint16_t*>(from + i + 2u) << 16;
+      }
+    }
+    *reinterpret_cast<uint4*>(out.at(o)) = make_uint4(w[0], w[1], w[2], w[3]);
   }
-  return salient_measure<DT>(warp_team, pl, plane, sal);
 }
 
 // What every thread of a CTA knows about the destination.
@@ -279,11 +202,6 @@ __device__ __forceinline__ Dest make_dest(const Plan& pl, const CompressArgs& a)
   return d;
 }
 
-__device__ __forceinline__ uint32_t salient_size(const Plan& pl, uint32_t nnz_s, uint32_t n_dense, uint32_t n_out_d) {
-  const uint32_t e = (uint32_t)pl.esize;
-  return 16u + 4u * pl.nbm + 4u * ((uint32_t)pl.H + 1u) + a4(2u * nnz_s) + a4(e * nnz_s) + 64u * n_dense +
-         a4(e * n_out_d);
-}
 // Overflow size, in 16-byte units, of a payload of `size` bytes.
 __device__ __forceinline__ uint32_t ovf_units(const Plan& pl, uint32_t size) {
   return a16(size) > pl.npay ? (a16(size) - pl.npay) >> 4 : 0u;
@@ -294,11 +212,12 @@ __device__ __forceinline__ uint32_t plane_units(const Plan& pl, const SalientInf
   return ovf_units(pl, raw ? (uint32_t)pl.plane_bytes : info.size);
 }
 
-// Per-call counters of a tile's outlier-rich planes (one thread): nsal and nraw share a word.
-__device__ __forceinline__ void count_blockwise(const CompressArgs& a, uint32_t units, uint32_t nsal, uint32_t nraw) {
-  if (units | nsal | nraw) *cta_dirty() = 1u;
-  if (units) atomicAdd(&a.sc->ovf16, (unsigned long long)units);
-  if (nsal | nraw) atomicAdd(&a.sc->nsal, (unsigned long long)nsal | ((unsigned long long)nraw << 32));
+// A tile's outlier-rich planes are added to the CTA's totals (one thread).
+__device__ __forceinline__ void count_blockwise(uint32_t units, uint32_t nsal, uint32_t nraw) {
+  CtaTotals* t = cta_totals();
+  if (units) atomicAdd(&t->units, units);
+  if (nsal) atomicAdd(&t->nsal, nsal);
+  if (nraw) atomicAdd(&t->nraw, nraw);
 }
 
 // Writes the payload of the measured plane gp (`plane` in shared memory, `info` and `sal` from
@@ -322,46 +241,9 @@ __device__ __forceinline__ void write_blockwise(const Team& t, const Plan& pl, c
         make_uint4(my_units ? (uint32_t)off16 : 0u, (raw ? kClsRaw : kClsSalient) | (n_out << 2), 0u, 0u);
 }
 
-// A warp measures the outlier-rich plane gp (in shared memory) and writes it with its overflow part `at` units
-// into the overflow region: small planes in registers, others through the measuring scratch `sal`.
-template <int DT>
-__device__ __forceinline__ void warp_plane_write(const Team& warp_team, const Plan& pl, const Dest& d, uint64_t gp,
-                                                 const uint8_t* plane, uint32_t* sal, uint32_t n_out, uint32_t at) {
-  if (!is_small_plane(pl)) {
-    const SalientInfo info = salient_measure<DT>(warp_team, pl, plane, sal);
-    write_blockwise<DT>(warp_team, pl, d, gp, plane, info, sal, n_out, at);
-    return;
-  }
-  SmallBlocks sb;
-  small_blocks<DT>(pl, plane, sb);
-  bool raw;
-  const uint32_t my_units = plane_units(pl, sb.info, raw);
-  const unsigned long long off16 = (pl.ovf_off >> 4) + at;
-  if (!d.fits || (off16 + my_units) * 16ull > d.capacity) return;  // never write past the capacity
-  SplitOut out;
-  out.slot = d.dst + pl.slots_off + gp * pl.npay;
-  out.ovf = d.dst + off16 * 16ull;
-  out.npay = pl.npay;
-  if (raw) raw_write(warp_team, pl, plane, out);
-  else small_write<DT>(pl, sb, out);
-  if (warp_team.lane == 0)
-    reinterpret_cast<uint4*>(d.dst + 64)[gp] =
-        make_uint4(my_units ? (uint32_t)off16 : 0u, (raw ? kClsRaw : kClsSalient) | (n_out << 2), 0u, 0u);
-}
-
-// One thread, after everything else of the call is done: header, result words, and every counter the
-// call touched back to zero.
-// `touched`: some CTA of the call has changed a counter; otherwise all of them are known to be zero.
-__device__ __forceinline__ void finalize(const Plan& pl, const CompressArgs& a, const Dest& d, bool touched) {
-  unsigned long long ovf16 = 0, cnt = 0;
-  uint32_t code = kErrNone;
-  if (touched) {
-    __threadfence();  // the counters as the other CTAs left them before they were counted out
-    ovf16 = ld_relaxed(&a.sc->ovf16);
-    cnt = ld_relaxed(&a.sc->nsal);
-    code = (uint32_t)ld_relaxed(&a.sc->status);
-  }
-  const uint32_t nsal = (uint32_t)cnt, nraw = (uint32_t)(cnt >> 32);
+// One thread, after everything else of the call is done: header and result words.
+__device__ __forceinline__ void finalize(const Plan& pl, const CompressArgs& a, const Dest& d, unsigned long long ovf16, uint32_t nsal,
+                                         uint32_t nraw, uint32_t code) {
   const unsigned long long total = pl.ovf_off + ovf16 * 16ull;
   if (total > d.capacity && code < kErrCapacity) code = kErrCapacity;
   if (d.capacity >= 64) {
@@ -380,39 +262,66 @@ __device__ __forceinline__ void finalize(const Plan& pl, const CompressArgs& a, 
     a.out2[1] = status_word(code);
   }
   if (a.d_off_out) *a.d_off_out = code == kErrNone ? d.off_in + ((total + 255ull) & ~255ull) : (~0ull >> 1);
-  if (ovf16) st_relaxed(&a.sc->ovf16, 0ull);
-  if (cnt) st_relaxed(&a.sc->nsal, 0ull);
-  if (code) st_relaxed(&a.sc->status, 0ull);
 }
 
 // Last step of every CTA: the last CTA to leave returns the group sums of the previous call's placement scan and
 // the hand-out counters to zero and finishes the container.
-// The exit counter carries the CTAs that have left in its low half and, in its high half, how many of them had
-// changed a counter of the call (cta_dirty); only such a CTA fences -- its updates must be performed before it is
-// counted out -- so a call without outlier-rich planes and without errors ends with one atomic per CTA and no
-// read-back.  The container itself needs no fence: its readers are later kernels.
+// The exit word carries the CTAs that have left, how many of them had something to add, and the overflow units of all:
+//   CTAs | CTAs with something << 13 | units << 26
+// The numbers of planes go the same way, each next to a count of the CTAs that added to it, by which the last CTA knows
+// that a sum is complete: nothing has to be ordered, so that only a CTA with an error to report fences (the number of these
+// is the topmost part of one of the sums).  (With counters
+// changed while the CTA worked, a fence ahead of the exit word and another ahead of reading them back, a call with
+// outlier-rich planes took 2.0 us from its last CTA's last store to its end, one without 0.5.)  The container itself
+// needs no fence either: its readers are later kernels.
+constexpr uint32_t kExitBits = 13, kExitMask = (1u << kExitBits) - 1u;  // (a grid has at most 32 CTAs per SM)
+__device__ __forceinline__ bool has_totals(const CtaTotals& t) { return (t.units | t.nsal | t.nraw | t.err) != 0u; }
 __device__ __forceinline__ void cta_exit(const Plan& pl, const CompressArgs& a, const Dest& d, uint32_t* s_last) {
-  __syncthreads();  // every thread's note in the flag is in
-  const bool dirty = *cta_dirty() != 0u;  // (the same for every thread)
-  if (dirty) {
-    __threadfence();
-    __syncthreads();
-  }
+  __syncthreads();  // every thread's notes are in
+  const CtaTotals t = *cta_totals();
+  unsigned long long now = 0;
   if (threadIdx.x == 0) {
-    const unsigned long long old = atomicAdd(&a.sc->exited, 1ull | (dirty ? 1ull << 32 : 0ull));
-    const bool last = (uint32_t)old == gridDim.x - 1u;
-    *s_last = last ? (((old >> 32) != 0ull || dirty) ? 3u : 1u) : 0u;
+    const bool some = has_totals(t);
+    if (t.err) __threadfence();  // the error code before the CTA is counted out
+    if (some) {
+      atomicAdd(&a.sc->nsal, 1ull | (unsigned long long)t.nsal << kExitBits);
+      atomicAdd(&a.sc->nraw, 1ull | (unsigned long long)t.nraw << kExitBits | (t.err ? 1ull << (64 - kExitBits) : 0ull));
+    }
+    const unsigned long long mine = 1ull | (some ? 1ull << kExitBits : 0ull) | (unsigned long long)t.units << (2 * kExitBits);
+    now = atomicAdd(&a.sc->exited, mine) + mine;
+    *s_last = ((uint32_t)now & kExitMask) == gridDim.x ? 1u : 0u;
   }
   __syncthreads();
-  const uint32_t last = *s_last;
-  if (!last) return;
+  if (!*s_last) return;
   if (pl.mode != kModeOff)
     for (uint32_t k = threadIdx.x; k < a.scan.clear_groups; k += blockDim.x) a.scan.grp_clear[k] = 0ull;
   if (threadIdx.x != 0) return;
   // (what follows is read by later kernels only, which start work after this one has completed: no fence)
   st_relaxed(&a.sc->ticket[a.parity], 0ull);
   st_relaxed(&a.sc->exited, 0ull);
-  finalize(pl, a, d, (last & 2u) != 0u);
+  const uint32_t adders = (uint32_t)(now >> kExitBits) & kExitMask;
+  unsigned long long vs = 0, vr = 0;
+  uint32_t code = kErrNone;
+  if (adders) {
+    for (uint32_t k = 0; k < (1u << 22); ++k) {
+      vs = ld_relaxed(&a.sc->nsal);
+      vr = ld_relaxed(&a.sc->nraw);
+      if (((uint32_t)vs & kExitMask) == adders && ((uint32_t)vr & kExitMask) == adders) break;
+    }
+    if (vr >> (64 - kExitBits)) {  // somebody has reported an error
+      __threadfence();
+      code = (uint32_t)ld_relaxed(&a.sc->status);
+      st_relaxed(&a.sc->status, 0ull);
+    }
+    st_relaxed(&a.sc->nsal, 0ull);
+    st_relaxed(&a.sc->nraw, 0ull);
+    st_relaxed(&a.sc->done, 0ull);
+    st_relaxed(&a.sc->queue, 0ull);
+  }
+  finalize(pl, a, d, now >> (2 * kExitBits), (uint32_t)(vs >> kExitBits), (uint32_t)(vr >> kExitBits), code);
+  // after an error, entries may be left of tiles that were put off: they are zero between calls
+  if (code && pl.mode != kModeOff)
+    for (uint32_t k = 0; k < pl.ntiles; ++k) a.defer_next[k] = 0u;
 }
 
 __device__ __forceinline__ void store_table_entry(const Dest& d, uint64_t plane, uint32_t off16, uint32_t meta, float lo,
@@ -421,9 +330,10 @@ __device__ __forceinline__ void store_table_entry(const Dest& d, uint64_t plane,
 }
 
 // Table entry of a plane that takes the block-wise path, until its payload is written: class salient, the
-// three-sigma count; phase 1 leaves the plane's overflow size (16-byte units) where the offset will go.
-__device__ __forceinline__ void store_marker(const Dest& d, uint64_t plane, uint32_t meta, uint32_t units) {
-  reinterpret_cast<uint4*>(d.dst + 64)[plane] = make_uint4(units, (meta & ~3u) | kClsSalient, 0u, 0u);
+// three-sigma count; phase 1 leaves the plane's overflow size (16-byte units) where the offset will go, and of a small
+// plane the bytes to store and whether it is raw.
+__device__ __forceinline__ void store_marker(const Dest& d, uint64_t plane, uint32_t meta, uint32_t units, uint32_t bytes = 0, bool raw = false) {
+  reinterpret_cast<uint4*>(d.dst + 64)[plane] = make_uint4(units, (meta & ~3u) | kClsSalient, bytes, raw ? 1u : 0u);
 }
 __device__ __forceinline__ uint2 load_marker(const Dest& d, uint64_t plane) {
   const volatile uint32_t* e = reinterpret_cast<const volatile uint32_t*>(d.dst + 64 + 16ull * plane);
@@ -432,36 +342,50 @@ __device__ __forceinline__ uint2 load_marker(const Dest& d, uint64_t plane) {
 
 // The block-wise path runs in two phases so that nothing in the streaming phase ever waits for another CTA.
 // Phase 1, while a tile lies in shared memory: its outlier-rich planes are measured, the tile publishes the
-// overflow size of its planes to the scan, and the CTA links the tile into its own list (newest first;
-// `defer_next[tile]` holds the tile listed before it).  Phase 2, when the CTA has run out of tiles: it takes
-// its listed tiles again (they come from the L2 cache when the tensor is small), obtains each tile's place
-// from the scan -- every tile before it has been published, or is about to be, by a CTA in phase 1 -- and
-// writes the payloads.  This block sits in shared memory: what the outlined functions of both phases need.
+// overflow size of its planes to the scan and is put off.  Phase 2, when the CTA has run out of tiles: tiles put off are
+// taken again (they come from the L2 cache when the tensor is small), obtain their place from the scan -- every tile
+// before one has been published, or is about to be, by a CTA in phase 1 -- and the payloads are written.  Tiles put off
+// wait in `defer_next`: linked from the CTA's own list (entry [tile]: the tile listed before it), or, in the CTA-team
+// kernels, in a queue that all CTAs share (entry [n]: the n-th tile put off, plus one); an entry is returned to zero by
+// who takes it.  This block sits in shared memory: what the outlined functions of both phases need.
 constexpr uint32_t kNoTile = 0xFFFFFFFFu;
 struct BlockCtl {
   Plan pl;
   CompressArgs a;
   Dest d;
   uint32_t U[kMaxStages], C[kMaxStages], arr[kMaxStages];  // warp-team kernel, per stage: units, counts, warps done
-  uint32_t wcnt[kMaxWarps];                                // phase 2: outlier-rich planes per warp's slice
   uint32_t base, ok;
   uint32_t head;                                           // the tile this CTA listed last
   uint32_t held[kMaxStages];                               // the tile each stage buffer holds
-  uint32_t measured;                                       // CTA-team kernels: the plane the measuring scratch is about ...
-  SalientInfo measured_info;                               // ... and its sizes
+  uint32_t next, ahead;                                    // CTA-team kernels, phase 2: the plane in hand, the one after it
+  uint32_t own, own_stage, own_held;                       // ... the plane the measuring scratch is about (kNoTile: none), its stage, whether it still lies there ...
+  SalientInfo own_info;                                    // ... and its sizes
 };
 
-struct BlockList {
-  // phase 2 of the warp-team kernel: the outlier-rich planes of the tile in hand, in plane order
-  uint32_t list_at[256];                                   // overflow units, then (scanned) the place within the tile's part
-  uint32_t list_meta[256];
-  uint16_t list_lp[256];
+// Warp-team kernel: what the tiles in the stages have gathered so far, and the tiles put off, as far as there is room (the
+// others are linked like those of the CTA-team kernels).  A slice is what one warp sweeps of a tile.
+constexpr uint32_t kListed = 32, kListedPlanes = 128;  // (static shared memory stays below what kSmemLimit leaves)
+struct WarpList {
+  uint32_t sum[kMaxStages][kWarps];  // overflow units of a slice (when the slice has outlier-rich planes)
+  uint32_t mask[kMaxStages];         // slices that have some
+  uint32_t count;                    // tiles put off
+  uint32_t handed[2];                // phase 2: items handed out in each of its passes
+  uint32_t tile[kListed];
+  uint32_t units[kListed], base[kListed];  // the tile's overflow units and, in phase 2, its place (kNoTile: not to be had)
+  uint32_t before[kListed][kWarps];  // units of the tile's slices before this one
+  uint8_t stage[kListed], slices[kListed];
+  uint16_t n[kListed];               // outlier-rich planes of the tile
+  // phase 2, planes of more than four blocks: those of the listed tiles
+  uint32_t planes;
+  uint32_t place[kListedPlanes], meta[kListedPlanes];
+  uint16_t lp[kListedPlanes];
+  uint8_t of[kListedPlanes];         // whose entry (kListed: nobody's)
 };
 
 // One thread: tile `tile` has `units` of overflow in `nsal` salient and `nraw` raw planes.
 __device__ __forceinline__ void publish_tile(BlockCtl* c, uint32_t tile, uint32_t units, uint32_t nsal, uint32_t nraw) {
   scan_publish(c->a.scan, tile, units);
-  count_blockwise(c->a, units, nsal, nraw);
+  count_blockwise(units, nsal, nraw);
   if ((nsal | nraw) && c->d.fits) c->a.defer_next[tile] = atomicExch(&c->head, tile);
 }
 
@@ -511,12 +435,12 @@ __global__ void __launch_bounds__(kThreads) compress_generic(const Plan pl, cons
   __shared__ BlockCtl s_ctl;
 
   const uint32_t tid = threadIdx.x;
-  if (tid == 0) *cta_dirty() = 0u;
+  if (tid == 0) *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
   if (tid == 0 && a.early_ticket) s_tile = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
   if (tid == 0 && pl.mode != kModeOff) {  // (before the wait for the previous kernel, whose tail hides it)
     s_ctl.pl = pl;
     s_ctl.a = a;
-    s_ctl.head = kNoTile;
+    s_ctl.head = s_ctl.own = kNoTile;
   }
   dep_wait();     // the previous kernel on the stream has completed
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
@@ -715,6 +639,7 @@ __global__ void __launch_bounds__(kThreads) compress_generic(const Plan pl, cons
       }
     }
     __syncthreads();
+    if (tid == 0) a.defer_next[tile] = 0u;
     tile = next;
   }
   cta_exit(pl, a, d, &s_last);
@@ -1043,119 +968,354 @@ __device__ __forceinline__ uint32_t plane_sweep(const Team& team, const Plan& pl
 // -------------------------------------------------------------------------------------------------
 constexpr int kWarpKernelThreads = kThreads + 32;
 
-// Phase 1, a warp with outlier-rich planes in its slice (`leaders`: the first lanes of their teams; lp0: first
-// plane of the warp's slice): they are measured, their sizes go into the sums of the tile in stage s and into
-// their table markers.
-template <int DT, int TT>
-__device__ __noinline__ void warp_tile_measure(BlockCtl* c, const uint8_t* tbuf, uint64_t p0, uint32_t s, uint32_t lp0,
-                                               uint32_t leaders, uint32_t meta, uint32_t* sal) {
-  const Team team = make_warp_team(nullptr);
-  const Plan& pl = c->pl;
-  uint32_t total = 0, nraw = 0, n = 0;
-  for (uint32_t m = leaders; m; m &= m - 1u, ++n) {
-    const uint32_t src = (uint32_t)__ffs((int)m) - 1u, lp = lp0 + src / TT;
-    if (n) __syncwarp();
-    const SalientInfo info = warp_plane_measure<DT>(team, pl, tbuf + (uint64_t)lp * pl.plane_bytes, sal);
-    bool raw;
-    const uint32_t u = plane_units(pl, info, raw);
-    total += u;
-    nraw += raw ? 1u : 0u;
-    const uint32_t mt = __shfl_sync(0xFFFFFFFFu, meta, (int)src);
-    if (team.lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
+// What was measured of a plane of more than four blocks waits for phase 2 in the plane's own slot, when that holds it:
+// sizes, the measuring scratch and, with the Huffman stage, the code.  (Measuring a second time was half of phase 2.)
+__device__ __forceinline__ uint32_t scratch_words(const Plan& pl) {
+  return (uint32_t)pl.H + 1u + 2u * (pl.nsr + 1u) + pl.nbm + (pl.entropy ? pl.nsr + 1u : 0u);
+}
+__device__ __forceinline__ bool scratch_saved(const Plan& pl) {
+  return 32u + 4u * scratch_words(pl) + (pl.entropy ? 4u * 256u : 0u) <= pl.npay;
+}
+__device__ __forceinline__ void scratch_save(const Team& t, const Plan& pl, const Dest& d, uint64_t gp, const SalientInfo& info, uint32_t* sal) {
+  uint4* slot = reinterpret_cast<uint4*>(d.dst + pl.slots_off + gp * pl.npay);
+  const HufEncode* h = sal_scratch(Geometry(pl), sal).huf;
+  if (t.lane == 0) {
+    slot[0] = make_uint4(info.nnz_s, info.n_dense, info.n_out_d, info.size);
+    slot[1] = pl.entropy ? make_uint4(info.coded, h->nlens, h->smin, h->smax) : make_uint4(0u, 0u, 0u, 0u);
   }
-  if (team.lane == 0) {
+  uint32_t* w = reinterpret_cast<uint32_t*>(slot + 2);
+  const uint32_t n = scratch_words(pl);
+  for (uint32_t i = t.lane; i < n; i += t.size) w[i] = sal[i];
+  if (info.coded)
+    for (uint32_t i = t.lane; i < 256u; i += t.size) w[n + i] = h->code[i];
+}
+__device__ __forceinline__ SalientInfo scratch_load(const Team& t, const Plan& pl, const Dest& d, uint64_t gp, uint32_t* sal) {
+  const uint4* slot = reinterpret_cast<const uint4*>(d.dst + pl.slots_off + gp * pl.npay);
+  HufEncode* h = sal_scratch(Geometry(pl), sal).huf;
+  const uint4 v = __ldcg(slot), x = __ldcg(slot + 1);
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(slot + 2);
+  const uint32_t n = scratch_words(pl);
+  for (uint32_t i = t.lane; i < n; i += t.size) sal[i] = __ldcg(w + i);
+  if (x.x) {
+    for (uint32_t i = t.lane; i < 256u; i += t.size) h->code[i] = __ldcg(w + n + i);
+    if (t.lane == 0) {
+      h->nlens = x.y;
+      h->smin = x.z;
+      h->smax = x.w;
+    }
+  }
+  SalientInfo info;
+  info.nnz_s = v.x;
+  info.n_dense = v.y;
+  info.n_out_d = v.z;
+  info.size = v.w;
+  info.coded = x.x;
+  return info;
+}
+
+// The lane that holds the k-th set bit of m (m has more than k).
+__device__ __forceinline__ uint32_t nth_bit(uint32_t m, uint32_t k) {
+  for (; k; --k) m &= m - 1u;
+  return (uint32_t)__ffs((int)m) - 1u;
+}
+
+// Encodes small planes of a warp's slice where they lie, `plane_of(k)` the k-th of them, and passes their sizes on:
+// done(k, size, raw) runs in one lane per plane.
+template <int DT, typename PlaneOf, typename Done>
+__device__ __forceinline__ void encode_small(const Plan& pl, uint32_t n, PlaneOf plane_of, Done done) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t size;
+  bool raw;
+  if (pl.nblk == 1u) {
+    for (uint32_t k0 = 0; k0 < n; k0 += 4u) {
+      const uint32_t k = k0 + (lane & 3u);
+      encode_few<DT, true>(pl, plane_of(min(k, n - 1u)), k < n, size, raw);
+      if (lane < 4u && k < n) done(k, size, raw);
+    }
+  } else {
+    for (uint32_t k = 0; k < n; ++k) {
+      encode_few<DT, false>(pl, plane_of(k), true, size, raw);
+      if (lane == 0u) done(k, size, raw);
+    }
+  }
+}
+
+// Phase 1, a warp with outlier-rich planes in its slice (`leaders`: the first lanes of their teams; lp0: first
+// plane of the slice): they are measured, their sizes go into the sums of the tile in stage s and into their table
+// markers.
+template <int DT, int TT>
+__device__ __noinline__ void warp_tile_measure(BlockCtl* c, WarpList* l, uint8_t* tbuf, uint64_t p0, uint32_t s, uint32_t slice,
+                                               uint32_t leaders, uint32_t meta, uint32_t* sal) {
+  const Plan& pl = c->pl;
+  const uint32_t lane = threadIdx.x & 31u, lp0 = slice * (32u / TT), n = __popc(leaders), full = 0xFFFFFFFFu;
+  uint32_t total = 0, nraw = 0;
+  if (is_small_plane(pl)) {
+    const uint32_t fits = c->d.fits;
+    encode_small<DT>(
+        pl, n, [&](uint32_t k) { return tbuf + (uint64_t)(lp0 + nth_bit(leaders, k) / TT) * pl.plane_bytes; },
+        [&](uint32_t k, uint32_t size, bool raw) {
+          const uint32_t bytes = raw ? (uint32_t)pl.plane_bytes : size, u = ovf_units(pl, bytes);
+          total += u;
+          nraw += raw ? 1u : 0u;
+          // (the leader's lane adds class and count afterwards)
+          if (fits) store_marker(c->d, p0 + lp0 + nth_bit(leaders, k) / TT, 0u, u, bytes, raw);
+        });
+    __syncwarp();
+    if (fits && ((leaders >> lane) & 1u))
+      reinterpret_cast<uint32_t*>(c->d.dst + 64)[4ull * (p0 + lp0 + lane / TT) + 1ull] = (meta & ~3u) | kClsSalient;
+    total += __shfl_xor_sync(full, total, 1);
+    total += __shfl_xor_sync(full, total, 2);
+    nraw += __shfl_xor_sync(full, nraw, 1);
+    nraw += __shfl_xor_sync(full, nraw, 2);
+  } else {
+    const Team team = make_warp_team(nullptr);
+    for (uint32_t m = leaders; m; m &= m - 1u) {
+      const uint32_t src = (uint32_t)__ffs((int)m) - 1u, lp = lp0 + src / TT;
+      const SalientInfo info = salient_measure<DT>(team, pl, tbuf + (uint64_t)lp * pl.plane_bytes, sal);
+      bool raw;
+      const uint32_t u = plane_units(pl, info, raw);
+      total += u;
+      nraw += raw ? 1u : 0u;
+      const uint32_t mt = __shfl_sync(full, meta, (int)src);
+      if (lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
+      if (c->d.fits && scratch_saved(pl)) scratch_save(team, pl, c->d, p0 + lp, info, sal);
+      __syncwarp();
+    }
+  }
+  if (lane == 0) {
+    l->sum[s][slice] = total;
+    atomicOr(&l->mask[s], 1u << slice);
     if (total) atomicAdd(&c->U[s], total);
     atomicAdd(&c->C[s], (n - nraw) | (nraw << 16));
   }
 }
 
 // Phase 1, the last of a tile's eight warps (one thread): the tile's sums are complete.
-static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, uint32_t s, uint32_t tile) {
+static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, WarpList* l, uint32_t s, uint32_t tile) {
   __threadfence_block();  // the other warps' sums after their arrivals
   const uint32_t U = c->U[s], C = c->C[s];
+  scan_publish(c->a.scan, tile, U);
+  if (C == 0u) return;
+  count_blockwise(U, C & 0xFFFFu, C >> 16);
+  const uint32_t mask = l->mask[s];
   c->U[s] = 0;
   c->C[s] = 0;
-  publish_tile(c, tile, U, C & 0xFFFFu, C >> 16);
+  l->mask[s] = 0;
+  if (!c->d.fits) return;
+  const uint32_t i = atomicAdd(&l->count, 1u);
+  if (i >= kListed) {
+    c->a.defer_next[tile] = atomicExch(&c->head, tile);
+    return;
+  }
+  l->tile[i] = tile;
+  l->units[i] = U;
+  l->n[i] = (uint16_t)((C & 0xFFFFu) + (C >> 16));
+  l->stage[i] = (uint8_t)s;
+  l->slices[i] = (uint8_t)mask;
+  uint32_t run = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < (uint32_t)kWarps; ++k) {
+    l->before[i][k] = run;
+    run += ((mask >> k) & 1u) ? l->sum[s][k] : 0u;
+  }
 }
 
-// Phase 2 of the warp-team kernel: every tile the CTA has put off, newest first.  The tile's outlier-rich
-// planes are listed in plane order (their markers carry class, count and size), placed by one scan over
-// the list, and dealt out to the warps in turn.
-template <int DT, int TT>
-__device__ __noinline__ void warp_phase2(BlockCtl* c, BlockList* l, uint8_t* stages, uint8_t* sal_base) {
+// `lanes` lanes (this is number j of them) fetch plane gp with the 16-byte chunks around it; returns where it starts.
+__device__ __forceinline__ uint8_t* fetch_plane(const Plan& pl, const uint8_t* src, uint64_t gp, uint8_t* to, uint32_t j, uint32_t lanes,
+                                                bool mine) {
+  const uint64_t start = gp * pl.plane_bytes, end = start + pl.plane_bytes, a0 = start & ~15ull, whole = pl.dense_bytes & ~15ull;
+  if (mine)
+    for (uint64_t o = a0 + 16u * j; o < end; o += 16u * lanes) {
+      if (o < whole) {
+        *reinterpret_cast<uint4*>(to + (o - a0)) = __ldg(reinterpret_cast<const uint4*>(src + o));
+      } else {
+        for (uint64_t i = o; i < pl.dense_bytes; i += 2) *reinterpret_cast<uint16_t*>(to + (i - a0)) = *reinterpret_cast<const uint16_t*>(src + i);
+      }
+    }
+  return to + (start - a0);
+}
+
+// Phase 2, a warp: an outlier-rich plane of more than four blocks, whose overflow part starts `place` units into the region.
+// `plane`: where it still lies, or null.
+template <int DT>
+__device__ __noinline__ void warp_plane_write(BlockCtl* c, uint64_t gp, const uint8_t* plane, uint32_t meta, uint32_t place, uint8_t* buf,
+                                              uint32_t* sal) {
   const Plan& pl = c->pl;
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const Team team = make_warp_team(nullptr);
+  if (!plane) plane = fetch_plane(pl, c->a.src, gp, buf, team.lane, 32u, true);
+  __syncwarp();
+  const SalientInfo info = scratch_saved(pl) ? scratch_load(team, pl, c->d, gp, sal) : salient_measure<DT>(team, pl, plane, sal);
+  __syncwarp();
+  write_blockwise<DT>(team, pl, c->d, gp, plane, info, sal, meta >> 2, place);
+  __syncwarp();
+}
+
+// Phase 2, a warp: the outlier-rich planes of one slice of a tile, whose overflow parts start `at` units into the region.
+// `staged`: where the tile still lies (null: nowhere, the planes are fetched again into `buf`).  Returns the slice's
+// units.
+template <int DT, int TT>
+__device__ __noinline__ uint32_t warp_slice_write(BlockCtl* c, uint32_t tile, uint32_t slice, uint32_t at, uint8_t* staged, uint8_t* buf,
+                                                  uint32_t* sal) {
+  const Plan& pl = c->pl;
+  const Dest& d = c->d;
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, lp0 = slice * (32u / TT);
+  const uint64_t p0 = (uint64_t)tile * pl.ppt;
+  const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0), pb = (uint32_t)pl.plane_bytes;
+  uint4 mk = make_uint4(0u, 0u, 0u, 0u);
+  if (lane < 32u / TT && lp0 + lane < np) {
+    mk = __ldcg(reinterpret_cast<const uint4*>(d.dst + 64) + p0 + lp0 + lane);
+  }
+  const uint32_t planes = __ballot_sync(full, (mk.y & 3u) != kClsNormal), n = __popc(planes);
+  if (n == 0u) return 0u;
+  const uint32_t u = (mk.y & 3u) != kClsNormal ? mk.x : 0u;
+  uint32_t incl = u;
+#pragma unroll
+  for (uint32_t o = 1; o < 32u; o <<= 1) {
+    const uint32_t up = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += up;
+  }
+  const uint32_t all = __shfl_sync(full, incl, 31);
+  const uint32_t place = at + incl - u;  // (of the lane's plane)
+  if (is_small_plane(pl)) {
+    // as many planes at a time as have room in the buffer (at least four: a quarter of a stage), eight lanes or all to one
+    const uint32_t lanes = pl.nblk == 1u ? 8u : 32u, step = pl.nblk == 1u ? 4u : 1u, room = a16(pb + 16u);
+    for (uint32_t k0 = 0; k0 < n; k0 += step) {
+      const uint32_t here = min(step, n - k0), k = k0 + lane / lanes, j = lane & (lanes - 1u);
+      const bool mine = lane / lanes < here;
+      const uint32_t b = nth_bit(planes, mine ? k : k0);
+      const uint64_t gp = p0 + lp0 + b;
+      uint32_t w = __shfl_sync(full, mk.w, (int)b);
+      const uint32_t bytes = __shfl_sync(full, mk.z, (int)b), meta = __shfl_sync(full, mk.y, (int)b),
+                     units = __shfl_sync(full, mk.x, (int)b), off = __shfl_sync(full, place, (int)b);
+      uint8_t* plane;
+      if (staged) {
+        plane = staged + (uint64_t)(lp0 + b) * pb;
+      } else {
+        auto at_buf = [&](uint32_t i) { return buf + i * room + ((uint32_t)((p0 + lp0 + nth_bit(planes, k0 + i)) * pb) & 15u); };
+        plane = fetch_plane(pl, c->a.src, gp, buf + (lane / lanes) * room, j, lanes, mine);
+        __syncwarp();
+        encode_small<DT>(pl, here, at_buf, [](uint32_t, uint32_t, bool) {});
+        __syncwarp();
+      }
+      const unsigned long long off16 = (pl.ovf_off >> 4) + off;
+      if (mine && (off16 + units) * 16ull <= d.capacity) {  // (never write past the capacity)
+        SplitOut out;
+        out.slot = d.dst + pl.slots_off + gp * pl.npay;
+        out.ovf = d.dst + off16 * 16ull;
+        out.npay = pl.npay;
+        payload_copy(w ? plane : small_payload(plane), bytes, out, j, lanes);
+        if (j == 0u)
+          reinterpret_cast<uint4*>(d.dst + 64)[gp] = make_uint4(units ? (uint32_t)off16 : 0u, (w ? kClsRaw : kClsSalient) | (meta & ~3u), 0u, 0u);
+      }
+      __syncwarp();
+    }
+  } else {
+    for (uint32_t m = planes; m; m &= m - 1u) {
+      const uint32_t b = (uint32_t)__ffs((int)m) - 1u;
+      warp_plane_write<DT>(c, p0 + lp0 + b, nullptr, __shfl_sync(full, mk.y, (int)b), __shfl_sync(full, place, (int)b), buf, sal);
+    }
+  }
+  return all;
+}
+
+// Phase 2 of the warp-team kernel.  The places of the listed tiles first, a warp to a tile (a look-up by every warp that
+// needs one had thousands of warps polling the same words: 7 x 7 planes, fp32: 25 -> 45 us).  Then the slices are handed
+// out to the warps, which need nothing of one another, in two passes: tiles that still lie in a stage (the last ones the
+// CTA streamed: all of them when the tensor is small), then the others, whose planes the warps fetch into their part of
+// the stages.  (Tile by tile with the whole CTA, a 28 x 28 bf16 tensor with every eighth channel outlier-rich had one warp
+// working and seven waiting.)
+template <int DT, int TT>
+__device__ __noinline__ void warp_phase2(BlockCtl* c, WarpList* l, uint8_t* stages, uint8_t* sal_base) {
+  const Plan& pl = c->pl;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, full = 0xFFFFFFFFu;
   uint32_t* sal = reinterpret_cast<uint32_t*>(sal_base + min(warp, (uint32_t)kWarps - 1u) * pl.sal_stride);
-  // Two walks over the list: first the tiles that still lie in a stage buffer (the last ones the CTA streamed:
-  // all of them when the tensor is small), then the others, fetched again into the first buffer.
-  for (uint32_t walk = 0; walk < 2u; ++walk) {
-    for (uint32_t tile = c->head; tile != kNoTile;) {
-      const uint32_t next = c->a.defer_next[tile];
-      uint32_t at_stage = kMaxStages;
-      for (uint32_t s = 0; s < pl.nstage; ++s)
-        if (c->held[s] == tile) at_stage = s;
-      if ((at_stage < (uint32_t)kMaxStages) != (walk == 0u)) {  // (the same for every thread)
-        tile = next;
+  uint8_t* buf = stages + min(warp, (uint32_t)kWarps - 1u) * ((pl.sm_sal / (uint32_t)kWarps) & ~15u);
+  const uint32_t n = min(l->count, kListed);
+  const bool small = is_small_plane(pl);
+  auto place_of = [&](uint32_t tile) {
+    uint32_t base = 0;
+    if (scan_prefix(c->a.scan, tile, base)) return base;
+    if (lane == 0) report_error(c->a, kErrTimeout);
+    return kNoTile;  // (no place: units are below 2^32 - 1)
+  };
+  for (uint32_t i = warp; i < n; i += (uint32_t)kWarps + 1u) {
+    const uint32_t tile = l->tile[i];
+    uint32_t base = l->units[i] ? place_of(tile) : 0u;
+    if (!small && base != kNoTile) {  // the tile's planes join the list; without room there, the tile joins the others
+      uint32_t at = 0;
+      if (lane == 0) at = atomicAdd(&l->planes, (uint32_t)l->n[i]);
+      at = __shfl_sync(full, at, 0);
+      const bool room = at + l->n[i] <= kListedPlanes;
+      if (!room) {
+        for (uint32_t k = at + lane; k < kListedPlanes; k += 32u) l->of[k] = (uint8_t)kListed;
+        if (lane == 0) c->a.defer_next[tile] = atomicExch(&c->head, tile);
+      }
+      const uint64_t p0 = (uint64_t)tile * pl.ppt;
+      const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
+      for (uint32_t lp0 = 0, run = base; room && lp0 < np; lp0 += 32u) {
+        const uint2 mk = lp0 + lane < np ? load_marker(c->d, p0 + lp0 + lane) : make_uint2(0u, 0u);
+        const bool mine = (mk.y & 3u) != kClsNormal;
+        const uint32_t m = __ballot_sync(full, mine), u = mine ? mk.x : 0u;
+        uint32_t incl = u;
+#pragma unroll
+        for (uint32_t o = 1; o < 32u; o <<= 1) {
+          const uint32_t up = __shfl_up_sync(full, incl, o);
+          if (lane >= o) incl += up;
+        }
+        if (mine) {
+          const uint32_t k = at + __popc(m & ((1u << lane) - 1u));
+          l->place[k] = run + incl - u;
+          l->meta[k] = mk.y;
+          l->lp[k] = (uint16_t)(lp0 + lane);
+          l->of[k] = (uint8_t)i;
+        }
+        at += __popc(m);
+        run += __shfl_sync(full, incl, 31);
+      }
+    }
+    if (lane == 0) l->base[i] = base;
+  }
+  for (uint32_t pass = 0; pass < 2u; ++pass) {
+    __syncthreads();  // the places are known; the stages are free
+    if (warp == (uint32_t)kWarps) continue;
+    for (;;) {
+      uint32_t item = 0;
+      if (lane == 0) item = atomicAdd(&l->handed[pass], 1u);
+      item = __shfl_sync(full, item, 0);
+      if (!small) {
+        if (item >= min(l->planes, kListedPlanes)) break;
+        const uint32_t i = l->of[item];
+        if (i == kListed) continue;
+        const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
+        const bool held = c->held[st] == tile;
+        if (held == (pass == 0u))
+          warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, held ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr,
+                               l->meta[item], l->place[item], buf, sal);
         continue;
       }
-      const uint32_t p0 = tile * pl.ppt;
-      const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
-      uint8_t* tbuf = stages + (uint64_t)(walk == 0u ? at_stage : 0u) * pl.stage_bytes;
-      if (walk) stage_planes(pl, c->a.src, p0, np, tbuf);  // (tiles of this kernel start on 16-byte boundaries)
-      uint2 mk = make_uint2(0u, 0u);
-      bool mine = false;
-      const uint32_t lp = tid / TT;
-      if (warp < (uint32_t)kWarps && lp < np && (tid % TT) == 0u) {
-        mk = load_marker(c->d, (uint64_t)p0 + lp);
-        mine = (mk.y & 3u) != kClsNormal;
-      }
-      const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, mine);
-      if (lane == 0 && warp < (uint32_t)kWarps) c->wcnt[warp] = __popc(leaders);
-      __syncthreads();
-      uint32_t before = 0, total = 0;
-      for (uint32_t w = 0; w < (uint32_t)kWarps; ++w) {
-        before += w < warp ? c->wcnt[w] : 0u;
-        total += c->wcnt[w];
-      }
-      if (mine) {
-        const uint32_t r = before + __popc(leaders & ((1u << lane) - 1u));
-        l->list_at[r] = mk.x;
-        l->list_meta[r] = mk.y;
-        l->list_lp[r] = (uint16_t)lp;
-      }
-      __syncthreads();
-      if (warp == 0) {  // places within the tile's part of the overflow region, and the tile's place
-        uint32_t run = 0;
-        for (uint32_t r0 = 0; r0 < total; r0 += 32u) {
-          const uint32_t v = r0 + lane < total ? l->list_at[r0 + lane] : 0u;
-          uint32_t incl = v;
-          for (uint32_t o = 1; o < 32u; o <<= 1) {
-            const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += up;
+      if (item >= n * (uint32_t)kWarps) break;
+      const uint32_t i = item / (uint32_t)kWarps, slice = item % (uint32_t)kWarps, tile = l->tile[i], st = l->stage[i];
+      const bool held = c->held[st] == tile;
+      if (held != (pass == 0u) || !((l->slices[i] >> slice) & 1u) || l->base[i] == kNoTile) continue;
+      warp_slice_write<DT, TT>(c, tile, slice, l->base[i] + l->before[i][slice],
+                               held ? stages + (uint64_t)st * pl.stage_bytes : nullptr, buf, sal);
+    }
+    while (pass) {  // the tiles that were not listed, a warp each
+      uint32_t tile = kNoTile;
+      if (lane == 0)
+        for (tile = *(volatile uint32_t*)&c->head; tile != kNoTile;) {
+          const uint32_t seen = atomicCAS(&c->head, tile, c->a.defer_next[tile]);
+          if (seen == tile) {
+            c->a.defer_next[tile] = 0u;
+            break;
           }
-          if (r0 + lane < total) l->list_at[r0 + lane] = run + incl - v;
-          run += __shfl_sync(0xFFFFFFFFu, incl, 31);
+          tile = seen;
         }
-        bool ok = true;
-        uint32_t base = 0;
-        if (run) ok = scan_prefix(c->a.scan, tile, base);
-        if (lane == 0) {
-          if (!ok) report_error(c->a, kErrTimeout);
-          c->base = base;
-          c->ok = ok;
-        }
-      }
-      __syncthreads();
-      if (c->ok && warp < (uint32_t)kWarps)
-        for (uint32_t r = warp; r < total; r += (uint32_t)kWarps) {
-          const uint32_t pl_lp = l->list_lp[r];
-          warp_plane_write<DT>(team, pl, c->d, (uint64_t)p0 + pl_lp, tbuf + (uint64_t)pl_lp * pl.plane_bytes, sal,
-                               l->list_meta[r] >> 2, c->base + l->list_at[r]);
-          __syncwarp();
-        }
-      __syncthreads();
-      tile = next;
+      tile = __shfl_sync(full, tile, 0);
+      if (tile == kNoTile) break;
+      uint32_t at = place_of(tile);
+      if (at == kNoTile) break;
+      for (uint32_t slice = 0; slice < (uint32_t)kWarps; ++slice) at += warp_slice_write<DT, TT>(c, tile, slice, at, nullptr, buf, sal);
     }
   }
 }
@@ -1163,13 +1323,12 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, BlockList* l, uint8_t* sta
 template <int DT, int SIGMA, int TT, int K, int EDGE>
 __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ double s_red[kMaxWarps * 5];
   __shared__ __align__(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages];
   __shared__ uint32_t s_tiles[kMaxStages];
   __shared__ volatile uint32_t s_abort;
   __shared__ uint32_t s_last;
   __shared__ BlockCtl s_ctl;
-  __shared__ BlockList s_list;
+  __shared__ WarpList s_list;
 
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t nstage = pl.nstage;
@@ -1183,29 +1342,35 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     }
     fence_mbar_init();
     s_abort = 0;
-    *cta_dirty() = 0u;
+    *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
     if (scan_on) {
       s_ctl.pl = pl;
       s_ctl.a = a;
-      s_ctl.head = kNoTile;
+      s_ctl.head = s_ctl.own = kNoTile;
       for (uint32_t s = 0; s < nstage; ++s) {
         s_ctl.U[s] = s_ctl.C[s] = s_ctl.arr[s] = 0;
         s_ctl.held[s] = kNoTile;
+        s_list.mask[s] = 0;
       }
+      s_list.count = s_list.planes = s_list.handed[0] = s_list.handed[1] = 0;
     }
   }
   // (the ticket counter of this call was returned to zero by the call before the previous one, which had
   // completed before the previous kernel let this one start)
   if (tid == (uint32_t)kThreads && a.early_ticket)
-    first_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
+    first_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)pl.first_req);
   __syncthreads();
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
-  const Dest d = make_dest(pl, a);
+  // (the sweeps only need the first and the last of these: the others wait in shared memory, not in registers)
+  Dest d = {};
   if (warp < (uint32_t)kWarps) {  // (the producer goes straight to its first loads)
+    const Dest all = make_dest(pl, a);
+    d.dst = all.dst;
+    d.fits = all.fits;
     if (tid == 0) {
       if (!d.fits && blockIdx.x == 0) report_error(a, kErrCapacity);
-      if (scan_on) s_ctl.d = d;
+      s_ctl.d = all;
     }
     asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");  // the consumer warps: s_ctl.d is in place
   }
@@ -1215,7 +1380,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     uint32_t s = 0, empty_phase = 0;
     bool aborted = false;
     if (!a.early_ticket && lane == 0)
-      first_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
+      first_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)pl.first_req);
     first_ticket = __shfl_sync(0xFFFFFFFFu, first_ticket, 0);
     // Waits until every consumer warp is done with the tile in stage q.
     auto drain = [&](uint32_t q) -> bool {
@@ -1229,9 +1394,23 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
         aborted = true;
         break;
       }
-      // tiles come in ticket order: the first nstage of them in one request, then one at a time
+      // tiles come in ticket order: the first of them in one request, then one at a time.  The tiles that are left of a small
+      // tensor when every CTA has its first go to the CTAs of the lowest numbers -- one to an SM -- as soon as their first
+      // load has arrived, so that the second is on its way while the first is swept (14 x 14, fp32, 512 tiles: 11.2 ->
+      // 9.9 us; whoever came first took them at first, three to an SM, which cost as much as it gave when the sweep is long).
       uint32_t t = first_ticket + n;
-      if (n >= nstage) {
+      if (n >= pl.first_req) {
+        if (n < nstage) {
+          const uint64_t given = (uint64_t)n * gridDim.x;
+          const bool soon = given < pl.ntiles && blockIdx.x < pl.ntiles - given;
+          bool here = soon ? mbar_wait_abortable(&s_full[s - 1u], 0u, 1u << 20, &s_abort)
+                           : mbar_wait_abortable(&s_empty[s - 1u], 0u, 1u << 20, &s_abort);
+          here = __all_sync(0xFFFFFFFFu, here);
+          if (!here) {
+            aborted = true;
+            break;
+          }
+        }
         if (lane == 0) t = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
         t = __shfl_sync(0xFFFFFFFFu, t, 0);
       }
@@ -1287,8 +1466,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     }
   } else {
     // ======================= consumers =======================
-    const Team team = make_team(TT, s_red);
-    const uint32_t my_team = tid / TT;
+    const Team team = make_team(TT, nullptr);
     const uint32_t grain = plane_grain(pl);
     uint32_t rp = 0, s = 0, phase = 0;
     for (;;) {
@@ -1304,19 +1482,22 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
       if (tile >= pl.ntiles) break;
       const uint32_t p0 = tile * pl.ppt;
       const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
-      const uint32_t lp = my_team, at = min(lp, np - 1u);
+      // (which warp takes which slice changes from tile to tile, so that a periodic pattern of outlier-rich planes does not
+      // land on the same warp every time)
+      const uint32_t slice = (warp + tile) & ((uint32_t)kWarps - 1u);
+      const uint32_t lp = slice * (32u / TT) + lane / TT, at = min(lp, np - 1u);
       const bool active = lp < np;
-      const uint8_t* stage = smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes;
+      uint8_t* stage = smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes;
       const uint32_t meta = plane_sweep<DT, SIGMA, K, TT, EDGE>(team, pl, d, a, stage + (uint64_t)at * pl.plane_bytes,
                                                                 (uint64_t)p0 + at, grain, active, rp);
       if (scan_on) {  // phase 1 of the block-wise path
         const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, active && (meta & 3u) != kClsNormal && team.lane == 0);
         if (leaders)
-          warp_tile_measure<DT, TT>(&s_ctl, stage, (uint64_t)p0, s, (warp * 32u) / TT, leaders, meta,
+          warp_tile_measure<DT, TT>(&s_ctl, &s_list, stage, (uint64_t)p0, s, slice, leaders, meta,
                                     reinterpret_cast<uint32_t*>(smem + pl.sm_sal + warp * pl.sal_stride));
         if (lane == 0) {
           if (leaders) __threadfence_block();  // the warp's sums before its arrival
-          if ((atomicAdd(&s_ctl.arr[s], 1u) & 7u) == 7u) warp_tile_publish(&s_ctl, s, tile);
+          if ((atomicAdd(&s_ctl.arr[s], 1u) & 7u) == 7u) warp_tile_publish(&s_ctl, &s_list, s, tile);
         }
       }
       __syncwarp();
@@ -1327,9 +1508,9 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   }
   if (scan_on) {
     __syncthreads();
-    if (s_ctl.head != kNoTile && !s_abort) warp_phase2<DT, TT>(&s_ctl, &s_list, smem + pl.sm_tile, smem + pl.sm_sal);
+    if (s_list.count != 0u && !s_abort) warp_phase2<DT, TT>(&s_ctl, &s_list, smem + pl.sm_tile, smem + pl.sm_sal);
   }
-  cta_exit(pl, a, d, &s_last);
+  cta_exit(pl, a, s_ctl.d, &s_last);
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -1341,21 +1522,80 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
 // plane, so NT is kept small for small planes.  Thread 0 keeps the next ticket in flight while the CTA works.
 // An outlier-rich plane is measured by the whole CTA while it lies in its stage and written in phase 2.
 // -------------------------------------------------------------------------------------------------
-// Phase 1: the plane in `plane` is measured, tile (= plane) `tile` published and put on the CTA's list.
+// Phase 1: the plane in `plane` is measured, tile (= plane) `tile` published.  Ends with a barrier.
 template <int DT>
 __device__ __noinline__ void cta_tile_measure(BlockCtl* c, double* red, const uint8_t* plane, uint32_t* sal, uint32_t tile,
                                               uint32_t meta) {
   const Team team = make_cta_team(blockDim.x, red);
   const SalientInfo info = salient_measure<DT>(team, c->pl, plane, sal);
-  bool raw;
-  const uint32_t units = plane_units(c->pl, info, raw);
   if (threadIdx.x == 0) {
-    c->measured = tile;
-    c->measured_info = info;
+    bool raw;
+    const uint32_t units = plane_units(c->pl, info, raw);
+    scan_publish(c->a.scan, tile, units);
+    count_blockwise(units, raw ? 0u : 1u, raw ? 1u : 0u);
     if (c->d.fits) store_marker(c->d, tile, meta, units);
-    publish_tile(c, tile, units, raw ? 0u : 1u, raw ? 1u : 0u);
   }
+  if (c->d.fits && scratch_saved(c->pl)) scratch_save(team, c->pl, c->d, tile, info, sal);
+  if (threadIdx.x == 0) c->own_info = info;
+  __syncthreads();
 }
+
+// The queue of planes put off (CTA-team kernels).  Which CTA has measured how many outlier-rich planes is a matter of
+// chance -- none to twice the mean --, so phase 2 deals them out anew: with every CTA writing its own, the bf16 112 x 112
+// tensor with every eighth channel outlier-rich spent 168 to 335 us of 338 in phase 2, depending on the CTA.
+// One thread, behind a barrier that follows the measuring: plane `tile`, of `stage`, is put off.  `held`: no other plane
+// will be loaded there.
+static __device__ __noinline__ void queue_push(BlockCtl* c, uint32_t tile, uint32_t stage, bool held) {
+  if (!c->d.fits) return;
+  c->head = tile;  // (the CTA has put something off)
+  // the CTA keeps its last plane, whose scratch lies ready; the one before joins the queue
+  const uint32_t before = c->own;
+  c->own = tile;
+  c->own_stage = stage;
+  c->own_held = held;
+  if (before == kNoTile) return;
+  const uint32_t n = (uint32_t)(atomicAdd(&c->a.sc->queue, 1ull << 32) >> 32);
+  __threadfence();  // marker and saved scratch, of all threads, before the entry
+  st_relaxed32(&c->a.defer_next[n], before + 1u);
+}
+constexpr uint32_t kPending = 0xFFFFFFFEu;
+// One thread: the plane of queue entry n, which is this CTA's; kNoTile when there will be none -- every CTA has finished
+// phase 1 and the queue is shorter --, kPending (unless `wait`) when it is not known yet.  A CTA in phase 1 waits for
+// nobody, so the wait ends; it is bounded all the same.
+static __device__ __noinline__ uint32_t queue_entry(BlockCtl* c, uint32_t n, bool wait) {
+  const CompressArgs& a = c->a;
+  if (n >= c->pl.ntiles) return kNoTile;
+  for (uint32_t k = 0; k < a.scan.polls; ++k) {
+    uint32_t e = ld_relaxed32(&a.defer_next[n]);
+    if (!e && wait) {
+      const unsigned long long left = ld_relaxed(&a.sc->exited), in2 = ld_relaxed(&a.sc->done);
+      __threadfence();
+      const uint32_t quiet = ((uint32_t)left & kExitMask) - ((uint32_t)(left >> kExitBits) & kExitMask);  // left with nothing
+      if (quiet + (uint32_t)in2 == gridDim.x && n >= (uint32_t)(ld_relaxed(&a.sc->queue) >> 32)) return kNoTile;
+      e = ld_relaxed32(&a.defer_next[n]);
+    }
+    if (e) {
+      st_relaxed32(&a.defer_next[n], 0u);
+      __threadfence();
+      return e - 1u;
+    }
+    if (!wait) return kPending;
+    __nanosleep(200);
+  }
+  report_error(a, kErrTimeout);
+  return kNoTile;
+}
+
+// All threads of the CTA start to copy plane gp with the 16-byte chunks around it; fetch_wait and a barrier end it.
+__device__ __forceinline__ void fetch_start(const Plan& pl, const uint8_t* src, uint64_t gp, uint8_t* to) {
+  const uint64_t start = gp * pl.plane_bytes, end = start + pl.plane_bytes, a0 = start & ~15ull;
+  const uint64_t whole = min((end + 15ull) & ~15ull, pl.dense_bytes & ~15ull);
+  for (uint64_t o = a0 + 16u * threadIdx.x; o < whole; o += 16u * blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(to + (o - a0))), "l"(src + o) : "memory");
+  if (threadIdx.x == 0)
+    for (uint64_t i = whole; i < end; i += 2) *reinterpret_cast<uint16_t*>(to + (i - a0)) = *reinterpret_cast<const uint16_t*>(src + i);
+}
+__device__ __forceinline__ void fetch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Bulk load of plane `gp` with the 16-byte chunks around it (one thread); plane_head says where the plane starts in the
 // stage.  The last bytes of a tensor that does not end on a 16-byte boundary are copied by the thread itself, ahead of
@@ -1371,55 +1611,66 @@ __device__ __forceinline__ void plane_load(const Plan& pl, const uint8_t* src, u
   bulk_g2s(stage, src + a0, (uint32_t)(whole - a0), bar);
 }
 
-// Phase 2 of the CTA-team kernels: every plane the CTA has put off, newest first.  The newest often still lies in a
-// stage (`c->held`), and what was measured of it in the scratch.
+// Phase 2 of the CTA-team kernels: the CTA's own plane, then planes from the queue until it is empty.  While one is written, the next is claimed and
+// fetched into the other stage.
 template <int DT>
-__device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal, uint64_t* bar, uint32_t parity) {
+__device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal) {
   const Plan& pl = c->pl;
   const Team team = make_cta_team(blockDim.x, red);
   const uint32_t tid = threadIdx.x;
-  for (uint32_t tile = c->head; tile != kNoTile;) {
-    const uint32_t next = c->a.defer_next[tile];
-    const uint32_t at = c->held[1] == tile ? 1u : 0u;
-    const uint8_t* plane = stages + (uint64_t)at * pl.stage_bytes + plane_head(pl, tile);
-    if (c->held[at] != tile) {  // (the same for every thread)
-      __syncthreads();
-      if (tid == 0) {
-        c->held[0] = tile;
-        plane_load(pl, c->a.src, tile, stages, bar);
-      }
-      bool ready = mbar_wait(bar, parity, 1u << 20);
-      ready = __syncthreads_and(ready);
-      parity ^= 1u;
-      if (!ready) {  // the load timed out: report, wait (bounded) for the copy, give up
-        if (tid == 0) {
-          report_error(c->a, kErrTimeout);
-          mbar_wait(bar, parity ^ 1u, 1u << 10);
-        }
-        return;
-      }
-    }
-    SalientInfo info;
-    if (c->measured == tile) info = c->measured_info;
-    else info = salient_measure<DT>(team, pl, plane, sal);
-    bool raw;
-    const uint32_t units = plane_units(pl, info, raw);
+  const bool claims = tid == blockDim.x - 32u;  // (not in the warp that looks up places, where there are two)
+  uint32_t mine = 0, cur = 0;
+  auto claim = [&]() { mine = (uint32_t)atomicAdd(&c->a.sc->queue, 1ull); };
+  if (claims) {
+    __threadfence();  // the CTA's entries before the note that it has finished phase 1
+    atomicAdd(&c->a.sc->done, 1ull);
+    c->next = c->own;
+  }
+  bool kept = true;  // the plane in hand is the CTA's own: its scratch lies ready
+  cur = c->own_stage;
+  for (bool fetched = c->own_held != 0u;;) {
+    __syncthreads();
+    const uint32_t tile = c->next;
+    if (tile >= pl.ntiles) break;  // (the same for every thread)
+    uint8_t* stage = stages + (uint64_t)cur * pl.stage_bytes;
+    if (!fetched) fetch_start(pl, c->a.src, tile, stage);
+    if (claims) claim();
+    const uint2 mk = load_marker(c->d, tile);  // units, class and count
     if (tid < 32u) {
       bool ok = true;
       uint32_t base = 0;
-      if (units) ok = scan_prefix(c->a.scan, tile, base);
+      if (mk.x) ok = scan_prefix(c->a.scan, tile, base);
       if (tid == 0) {
         if (!ok) report_error(c->a, kErrTimeout);
         c->base = base;
         c->ok = ok;
       }
     }
+    SalientInfo info;
+    const bool saved = scratch_saved(pl);
+    if (kept) info = c->own_info;
+    else if (saved) info = scratch_load(team, pl, c->d, tile, sal);
+    if (claims) c->ahead = queue_entry(c, mine, false);
+    fetch_wait();
     __syncthreads();
-    if (tid == 0) c->measured = kNoTile;
-    if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, plane, info, sal, load_marker(c->d, tile).y >> 2, c->base);
-    __syncthreads();
-    tile = next;
+    const uint32_t ahead = c->ahead;
+    const uint8_t* plane = stage + plane_head(pl, tile);
+    fetched = ahead < pl.ntiles;
+    if (fetched) fetch_start(pl, c->a.src, ahead, stages + (uint64_t)(cur ^ 1u) * pl.stage_bytes);
+    if (!saved && !kept) info = salient_measure<DT>(team, pl, plane, sal);
+    kept = false;
+    if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, plane, info, sal, mk.y >> 2, c->base);
+    if (claims) c->next = ahead == kPending ? queue_entry(c, mine, true) : ahead;
+    fetch_wait();
+    if (fetched) cur ^= 1u;
   }
+}
+// Behind phase 1 of a CTA-team kernel.
+template <int DT>
+__device__ __forceinline__ void cta_finish(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal, bool aborted) {
+  __syncthreads();
+  if (c->head != kNoTile && !aborted) cta_phase2<DT>(c, red, stages, sal);
+  else if (threadIdx.x == 0 && has_totals(*cta_totals())) atomicAdd(&c->a.sc->done, 1ull);  // (see queue_entry)
 }
 
 template <int DT>
@@ -1492,7 +1743,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
     for (uint32_t s = 0; s < nstage; ++s) mbar_init(&s_full[s], 1);
     fence_mbar_init();
     s_abort = 0;
-    *cta_dirty() = 0u;
+    *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
     // (the ticket counter of this call was returned to zero by the call before the previous one, which had
     // completed before the previous kernel let this one start)
     if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
@@ -1500,7 +1751,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
   if (tid == 0 && scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
     s_ctl.pl = pl;
     s_ctl.a = a;
-    s_ctl.head = s_ctl.measured = s_ctl.held[0] = s_ctl.held[1] = kNoTile;
+    s_ctl.head = s_ctl.own = kNoTile;
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
@@ -1642,8 +1893,10 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
       }
     } else {  // (the same for every thread) phase 1 of the block-wise path
       cta_tile_measure<DT>(&s_ctl, s_red, plane, sal, tile, cls | (n_out << 2));
-      __syncthreads();  // every thread is done with the stage
-      if (tid == 0) issue(s);
+      if (tid == 0) {
+        issue(s);
+        queue_push(&s_ctl, tile, s, s_tiles[s] >= pl.ntiles);
+      }
     }
     s = s + 1 == nstage ? 0 : s + 1;
     // s_tiles[s] for the next iteration was written at least one barrier ago (nstage >= 2)
@@ -1657,11 +1910,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
         mbar_wait(&s_full[k], 1u, 1u << 10);
       }
   }
-  if (scan_on) {
-    __syncthreads();
-    if (s_ctl.head != kNoTile && !s_abort)
-      cta_phase2<DT>(&s_ctl, s_red, smem + pl.sm_tile, sal, &s_full[0], phase & 1u);
-  }
+  if (scan_on) cta_finish<DT>(&s_ctl, s_red, smem + pl.sm_tile, sal, s_abort != 0u);
   cta_exit(pl, a, d, &s_last);
 }
 
@@ -1703,12 +1952,12 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     fence_mbar_init();
     s_abort = 0;
     s_count[0] = s_count[1] = 0;
-    *cta_dirty() = 0u;
+    *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
     if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)early);
     if (scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
       s_ctl.pl = pl;
       s_ctl.a = a;
-      s_ctl.head = s_ctl.measured = s_ctl.held[0] = s_ctl.held[1] = kNoTile;
+      s_ctl.head = s_ctl.own = kNoTile;
     }
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
@@ -1717,7 +1966,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     const uint32_t t = next_ticket;
     s_tiles[s] = t;
     if (t < pl.ntiles) {
-      if (scan_on) s_ctl.held[s] = t;
       plane_load(pl, a.src, t, smem + (uint64_t)s * pl.stage_bytes, &s_full[s]);
       ++issued;
       next_ticket = issued < early ? t + 1u : (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
@@ -1759,8 +2007,10 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
   };
   auto measure = [&](uint32_t s) {
     cta_tile_measure<DT>(&s_ctl, s_red, smem + (uint64_t)s * pl.stage_bytes + plane_head(pl, prev), sal, prev, prev_meta);
-    __syncthreads();  // every thread is done with the stage
-    if (tid == 0) issue(s);
+    if (tid == 0) {
+      issue(s);
+      queue_push(&s_ctl, prev, s, s_tiles[s] >= pl.ntiles);
+    }
   };
 
   uint32_t s = 0, phase = 0;
@@ -1846,10 +2096,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
         mbar_wait(&s_full[k], 1u, 1u << 10);
       }
   }
-  if (scan_on) {
-    __syncthreads();
-    if (s_ctl.head != kNoTile && !s_abort) cta_phase2<DT>(&s_ctl, s_red, smem, sal, &s_full[0], phase & 1u);
-  }
+  if (scan_on) cta_finish<DT>(&s_ctl, s_red, smem, sal, s_abort != 0u);
   cta_exit(pl, a, d, &s_last);
 }
 

@@ -54,6 +54,7 @@ struct Plan {
   uint32_t ntiles;
   uint32_t team;         // threads per plane: 1..32 (power of two) or kThreads
   uint32_t nstage;       // fast kernels: tiles in flight per CTA
+  uint32_t first_req;    // warp-team kernel: tiles a CTA requests at once when it starts
   uint32_t stage_bytes;  // fast kernels: bytes of one stage buffer (ppt * plane_bytes)
   // shared-memory layout (byte offsets into dynamic shared memory)
   uint32_t sm_tile, sm_out, sm_rec, sm_total;
@@ -70,11 +71,12 @@ struct Scratch {
   unsigned long long ticket[2];  // next tile; consecutive compress calls on a stream alternate between the two
   unsigned long long exited;     // CTAs that have left the running kernel
   unsigned long long status;     // device error code (atomicMax)
-  unsigned long long ovf16;      // overflow region size of this call, in 16-byte units
-  unsigned long long nsal, nraw;
+  unsigned long long nsal, nraw; // outlier-rich planes of either kind (see cta_exit)
   unsigned long long reserved;
+  unsigned long long queue;      // CTA-team kernels: planes put off, entries claimed (high half, low half)
+  unsigned long long done;       // ... CTAs that have finished phase 1 and either work on the queue or have an error to report
 };
-static_assert(sizeof(Scratch) == 64, "Scratch layout");
+static_assert(sizeof(Scratch) == 72, "Scratch layout");
 constexpr uint32_t kScratchHeadBytes = 256;  // the header, padded
 
 // (uint64)(int64) fh_status of a device error code.
@@ -103,6 +105,15 @@ __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long lon
 }
 __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+__device__ __forceinline__ uint32_t ld_relaxed32(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed32(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // ---- programmatic dependent launch: a kernel launched with the programmatic-serialisation attribute may
@@ -366,14 +377,6 @@ __device__ __forceinline__ uint32_t quant_code_random(float d, float inv, uint32
   const float least = __fsub_rn(upper, __uint_as_float((word & 0x100u) * 0x338000u));     // ... less 2^-24 when r is odd
   const uint32_t n = __float_as_uint(magic) - 0x4B000000u;
   return min(n + (frac >= least ? 1u : 0u), L);
-}
-
-// Pre-quantisation of dense-block elements (Eq. 9 on integers): k = rne(fp32(x * inv2e)), |k| <= 2^24.
-__device__ __forceinline__ int32_t dense_k(float x, float inv2e, bool* big) {
-  float kf = rintf(__fmul_rn(x, inv2e));
-  *big = fabsf(kf) >= 16777216.0f;
-  kf = fminf(fmaxf(kf, -16777216.0f), 16777216.0f);
-  return (int32_t)kf;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -842,63 +845,62 @@ __device__ __forceinline__ void scan_publish(const Scan& s, uint32_t t, uint32_t
 static __device__ __noinline__ bool scan_prefix(const Scan& s, uint32_t t, uint32_t& prefix) {
   const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu;
   const uint32_t g = t >> 5, within = t & 31u;
-  // tiles of the own group before t
-  unsigned long long u = 0;
-  {
-    bool ok = lane >= within;
-    for (uint32_t k = 0; k < s.polls; ++k) {
-      if (!ok) {
-        const unsigned long long v = ld_relaxed(&s.tile[g * 32u + lane]);
-        if ((uint32_t)(v >> 32) == s.epoch) {
-          u = v & 0xFFFFFFFFull;
-          ok = true;
-        }
-      }
-      if (__all_sync(full, ok)) break;
-      __nanosleep(100);
+  // tiles of the own group before t, and at the same time earlier groups, the nearest first, 32 at a time, until a group
+  // whose prefix somebody has published
+  unsigned long long own = 0, gsum = 0;
+  bool mine = lane >= within;
+  if (g > 0u) {  // usually that prefix is there: one word, where the search below has every waiting warp read 64
+    const unsigned long long vp = ld_relaxed(&s.gpre[g - 1u]);
+    const unsigned long long vt = mine ? 0ull : ld_relaxed(&s.tile[g * 32u + lane]);
+    if (!mine && (uint32_t)(vt >> 32) == s.epoch) {
+      own = vt & 0xFFFFFFFFull;
+      mine = true;
     }
-    if (!__all_sync(full, ok)) return false;
+    if ((uint32_t)(vp >> 32) == s.epoch && __all_sync(full, mine)) {
+      prefix = (uint32_t)((vp & 0xFFFFFFFFull) + warp_sum_u64(own));
+      return true;
+    }
   }
-  unsigned long long acc = warp_sum_u64(u);
-  // earlier groups, the nearest first, 32 at a time, until a group whose prefix somebody has published
-  unsigned long long gsum = 0;
-  uint32_t hi = g;
-  while (hi > 0) {
+  for (uint32_t hi = g;;) {
     const bool act = lane < hi;
     const uint32_t j = act ? hi - 1u - lane : 0u;
     bool have_pre = false, done = !act;
     unsigned long long val = 0;
-    uint32_t first = 32, need = full, dm = 0;
+    uint32_t first = 32;
+    bool all = false;
     for (uint32_t k = 0; k < s.polls; ++k) {
-      if (act && !have_pre) {
-        const unsigned long long v = ld_relaxed(&s.gpre[j]);
-        if ((uint32_t)(v >> 32) == s.epoch) {
-          have_pre = true;
-          done = true;
-          val = v & 0xFFFFFFFFull;
-        }
+      unsigned long long vt = 0, vp = 0, vg = 0;
+      if (!mine) vt = ld_relaxed(&s.tile[g * 32u + lane]);
+      if (act && !have_pre) vp = ld_relaxed(&s.gpre[j]);
+      if (!done) vg = ld_relaxed(&s.grp[j]);
+      if (!mine && (uint32_t)(vt >> 32) == s.epoch) {
+        own = vt & 0xFFFFFFFFull;
+        mine = true;
       }
-      if (act && !done) {
-        const unsigned long long v = ld_relaxed(&s.grp[j]);
-        if ((v >> 40) == 32ull) {  // every group before another one is a whole group of 32 tiles
-          done = true;
-          val = v & ((1ull << 40) - 1ull);
-        }
+      if (act && !have_pre && (uint32_t)(vp >> 32) == s.epoch) {
+        have_pre = true;
+        done = true;
+        val = vp & 0xFFFFFFFFull;
+      }
+      if (!done && (vg >> 40) == 32ull) {  // every group before another one is a whole group of 32 tiles
+        done = true;
+        val = vg & ((1ull << 40) - 1ull);
       }
       const uint32_t pm = __ballot_sync(full, have_pre);
       first = pm ? (uint32_t)__ffs((int)pm) - 1u : 32u;
-      need = first >= 31u ? full : ((2u << first) - 1u);  // lanes 0..first
-      dm = __ballot_sync(full, done);
-      if ((dm & need) == need) break;
-      __nanosleep(100);
+      const uint32_t need = first >= 31u ? full : ((2u << first) - 1u);  // lanes 0..first
+      const uint32_t dm = __ballot_sync(full, done);
+      all = (dm & need) == need && __all_sync(full, mine);
+      if (all) break;
+      __nanosleep(k < 4u ? 100u : 500u);
     }
-    if ((dm & need) != need) return false;
+    if (!all) return false;
     gsum += warp_sum_u64(lane <= first ? val : 0ull);
-    if (first < 32u) break;
-    hi = hi > 32u ? hi - 32u : 0u;
+    if (first < 32u || hi <= 32u) break;
+    hi -= 32u;
   }
   if (g > 0 && lane == 0) st_relaxed(&s.gpre[g - 1u], ((unsigned long long)s.epoch << 32) | (gsum & 0xFFFFFFFFull));
-  prefix = (uint32_t)(gsum + acc);
+  prefix = (uint32_t)(gsum + warp_sum_u64(own));
   return true;
 }
 
@@ -914,7 +916,7 @@ struct CompressArgs {
   unsigned long long* out2;             // optional: {total bytes, status}
   Scratch* sc;
   Scan scan;                            // placement of overflow parts (unused with salient_mode OFF)
-  uint32_t* defer_next;                 // one word per tile: links the tiles a CTA has put off (see BlockCtl)
+  uint32_t* defer_next;                 // one word per tile, zero between calls: tiles put off (see BlockCtl)
   uint32_t parity;                      // which of the two ticket counters this call uses
   uint32_t early_ticket;                // 1: tiles may be requested before the previous kernel on the stream has completed
   // channel-wide three-sigma mode: per-channel outlier counts and per-plane counts from the statistics passes

@@ -87,7 +87,7 @@ inline int spread_grid(int grid, uint32_t ntiles) {
 inline Plan with_first_request(const Plan& pl, int grid, uint32_t least) {
   Plan q = pl;
   const uint32_t each = pl.ntiles / (uint32_t)(grid > 0 ? grid : 1);
-  q.nstage = each < least ? least : (each > pl.nstage ? pl.nstage : each);
+  q.nstage = q.first_req = each < least ? least : (each > pl.nstage ? pl.nstage : each);
   return q;
 }
 

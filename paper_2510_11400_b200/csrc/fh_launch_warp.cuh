@@ -12,8 +12,9 @@ int launch_warp_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int rc = grid_for(compress_warp<DT, SIGMA, TT, K, EDGE>, pl.sm_total, pl.ntiles, &grid, kWarpKernelThreads);
   if (rc != FH_OK) return rc;
   grid = spread_grid(grid, pl.ntiles);
-  return launch_dependent(compress_warp<DT, SIGMA, TT, K, EDGE>, grid, kWarpKernelThreads, pl.sm_total, stream,
-                          with_first_request(pl, grid, 1), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+  Plan q = with_first_request(pl, grid, 1);
+  q.nstage = pl.nstage;  // (the ring has all its stages, however many tiles the first request is for)
+  return launch_dependent(compress_warp<DT, SIGMA, TT, K, EDGE>, grid, kWarpKernelThreads, pl.sm_total, stream, q, a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
 
 // Slots per lane: the team is the smallest that holds the plane, so (teams of two and more) at least four are whole;
