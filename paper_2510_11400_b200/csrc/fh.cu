@@ -285,8 +285,9 @@ struct StreamScratch {
   uint32_t prev_groups = 0;              // groups of 32 tiles the last of them used (the next one clears that set)
   uint32_t* plane_nout = nullptr;        // channel-wide three-sigma mode: per-plane counts ...
   size_t pn_cap = 0;
-  fh::ChanStat* chan = nullptr;          // ... and per-channel statistics
+  fh::ChanStat* chan = nullptr;          // ... and per-channel statistics: two sets, which alternate between calls
   size_t chan_cap = 0;
+  uint32_t chan_calls = 0, chan_used[2] = {0, 0};  // which set is next; entries of a set that may not be zero
   SchedSpace* sched = nullptr;           // schedule runner: the workspace that is not in use, if any
 };
 // tile words | two sets of group sums | group prefixes | tile links (32-bit)
@@ -373,7 +374,7 @@ int next_call(uint32_t* calls, unsigned long long* scan, size_t tile_cap, Stream
 }
 
 // Scratch of the channel-wide three-sigma mode (grown on demand like the per-stream scratch).
-int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels) {
+int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels, cudaStream_t stream) {
   if (planes > s->pn_cap) {
     size_t cap = s->pn_cap ? s->pn_cap : 65536;
     while (cap < planes) cap *= 2;
@@ -395,8 +396,10 @@ int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels) {
       s->chan = nullptr;
       s->chan_cap = 0;
     }
-    if (cudaMalloc(&s->chan, cap * sizeof(fh::ChanStat)) != cudaSuccess) return FH_ERR_CUDA;
+    if (cudaMalloc(&s->chan, 2 * cap * sizeof(fh::ChanStat)) != cudaSuccess) return FH_ERR_CUDA;
+    if (cudaMemsetAsync(s->chan, 0, 2 * cap * sizeof(fh::ChanStat), stream) != cudaSuccess) return FH_ERR_CUDA;
     s->chan_cap = cap;
+    s->chan_used[0] = s->chan_used[1] = 0;
   }
   return FH_OK;
 }
@@ -435,17 +438,22 @@ int enqueue_compress(const fh_tensor_desc* desc, const fh_params* params, const 
   a.chan_nout = nullptr;
   a.plane_nout = nullptr;
   if (pl.mode >= fh::kModeChannel) {  // statistics per channel over the batch, or over the tensor: three passes ahead of the streaming kernel
-    rc = get_channel_scratch(s, pl.P, pl.C);
+    rc = get_channel_scratch(s, pl.P, pl.C, stream);
     if (rc != FH_OK) return rc;
-    fh::ChannelArgs ca;
+    const uint32_t set = s->chan_calls++ & 1u;
+    fh::ChannelArgs ca = {};
     ca.src = (const uint8_t*)d_src;
-    ca.chan = s->chan;
+    ca.chan = s->chan + set * s->chan_cap;
+    ca.next = s->chan + (1u - set) * s->chan_cap;
+    ca.clear = s->chan_used[1u - set];
+    s->chan_used[set] = pl.mode == fh::kModeTensor ? 1u : pl.C;
+    s->chan_used[1u - set] = 0;
     ca.plane_nout = s->plane_nout;
     ca.inv_nhw = 1.0 / ((double)(pl.mode == fh::kModeTensor ? pl.P : pl.N) * (double)pl.HW);
     rc = fh::launch_channel_passes(pl, ca, stream);
     if (rc != FH_OK) return rc;
     g_launches.fetch_add(3);
-    a.chan_nout = reinterpret_cast<const unsigned long long*>(s->chan) + 3;
+    a.chan_nout = reinterpret_cast<const unsigned long long*>(ca.chan) + 3;
     a.plane_nout = s->plane_nout;
   }
   return launch_compress(pl, v, a, stream);

@@ -2,13 +2,17 @@
 // over the N planes (n, c) of a channel c together, and the channel as a whole is normal or outlier-rich.
 // Tensor-wide statistics (salient_mode = TENSOR) run through the same passes with the whole tensor as the
 // one "channel"; a plane's class then follows from its own count.
-// Three passes over the tensor, a warp per plane, results gathered per channel with atomics:
+// Three passes over the tensor, a team of lanes per plane (of at most 512 groups: larger ones go in pieces), results
+// gathered per channel with atomics:
 //   pass 0: minimum and maximum of the channel (the moments are taken of the distances from the minimum, and the
 //           range fixes the scale of the integer sums);
 //   pass 1: integer moment sums of the channel (exact, so the order of the atomics is immaterial);
 //   pass 2: thresholds from the sums; outliers per plane (kept for the plane table) and per channel.
-// The streaming kernel then reads a plane's class from its channel's count.  This mode is not tuned: it
-// reads the tensor four times where the per-plane mode reads it once.
+// The streaming kernel then reads a plane's class from its channel's count, so the tensor is read four times; what fits
+// the L2 cache comes from there from the second time on.  A lane has 64 bytes in flight; the
+// passes follow one another by programmatic launch; no memset between them (pass 0 clears the statistics that the call
+// after this one will use).  Element by element with a warp per plane the three took 162 us for 32 x 96 bf16 planes of
+// 112 x 112 (77 MB) and 27 us for 32 x 960 of 7 x 7; now 67 and 17.
 #pragma once
 
 #include "fh_device.cuh"
@@ -25,100 +29,151 @@ __device__ __forceinline__ float key_float(unsigned int k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
 
-template <int DT>
-__device__ __forceinline__ void load_group_global(const uint8_t* plane, uint32_t g, uint32_t HW, float v[4]) {
+// Group g of a plane as it lies there: four fp32 values, or two words of two bf16.  VEC: planes are whole groups on
+// group-sized boundaries; otherwise positions past HW read as the plane's last element.  (The choice is made at compile
+// time: a branch per load keeps the compiler from issuing the loads together.)
+template <int DT, bool VEC>
+__device__ __forceinline__ void load_group_raw(const uint8_t* plane, uint32_t g, uint32_t HW, uint32_t (&w)[4]) {
+  if (VEC) {
+    if (DT == kF32) {
+      const uint4 t = __ldg(reinterpret_cast<const uint4*>(plane) + g);
+      w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+    } else {
+      const uint2 t = __ldg(reinterpret_cast<const uint2*>(plane) + g);
+      w[0] = t.x; w[1] = t.y;
+    }
+    return;
+  }
+  uint32_t e[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint32_t i = g * 4u + k;
-    float x = 0.0f;
-    if (i < HW) x = DT == kF32 ? __ldg(reinterpret_cast<const float*>(plane) + i)
-                               : bf16_bits_to_f32(__ldg(reinterpret_cast<const uint16_t*>(plane) + i));
-    v[k] = x;
+  for (uint32_t k = 0; k < 4u; ++k) {
+    const uint32_t i = min(g * 4u + k, HW - 1u);
+    e[k] = DT == kF32 ? __ldg(reinterpret_cast<const uint32_t*>(plane) + i) : (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(plane) + i);
+  }
+  if (DT == kF32) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = e[k];
+  } else {
+    w[0] = e[0] | e[1] << 16;
+    w[1] = e[2] | e[3] << 16;
   }
 }
 
-template <int DT, int PASS>
-__global__ void __launch_bounds__(kThreads) channel_pass(const Plan pl, const ChannelArgs a) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t warps = (uint64_t)gridDim.x * kWarps, first = (uint64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
-  // Tensor-wide statistics have a single destination: a warp gathers over its planes, the CTA's warps are
+constexpr uint32_t kChanPiece = 512;  // groups of a piece: their integer sums fit 32 bits
+
+template <int DT, int PASS, bool VEC>
+__global__ void __launch_bounds__(kThreads, 4) channel_pass(const Plan pl, const ChannelArgs a) {
+  const uint32_t tt = a.team, lane = threadIdx.x & 31u, tl = lane & (tt - 1u), full = 0xFFFFFFFFu;
+  // Tensor-wide statistics have a single destination: a team gathers over its planes, the CTA's teams are
   // combined in shared memory, and one thread per CTA issues the atomics.
   const bool whole = pl.mode == kModeTensor;
   __shared__ float s_lo[kWarps], s_hi[kWarps];
-  __shared__ long long s_s[kWarps], s_q[kWarps];
+  __shared__ unsigned long long s_s[kWarps], s_q[kWarps];
   float wlo = __int_as_float(0x7F800000), whi = __int_as_float(0xFF800000);
-  long long ws = 0, wq = 0;
-  for (uint64_t p = first; p < pl.P; p += warps) {
+  unsigned long long ws = 0, wq = 0;
+  const uint32_t pieces = (pl.groups + kChanPiece - 1u) / kChanPiece;
+  const uint64_t items = pl.P * pieces, step = (uint64_t)gridDim.x * (kThreads / tt);
+  dep_trigger();
+  dep_wait();
+  if (PASS == 0)
+    for (uint32_t k = blockIdx.x * kThreads + threadIdx.x; k < 4u * a.clear; k += gridDim.x * kThreads)
+      reinterpret_cast<unsigned long long*>(a.next)[k] = 0ull;
+  for (uint64_t base = (uint64_t)blockIdx.x * (kThreads / tt); base < items; base += step) {  // (the warp stays together)
+    const uint64_t item = base + threadIdx.x / tt;
+    const bool there = item < items;
+    const uint32_t p = !there ? 0u : (pieces == 1u ? (uint32_t)item : (uint32_t)(item / pieces));
+    const uint32_t g0 = there ? (uint32_t)(item - (uint64_t)p * pieces) * kChanPiece : 0u, g1 = there ? min(pl.groups, g0 + kChanPiece) : 0u;
     const uint8_t* plane = a.src + p * pl.plane_bytes;
-    ChanStat* cs = a.chan + (pl.mode == kModeTensor ? 0ull : p % pl.C);
-    if (PASS == 0) {
-      float lo = __int_as_float(0x7F800000), hi = __int_as_float(0xFF800000);
-      for (uint32_t i = lane; i < pl.HW; i += 32u) {
-        const float x = DT == kF32 ? __ldg(reinterpret_cast<const float*>(plane) + i)
-                                   : bf16_bits_to_f32(__ldg(reinterpret_cast<const uint16_t*>(plane) + i));
-        lo = fminf(lo, x);   // non-finite input is reported by the streaming kernel; here it only must not trap
-        hi = fmaxf(hi, x);
-      }
-      for (uint32_t o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-      }
-      if (whole) {
-        wlo = fminf(wlo, lo);
-        whi = fmaxf(whi, hi);
-      } else if (lane == 0) {
-        atomicMax(&cs->lo_inv, ~float_key(lo));
-        atomicMax(&cs->hi_key, float_key(hi));
-      }
-    } else {
-      const float clo = key_float(~cs->lo_inv), chi = key_float(cs->hi_key);
-      const SigmaScale sc = sigma_scale(__fsub_rn(chi, clo));
-      if (!sc.applies) {  // constant channel, or a range outside the rule's domain: no outliers
-        if (PASS == 2 && lane == 0) a.plane_nout[p] = 0;
-        continue;
-      }
-      if (PASS == 1) {
-        long long s = 0, q = 0;
-        for (uint32_t g = lane; g < pl.groups; g += 32u) {
-          float v[4];
-          load_group_global<DT>(plane, g, pl.HW, v);
+    ChanStat* cs = a.chan + (whole ? 0u : p % pl.C);
+    float clo = 0.0f, dlo = 0.0f, dhi = 0.0f;
+    SigmaScale sc = {};
+    if (PASS > 0) {
+      clo = key_float(~cs->lo_inv);
+      sc = sigma_scale(__fsub_rn(key_float(cs->hi_key), clo));  // (not `applies`: a constant channel, or a range outside the rule's domain)
+      if (PASS == 2) sigma_thresholds((long long)cs->Is, (long long)cs->Iq, sc, a.inv_nhw, dlo, dhi);
+    }
+    float lo = __int_as_float(0x7F800000), hi = __int_as_float(0xFF800000);
+    uint32_t as = 0, aq = 0, n = 0;
+    constexpr uint32_t U = DT == kF32 ? 4u : 8u;  // groups in flight: 64 bytes a lane
+    for (uint32_t g = g0 + tl; g < g1; g += U * tt) {
+      uint32_t w[U][4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) v[k] = (g * 4u + k < pl.HW) ? __fsub_rn(v[k], clo) : 0.0f;
-          uint32_t as = 0, aq = 0;
-          sigma_addends(v, sc, as, aq);
-          s += (int32_t)(as - kMagicBits);
-          q += (int32_t)(aq - kMagicBits);
+      for (uint32_t u = 0; u < U; ++u) load_group_raw<DT, VEC>(plane, min(g + u * tt, g1 - 1u), pl.HW, w[u]);
+#pragma unroll
+      for (uint32_t u = 0; u < U; ++u) {
+        float v[4];
+        if (DT == kF32) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = __uint_as_float(w[u][k]);
+        } else {
+          v[0] = __uint_as_float(w[u][0] << 16); v[1] = __uint_as_float(w[u][0] & 0xFFFF0000u);
+          v[2] = __uint_as_float(w[u][1] << 16); v[3] = __uint_as_float(w[u][1] & 0xFFFF0000u);
         }
-        for (uint32_t o = 16; o > 0; o >>= 1) {
-          s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-          q += __shfl_xor_sync(0xFFFFFFFFu, q, o);
+        if (PASS == 0) {  // (an element read twice changes nothing; non-finite input is reported by the streaming kernel)
+          lo = fminf(lo, fminf(fminf(v[0], v[1]), fminf(v[2], v[3])));
+          hi = fmaxf(hi, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+        } else {
+          const uint32_t in = g + u * tt < g1 ? (VEC ? 4u : min(4u, pl.HW - 4u * (g + u * tt))) : 0u;
+          float d[4];
+#pragma unroll
+          for (uint32_t k = 0; k < 4u; ++k) d[k] = k < in ? __fsub_rn(v[k], clo) : 0.0f;
+          if (PASS == 1) {
+            if (in) {
+              sigma_addends(d, sc, as, aq);
+              ++n;
+            }
+          } else {
+#pragma unroll
+            for (uint32_t k = 0; k < 4u; ++k) n += k < in && (d[k] > dhi || d[k] < dlo);
+          }
         }
-        if (whole) {
-          ws += s;
-          wq += q;
-        } else if (lane == 0) {
+      }
+    }
+    if (PASS == 0) {
+      for (uint32_t o = tt >> 1; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(full, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(full, hi, o));
+      }
+      wlo = fminf(wlo, lo);
+      whi = fmaxf(whi, hi);
+      if (there && tl == 0) {
+        if (!whole) {
+          atomicMax(&cs->lo_inv, ~float_key(lo));
+          atomicMax(&cs->hi_key, float_key(hi));
+        }
+        if (g0 == 0u) a.plane_nout[p] = 0;
+      }
+    } else if (PASS == 1) {
+      uint32_t s = sc.applies ? as - n * kMagicBits : 0u, q = sc.applies ? aq - n * kMagicBits : 0u;
+      for (uint32_t o = tt >> 1; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(full, s, o);
+        q += __shfl_xor_sync(full, q, o);
+      }
+      if (there && tl == 0) {
+        ws += s;
+        wq += q;
+        if (!whole && sc.applies) {
           atomicAdd(&cs->Is, (unsigned long long)s);
           atomicAdd(&cs->Iq, (unsigned long long)q);
         }
-      } else {
-        float dlo, dhi;
-        sigma_thresholds((long long)cs->Is, (long long)cs->Iq, sc, a.inv_nhw, dlo, dhi);
-        uint32_t cnt = 0;
-        for (uint32_t i = lane; i < pl.HW; i += 32u) {
-          const float x = DT == kF32 ? __ldg(reinterpret_cast<const float*>(plane) + i)
-                                     : bf16_bits_to_f32(__ldg(reinterpret_cast<const uint16_t*>(plane) + i));
-          const float dd = __fsub_rn(x, clo);
-          cnt += (dd > dhi) || (dd < dlo);
-        }
-        asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(cnt) : "r"(0xFFFFFFFFu));
-        if (lane == 0) {
-          a.plane_nout[p] = cnt;
-          if (cnt && !whole) atomicAdd(&cs->nout, (unsigned long long)cnt);  // the tensor-wide mode classifies by the plane's count
-        }
+      }
+    } else {
+      if (!sc.applies) n = 0;
+      for (uint32_t o = tt >> 1; o > 0; o >>= 1) n += __shfl_xor_sync(full, n, o);
+      if (there && tl == 0 && n) {
+        if (pieces == 1u) a.plane_nout[p] = n;
+        else atomicAdd(&a.plane_nout[p], n);
+        if (!whole) atomicAdd(&cs->nout, (unsigned long long)n);  // the tensor-wide mode classifies by the plane's count
       }
     }
   }
   if (whole && PASS < 2) {
+    for (uint32_t o = 16; o > 0; o >>= 1) {
+      wlo = fminf(wlo, __shfl_xor_sync(full, wlo, o));
+      whi = fmaxf(whi, __shfl_xor_sync(full, whi, o));
+    }
+    ws = warp_sum_u64(ws);
+    wq = warp_sum_u64(wq);
     const uint32_t warp = threadIdx.x >> 5;
     if (lane == 0) {
       s_lo[warp] = wlo;
@@ -134,12 +189,12 @@ __global__ void __launch_bounds__(kThreads) channel_pass(const Plan pl, const Ch
         ws += s_s[k];
         wq += s_q[k];
       }
-      if (PASS == 0) {  // (every CTA of the grid owns at least one plane, so both values are finite numbers of the input)
+      if (PASS == 0) {  // (every CTA of the grid owns at least one plane, so both values are numbers of the input)
         atomicMax(&a.chan->lo_inv, ~float_key(wlo));
         atomicMax(&a.chan->hi_key, float_key(whi));
       } else {
-        atomicAdd(&a.chan->Is, (unsigned long long)ws);
-        atomicAdd(&a.chan->Iq, (unsigned long long)wq);
+        atomicAdd(&a.chan->Is, ws);
+        atomicAdd(&a.chan->Iq, wq);
       }
     }
   }

@@ -945,8 +945,11 @@ static_assert(sizeof(ChanStat) == 32, "ChanStat layout");
 
 struct ChannelArgs {
   const uint8_t* src;
-  ChanStat* chan;        // C entries (one in the tensor-wide mode), zeroed before pass 0
-  uint32_t* plane_nout;  // P entries, written by pass 2
+  ChanStat* chan;        // C entries (one in the tensor-wide mode), zero ahead of pass 0
+  ChanStat* next;        // those of the next call on the stream: pass 0 returns the first `clear` of them to zero
+  uint32_t clear;
+  uint32_t team;         // lanes per plane: a power of two, at most a warp
+  uint32_t* plane_nout;  // P entries, zeroed by pass 0, written by pass 2
   double inv_nhw;        // 1 / (N * HW); tensor-wide: 1 / (N * C * HW)
 };
 

@@ -14,18 +14,24 @@ int launch_generic_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream)
              ? FH_OK : FH_ERR_CUDA;
 }
 
-template <int DT>
-int launch_channel_passes_t(const Plan& pl, const ChannelArgs& ca, cudaStream_t stream) {
-  const int sms = sm_count();
-  if (sms < 1) return FH_ERR_CUDA;
-  const uint64_t want = (pl.P + kWarps - 1) / kWarps, most = (uint64_t)sms * 8;
-  const int grid = (int)(want < most ? want : most);
-  if (cudaMemsetAsync(ca.chan, 0, pl.C * sizeof(ChanStat), stream) != cudaSuccess) return FH_ERR_CUDA;
-  channel_pass<DT, 0><<<grid, kThreads, 0, stream>>>(pl, ca);
-  channel_pass<DT, 1><<<grid, kThreads, 0, stream>>>(pl, ca);
-  channel_pass<DT, 2><<<grid, kThreads, 0, stream>>>(pl, ca);
-  if (cudaGetLastError() != cudaSuccess) return FH_ERR_CUDA;
-  return FH_OK;
+template <int DT, int PASS, bool VEC>
+int launch_channel_pass(const Plan& pl, const ChannelArgs& ca, cudaStream_t stream) {
+  int grid = 0;
+  const uint64_t items = pl.P * ((pl.groups + kChanPiece - 1) / kChanPiece), per = kThreads / ca.team, want = (items + per - 1) / per;
+  const int rc = grid_for(channel_pass<DT, PASS, VEC>, 0, (uint32_t)(want < 0x7FFFFFFFull ? want : 0x7FFFFFFFull), &grid);
+  if (rc != FH_OK) return rc;
+  return launch_dependent(channel_pass<DT, PASS, VEC>, grid, kThreads, 0, stream, pl, ca) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+}
+
+template <int DT, bool VEC>
+int launch_channel_passes_t(const Plan& pl, const ChannelArgs& args, cudaStream_t stream) {
+  ChannelArgs ca = args;  // a team takes four groups per lane at once: more lanes than that have nothing to do
+  ca.team = 1;
+  while (ca.team < 32u && ca.team * 4u < pl.groups) ca.team *= 2u;
+  int rc = launch_channel_pass<DT, 0, VEC>(pl, ca, stream);
+  if (rc == FH_OK) rc = launch_channel_pass<DT, 1, VEC>(pl, ca, stream);
+  if (rc == FH_OK) rc = launch_channel_pass<DT, 2, VEC>(pl, ca, stream);
+  return rc;
 }
 
 }  // namespace
@@ -41,7 +47,9 @@ int launch_compress_generic(const Plan& pl, const CompressArgs& a, cudaStream_t 
 }
 
 int launch_channel_passes(const Plan& pl, const ChannelArgs& ca, cudaStream_t stream) {
-  return pl.dtype == kF32 ? launch_channel_passes_t<kF32>(pl, ca, stream) : launch_channel_passes_t<kBF16>(pl, ca, stream);
+  const bool vec = pl.HW % 4 == 0;
+  if (pl.dtype == kF32) return vec ? launch_channel_passes_t<kF32, true>(pl, ca, stream) : launch_channel_passes_t<kF32, false>(pl, ca, stream);
+  return vec ? launch_channel_passes_t<kBF16, true>(pl, ca, stream) : launch_channel_passes_t<kBF16, false>(pl, ca, stream);
 }
 
 }  // namespace fh
