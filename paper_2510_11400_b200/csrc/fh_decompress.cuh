@@ -789,6 +789,8 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
 // Tiles (256 / team planes) start on 16-byte boundaries; two buffers alternate.
 // -------------------------------------------------------------------------------------------------
 
+constexpr uint32_t kSmallGroups = 8;  // a lane restores at most so many groups
+
 template <int DT>
 __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, const DecompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -804,6 +806,13 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
   const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
   const uint8_t* src = a.src_base + off_in;
   const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;
+  // table entry of the team's plane: the first is fetched along with the header, a tile's while the one before is restored
+  const uint32_t tt = pl.team, lane = tid & (tt - 1u), lp = tid / tt;
+  auto entry_of = [&](uint32_t tile) {
+    const uint64_t gp = (uint64_t)tile * pl.ppt + lp;
+    return tile < pl.ntiles && lp < pl.ppt && gp < pl.P ? __ldg(reinterpret_cast<const uint4*>(src + 64) + gp) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  uint4 en = src_bytes >= 64ull + 16ull * pl.P ? entry_of(blockIdx.x) : make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
     uint32_t bits = 0;
     float eps = 0.0f;
@@ -822,37 +831,46 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
     const unsigned long long total = s_total;
     const uint32_t npay = a16(4u * ((pl.HW * bits + 31u) / 32u));
     const unsigned long long slots_off = 64ull + 16ull * pl.P, ovf_off = slots_off + pl.P * (unsigned long long)npay;
-    const uint32_t tt = pl.team, lane = tid & (tt - 1u), my_team = tid / tt;
     const Team warp_team = make_warp_team(s_red);
     const bool vec = (pl.plane_bytes & (DT == kF32 ? 15u : 7u)) == 0u;  // planes start on vector boundaries in the tile buffer
     const uint32_t tile_bytes_max = pl.stage_bytes;
     uint32_t buf = 0;
     for (uint32_t tile = blockIdx.x; tile < pl.ntiles; tile += gridDim.x, buf ^= 1u) {
       uint8_t* tbuf = smem + (uint64_t)buf * tile_bytes_max;
-      if (tid == 0) bulk_wait_read<1>();  // the store that left this buffer two tiles ago has read it
-      __syncthreads();
       const uint64_t p0 = (uint64_t)tile * pl.ppt;
       const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
-      const uint32_t lp = my_team;
+      // the codes are requested before the entry is looked at (what another plane keeps in its slot is read and dropped)
+      uint32_t code[kSmallGroups];
+#pragma unroll
+      for (uint32_t k = 0; k < kSmallGroups; ++k) {
+        const uint32_t g = lane + k * tt;
+        const uint8_t* slot = src + slots_off + (p0 + lp) * npay;
+        code[k] = 0;
+        if (lp < np && g < pl.groups)
+          code[k] = bits == 2u ? (uint32_t)__ldg(slot + g)
+                               : (bits == 4u ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(slot) + g)
+                                             : __ldg(reinterpret_cast<const uint32_t*>(slot) + g));
+      }
+      const uint4 ahead = entry_of(tile + gridDim.x);
+      if (tid == 0) bulk_wait_read<1>();  // the store that left this buffer two tiles ago has read it
+      __syncthreads();
       bool salient = false, raw = false;
       uint32_t my_off16 = 0;
       if (lp < np) {
         const uint64_t gp = p0 + lp;
-        const uint4 en = __ldg(reinterpret_cast<const uint4*>(src + 64) + gp);
         my_off16 = en.x;
         const unsigned long long off = (unsigned long long)en.x * 16ull;
         const uint32_t cls = en.y & 3u;
         uint8_t* out = tbuf + (uint64_t)lp * pl.plane_bytes;
-        const uint8_t* slot = src + slots_off + gp * npay;
         if (cls == kClsNormal) {
           if (off != slots_off + gp * npay) {
             bad = true;
           } else {
             const float lo = __uint_as_float(en.z), scale = __uint_as_float(en.w);
-            for (uint32_t g = lane; g < pl.groups; g += tt) {
-              const uint32_t word = bits == 2u ? (uint32_t)__ldg(slot + g)
-                                               : (bits == 4u ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(slot) + g)
-                                                             : __ldg(reinterpret_cast<const uint32_t*>(slot) + g));
+#pragma unroll
+            for (uint32_t k0 = 0; k0 < kSmallGroups; ++k0) {
+              const uint32_t g = lane + k0 * tt, word = code[k0];
+              if (g >= pl.groups) break;
               const uint32_t i = 4u * g;
               if (vec && i + 3u < pl.HW) {  // whole group of a plane on a vector boundary: one store
                 store_group<DT>(out, g, dequant(word & L, scale, lo), dequant((word >> bits) & L, scale, lo),
@@ -939,6 +957,7 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
         }
         __syncwarp();
       }
+      en = ahead;
       __syncthreads();
       // the tile leaves: one bulk store when it is whole 16-byte chunks, plain stores otherwise
       const uint32_t bytes = np * (uint32_t)pl.plane_bytes;
