@@ -380,6 +380,9 @@ struct WarpList {
   uint32_t place[kListedPlanes], meta[kListedPlanes];
   uint16_t lp[kListedPlanes];
   uint8_t of[kListedPlanes];         // whose entry (kListed: nobody's)
+  // where the slot cannot hold measurements: the plane that a warp's scratch is about (kNoTile: none), and its sizes
+  uint32_t own[kWarps];
+  SalientInfo own_info[kWarps];
 };
 
 // One thread: tile `tile` has `units` of overflow in `nsal` salient and `nraw` raw planes.
@@ -1078,7 +1081,12 @@ __device__ __noinline__ void warp_tile_measure(BlockCtl* c, WarpList* l, uint8_t
       nraw += raw ? 1u : 0u;
       const uint32_t mt = __shfl_sync(full, meta, (int)src);
       if (lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
-      if (c->d.fits && scratch_saved(pl)) scratch_save(team, pl, c->d, p0 + lp, info, sal);
+      if (scratch_saved(pl)) {
+        if (c->d.fits) scratch_save(team, pl, c->d, p0 + lp, info, sal);
+      } else if (lane == 0) {
+        l->own[threadIdx.x >> 5] = (uint32_t)(p0 + lp);
+        l->own_info[threadIdx.x >> 5] = info;
+      }
       __syncwarp();
     }
   }
@@ -1136,15 +1144,18 @@ __device__ __forceinline__ uint8_t* fetch_plane(const Plan& pl, const uint8_t* s
 }
 
 // Phase 2, a warp: an outlier-rich plane of more than four blocks, whose overflow part starts `place` units into the region.
-// `plane`: where it still lies, or null.
+// `plane`: where it still lies, or null; `ready`: its sizes, when the warp's scratch is about it already.
 template <int DT>
 __device__ __noinline__ void warp_plane_write(BlockCtl* c, uint64_t gp, const uint8_t* plane, uint32_t meta, uint32_t place, uint8_t* buf,
-                                              uint32_t* sal) {
+                                              uint32_t* sal, const SalientInfo* ready = nullptr) {
   const Plan& pl = c->pl;
   const Team team = make_warp_team(nullptr);
   if (!plane) plane = fetch_plane(pl, c->a.src, gp, buf, team.lane, 32u, true);
   __syncwarp();
-  const SalientInfo info = scratch_saved(pl) ? scratch_load(team, pl, c->d, gp, sal) : salient_measure<DT>(team, pl, plane, sal);
+  SalientInfo info;
+  if (ready) info = *ready;
+  else if (scratch_saved(pl)) info = scratch_load(team, pl, c->d, gp, sal);
+  else info = salient_measure<DT>(team, pl, plane, sal);
   __syncwarp();
   write_blockwise<DT>(team, pl, c->d, gp, plane, info, sal, meta >> 2, place);
   __syncwarp();
@@ -1275,9 +1286,25 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, WarpList* l, uint8_t* stag
     }
     if (lane == 0) l->base[i] = base;
   }
+  const bool owns = !small && !scratch_saved(pl);
+  if (owns && warp < (uint32_t)kWarps && l->own[warp] != kNoTile) {  // (a plane that has to be fetched again is not kept)
+    const bool held = lane < pl.nstage && c->held[lane] == l->own[warp] / pl.ppt;
+    if (!__any_sync(full, held) && lane == 0) l->own[warp] = kNoTile;
+  }
   for (uint32_t pass = 0; pass < 2u; ++pass) {
     __syncthreads();  // the places are known; the stages are free
     if (warp == (uint32_t)kWarps) continue;
+    if (owns && pass == 0u && l->own[warp] != kNoTile) {  // the plane that the warp's scratch is about comes first
+      const uint32_t gp = l->own[warp], np = min(l->planes, kListedPlanes);
+      for (uint32_t k = lane; k < ((np + 31u) & ~31u); k += 32u) {
+        const bool mine = k < np && l->of[k] != (uint8_t)kListed && l->tile[l->of[k]] * pl.ppt + l->lp[k] == gp;
+        const uint32_t m = __ballot_sync(full, mine);
+        if (!m) continue;
+        const uint32_t at = k - lane + (uint32_t)__ffs((int)m) - 1u, st = l->stage[l->of[at]];
+        warp_plane_write<DT>(c, gp, stages + (uint64_t)st * pl.stage_bytes + (uint64_t)l->lp[at] * pl.plane_bytes, l->meta[at], l->place[at],
+                             buf, sal, &l->own_info[warp]);
+      }
+    }
     for (;;) {
       uint32_t item = 0;
       if (lane == 0) item = atomicAdd(&l->handed[pass], 1u);
@@ -1288,6 +1315,7 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, WarpList* l, uint8_t* stag
         if (i == kListed) continue;
         const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
         const bool held = c->held[st] == tile;
+        if (owns && __any_sync(full, lane < (uint32_t)kWarps && l->own[lane & 7u] == tile * pl.ppt + lp)) continue;  // (its owner's)
         if (held == (pass == 0u))
           warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, held ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr,
                                l->meta[item], l->place[item], buf, sal);
@@ -1352,6 +1380,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
         s_ctl.held[s] = kNoTile;
         s_list.mask[s] = 0;
       }
+      for (uint32_t w = 0; w < (uint32_t)kWarps; ++w) s_list.own[w] = kNoTile;
       s_list.count = s_list.planes = s_list.handed[0] = s_list.handed[1] = 0;
     }
   }
