@@ -1013,16 +1013,6 @@ __device__ __forceinline__ SalientInfo scratch_load(const Team& t, const Plan& p
   return info;
 }
 
-// Huffman stage, warp-team kernel: which plane a warp's scratch is about (kNoTile: none), and its sizes; behind the scratch.
-struct OwnPlane {
-  uint32_t gp;
-  SalientInfo info;
-};
-static_assert(sizeof(OwnPlane) <= kOwnBytes, "room behind the scratch");
-__device__ __forceinline__ OwnPlane* own_plane(const Plan& pl, uint8_t* sal_base, uint32_t warp) {
-  return reinterpret_cast<OwnPlane*>(sal_base + (warp + 1u) * pl.sal_stride - kOwnBytes);
-}
-
 // The lane that holds the k-th set bit of m (m has more than k).
 __device__ __forceinline__ uint32_t nth_bit(uint32_t m, uint32_t k) {
   for (; k; --k) m &= m - 1u;
@@ -1088,13 +1078,7 @@ __device__ __noinline__ void warp_tile_measure(BlockCtl* c, WarpList* l, uint8_t
       nraw += raw ? 1u : 0u;
       const uint32_t mt = __shfl_sync(full, meta, (int)src);
       if (lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
-      if (scratch_saved(pl)) {
-        if (c->d.fits) scratch_save(team, pl, c->d, p0 + lp, info, sal);
-      } else if (pl.entropy && lane == 0) {
-        OwnPlane* own = own_plane(pl, reinterpret_cast<uint8_t*>(sal), 0u);
-        own->gp = (uint32_t)(p0 + lp);
-        own->info = info;
-      }
+      if (c->d.fits && scratch_saved(pl)) scratch_save(team, pl, c->d, p0 + lp, info, sal);
       __syncwarp();
     }
   }
@@ -1152,18 +1136,15 @@ __device__ __forceinline__ uint8_t* fetch_plane(const Plan& pl, const uint8_t* s
 }
 
 // Phase 2, a warp: an outlier-rich plane of more than four blocks, whose overflow part starts `place` units into the region.
-// `plane`: where it still lies, or null; `ready`: its sizes, when the warp's scratch is about it already.
+// `plane`: where it still lies, or null.
 template <int DT>
 __device__ __noinline__ void warp_plane_write(BlockCtl* c, uint64_t gp, const uint8_t* plane, uint32_t meta, uint32_t place, uint8_t* buf,
-                                              uint32_t* sal, const SalientInfo* ready = nullptr) {
+                                              uint32_t* sal) {
   const Plan& pl = c->pl;
   const Team team = make_warp_team(nullptr);
   if (!plane) plane = fetch_plane(pl, c->a.src, gp, buf, team.lane, 32u, true);
   __syncwarp();
-  SalientInfo info;
-  if (ready) info = *ready;
-  else if (scratch_saved(pl)) info = scratch_load(team, pl, c->d, gp, sal);
-  else info = salient_measure<DT>(team, pl, plane, sal);
+  const SalientInfo info = scratch_saved(pl) ? scratch_load(team, pl, c->d, gp, sal) : salient_measure<DT>(team, pl, plane, sal);
   __syncwarp();
   write_blockwise<DT>(team, pl, c->d, gp, plane, info, sal, meta >> 2, place);
   __syncwarp();
@@ -1294,27 +1275,9 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, WarpList* l, uint8_t* stag
     }
     if (lane == 0) l->base[i] = base;
   }
-  const bool owns = pl.entropy && !scratch_saved(pl);
-  OwnPlane* own = own_plane(pl, sal_base, min(warp, (uint32_t)kWarps - 1u));
-  if (owns && warp < (uint32_t)kWarps && own->gp != kNoTile) {  // (a plane that has to be fetched again is not kept)
-    const bool held = lane < pl.nstage && c->held[lane] == own->gp / pl.ppt;
-    __syncwarp();
-    if (!__any_sync(full, held) && lane == 0) own->gp = kNoTile;
-  }
   for (uint32_t pass = 0; pass < 2u; ++pass) {
     __syncthreads();  // the places are known; the stages are free
     if (warp == (uint32_t)kWarps) continue;
-    if (owns && pass == 0u && own->gp != kNoTile) {  // the plane that the warp's scratch is about comes first
-      const uint32_t gp = own->gp, np = min(l->planes, kListedPlanes);
-      for (uint32_t k = lane; k < ((np + 31u) & ~31u); k += 32u) {
-        const bool mine = k < np && l->of[k] != (uint8_t)kListed && l->tile[l->of[k]] * pl.ppt + l->lp[k] == gp;
-        const uint32_t m = __ballot_sync(full, mine);
-        if (!m) continue;
-        const uint32_t at = k - lane + (uint32_t)__ffs((int)m) - 1u, st = l->stage[l->of[at]];
-        warp_plane_write<DT>(c, gp, stages + (uint64_t)st * pl.stage_bytes + (uint64_t)l->lp[at] * pl.plane_bytes, l->meta[at], l->place[at],
-                             buf, sal, &own->info);
-      }
-    }
     for (;;) {
       uint32_t item = 0;
       if (lane == 0) item = atomicAdd(&l->handed[pass], 1u);
@@ -1325,7 +1288,6 @@ __device__ __noinline__ void warp_phase2(BlockCtl* c, WarpList* l, uint8_t* stag
         if (i == kListed) continue;
         const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
         const bool held = c->held[st] == tile;
-        if (owns && __any_sync(full, lane < (uint32_t)kWarps && own_plane(pl, sal_base, lane & 7u)->gp == tile * pl.ppt + lp)) continue;  // (its owner's)
         if (held == (pass == 0u))
           warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, held ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr,
                                l->meta[item], l->place[item], buf, sal);
@@ -1373,7 +1335,6 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   const bool scan_on = pl.mode != kModeOff;
   uint32_t first_ticket = 0;
   // Everything that needs no global memory comes before the wait for the previous kernel, whose tail hides it.
-  if (pl.entropy && tid < (uint32_t)kWarps) own_plane(pl, smem + pl.sm_sal, tid)->gp = kNoTile;
   if (tid == 0) {
     for (uint32_t s = 0; s < nstage; ++s) {
       mbar_init(&s_full[s], 1);

@@ -21,7 +21,6 @@ constexpr uint32_t kClsNormal = 0, kClsSalient = 1, kClsRaw = 2;
 constexpr int kModeAuto = 0, kModeOff = 1, kModeAll = 2, kModeChannel = 3, kModeTensor = 4;
 constexpr int kF32 = 0, kBF16 = 1;
 constexpr int kMaxStages = 4;
-constexpr uint32_t kOwnBytes = 32;        // Huffman stage: behind the measuring scratch of a unit (see OwnPlane)
 constexpr float kMagicF = 12582912.0f;    // 1.5 * 2^23: fma(v, c, kMagicF) leaves rne(v*c) in the mantissa
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
