@@ -183,8 +183,8 @@ __device__ __forceinline__ uint32_t count_verbatim(const uint32_t (&codes)[16]) 
 // what counts for planes of few blocks (14 x 14, fp32, 67 outlier-rich planes of 16,384: 22.6 -> 13.7 us a call).
 //   code_at(i)  the lane's code byte of row i;  dense  the lane's block is one (the others take part with codes of 128)
 //   out, y0, x0 where the block's elements go
-// `locate` is told the number of verbatim elements of the lane's block (all lanes call it) and returns the payload offset
-// of the first.
+// `locate` is told the number of verbatim elements of the lane's block (all lanes call it) and says where in the payload the
+// first lies, or that the payload does not hold as many: their values are then not read.
 template <int DT, typename In, typename CodeAt, typename Locate>
 __device__ __forceinline__ void restore_columns(const In& in, CodeAt code_at, Locate locate, bool dense, float two_eps, float inv2e,
                                                 uint8_t* out, uint32_t H, uint32_t W, uint32_t y0, uint32_t x0) {
@@ -204,18 +204,18 @@ __device__ __forceinline__ void restore_columns(const In& in, CodeAt code_at, Lo
   float raw[8];
   int32_t kv[8];
   if (any) {
-    uint32_t o = locate(n);
+    uint32_t o = 0;
+    const bool held = locate(n, o);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const uint32_t at = o + (DT == kF32 ? 4u : 2u) * __popc(mask[i] & ((1u << j) - 1u));
       raw[i] = 0.0f;
-      if ((mask[i] >> j) & 1u) raw[i] = DT == kF32 ? __uint_as_float(in.ld32(at)) : bf16_bits_to_f32(in.ld16(at));
+      if (held && ((mask[i] >> j) & 1u)) raw[i] = DT == kF32 ? __uint_as_float(in.ld32(at)) : bf16_bits_to_f32(in.ld16(at));
       o += (DT == kF32 ? 4u : 2u) * __popc(mask[i]);
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) kv[i] = max(min(__float2int_rn(__fmul_rn(raw[i], inv2e)), 1 << 24), -(1 << 24));
   } else {
-    locate(0u);
 #pragma unroll
     for (int i = 0; i < 8; ++i) raw[i] = 0.0f, kv[i] = 0;
   }
@@ -414,17 +414,16 @@ __device__ __noinline__ bool decode_few(const Plan& pl, const FlatIn in, uint32_
     const float two_eps = __fmul_rn(2.0f, eps);
     restore_columns<DT>(
         in, [&](int i) { return in.ld8(o_codes + 64u * rank + 8u * i + j); },
-        [&](uint32_t n) {
+        [&](uint32_t n, uint32_t& o) {
           uint32_t first = 0;
           if (!FOUR) {
             const uint32_t n0 = __shfl_sync(full, n, 0), n1 = __shfl_sync(full, n, 8), n2 = __shfl_sync(full, n, 16);
             first = (q > 0u ? n0 : 0u) + (q > 1u ? n1 : 0u) + (q > 2u ? n2 : 0u);
           }
-          if (dense && first + n > n_out_d) {  // (reads stay within the payload)
-            ok = false;
-            return 0u;
-          }
-          return o_outl + e * first;
+          o = o_outl + e * first;
+          const bool held = first + n <= n_out_d;
+          if (dense && !held) ok = false;
+          return held;
         },
         dense, two_eps, __fdiv_rn(1.0f, two_eps), out, H, W, by * 8u, bx * 8u);
   }
