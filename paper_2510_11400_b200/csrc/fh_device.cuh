@@ -855,7 +855,8 @@ static __device__ __noinline__ bool scan_prefix(const Scan& s, uint32_t t, uint3
       own = vt & 0xFFFFFFFFull;
       mine = true;
     }
-    if ((uint32_t)(vp >> 32) == s.epoch && __all_sync(full, mine)) {
+    // (one vote of all lanes on the whole condition: another CTA may store the word between two lanes' loads of it)
+    if (__all_sync(full, mine && (uint32_t)(vp >> 32) == s.epoch)) {
       prefix = (uint32_t)((vp & 0xFFFFFFFFull) + warp_sum_u64(own));
       return true;
     }
