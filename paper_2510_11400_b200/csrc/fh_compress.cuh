@@ -315,7 +315,6 @@ __device__ __forceinline__ void cta_exit(const Plan& pl, const CompressArgs& a, 
     }
     st_relaxed(&a.sc->nsal, 0ull);
     st_relaxed(&a.sc->nraw, 0ull);
-    st_relaxed(&a.sc->done, 0ull);
     st_relaxed(&a.sc->queue, 0ull);
   }
   finalize(pl, a, d, now >> (2 * kExitBits), (uint32_t)(vs >> kExitBits), (uint32_t)(vr >> kExitBits), code);
@@ -339,6 +338,10 @@ __device__ __forceinline__ uint2 load_marker(const Dest& d, uint64_t plane) {
   const volatile uint32_t* e = reinterpret_cast<const volatile uint32_t*>(d.dst + 64 + 16ull * plane);
   return make_uint2(e[0], e[1]);
 }
+// ... the marker's word that links the planes a CTA keeps for itself (CTA-team kernels).
+__device__ __forceinline__ volatile uint32_t& marker_link(const Dest& d, uint64_t plane) {
+  return reinterpret_cast<volatile uint32_t*>(d.dst + 64 + 16ull * plane)[2];
+}
 
 // The block-wise path runs in two phases so that nothing in the streaming phase ever waits for another CTA.
 // Phase 1, while a tile lies in shared memory: its outlier-rich planes are measured, the tile publishes the
@@ -346,7 +349,7 @@ __device__ __forceinline__ uint2 load_marker(const Dest& d, uint64_t plane) {
 // taken again (they come from the L2 cache when the tensor is small), obtain their place from the scan -- every tile
 // before one has been published, or is about to be, by a CTA in phase 1 -- and the payloads are written.  Tiles put off
 // wait in `defer_next`: linked from the CTA's own list (entry [tile]: the tile listed before it), or, in the CTA-team
-// kernels, in a queue that all CTAs share (entry [n]: the n-th tile put off, plus one); an entry is returned to zero by
+// kernels, in a queue that all CTAs share (entry [n]: the n-th tile queued, plus one); an entry is returned to zero by
 // who takes it.  This block sits in shared memory: what the outlined functions of both phases need.
 constexpr uint32_t kNoTile = 0xFFFFFFFFu;
 struct BlockCtl {
@@ -355,11 +358,12 @@ struct BlockCtl {
   Dest d;
   uint32_t U[kMaxStages], C[kMaxStages], arr[kMaxStages];  // warp-team kernel, per stage: units, counts, warps done
   uint32_t base, ok;
-  uint32_t head;                                           // the tile this CTA listed last
+  uint32_t head;                                           // warp-team and generic kernel: the tile this CTA listed last
   uint32_t held[kMaxStages];                               // the tile each stage buffer holds
   uint32_t next, ahead;                                    // CTA-team kernels, phase 2: the plane in hand, the one after it
   uint32_t own, own_stage, own_held;                       // ... the plane the measuring scratch is about (kNoTile: none), its stage, whether it still lies there ...
   SalientInfo own_info;                                    // ... and its sizes
+  uint32_t kept;                                           // ... the first of the planes the CTA keeps for itself (kNoTile: none)
 };
 
 // Warp-team kernel: what the tiles in the stages have gathered so far, and the tiles put off, as far as there is room (the
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(kThreads) compress_generic(const Plan pl, cons
   if (tid == 0 && pl.mode != kModeOff) {  // (before the wait for the previous kernel, whose tail hides it)
     s_ctl.pl = pl;
     s_ctl.a = a;
-    s_ctl.head = s_ctl.own = kNoTile;
+    s_ctl.head = kNoTile;
   }
   dep_wait();     // the previous kernel on the stream has completed
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
@@ -1346,7 +1350,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     if (scan_on) {
       s_ctl.pl = pl;
       s_ctl.a = a;
-      s_ctl.head = s_ctl.own = kNoTile;
+      s_ctl.head = kNoTile;
       for (uint32_t s = 0; s < nstage; ++s) {
         s_ctl.U[s] = s_ctl.C[s] = s_ctl.arr[s] = 0;
         s_ctl.held[s] = kNoTile;
@@ -1543,44 +1547,45 @@ __device__ __noinline__ void cta_tile_measure(BlockCtl* c, double* red, const ui
 // The queue of planes put off (CTA-team kernels).  Which CTA has measured how many outlier-rich planes is a matter of
 // chance -- none to twice the mean --, so phase 2 deals them out anew: with every CTA writing its own, the bf16 112 x 112
 // tensor with every eighth channel outlier-rich spent 168 to 335 us of 338 in phase 2, depending on the CTA.
+// One word counts the planes queued (high half) and the entries claimed (low half).  A CTA that claims when all entries are
+// taken leaves; it never waits for entries to come, since those who would queue them may be CTAs that have not started yet
+// and find no room while it stays.  The entry it has claimed is then nobody's: whoever would queue that one sees so from the
+// same word and keeps the plane for itself, linked to the others that it keeps through the third word of the planes' markers.
+//
 // One thread, behind a barrier that follows the measuring: plane `tile`, of `stage`, is put off.  `held`: no other plane
 // will be loaded there.
 static __device__ __noinline__ void queue_push(BlockCtl* c, uint32_t tile, uint32_t stage, bool held) {
   if (!c->d.fits) return;
-  c->head = tile;  // (the CTA has put something off)
   // the CTA keeps its last plane, whose scratch lies ready; the one before joins the queue
   const uint32_t before = c->own;
   c->own = tile;
   c->own_stage = stage;
   c->own_held = held;
   if (before == kNoTile) return;
-  const uint32_t n = (uint32_t)(atomicAdd(&c->a.sc->queue, 1ull << 32) >> 32);
+  const unsigned long long q = atomicAdd(&c->a.sc->queue, 1ull << 32);
+  const uint32_t n = (uint32_t)(q >> 32);
+  if ((uint32_t)q > n) {
+    marker_link(c->d, before) = c->kept;
+    c->kept = before;
+    return;
+  }
   __threadfence();  // marker and saved scratch, of all threads, before the entry
   st_relaxed32(&c->a.defer_next[n], before + 1u);
 }
 constexpr uint32_t kPending = 0xFFFFFFFEu;
-// One thread: the plane of queue entry n, which is this CTA's; kNoTile when there will be none -- every CTA has finished
-// phase 1 and the queue is shorter --, kPending (unless `wait`) when it is not known yet.  A CTA in phase 1 waits for
-// nobody, so the wait ends; it is bounded all the same.
+// One thread: the plane of queue entry n, which this CTA has claimed.  It has been counted, so its place is about to be
+// filled by a CTA that is running; unless `wait`, kPending when it is not yet.  The wait is bounded all the same.
 static __device__ __noinline__ uint32_t queue_entry(BlockCtl* c, uint32_t n, bool wait) {
   const CompressArgs& a = c->a;
-  if (n >= c->pl.ntiles) return kNoTile;
   for (uint32_t k = 0; k < a.scan.polls; ++k) {
-    uint32_t e = ld_relaxed32(&a.defer_next[n]);
-    if (!e && wait) {
-      const unsigned long long left = ld_relaxed(&a.sc->exited), in2 = ld_relaxed(&a.sc->done);
-      __threadfence();
-      const uint32_t quiet = ((uint32_t)left & kExitMask) - ((uint32_t)(left >> kExitBits) & kExitMask);  // left with nothing
-      if (quiet + (uint32_t)in2 == gridDim.x && n >= (uint32_t)(ld_relaxed(&a.sc->queue) >> 32)) return kNoTile;
-      e = ld_relaxed32(&a.defer_next[n]);
-    }
+    const uint32_t e = ld_relaxed32(&a.defer_next[n]);
     if (e) {
       st_relaxed32(&a.defer_next[n], 0u);
       __threadfence();
       return e - 1u;
     }
     if (!wait) return kPending;
-    __nanosleep(200);
+    __nanosleep(100);
   }
   report_error(a, kErrTimeout);
   return kNoTile;
@@ -1611,21 +1616,18 @@ __device__ __forceinline__ void plane_load(const Plan& pl, const uint8_t* src, u
   bulk_g2s(stage, src + a0, (uint32_t)(whole - a0), bar);
 }
 
-// Phase 2 of the CTA-team kernels: the CTA's own plane, then planes from the queue until it is empty.  While one is written, the next is claimed and
-// fetched into the other stage.
+// Phase 2 of the CTA-team kernels: the CTA's own plane, then planes from the queue until it is empty, then those that the CTA
+// had to keep.  While one is written, the next is claimed and fetched into the other stage.
 template <int DT>
 __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal) {
   const Plan& pl = c->pl;
   const Team team = make_cta_team(blockDim.x, red);
   const uint32_t tid = threadIdx.x;
   const bool claims = tid == blockDim.x - 32u;  // (not in the warp that looks up places, where there are two)
-  uint32_t mine = 0, cur = 0;
-  auto claim = [&]() { mine = (uint32_t)atomicAdd(&c->a.sc->queue, 1ull); };
-  if (claims) {
-    __threadfence();  // the CTA's entries before the note that it has finished phase 1
-    atomicAdd(&c->a.sc->done, 1ull);
-    c->next = c->own;
-  }
+  unsigned long long claim = 0;  // the queue's word before this CTA's latest claim
+  bool more = true;
+  uint32_t cur = 0;
+  if (claims) c->next = c->own;
   bool kept = true;  // the plane in hand is the CTA's own: its scratch lies ready
   cur = c->own_stage;
   for (bool fetched = c->own_held != 0u;;) {
@@ -1634,7 +1636,7 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     if (tile >= pl.ntiles) break;  // (the same for every thread)
     uint8_t* stage = stages + (uint64_t)cur * pl.stage_bytes;
     if (!fetched) fetch_start(pl, c->a.src, tile, stage);
-    if (claims) claim();
+    if (claims && more) claim = atomicAdd(&c->a.sc->queue, 1ull);
     const uint2 mk = load_marker(c->d, tile);  // units, class and count
     if (tid < 32u) {
       bool ok = true;
@@ -1650,7 +1652,15 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     const bool saved = scratch_saved(pl);
     if (kept) info = c->own_info;
     else if (saved) info = scratch_load(team, pl, c->d, tile, sal);
-    if (claims) c->ahead = queue_entry(c, mine, false);
+    if (claims) {
+      more = more && (uint32_t)claim < (uint32_t)(claim >> 32);
+      if (more) {
+        c->ahead = queue_entry(c, (uint32_t)claim, false);
+      } else {
+        c->ahead = c->kept;
+        if (c->kept != kNoTile) c->kept = marker_link(c->d, c->kept);
+      }
+    }
     fetch_wait();
     __syncthreads();
     const uint32_t ahead = c->ahead;
@@ -1660,7 +1670,7 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     if (!saved && !kept) info = salient_measure<DT>(team, pl, plane, sal);
     kept = false;
     if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, plane, info, sal, mk.y >> 2, c->base);
-    if (claims) c->next = ahead == kPending ? queue_entry(c, mine, true) : ahead;
+    if (claims) c->next = ahead == kPending ? queue_entry(c, (uint32_t)claim, true) : ahead;
     fetch_wait();
     if (fetched) cur ^= 1u;
   }
@@ -1669,8 +1679,7 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
 template <int DT>
 __device__ __forceinline__ void cta_finish(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal, bool aborted) {
   __syncthreads();
-  if (c->head != kNoTile && !aborted) cta_phase2<DT>(c, red, stages, sal);
-  else if (threadIdx.x == 0 && has_totals(*cta_totals())) atomicAdd(&c->a.sc->done, 1ull);  // (see queue_entry)
+  if (c->own != kNoTile && !aborted) cta_phase2<DT>(c, red, stages, sal);
 }
 
 template <int DT>
@@ -1751,7 +1760,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
   if (tid == 0 && scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
     s_ctl.pl = pl;
     s_ctl.a = a;
-    s_ctl.head = s_ctl.own = kNoTile;
+    s_ctl.own = s_ctl.kept = kNoTile;
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
@@ -1957,7 +1966,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     if (scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
       s_ctl.pl = pl;
       s_ctl.a = a;
-      s_ctl.head = s_ctl.own = kNoTile;
+      s_ctl.own = s_ctl.kept = kNoTile;
     }
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on

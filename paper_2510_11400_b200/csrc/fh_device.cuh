@@ -73,10 +73,9 @@ struct Scratch {
   unsigned long long status;     // device error code (atomicMax)
   unsigned long long nsal, nraw; // outlier-rich planes of either kind (see cta_exit)
   unsigned long long reserved;
-  unsigned long long queue;      // CTA-team kernels: planes put off, entries claimed (high half, low half)
-  unsigned long long done;       // ... CTAs that have finished phase 1 and either work on the queue or have an error to report
+  unsigned long long queue;      // CTA-team kernels: planes queued, entries claimed (high half, low half; see queue_push)
 };
-static_assert(sizeof(Scratch) == 72, "Scratch layout");
+static_assert(sizeof(Scratch) == 64, "Scratch layout");
 constexpr uint32_t kScratchHeadBytes = 256;  // the header, padded
 
 // (uint64)(int64) fh_status of a device error code.

@@ -3,8 +3,9 @@ lists, planes that pass through the queue of the CTA-team kernels (measurements 
 Huffman code, or too large for it), statistics over channels in pieces and over many small planes, from call to call."""
 import pytest
 
+from oracle import fho
 from paper_2510_11400_b200 import api, synth
-from tests.test_gpu_parity import full_parity
+from tests.test_gpu_parity import full_parity, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +32,26 @@ def test_parity_with_every_plane_put_off(shape, dtype, kind, kw):
 def test_parity_of_channel_statistics(mode, dtype):
     for shape in [(5, 3, 150, 151), (3, 700, 3, 3), (4, 33, 64, 72), (2, 17, 45, 47), (9, 1, 1, 1), (3, 700, 8, 8)]:
         full_parity(synth.TensorSpec("t", shape, dtype, "spiky_relu", 42), bits=4, salient_mode=mode)
+
+
+def test_parity_of_overlapping_calls_on_two_streams():
+    """Kernels with planes put off on two streams at once, each with more CTAs than find room beside the other's: every call
+    must come through with the bytes of a call alone."""
+    import torch
+    calls, p = [], api.default_params(bits=4, salient_mode=api.FH_SALIENT_ALL)
+    for i, (shape, dtype) in enumerate([((2, 350, 112, 112), synth.BF16), ((2, 700, 56, 56), synth.F32)]):
+        raw = synth.make(synth.TensorSpec("t", shape, dtype, "spiky_relu", 43 + i))
+        st, buf, total = fho.compress(raw, fho.desc(shape, dtype), fho.params(bits=4, salient_mode=fho.ALL))
+        assert st == fho.OK
+        d = api.desc(shape, dtype)
+        dst = [torch.zeros(api.compressed_bytes(d, p, 1), dtype=torch.uint8, device="cuda") for _ in range(6)]
+        calls.append((to_dev(raw), d, buf, total, dst, torch.zeros(6, 2, dtype=torch.int64, device="cuda"), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for k in range(6):
+        for x, d, _, _, dst, out2, stream in calls:
+            assert api.fh_compress(d, p, x, dst[k], out2[k], stream=stream) == api.FH_OK
+    torch.cuda.synchronize()
+    for _, _, buf, total, dst, out2, _ in calls:
+        want = to_dev(buf)
+        assert out2.tolist() == [[total, api.FH_OK]] * 6
+        assert all(torch.equal(t[:total], want) for t in dst)
