@@ -315,6 +315,7 @@ __device__ __forceinline__ void cta_exit(const Plan& pl, const CompressArgs& a, 
     }
     st_relaxed(&a.sc->nsal, 0ull);
     st_relaxed(&a.sc->nraw, 0ull);
+    st_relaxed(&a.sc->done, 0ull);
     st_relaxed(&a.sc->queue, 0ull);
   }
   finalize(pl, a, d, now >> (2 * kExitBits), (uint32_t)(vs >> kExitBits), (uint32_t)(vr >> kExitBits), code);
@@ -338,10 +339,6 @@ __device__ __forceinline__ uint2 load_marker(const Dest& d, uint64_t plane) {
   const volatile uint32_t* e = reinterpret_cast<const volatile uint32_t*>(d.dst + 64 + 16ull * plane);
   return make_uint2(e[0], e[1]);
 }
-// ... the marker's word that links the planes a CTA keeps for itself (CTA-team kernels).
-__device__ __forceinline__ volatile uint32_t& marker_link(const Dest& d, uint64_t plane) {
-  return reinterpret_cast<volatile uint32_t*>(d.dst + 64 + 16ull * plane)[2];
-}
 
 // The block-wise path runs in two phases so that nothing in the streaming phase ever waits for another CTA.
 // Phase 1, while a tile lies in shared memory: its outlier-rich planes are measured, the tile publishes the
@@ -363,7 +360,6 @@ struct BlockCtl {
   uint32_t next, ahead;                                    // CTA-team kernels, phase 2: the plane in hand, the one after it
   uint32_t own, own_stage, own_held;                       // ... the plane the measuring scratch is about (kNoTile: none), its stage, whether it still lies there ...
   SalientInfo own_info;                                    // ... and its sizes
-  uint32_t kept;                                           // ... the first of the planes the CTA keeps for itself (kNoTile: none)
 };
 
 // Warp-team kernel: what the tiles in the stages have gathered so far, and the tiles put off, as far as there is room (the
@@ -1547,13 +1543,15 @@ __device__ __noinline__ void cta_tile_measure(BlockCtl* c, double* red, const ui
 // The queue of planes put off (CTA-team kernels).  Which CTA has measured how many outlier-rich planes is a matter of
 // chance -- none to twice the mean --, so phase 2 deals them out anew: with every CTA writing its own, the bf16 112 x 112
 // tensor with every eighth channel outlier-rich spent 168 to 335 us of 338 in phase 2, depending on the CTA.
-// One word counts the planes queued (high half) and the entries claimed (low half).  A CTA that claims when all entries are
-// taken leaves; it never waits for entries to come, since those who would queue them may be CTAs that have not started yet
-// and find no room while it stays.  The entry it has claimed is then nobody's: whoever would queue that one sees so from the
-// same word and keeps the plane for itself, linked to the others that it keeps through the third word of the planes' markers.
+// A CTA that has claimed an entry that is not there yet waits for it until no CTA can queue another plane.  Those that can
+// are CTAs that have started, as the ticket word counts them along with its tickets: whoever starts once the tickets are
+// used up gets no tile.  It must not wait for CTAs that have not started, which may find no room while it stays (kernels on
+// other streams hold the rest of the GPU).  Leaving at once when the queue is empty, instead of waiting, left the last planes
+// to the CTAs that had measured them: 128 x 144 bf16 planes of 56 x 56, 125 -> 141 us.
 //
 // One thread, behind a barrier that follows the measuring: plane `tile`, of `stage`, is put off.  `held`: no other plane
 // will be loaded there.
+constexpr unsigned long long kStarted = 1ull << 32;  // added to the ticket word with a CTA's first request
 static __device__ __noinline__ void queue_push(BlockCtl* c, uint32_t tile, uint32_t stage, bool held) {
   if (!c->d.fits) return;
   // the CTA keeps its last plane, whose scratch lies ready; the one before joins the queue
@@ -1562,30 +1560,34 @@ static __device__ __noinline__ void queue_push(BlockCtl* c, uint32_t tile, uint3
   c->own_stage = stage;
   c->own_held = held;
   if (before == kNoTile) return;
-  const unsigned long long q = atomicAdd(&c->a.sc->queue, 1ull << 32);
-  const uint32_t n = (uint32_t)(q >> 32);
-  if ((uint32_t)q > n) {
-    marker_link(c->d, before) = c->kept;
-    c->kept = before;
-    return;
-  }
+  const uint32_t n = (uint32_t)(atomicAdd(&c->a.sc->queue, 1ull << 32) >> 32);
   __threadfence();  // marker and saved scratch, of all threads, before the entry
   st_relaxed32(&c->a.defer_next[n], before + 1u);
 }
 constexpr uint32_t kPending = 0xFFFFFFFEu;
-// One thread: the plane of queue entry n, which this CTA has claimed.  It has been counted, so its place is about to be
-// filled by a CTA that is running; unless `wait`, kPending when it is not yet.  The wait is bounded all the same.
+// One thread: the plane of queue entry n, which is this CTA's; kNoTile when there will be none -- every CTA that has started
+// has finished phase 1 and the queue is shorter --, kPending (unless `wait`) when it is not known yet.  A CTA in phase 1 waits
+// for nobody, so the wait ends; it is bounded all the same.
 static __device__ __noinline__ uint32_t queue_entry(BlockCtl* c, uint32_t n, bool wait) {
   const CompressArgs& a = c->a;
+  if (n >= c->pl.ntiles) return kNoTile;
   for (uint32_t k = 0; k < a.scan.polls; ++k) {
-    const uint32_t e = ld_relaxed32(&a.defer_next[n]);
+    uint32_t e = ld_relaxed32(&a.defer_next[n]);
+    if (!e && wait) {
+      const unsigned long long left = ld_relaxed(&a.sc->exited), in2 = ld_relaxed(&a.sc->done);
+      __threadfence();  // (those that have finished before those that have started: the latter can only be more)
+      const uint32_t quiet = ((uint32_t)left & kExitMask) - ((uint32_t)(left >> kExitBits) & kExitMask);  // left with nothing
+      const uint32_t started = (uint32_t)(ld_relaxed(&a.sc->ticket[a.parity]) / kStarted);
+      if (quiet + (uint32_t)in2 == started && n >= (uint32_t)(ld_relaxed(&a.sc->queue) >> 32)) return kNoTile;
+      e = ld_relaxed32(&a.defer_next[n]);
+    }
     if (e) {
       st_relaxed32(&a.defer_next[n], 0u);
       __threadfence();
       return e - 1u;
     }
     if (!wait) return kPending;
-    __nanosleep(100);
+    __nanosleep(200);
   }
   report_error(a, kErrTimeout);
   return kNoTile;
@@ -1616,18 +1618,21 @@ __device__ __forceinline__ void plane_load(const Plan& pl, const uint8_t* src, u
   bulk_g2s(stage, src + a0, (uint32_t)(whole - a0), bar);
 }
 
-// Phase 2 of the CTA-team kernels: the CTA's own plane, then planes from the queue until it is empty, then those that the CTA
-// had to keep.  While one is written, the next is claimed and fetched into the other stage.
+// Phase 2 of the CTA-team kernels: the CTA's own plane, then planes from the queue until it is empty.  While one is written,
+// the next is claimed and fetched into the other stage.
 template <int DT>
 __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal) {
   const Plan& pl = c->pl;
   const Team team = make_cta_team(blockDim.x, red);
   const uint32_t tid = threadIdx.x;
   const bool claims = tid == blockDim.x - 32u;  // (not in the warp that looks up places, where there are two)
-  unsigned long long claim = 0;  // the queue's word before this CTA's latest claim
-  bool more = true;
-  uint32_t cur = 0;
-  if (claims) c->next = c->own;
+  uint32_t mine = 0, cur = 0;
+  auto claim = [&]() { mine = (uint32_t)atomicAdd(&c->a.sc->queue, 1ull); };
+  if (claims) {
+    __threadfence();  // the CTA's entries before the note that it has finished phase 1
+    atomicAdd(&c->a.sc->done, 1ull);
+    c->next = c->own;
+  }
   bool kept = true;  // the plane in hand is the CTA's own: its scratch lies ready
   cur = c->own_stage;
   for (bool fetched = c->own_held != 0u;;) {
@@ -1636,7 +1641,7 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     if (tile >= pl.ntiles) break;  // (the same for every thread)
     uint8_t* stage = stages + (uint64_t)cur * pl.stage_bytes;
     if (!fetched) fetch_start(pl, c->a.src, tile, stage);
-    if (claims && more) claim = atomicAdd(&c->a.sc->queue, 1ull);
+    if (claims) claim();
     const uint2 mk = load_marker(c->d, tile);  // units, class and count
     if (tid < 32u) {
       bool ok = true;
@@ -1652,15 +1657,7 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     const bool saved = scratch_saved(pl);
     if (kept) info = c->own_info;
     else if (saved) info = scratch_load(team, pl, c->d, tile, sal);
-    if (claims) {
-      more = more && (uint32_t)claim < (uint32_t)(claim >> 32);
-      if (more) {
-        c->ahead = queue_entry(c, (uint32_t)claim, false);
-      } else {
-        c->ahead = c->kept;
-        if (c->kept != kNoTile) c->kept = marker_link(c->d, c->kept);
-      }
-    }
+    if (claims) c->ahead = queue_entry(c, mine, false);
     fetch_wait();
     __syncthreads();
     const uint32_t ahead = c->ahead;
@@ -1670,7 +1667,7 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     if (!saved && !kept) info = salient_measure<DT>(team, pl, plane, sal);
     kept = false;
     if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, plane, info, sal, mk.y >> 2, c->base);
-    if (claims) c->next = ahead == kPending ? queue_entry(c, (uint32_t)claim, true) : ahead;
+    if (claims) c->next = ahead == kPending ? queue_entry(c, mine, true) : ahead;
     fetch_wait();
     if (fetched) cur ^= 1u;
   }
@@ -1680,6 +1677,7 @@ template <int DT>
 __device__ __forceinline__ void cta_finish(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal, bool aborted) {
   __syncthreads();
   if (c->own != kNoTile && !aborted) cta_phase2<DT>(c, red, stages, sal);
+  else if (threadIdx.x == 0 && has_totals(*cta_totals())) atomicAdd(&c->a.sc->done, 1ull);  // (see queue_entry)
 }
 
 template <int DT>
@@ -1755,12 +1753,12 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
     *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
     // (the ticket counter of this call was returned to zero by the call before the previous one, which had
     // completed before the previous kernel let this one start)
-    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
+    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + nstage);
   }
   if (tid == 0 && scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
     s_ctl.pl = pl;
     s_ctl.a = a;
-    s_ctl.own = s_ctl.kept = kNoTile;
+    s_ctl.own = kNoTile;
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
@@ -1777,7 +1775,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
     }
   };
   if (tid == 0) {  // the first loads before anything else
-    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)nstage);
+    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + nstage);
     for (uint32_t s = 0; s < nstage; ++s) issue(s);
   }
   const Dest d = make_dest(pl, a);
@@ -1962,11 +1960,11 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     s_abort = 0;
     s_count[0] = s_count[1] = 0;
     *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
-    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)early);
+    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + early);
     if (scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
       s_ctl.pl = pl;
       s_ctl.a = a;
-      s_ctl.own = s_ctl.kept = kNoTile;
+      s_ctl.own = kNoTile;
     }
   }
   dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
@@ -1981,7 +1979,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     }
   };
   if (tid == 0) {  // the first loads before anything else
-    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)early);
+    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + early);
     issue(0);
     issue(1);
   }

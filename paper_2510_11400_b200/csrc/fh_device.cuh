@@ -68,14 +68,16 @@ struct Plan {
 // placement of overflow parts (see "Placement scan" below).  Everything in the header that a call changes
 // is returned to zero by the last CTA of its kernel.
 struct Scratch {
-  unsigned long long ticket[2];  // next tile; consecutive compress calls on a stream alternate between the two
+  unsigned long long ticket[2];  // next tile (low half; high half, CTA-team kernels: CTAs that have started); consecutive
+                                 // compress calls on a stream alternate between the two
   unsigned long long exited;     // CTAs that have left the running kernel
   unsigned long long status;     // device error code (atomicMax)
   unsigned long long nsal, nraw; // outlier-rich planes of either kind (see cta_exit)
   unsigned long long reserved;
-  unsigned long long queue;      // CTA-team kernels: planes queued, entries claimed (high half, low half; see queue_push)
+  unsigned long long queue;      // CTA-team kernels: planes put off, entries claimed (high half, low half)
+  unsigned long long done;       // ... CTAs that have finished phase 1 and either work on the queue or have an error to report
 };
-static_assert(sizeof(Scratch) == 64, "Scratch layout");
+static_assert(sizeof(Scratch) == 72, "Scratch layout");
 constexpr uint32_t kScratchHeadBytes = 256;  // the header, padded
 
 // (uint64)(int64) fh_status of a device error code.
