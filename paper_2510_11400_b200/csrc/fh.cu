@@ -285,9 +285,9 @@ struct StreamScratch {
   uint32_t prev_groups = 0;              // groups of 32 tiles the last of them used (the next one clears that set)
   uint32_t* plane_nout = nullptr;        // channel-wide three-sigma mode: per-plane counts ...
   size_t pn_cap = 0;
-  fh::ChanStat* chan = nullptr;          // ... and per-channel statistics: two sets, which alternate between calls
+  fh::ChanStat* chan = nullptr;          // ... and per-channel statistics, zero between calls
   size_t chan_cap = 0;
-  uint32_t chan_calls = 0, chan_used[2] = {0, 0};  // which set is next; entries of a set that may not be zero
+  bool chan_dirty = false;               // they may not be zero: the next call that uses them clears them first
   SchedSpace* sched = nullptr;           // schedule runner: the workspace that is not in use, if any
 };
 // tile words | two sets of group sums | group prefixes | tile links (32-bit)
@@ -396,11 +396,12 @@ int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels, cudaSt
       s->chan = nullptr;
       s->chan_cap = 0;
     }
-    if (cudaMalloc(&s->chan, 2 * cap * sizeof(fh::ChanStat)) != cudaSuccess) return FH_ERR_CUDA;
-    if (cudaMemsetAsync(s->chan, 0, 2 * cap * sizeof(fh::ChanStat), stream) != cudaSuccess) return FH_ERR_CUDA;
+    if (cudaMalloc(&s->chan, cap * sizeof(fh::ChanStat)) != cudaSuccess) return FH_ERR_CUDA;
     s->chan_cap = cap;
-    s->chan_used[0] = s->chan_used[1] = 0;
+    s->chan_dirty = true;
   }
+  if (s->chan_dirty && cudaMemsetAsync(s->chan, 0, s->chan_cap * sizeof(fh::ChanStat), stream) != cudaSuccess) return FH_ERR_CUDA;
+  s->chan_dirty = true;  // (until the whole call is launched)
   return FH_OK;
 }
 
@@ -435,28 +436,26 @@ int enqueue_compress(const fh_tensor_desc* desc, const fh_params* params, const 
   a.early_ticket = 1;
   rc = next_call(&s->calls, pl.mode == FH_SALIENT_OFF ? nullptr : s->scan, s->tile_cap, s, (pl.ntiles + 31u) / 32u, stream, &a);
   if (rc != FH_OK) return rc;
-  a.chan_nout = nullptr;
-  a.plane_nout = nullptr;
   if (pl.mode >= fh::kModeChannel) {  // statistics per channel over the batch, or over the tensor: three passes ahead of the streaming kernel
     rc = get_channel_scratch(s, pl.P, pl.C, stream);
     if (rc != FH_OK) return rc;
-    const uint32_t set = s->chan_calls++ & 1u;
     fh::ChannelArgs ca = {};
     ca.src = (const uint8_t*)d_src;
-    ca.chan = s->chan + set * s->chan_cap;
-    ca.next = s->chan + (1u - set) * s->chan_cap;
-    ca.clear = s->chan_used[1u - set];
-    s->chan_used[set] = pl.mode == fh::kModeTensor ? 1u : pl.C;
-    s->chan_used[1u - set] = 0;
+    ca.chan = s->chan;
     ca.plane_nout = s->plane_nout;
     ca.inv_nhw = 1.0 / ((double)(pl.mode == fh::kModeTensor ? pl.P : pl.N) * (double)pl.HW);
     rc = fh::launch_channel_passes(pl, ca, stream);
     if (rc != FH_OK) return rc;
     g_launches.fetch_add(3);
-    a.chan_nout = reinterpret_cast<const unsigned long long*>(ca.chan) + 3;
+    a.chan_stats = reinterpret_cast<unsigned long long*>(s->chan);
+    // one CTA returns 4,096 channels' statistics to zero in about a microsecond; more are left to a memset in the next call
+    const uint32_t used = pl.mode == fh::kModeTensor ? 1u : pl.C;
+    a.chan_words = used <= 4096u ? (uint32_t)(sizeof(fh::ChanStat) / 8) * used : 0u;
     a.plane_nout = s->plane_nout;
   }
-  return launch_compress(pl, v, a, stream);
+  rc = launch_compress(pl, v, a, stream);
+  if (rc == FH_OK && a.chan_words) s->chan_dirty = false;
+  return rc;
 }
 
 int enqueue_decompress(const void* d_src, size_t src_bytes, const fh_tensor_desc* expect, void* d_dst,
@@ -809,8 +808,6 @@ int fh_compress_static(const fh_tensor_desc* desc, const fh_params* params, cons
   a.early_ticket = 0;  // the counters are cleared by the memset just enqueued: nothing may touch them before it
   rc = next_call(&g_static_calls[dev], scan, cap, nullptr, 0, stream, &a);
   if (rc != FH_OK) return rc;
-  a.chan_nout = nullptr;
-  a.plane_nout = nullptr;
   std::lock_guard<std::mutex> lock2(g_mu);  // the launch helpers keep their occupancy cache under g_mu
   return launch_compress(pl, v, a, stream);
 }

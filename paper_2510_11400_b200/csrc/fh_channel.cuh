@@ -10,8 +10,8 @@
 //   pass 2: thresholds from the sums; outliers per plane (kept for the plane table) and per channel.
 // The streaming kernel then reads a plane's class from its channel's count, so the tensor is read four times; what fits
 // the L2 cache comes from there from the second time on.  A lane has 64 bytes in flight; the
-// passes follow one another by programmatic launch; no memset between them (pass 0 clears the statistics that the call
-// after this one will use).  Element by element with a warp per plane the three took 162 us for 32 x 96 bf16 planes of
+// passes follow one another by programmatic launch; no memset between them (the streaming kernel's last CTA returns the
+// statistics to zero).  Element by element with a warp per plane the three took 162 us for 32 x 96 bf16 planes of
 // 112 x 112 (77 MB) and 27 us for 32 x 960 of 7 x 7; now 67 and 17.
 #pragma once
 
@@ -75,9 +75,6 @@ __global__ void __launch_bounds__(kThreads, 4) channel_pass(const Plan pl, const
   const uint64_t items = pl.P * pieces, step = (uint64_t)gridDim.x * (kThreads / tt);
   dep_trigger();
   dep_wait();
-  if (PASS == 0)
-    for (uint32_t k = blockIdx.x * kThreads + threadIdx.x; k < 4u * a.clear; k += gridDim.x * kThreads)
-      reinterpret_cast<unsigned long long*>(a.next)[k] = 0ull;
   for (uint64_t base = (uint64_t)blockIdx.x * (kThreads / tt); base < items; base += step) {  // (the warp stays together)
     const uint64_t item = base + threadIdx.x / tt;
     const bool there = item < items;

@@ -30,7 +30,7 @@ __device__ __forceinline__ uint32_t channel_class(const Plan& pl, const Compress
   n_out = a.plane_nout[gp];
   if (pl.mode == kModeTensor)
     return (uint64_t)n_out * pl.rho_den > (uint64_t)pl.rho_num * pl.HW ? kClsSalient : kClsNormal;
-  const unsigned long long total = a.chan_nout[(gp % pl.C) * 4ull];
+  const unsigned long long total = a.chan_stats[(gp % pl.C) * 4ull + 3ull];  // (see ChanStat)
   return total * pl.rho_den > (unsigned long long)pl.rho_num * pl.N * pl.HW ? kClsSalient : kClsNormal;
 }
 
@@ -264,8 +264,8 @@ __device__ __forceinline__ void finalize(const Plan& pl, const CompressArgs& a, 
   if (a.d_off_out) *a.d_off_out = code == kErrNone ? d.off_in + ((total + 255ull) & ~255ull) : (~0ull >> 1);
 }
 
-// Last step of every CTA: the last CTA to leave returns the group sums of the previous call's placement scan and
-// the hand-out counters to zero and finishes the container.
+// Last step of every CTA: the last CTA to leave returns the group sums of the previous call's placement scan, the
+// hand-out counters and the statistics of the channel- and tensor-wide modes to zero and finishes the container.
 // The exit word carries the CTAs that have left, how many of them had something to add, and the overflow units of all:
 //   CTAs | CTAs with something << 13 | units << 26
 // The numbers of planes go the same way, each next to a count of the CTAs that added to it, by which the last CTA knows
@@ -295,6 +295,7 @@ __device__ __forceinline__ void cta_exit(const Plan& pl, const CompressArgs& a, 
   if (!*s_last) return;
   if (pl.mode != kModeOff)
     for (uint32_t k = threadIdx.x; k < a.scan.clear_groups; k += blockDim.x) a.scan.grp_clear[k] = 0ull;
+  for (uint32_t k = threadIdx.x; k < a.chan_words; k += blockDim.x) a.chan_stats[k] = 0ull;  // (every CTA has read what it needed)
   if (threadIdx.x != 0) return;
   // (what follows is read by later kernels only, which start work after this one has completed: no fence)
   st_relaxed(&a.sc->ticket[a.parity], 0ull);

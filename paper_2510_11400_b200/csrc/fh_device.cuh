@@ -920,8 +920,10 @@ struct CompressArgs {
   uint32_t* defer_next;                 // one word per tile, zero between calls: tiles put off (see BlockCtl)
   uint32_t parity;                      // which of the two ticket counters this call uses
   uint32_t early_ticket;                // 1: tiles may be requested before the previous kernel on the stream has completed
-  // channel-wide three-sigma mode: per-channel outlier counts and per-plane counts from the statistics passes
-  const unsigned long long* chan_nout;  // stride: 4 words (see ChanStat)
+  // channel- and tensor-wide three-sigma modes: the statistics passes' results per channel (ChanStat, four words each),
+  // the words that the call's last CTA returns to zero, and outlier counts per plane
+  unsigned long long* chan_stats;
+  uint32_t chan_words;
   const uint32_t* plane_nout;
 };
 
@@ -947,8 +949,6 @@ static_assert(sizeof(ChanStat) == 32, "ChanStat layout");
 struct ChannelArgs {
   const uint8_t* src;
   ChanStat* chan;        // C entries (one in the tensor-wide mode), zero ahead of pass 0
-  ChanStat* next;        // those of the next call on the stream: pass 0 returns the first `clear` of them to zero
-  uint32_t clear;
   uint32_t team;         // lanes per plane: a power of two, at most a warp
   uint32_t* plane_nout;  // P entries, zeroed by pass 0, written by pass 2
   double inv_nhw;        // 1 / (N * HW); tensor-wide: 1 / (N * C * HW)

@@ -1,6 +1,7 @@
 """Parity with the oracle where many outlier-rich planes are put off: more tiles or planes than a CTA of the warp-team kernel
 lists, planes that pass through the queue of the CTA-team kernels (measurements kept in the slot, with and without the
 Huffman code, or too large for it), statistics over channels in pieces and over many small planes, from call to call."""
+import numpy as np
 import pytest
 
 from oracle import fho
@@ -55,3 +56,31 @@ def test_parity_of_overlapping_calls_on_two_streams():
         want = to_dev(buf)
         assert out2.tolist() == [[total, api.FH_OK]] * 6
         assert all(torch.equal(t[:total], want) for t in dst)
+
+
+@pytest.mark.parametrize("mode", [api.FH_SALIENT_CHANNEL, api.FH_SALIENT_TENSOR])
+@pytest.mark.parametrize("shape", [(4, 6, 28, 28), (2, 5000, 7, 7)])   # statistics cleared by the call itself, and ahead of the next
+def test_channel_statistics_of_a_captured_call(mode, shape):
+    """A captured call starts from cleared statistics each time it is replayed, and so do calls made in between."""
+    import torch
+    rng = np.random.default_rng(45)   # (no outliers in uniform draws)
+    raws = [scale * rng.random(int(np.prod(shape)), dtype=np.float32) for scale in (np.float32(1), np.float32(-3))]
+    want = [to_dev(fho.compress(r, fho.desc(shape), fho.params(bits=4, salient_mode=mode))[1]) for r in raws]
+    assert all(fho.parse_header(w.cpu().numpy())["n_salient"] == 0 for w in want)
+    xs = [to_dev(r) for r in raws]
+    p, d = api.default_params(bits=4, salient_mode=mode), api.desc(shape)
+    x, dst = torch.empty_like(xs[0]), torch.zeros(api.compressed_bytes(d, p, 1), dtype=torch.uint8, device="cuda")
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        x.copy_(xs[0])
+        assert api.fh_compress(d, p, x, dst) == api.FH_OK
+        with torch.cuda.graph(graph, stream=stream):
+            assert api.fh_compress(d, p, x, dst) == api.FH_OK
+        for k in (0, 1, 1, 0):
+            x.copy_(xs[k])
+            for step in (graph.replay, graph.replay, lambda: api.fh_compress(d, p, x, dst)):
+                dst.zero_()
+                step()
+                assert torch.equal(dst[:want[k].numel()], want[k])
+    torch.cuda.synchronize()
