@@ -304,14 +304,16 @@ __device__ __forceinline__ void cta_exit(const Plan& pl, const CompressArgs& a, 
   unsigned long long vs = 0, vr = 0;
   uint32_t code = kErrNone;
   if (adders) {
-    for (uint32_t k = 0; k < (1u << 22); ++k) {
+    bool complete = false;
+    for (uint32_t k = 0; k < a.scan.polls && !complete; ++k) {
       vs = ld_relaxed(&a.sc->nsal);
       vr = ld_relaxed(&a.sc->nraw);
-      if (((uint32_t)vs & kExitMask) == adders && ((uint32_t)vr & kExitMask) == adders) break;
+      complete = ((uint32_t)vs & kExitMask) == adders && ((uint32_t)vr & kExitMask) == adders;
     }
+    if (!complete) code = kErrTimeout;
     if (vr >> (64 - kExitBits)) {  // somebody has reported an error
       __threadfence();
-      code = (uint32_t)ld_relaxed(&a.sc->status);
+      code = max(code, (uint32_t)ld_relaxed(&a.sc->status));
       st_relaxed(&a.sc->status, 0ull);
     }
     st_relaxed(&a.sc->nsal, 0ull);
