@@ -190,10 +190,10 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   if (!compress) {
     // Units of the block-wise path: a warp for planes of up to a lane per block, the CTA otherwise.  Scratch of a unit:
     // the bitmap and its prefix sums, a word per warp, the blocks by rank and, since planes may be Huffman-coded (the
-    // host cannot know), chunk offsets and tables.
+    // host cannot know), chunk offsets; then the Huffman tables.
     pl.team = pl.nblk <= 32 ? 32u : (uint32_t)fh::kThreads;
     const uint32_t units = pl.team == 32u ? (uint32_t)fh::kWarps : 1u;
-    const size_t base = A16(4 * (2 * (size_t)pl.nbm + 1 + fh::kMaxWarps + pl.nblk + 1) + sizeof(fh::HufDecode) + 2 * (size_t)pl.nblk);
+    const size_t base = A16(4 * (2 * (size_t)pl.nbm + 1 + fh::kMaxWarps + pl.nblk + 1) + 2 * (size_t)pl.nblk) + A16(sizeof(fh::HufDecode));
     // ... and a payload: as much as leaves room for four CTAs on an SM (a payload is shorter than its plane; one that
     // does not fit is read where it lies)
     size_t room = 48 * 1024 / units;

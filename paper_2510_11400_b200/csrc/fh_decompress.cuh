@@ -240,12 +240,12 @@ __device__ __forceinline__ void restore_columns(const In& in, CodeAt code_at, Lo
 // Outlier-rich plane: the inverse of salient_write.  Dense blocks a lane each, by rank (so that all lanes have one);
 // where a block's verbatim values start is a scan over the zero bytes of the codes.  Sparse blocks are
 // zeroed first, a lane per block row, and take their values entry by entry, eight lanes to a CSR row.  `scr` is the team's shared scratch, laid out by
-// make_plan; `ovf_avail` the number of readable bytes behind in.ovf; `version` the container's (2: the dense blocks'
+// make_plan, `hd` its tables for a Huffman-coded plane (touched only when the container is of version 2); `ovf_avail` the number of readable bytes behind in.ovf; `version` the container's (2: the dense blocks'
 // codes may be Huffman-coded, Section 4.4.1 "Decompression involves Huffman decoding").  Returns false in the threads
 // that found the payload inconsistent.
 template <int DT, typename In>
 __device__ __noinline__ bool decode_salient(const Team t, const Plan& pl, const In in, uint64_t ovf_avail, float eps, uint8_t* out,
-                                            uint32_t* scr, uint32_t version) {
+                                            uint32_t* scr, HufDecode* hd, uint32_t version) {
   const Geometry g(pl);
   const uint32_t H = g.H, W = g.W, nblk = g.nblk, nbx = g.nbx, nbm = g.nbm, e = g.esize, HW = g.HW;
   const uint32_t full = 0xFFFFFFFFu;
@@ -263,8 +263,7 @@ __device__ __noinline__ bool decode_salient(const Team t, const Plan& pl, const 
   uint32_t* wp = bm + nbm;         // dense blocks before each of its words
   uint32_t* wsum = wp + nbm + 1u;  // one word per warp
   uint32_t* cho = wsum + kMaxWarps;  // (Huffman) start of every chunk
-  HufDecode* hd = reinterpret_cast<HufDecode*>(cho + nblk + 1u);
-  uint16_t* block_of = reinterpret_cast<uint16_t*>(hd + 1);  // by rank
+  uint16_t* block_of = reinterpret_cast<uint16_t*>(cho + nblk + 1u);  // by rank
   bool ok = true;
   for (uint32_t w = t.lane; w < nbm; w += t.size) {
     uint32_t m = in.ld32(o_bm + 4u * w);
@@ -732,6 +731,7 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
       const uint32_t hop = (uint32_t)a.cta_stride, most = blockIdx.x < hop ? ((uint32_t)pl.P + hop - 1u) / hop : 0u;
       const Team unit = pl.team == 32u ? make_warp_team(s_red) : make_team(kThreads, s_red);
       uint32_t* scr = reinterpret_cast<uint32_t*>(smem + (pl.team == 32u ? (uint64_t)warp * pl.sal_stride : 0ull));
+      HufDecode* hd = reinterpret_cast<HufDecode*>(reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes) - 1;
       for (uint32_t base = 0; base < most; base += kThreads) {
         const uint64_t gp = blockIdx.x + (uint64_t)(base + tid) * hop;
         if (gp < pl.P && (__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp) + 1) & 3u) == kClsSalient)
@@ -764,9 +764,9 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
             FlatIn flat;
             flat.p = pay;
             flat.npay = got;
-            good = decode_salient<DT>(unit, s_pl, flat, 0ull, s_eps, a.dst + gp * pl.plane_bytes, scr, s_hdr_ok);
+            good = decode_salient<DT>(unit, s_pl, flat, 0ull, s_eps, a.dst + gp * pl.plane_bytes, scr, hd, s_hdr_ok);
           } else {
-            good = decode_salient<DT>(unit, s_pl, in, ovf_avail, s_eps, a.dst + gp * pl.plane_bytes, scr, s_hdr_ok);
+            good = decode_salient<DT>(unit, s_pl, in, ovf_avail, s_eps, a.dst + gp * pl.plane_bytes, scr, hd, s_hdr_ok);
           }
           if (!good) bad = true;
           team_sync(unit);  // the scratch is reused
@@ -790,10 +790,22 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
 
 constexpr uint32_t kSmallGroups = 8;  // a lane restores at most so many groups
 
+// Code words of groups lane, lane + tt, ... of a plane.
+template <int BITS>
+__device__ __forceinline__ void load_codes(const uint8_t* slot, uint32_t lane, uint32_t tt, uint32_t groups, uint32_t (&code)[kSmallGroups]) {
+#pragma unroll
+  for (uint32_t k = 0; k < kSmallGroups; ++k) {
+    const uint32_t g = lane + k * tt;
+    code[k] = 0;
+    if (g < groups)
+      code[k] = BITS == 2 ? (uint32_t)__ldg(slot + g)
+                          : (BITS == 4 ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(slot) + g) : __ldg(reinterpret_cast<const uint32_t*>(slot) + g));
+  }
+}
+
 template <int DT>
 __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, const DecompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ double s_red[kMaxWarps * 5];
   __shared__ uint32_t s_hdr_ok, s_bits;
   __shared__ float s_eps;
   __shared__ unsigned long long s_total;
@@ -805,7 +817,7 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
   const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
   const uint8_t* src = a.src_base + off_in;
   const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;
-  // table entry of the team's plane: the first is fetched along with the header, a tile's while the one before is restored
+  // table entry of the team's plane: the first is fetched along with the header, a tile's at the end of the one before
   const uint32_t tt = pl.team, lane = tid & (tt - 1u), lp = tid / tt;
   auto entry_of = [&](uint32_t tile) {
     const uint64_t gp = (uint64_t)tile * pl.ppt + lp;
@@ -830,28 +842,30 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
     const unsigned long long total = s_total;
     const uint32_t npay = a16(4u * ((pl.HW * bits + 31u) / 32u));
     const unsigned long long slots_off = 64ull + 16ull * pl.P, ovf_off = slots_off + pl.P * (unsigned long long)npay;
-    const Team warp_team = make_warp_team(s_red);
+    const Team warp_team = make_warp_team(nullptr);
     const bool vec = (pl.plane_bytes & (DT == kF32 ? 15u : 7u)) == 0u;  // planes start on vector boundaries in the tile buffer
-    const uint32_t tile_bytes_max = pl.stage_bytes;
-    uint32_t buf = 0;
-    for (uint32_t tile = blockIdx.x; tile < pl.ntiles; tile += gridDim.x, buf ^= 1u) {
-      uint8_t* tbuf = smem + (uint64_t)buf * tile_bytes_max;
+    // (the warps' tables for Huffman-coded planes lie where the second tile buffer is: a container that may hold such planes
+    // is restored with one buffer)
+    const uint32_t other = s_hdr_ok == 1u ? pl.stage_bytes : 0u;
+    uint32_t at = 0;
+    for (uint32_t tile = blockIdx.x; tile < pl.ntiles; tile += gridDim.x, at = other - at) {
+      uint8_t* tbuf = smem + at;
       const uint64_t p0 = (uint64_t)tile * pl.ppt;
       const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
       // the codes are requested before the entry is looked at (what another plane keeps in its slot is read and dropped)
-      uint32_t code[kSmallGroups];
-#pragma unroll
-      for (uint32_t k = 0; k < kSmallGroups; ++k) {
-        const uint32_t g = lane + k * tt;
+      uint32_t code[kSmallGroups], ln = lane, st = tt;
+      asm volatile("" : "+r"(ln), "+r"(st));  // (a lane's group numbers are worked out anew for each tile, not kept in registers)
+      {
         const uint8_t* slot = src + slots_off + (p0 + lp) * npay;
-        code[k] = 0;
-        if (lp < np && g < pl.groups)
-          code[k] = bits == 2u ? (uint32_t)__ldg(slot + g)
-                               : (bits == 4u ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(slot) + g)
-                                             : __ldg(reinterpret_cast<const uint32_t*>(slot) + g));
+        const uint32_t n = lp < np ? pl.groups : 0u;
+        if (bits == 2u) load_codes<2>(slot, ln, st, n, code);
+        else if (bits == 4u) load_codes<4>(slot, ln, st, n, code);
+        else load_codes<8>(slot, ln, st, n, code);
       }
-      const uint4 ahead = entry_of(tile + gridDim.x);
-      if (tid == 0) bulk_wait_read<1>();  // the store that left this buffer two tiles ago has read it
+      if (tid == 0) {  // the store that left this buffer last has read it
+        if (other) bulk_wait_read<1>();
+        else bulk_wait_read<0>();
+      }
       __syncthreads();
       bool salient = false, raw = false;
       uint32_t my_off16 = 0;
@@ -868,7 +882,7 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
             const float lo = __uint_as_float(en.z), scale = __uint_as_float(en.w);
 #pragma unroll
             for (uint32_t k0 = 0; k0 < kSmallGroups; ++k0) {
-              const uint32_t g = lane + k0 * tt, word = code[k0];
+              const uint32_t g = ln + k0 * st, word = code[k0];
               if (g >= pl.groups) break;
               const uint32_t i = 4u * g;
               if (vec && i + 3u < pl.HW) {  // whole group of a plane on a vector boundary: one store
@@ -891,28 +905,43 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
           bad = true;
         }
       }
-      // raw planes of the warp's slice, one after the other by the whole warp, a word per lane
-      for (uint32_t m = __ballot_sync(0xFFFFFFFFu, raw && lane == 0); m; m &= m - 1u) {
-        const uint32_t first = (uint32_t)__ffs((int)m) - 1u, rlp = (tid & ~31u) / tt + first / tt;
-        SplitIn in;
-        in.slot = src + slots_off + (p0 + rlp) * npay;
-        in.ovf = src + (unsigned long long)__shfl_sync(0xFFFFFFFFu, my_off16, (int)first) * 16ull;
-        in.npay = npay;
-        uint8_t* out = tbuf + (uint64_t)rlp * pl.plane_bytes;
-        for (uint32_t o = 4u * wlane; o < (uint32_t)pl.plane_bytes; o += 128u) {  // (payloads are padded to 16 bytes)
-          const uint32_t w = in.ld32(o);
-          if (DT == kF32) {
-            *reinterpret_cast<uint32_t*>(out + o) = w;
-          } else {
-            *reinterpret_cast<uint16_t*>(out + o) = (uint16_t)w;
-            if (o + 2u < (uint32_t)pl.plane_bytes) *reinterpret_cast<uint16_t*>(out + o + 2u) = (uint16_t)(w >> 16);
+      // raw planes of the warp's slice, a word per lane and turn: each by its own team, or, when there are fewer of them than a
+      // team would take rounds of eight loads, one after the other by the whole warp (always by the warp, 4,581,888 planes of
+      // 1 x 2 took 518 us, 91,500 of 7 x 7 in bf16 31)
+      if (uint32_t m = __ballot_sync(0xFFFFFFFFu, raw && lane == 0)) {
+        const uint32_t pb = (uint32_t)pl.plane_bytes;
+        auto copy = [&](uint32_t rlp, uint32_t off16, uint32_t j, uint32_t lanes) {
+          SplitIn in;
+          in.slot = src + slots_off + (p0 + rlp) * npay;
+          in.ovf = src + (unsigned long long)off16 * 16ull;
+          in.npay = npay;
+          uint8_t* out = tbuf + (uint64_t)rlp * pb;
+#pragma unroll 4
+          for (uint32_t o = 4u * j; o < pb; o += 4u * lanes) {
+            if (DT == kF32) {
+              *reinterpret_cast<uint32_t*>(out + o) = in.ld32(o);
+            } else if (o + 2u < pb) {
+              const uint32_t w = in.ld32(o);
+              *reinterpret_cast<uint16_t*>(out + o) = (uint16_t)w;
+              *reinterpret_cast<uint16_t*>(out + o + 2u) = (uint16_t)(w >> 16);
+            } else {
+              *reinterpret_cast<uint16_t*>(out + o) = (uint16_t)in.ld16(o);
+            }
+          }
+        };
+        if (32u * tt * __popc(m) > pb) {
+          if (raw) copy(lp, my_off16, lane, tt);
+        } else {
+          for (; m; m &= m - 1u) {
+            const uint32_t first = (uint32_t)__ffs((int)m) - 1u;
+            copy((tid & ~31u) / tt + first / tt, __shfl_sync(0xFFFFFFFFu, my_off16, (int)first), wlane, 32u);
           }
         }
       }
       // outlier-rich planes of the warp's slice, by the whole warp: four at a time when a plane is one block, one after
       // the other otherwise.  A payload (shorter than its plane, or it would have been stored raw) is copied to the
       // warp's scratch in one go, before its header is known, and decoded from there.
-      uint32_t* scr = reinterpret_cast<uint32_t*>(smem + 2ull * tile_bytes_max + (uint64_t)(tid >> 5) * pl.sal_stride);
+      uint32_t* scr = reinterpret_cast<uint32_t*>(smem + pl.sm_sal + (uint64_t)(tid >> 5) * pl.sal_stride);
       const bool four = pl.nblk == 1u;
       const uint32_t pay_max = a16((uint32_t)pl.plane_bytes), per = four ? 8u : 32u;
       uint8_t* pay = reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes + (four ? (wlane >> 3) * (pay_max + 16u) : 0u);
@@ -950,13 +979,14 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
             FlatIn one;
             one.p = (const uint8_t*)__shfl_sync(0xFFFFFFFFu, (unsigned long long)flat.p, (int)k);
             one.npay = __shfl_sync(0xFFFFFFFFu, avail, (int)k);
-            if (!decode_salient<DT>(warp_team, s_pl, one, 0ull, eps, to, scr, s_hdr_ok)) bad = true;
+            HufDecode* hd = reinterpret_cast<HufDecode*>(smem + pl.stage_bytes) + (tid >> 5);
+            if (!decode_salient<DT>(warp_team, s_pl, one, 0ull, eps, to, scr, hd, s_hdr_ok)) bad = true;
             __syncwarp();
           }
         }
         __syncwarp();
       }
-      en = ahead;
+      en = entry_of(tile + gridDim.x);
       __syncthreads();
       // the tile leaves: one bulk store when it is whole 16-byte chunks, plain stores otherwise
       const uint32_t bytes = np * (uint32_t)pl.plane_bytes;

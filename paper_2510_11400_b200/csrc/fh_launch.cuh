@@ -15,6 +15,7 @@
 namespace fh {
 
 constexpr size_t kSmemLimit = 227 * 1024 - 4096;  // dynamic shared memory a CTA may ask for
+constexpr uint32_t kSmemPerSm = 228 * 1024;       // shared memory of an SM
 
 inline size_t A16(size_t x) { return (x + 15) & ~(size_t)15; }
 
