@@ -198,6 +198,8 @@ def fh_run_schedule(items: List[SchedItem], p: fh_params, arena, stream=None) ->
     buf, at = bytearray(_SCHED_ENTRY.size * len(items)), 0
     for it in items:
         dense, restored = it.dense, it.restored
+        if not isinstance(it.desc, fh_tensor_desc):    # (anything has bytes)
+            raise TypeError(f"expected fh_tensor_desc, got {type(it.desc).__name__}")
         _SCHED_ENTRY.pack_into(buf, at, bytes(it.desc), it.action, 0 if dense is None else dense.data_ptr(),
                                0 if restored is None else restored.data_ptr())
         at += _SCHED_ENTRY.size

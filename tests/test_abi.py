@@ -90,3 +90,9 @@ def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(api, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(FileNotFoundError):
         api.lib()
+
+
+@pytest.mark.parametrize("desc", [api.fh_params(), 32, b"x" * 32, [0] * 32, (1, 2, 8, 8)])
+def test_a_schedule_takes_nothing_but_tensor_descriptions(desc):
+    with pytest.raises(TypeError, match="fh_tensor_desc"):
+        api.fh_run_schedule([api.SchedItem(desc, api.FH_KEEP, None, None)], api.fh_params(), None)
