@@ -15,7 +15,7 @@
 //       team per plane, groups kept in registers; a warp handles the outlier-rich planes of its slice;
 //   compress_cta_regs<DT, SIGMA, K, EDGE>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
 //   compress_cta<DT, SIGMA, NT>            still larger ones of whole 16-byte chunks: swept in shared memory;
-//   compress_generic<DT, BITS>             everything else (still larger ragged planes, random rounding outside the
+//   compress_generic<DT, BITS, ROUND>      everything else (still larger ragged planes, random rounding outside the
 //       plane-wise three-sigma mode).
 // The kernel's last CTA writes the header and the result words and returns the scratch to its idle state.
 #pragma once
@@ -429,9 +429,11 @@ struct Rec {
 // on a 16-byte boundary); a team per plane computes statistics and class; the codes of normal planes
 // are staged in shared memory and leave with 16-byte stores.  Outlier-rich planes of the tile are then
 // measured one after the other by the whole CTA, and written the same way in phase 2 (this kernel serves the
-// odd shapes and is not tuned).
-template <int DT, int BITS>
-__global__ void __launch_bounds__(kThreads) compress_generic(const Plan pl, const CompressArgs a) {
+// odd shapes and is not tuned).  ROUND: random rounding, which serves planes of any size in the modes without plane-wise
+// statistics and wants four CTAs to an SM (64 registers; with the 119 that the compiler takes, 64 x 64 fp32 planes of 56 x 56
+// in mode OFF took 68.5 us, now 48.0); otherwise planes are so large that one or two CTAs fit.
+template <int DT, int BITS, bool ROUND>
+__global__ void __launch_bounds__(kThreads, ROUND ? 4 : 1) compress_generic(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 5];
   __shared__ uint32_t s_tile, s_last;
@@ -550,12 +552,12 @@ __global__ void __launch_bounds__(kThreads) compress_generic(const Plan pl, cons
             float dd[4];
             load_dist<DT>(plane, g, HW, vec, lo, dd);
             uint32_t rnd[4] = {0, 0, 0, 0};
-            if (pl.rounding)  // one generator call per group: counter = (group, plane, tensor id), key = seed
+            if (ROUND)  // one generator call per group: counter = (group, plane, tensor id), key = seed
               philox4x32_10(g, (uint32_t)(p0 + lp), (uint32_t)pl.tensor_id, (uint32_t)(pl.tensor_id >> 32),
                             (uint32_t)pl.seed, (uint32_t)(pl.seed >> 32), rnd);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              uint32_t q = pl.rounding ? quant_code_random(dd[k], inv, L, rnd[k]) : quant_code(dd[k], inv, L);
+              uint32_t q = ROUND ? quant_code_random(dd[k], inv, L, rnd[k]) : quant_code(dd[k], inv, L);
               if (g * 4u + k >= HW) q = 0;
               word |= q << (k * BITS);
             }
@@ -868,14 +870,17 @@ __device__ __forceinline__ void run_codes(uint32_t lane, int32_t n, float inv, u
 // past the plane's end carry code 0 whatever the draw.  The run is read from its stage at `p` once more, in a loop: with
 // the distances held in registers the generator's rounds, unrolled over the slots, spilled and overran the instruction
 // cache (112 x 112: 150 us a call).  `g0`: the run's first group, whose codes go to `slot`.
-template <int DT>
+// GRAIN: the run's, when the kernel fixes it (runs of whole groups), so that the loop holds one form of load; -1: `grain`.
+// With width and grain looked at in the loop, 512 x 64 planes of 32 x 32 took 71.6 us, now 63.6.
+template <int DT, int BITS, int GRAIN>
 __device__ __forceinline__ void run_codes_random(const Plan& pl, const uint8_t* p, uint32_t grain, uint32_t lane, uint32_t step, int32_t n,
                                                  float lo, float inv, uint32_t g0, uint64_t gp, uint8_t* slot) {
-  const uint32_t bits = (uint32_t)pl.bits, L = (1u << bits) - 1u, groups = (uint32_t)(n + 3) >> 2;
+  constexpr uint32_t L = (1u << BITS) - 1u;
+  const uint32_t groups = (uint32_t)(n + 3) >> 2;
 #pragma unroll 2
   for (uint32_t v = lane; v < groups; v += step) {
     uint32_t w[4], rnd[4];
-    group_load<DT>(p, v, grain, w);
+    group_load<DT>(p, v, GRAIN < 0 ? grain : (uint32_t)GRAIN, w);
     philox4x32_10(g0 + v, (uint32_t)gp, (uint32_t)pl.tensor_id, (uint32_t)(pl.tensor_id >> 32), (uint32_t)pl.seed,
                   (uint32_t)(pl.seed >> 32), rnd);
     float x[4];
@@ -888,11 +893,11 @@ __device__ __forceinline__ void run_codes_random(const Plan& pl, const uint8_t* 
     }
     uint32_t word = 0;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) word |= quant_code_random(__fsub_rn(x[e], lo), inv, L, rnd[e]) << (e * bits);
+    for (int e = 0; e < 4; ++e) word |= quant_code_random(__fsub_rn(x[e], lo), inv, L, rnd[e]) << (e * BITS);
     const int32_t in = n - 4 * (int32_t)v;
-    if (in < 4) word &= (1u << ((uint32_t)in * bits)) - 1u;
-    if (bits == 2u) slot[v] = (uint8_t)word;
-    else if (bits == 4u) reinterpret_cast<uint16_t*>(slot)[v] = (uint16_t)word;
+    if (GRAIN < 0 && in < 4) word &= (1u << ((uint32_t)in * BITS)) - 1u;
+    if (BITS == 2) slot[v] = (uint8_t)word;
+    else if (BITS == 4) reinterpret_cast<uint16_t*>(slot)[v] = (uint16_t)word;
     else reinterpret_cast<uint32_t*>(slot)[v] = word;
   }
 }
@@ -901,8 +906,12 @@ template <int DT, int SIGMA, int K, int TT, int EDGE>
 __device__ __forceinline__ void run_codes_any(const Plan& pl, const uint8_t* p, uint32_t grain, uint32_t lane, int32_t n, float lo,
                                               float inv, uint32_t g0, uint64_t gp, uint8_t* slot, const float (&x)[K][4]) {
   uint8_t* at = slot + g0 * (uint32_t)pl.bits / 2u;
-  if (SIGMA == 2) run_codes_random<DT>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
-  else if (pl.bits == 2) run_codes<DT, K, TT, EDGE, 2>(lane, n, inv, at, x);
+  constexpr int GRAIN = EDGE == 0 ? 2 : -1;
+  if (SIGMA == 2) {
+    if (pl.bits == 2) run_codes_random<DT, 2, GRAIN>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+    else if (pl.bits == 4) run_codes_random<DT, 4, GRAIN>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+    else run_codes_random<DT, 8, GRAIN>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+  } else if (pl.bits == 2) run_codes<DT, K, TT, EDGE, 2>(lane, n, inv, at, x);
   else if (pl.bits == 4) run_codes<DT, K, TT, EDGE, 4>(lane, n, inv, at, x);
   else run_codes<DT, K, TT, EDGE, 8>(lane, n, inv, at, x);
 }

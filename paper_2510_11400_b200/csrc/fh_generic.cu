@@ -5,13 +5,20 @@
 namespace fh {
 namespace {
 
-template <int DT, int BITS>
+template <int DT, int BITS, bool ROUND>
 int launch_generic_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int grid = 0;
-  int rc = grid_for(compress_generic<DT, BITS>, pl.sm_total, pl.ntiles, &grid);
+  int rc = grid_for(compress_generic<DT, BITS, ROUND>, pl.sm_total, pl.ntiles, &grid);
   if (rc != FH_OK) return rc;
-  return launch_dependent(compress_generic<DT, BITS>, grid, kThreads, pl.sm_total, stream, pl, a) == cudaSuccess
+  return launch_dependent(compress_generic<DT, BITS, ROUND>, grid, kThreads, pl.sm_total, stream, pl, a) == cudaSuccess
              ? FH_OK : FH_ERR_CUDA;
+}
+
+template <int DT, bool ROUND>
+int launch_generic_dt(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+  return pl.bits == 2   ? launch_generic_t<DT, 2, ROUND>(pl, a, stream)
+         : pl.bits == 4 ? launch_generic_t<DT, 4, ROUND>(pl, a, stream)
+                        : launch_generic_t<DT, 8, ROUND>(pl, a, stream);
 }
 
 template <int DT, int PASS, bool VEC>
@@ -37,13 +44,8 @@ int launch_channel_passes_t(const Plan& pl, const ChannelArgs& args, cudaStream_
 }  // namespace
 
 int launch_compress_generic(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
-  if (pl.dtype == kF32)
-    return pl.bits == 2   ? launch_generic_t<kF32, 2>(pl, a, stream)
-           : pl.bits == 4 ? launch_generic_t<kF32, 4>(pl, a, stream)
-                          : launch_generic_t<kF32, 8>(pl, a, stream);
-  return pl.bits == 2   ? launch_generic_t<kBF16, 2>(pl, a, stream)
-         : pl.bits == 4 ? launch_generic_t<kBF16, 4>(pl, a, stream)
-                        : launch_generic_t<kBF16, 8>(pl, a, stream);
+  if (pl.dtype == kF32) return pl.rounding ? launch_generic_dt<kF32, true>(pl, a, stream) : launch_generic_dt<kF32, false>(pl, a, stream);
+  return pl.rounding ? launch_generic_dt<kBF16, true>(pl, a, stream) : launch_generic_dt<kBF16, false>(pl, a, stream);
 }
 
 int launch_channel_passes(const Plan& pl, const ChannelArgs& ca, cudaStream_t stream) {
