@@ -132,11 +132,23 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   if (pl.P > 0x7FFFFFFFull) return FH_ERR_UNSUPPORTED;
   // block-wise path: blocks per step side by side, rows of steps (see fh_blocks.cuh)
   pl.qs = pl.nbx >= 3 ? 2u : pl.nbx - 1u;
-  pl.nsr = (pl.nby + (4u >> pl.qs) - 1u) / (4u >> pl.qs);
+  const uint32_t step_rows = (pl.nby + (4u >> pl.qs) - 1u) / (4u >> pl.qs);
+  // Its warps take a row of steps each; where a team has more warps than the plane has rows, the rows go in parts (planes
+  // of 1 x 5000 are one row, which one warp of three took: 14 x 64 fp32 planes, every eighth outlier-rich,
+  // 240 us, now 98)
+  auto split_rows = [&](uint32_t warps) {
+    const uint32_t steps = (pl.nbx + (1u << pl.qs) - 1u) >> pl.qs;
+    uint32_t seg = step_rows < warps ? (warps + step_rows - 1u) / step_rows : 1u;
+    if (seg > steps) seg = steps;
+    pl.segb = ((steps + seg - 1u) / seg) << pl.qs;
+    pl.seg = (pl.nbx + pl.segb - 1u) / pl.segb;
+    pl.nsr = step_rows * pl.seg;
+  };
+  split_rows(1u);
   // its measuring scratch (of a team of `warps`): row pointers, two sums per step row, the bitmap; with the Huffman stage
   // one more sum and the encoder's tables
   auto sal_bytes_of = [&](uint32_t warps) {
-    const size_t words = (size_t)pl.H + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
+    const size_t words = (size_t)pl.H * pl.seg + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
                          (pl.entropy ? (size_t)pl.nsr + 1 + sizeof(fh::HufEncode) / 4 + (warps - 1) * 4 * fh::kHufStageWords : 0);
     return (uint32_t)A16(4 * words + 16);
   };
@@ -169,6 +181,7 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     // (CTA-team kernels: two stages; a third buys nothing that more resident CTAs do not give)
     const uint32_t ns_max = v.cta ? 2u : (uint32_t)fh::kMaxStages;
     ns = ns < 2 ? 2 : (ns > ns_max ? ns_max : ns);
+    split_rows(v.cta ? pl.team / 32 : 1u);
     const uint32_t sal_bytes = sal_bytes_of(v.cta ? pl.team / 32 : 1u);
     const uint32_t areas = blockwise ? (v.cta ? 1u : (uint32_t)fh::kWarps) : 0u;
     for (;;) {
@@ -220,6 +233,7 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     }
     pl.nstage = 0;
     pl.stage_bytes = 0;
+    split_rows(fh::kWarps);
     const uint32_t sal_bytes = sal_bytes_of(fh::kWarps);
     uint64_t ppt = kTileTarget / pl.plane_bytes;
     if (ppt < 1) ppt = 1;

@@ -6,7 +6,8 @@
 // differences come from lane l - 4, one shuffle per eight elements' column; a block's sums are three shuffles over the
 // lanes of its column of the warp, a plane row's running count is carried in the lanes that own the row.  The blocks of
 // a step lie side by side (planes of three block columns and more), in 2 x 2 (two columns) or below one another (one).
-// Warps take the plane's block rows ("step rows") in turn; only their sums -- CSR row lengths, dense blocks, verbatim
+// Warps take the plane's block rows ("step rows") in turn, a CTA's warps parts of them (PARTS) where there are fewer rows
+// than warps; only their sums -- CSR row lengths, dense blocks, verbatim
 // elements, chunk bytes per step row -- go through shared memory, and one pass of scans turns them into places.
 // What bounds it: instruction issue (about 25 instructions per element and pass); a 112 x 112 plane measured in
 // 13 us and written in 14 us with a warp per block and a lane per two elements, see the figures at the kernels.
@@ -42,16 +43,16 @@ struct Geometry {
         qs(pl.qs), esize((uint32_t)pl.esize) {}
 };
 
-// Shared scratch of one measured plane: words of rowp[H + 1], dense[nsr + 1], outl[nsr + 1], bitmap[nbm] and, with the
-// Huffman stage, chunks[nsr + 1] and a HufEncode.
+// Shared scratch of one measured plane: words of rowp[H * seg + 1] (a row's entries part by part), dense[nsr + 1],
+// outl[nsr + 1], bitmap[nbm] and, with the Huffman stage, chunks[nsr + 1] and a HufEncode.
 struct SalScratch {
   uint32_t *rowp, *dense, *outl, *bitmap, *chunks;
   HufEncode* huf;
 };
-__device__ __forceinline__ SalScratch sal_scratch(const Geometry& pl, uint32_t* sal) {
+__device__ __forceinline__ SalScratch sal_scratch(const Geometry& pl, uint32_t* sal, uint32_t seg) {
   SalScratch s;
   s.rowp = sal;
-  s.dense = s.rowp + pl.H + 1u;
+  s.dense = s.rowp + pl.H * seg + 1u;
   s.outl = s.dense + pl.nsr + 1u;
   s.bitmap = s.outl + pl.nsr + 1u;
   s.chunks = s.bitmap + pl.nbm;
@@ -59,6 +60,27 @@ __device__ __forceinline__ SalScratch sal_scratch(const Geometry& pl, uint32_t* 
   return s;
 }
 
+// Parts of a step row, block columns of a part.  (Fixed where a row is one part: the streaming kernels' sweeps lose 5 % to the
+// registers that these take in the outlined functions.)
+template <bool PARTS>
+struct Split {
+  uint32_t seg, segb;
+  __device__ __forceinline__ explicit Split(const Plan& pl) : seg(PARTS ? pl.seg : 1u), segb(PARTS ? pl.segb : pl.nbx) {}
+};
+// The `unit`-th part: its step row, its number within the row, its block columns.
+struct StepUnit {
+  uint32_t sr, part, bx0, bx1;
+};
+template <bool PARTS>
+__device__ __forceinline__ StepUnit step_unit(const Geometry& g, const Split<PARTS>& sp, uint32_t unit) {
+  if (!PARTS) return StepUnit{unit, 0u, 0u, g.nbx};
+  StepUnit u;
+  u.sr = sp.seg == 1u ? unit : unit / sp.seg;
+  u.part = unit - u.sr * sp.seg;
+  u.bx0 = u.part * sp.segb;
+  u.bx1 = min(g.nbx, u.bx0 + sp.segb);
+  return u;
+}
 // This lane's place in a step.
 struct StepLane {
   uint32_t r, q;    // row within the block, block within the step
@@ -202,10 +224,11 @@ __device__ __forceinline__ void warp_excl_scan(uint32_t* arr, uint32_t n) {
 
 // Measuring part: block classes, CSR row lengths, sizes.  The team is a whole warp or a whole CTA.  Leaves rowp, dense
 // and outl (and chunks) as exclusive prefix sums with the total behind the last entry, the bitmap and the code.
-template <int DT>
+template <int DT, bool PARTS>
 __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
   const Geometry g(pl);
-  const SalScratch sc = sal_scratch(g, sal);
+  const Split<PARTS> sp(pl);
+  const SalScratch sc = sal_scratch(g, sal, sp.seg);
   const uint32_t H = g.H, W = g.W, nsr = g.nsr, tau_den = pl.tau_den, full = 0xFFFFFFFFu;
   const bool entropy = pl.entropy != 0;
   const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane = threadIdx.x & 31u;
@@ -216,12 +239,13 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
   for (uint32_t i = t.lane; i < g.nbm; i += t.size) sc.bitmap[i] = 0;
   if (entropy)
     for (uint32_t i = t.lane; i < 256u; i += t.size) sc.huf->hist[i] = 0;
-  if (t.lane == 0) sc.rowp[H] = sc.dense[nsr] = sc.outl[nsr] = 0;
+  if (t.lane == 0) sc.rowp[H * sp.seg] = sc.dense[nsr] = sc.outl[nsr] = 0;
   team_sync(t);
   for (uint32_t sr = wid; sr < nsr; sr += nw) {
-    const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
+    const StepUnit un = step_unit(g, sp, sr);
+    const uint32_t by = un.sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
     uint32_t row = 0, n_dense = 0, n_out = 0;
-    for (uint32_t bx0 = 0; bx0 < g.nbx; bx0 += sl.qm + 1u) {
+    for (uint32_t bx0 = un.bx0; bx0 < un.bx1; bx0 += sl.qm + 1u) {
       const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u;
       const bool valid = by < g.nby && bx < g.nbx;
       const uint32_t nin = seg_in(g, valid, y, x0);
@@ -250,7 +274,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
     }
     if (g.qs > 0) row += __shfl_xor_sync(full, row, 1);
     if (g.qs > 1) row += __shfl_xor_sync(full, row, 2);
-    if ((sl.q & sl.qm) == 0u && y < H) sc.rowp[y] = row;
+    if ((sl.q & sl.qm) == 0u && y < H) sc.rowp[y * sp.seg + un.part] = row;
     asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_out) : "r"(full));
     if (lane == 0) {
       sc.dense[sr] = n_dense;
@@ -258,7 +282,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
     }
   }
   team_sync(t);
-  if (wid == 0) warp_excl_scan(sc.rowp, H + 1u);
+  if (wid == 0) warp_excl_scan(sc.rowp, H * sp.seg + 1u);
   if (wid == min(1u, nw - 1u)) {
     warp_excl_scan(sc.dense, nsr + 1u);
     warp_excl_scan(sc.outl, nsr + 1u);
@@ -266,7 +290,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
   team_sync(t);
   SalientInfo info;
   info.n_dense = sc.dense[nsr];
-  info.nnz_s = sc.rowp[H];
+  info.nnz_s = sc.rowp[H * sp.seg];
   info.n_out_d = sc.outl[nsr];
   info.coded = 0;
   if (entropy && info.n_dense) {
@@ -277,9 +301,10 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
     team_sync(t);
     if (h->maxlen <= kHufMaxLen) {
       for (uint32_t sr = wid; sr < nsr; sr += nw) {
-        const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
+        const StepUnit un = step_unit(g, sp, sr);
+        const uint32_t by = un.sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
         uint32_t bytes = 0;
-        for (uint32_t bx0 = 0; bx0 < g.nbx; bx0 += sl.qm + 1u) {
+        for (uint32_t bx0 = un.bx0; bx0 < un.bx1; bx0 += sl.qm + 1u) {
           const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u, b = by * g.nbx + bx;
           const bool valid = by < g.nby && bx < g.nbx;
           const bool dense = valid && ((sc.bitmap[b >> 5] >> (b & 31u)) & 1u);
@@ -312,11 +337,12 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
 
 // Writing part; `sal` holds what salient_measure left.  Every lane recomputes the codes of its block rows and stores
 // them (and the CSR entries and verbatim values) straight to their places.
-template <int DT>
+template <int DT, bool PARTS>
 __device__ __noinline__ void salient_write(const Team t, const Plan& pl, const uint8_t* plane, const SalientInfo info,
                                            uint32_t* sal, const SplitOut out) {
   const Geometry g(pl);
-  const SalScratch sc = sal_scratch(g, sal);
+  const Split<PARTS> sp(pl);
+  const SalScratch sc = sal_scratch(g, sal, sp.seg);
   const uint32_t H = g.H, W = g.W, nsr = g.nsr, e = g.esize, full = 0xFFFFFFFFu;
   const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane = threadIdx.x & 31u;
   const uint32_t o_bm = 16u, o_rp = o_bm + 4u * g.nbm, o_col = o_rp + 4u * (H + 1u);
@@ -336,7 +362,7 @@ __device__ __noinline__ void salient_write(const Team t, const Plan& pl, const u
   const uint32_t end = max(out.npay, a16(info.size));
   for (uint32_t o = info.size + 4u * t.lane; o < end; o += 4u * t.size) out.st32(o, 0);
   for (uint32_t w = t.lane; w < g.nbm; w += t.size) out.st32(o_bm + 4u * w, sc.bitmap[w]);
-  for (uint32_t y = t.lane; y <= H; y += t.size) out.st32(o_rp + 4u * y, sc.rowp[y]);
+  for (uint32_t y = t.lane; y <= H; y += t.size) out.st32(o_rp + 4u * y, sc.rowp[y * sp.seg]);
   const HufEncode* h = sc.huf;  // (only looked at when info.coded)
   uint32_t o_cb = 0, o_chunks = 0;
   if (info.coded) {  // the section's head: code lengths, then the bytes of every chunk; pads are zero
@@ -358,10 +384,11 @@ __device__ __noinline__ void salient_write(const Team t, const Plan& pl, const u
   const StepLane sl = step_lane(g);
   const bool vec = seg_vec<DT>(plane, W);
   for (uint32_t sr = wid; sr < nsr; sr += nw) {
-    const uint32_t by = sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
+    const StepUnit un = step_unit(g, sp, sr);
+    const uint32_t by = un.sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
     uint32_t rank0 = sc.dense[sr], outl0 = sc.outl[sr], chunk0 = info.coded ? sc.chunks[sr] : 0u;
-    uint32_t csr = y < H ? sc.rowp[y] : 0u;
-    for (uint32_t bx0 = 0; bx0 < g.nbx; bx0 += sl.qm + 1u) {
+    uint32_t csr = y < H ? sc.rowp[y * sp.seg + un.part] : 0u;
+    for (uint32_t bx0 = un.bx0; bx0 < un.bx1; bx0 += sl.qm + 1u) {
       const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u, b = by * g.nbx + bx;
       const bool valid = by < g.nby && bx < g.nbx;
       const uint32_t nin = seg_in(g, valid, y, x0);

@@ -13,7 +13,7 @@
 // Variants by plane size:
 //   compress_warp<DT, SIGMA, TT, K, EDGE>   planes of at most 256 groups: bulk-copy (TMA) pipeline, a sub-warp
 //       team per plane, groups kept in registers; a warp handles the outlier-rich planes of its slice;
-//   compress_cta_regs<DT, SIGMA, K, EDGE>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
+//   compress_cta_regs<DT, SIGMA, K, EDGE, PARTS>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
 //   compress_cta<DT, SIGMA, NT>            still larger ones of whole 16-byte chunks: swept in shared memory;
 //   compress_generic<DT, BITS, ROUND>      everything else (still larger ragged planes, random rounding outside the
 //       plane-wise three-sigma mode).
@@ -222,7 +222,7 @@ __device__ __forceinline__ void count_blockwise(uint32_t units, uint32_t nsal, u
 
 // Writes the payload of the measured plane gp (`plane` in shared memory, `info` and `sal` from
 // salient_measure) with its overflow part `at` units into the overflow region, and its table entry.
-template <int DT>
+template <int DT, bool PARTS>
 __device__ __forceinline__ void write_blockwise(const Team& t, const Plan& pl, const Dest& d, uint64_t gp,
                                                 const uint8_t* plane, const SalientInfo& info, uint32_t* sal,
                                                 uint32_t n_out, uint32_t at) {
@@ -235,7 +235,7 @@ __device__ __forceinline__ void write_blockwise(const Team& t, const Plan& pl, c
   out.ovf = d.dst + off16 * 16ull;
   out.npay = pl.npay;
   if (raw) raw_write(t, pl, plane, out);
-  else salient_write<DT>(t, pl, plane, info, sal, out);
+  else salient_write<DT, PARTS>(t, pl, plane, info, sal, out);
   if (t.lane == 0)
     reinterpret_cast<uint4*>(d.dst + 64)[gp] =
         make_uint4(my_units ? (uint32_t)off16 : 0u, (raw ? kClsRaw : kClsSalient) | (n_out << 2), 0u, 0u);
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(kThreads, ROUND ? 4 : 1) compress_generic(cons
       uint32_t U = 0, nsal = 0, nraw = 0;  // (every thread keeps the same figures)
       for (uint32_t lp = 0; lp < np; ++lp) {
         if ((rec[lp].meta & 3u) == kClsNormal) continue;
-        const SalientInfo info = salient_measure<DT>(cta, s_ctl.pl, tile_buf + head + (uint64_t)lp * pl.plane_bytes, sal);
+        const SalientInfo info = salient_measure<DT, true>(cta, s_ctl.pl, tile_buf + head + (uint64_t)lp * pl.plane_bytes, sal);
         bool raw;
         const uint32_t u = plane_units(pl, info, raw);
         if (tid == 0 && d.fits) store_marker(d, p0 + lp, rec[lp].meta, u);
@@ -637,8 +637,8 @@ __global__ void __launch_bounds__(kThreads, ROUND ? 4 : 1) compress_generic(cons
       for (uint32_t lp = 0; lp < np; ++lp) {
         if ((rec[lp].meta & 3u) == kClsNormal) continue;
         const uint8_t* plane = tile_buf + head + (uint64_t)lp * pl.plane_bytes;
-        const SalientInfo info = salient_measure<DT>(cta, s_ctl.pl, plane, sal);
-        write_blockwise<DT>(cta, s_ctl.pl, d, p0 + lp, plane, info, sal, rec[lp].meta >> 2, at);
+        const SalientInfo info = salient_measure<DT, true>(cta, s_ctl.pl, plane, sal);
+        write_blockwise<DT, true>(cta, s_ctl.pl, d, p0 + lp, plane, info, sal, rec[lp].meta >> 2, at);
         at += rec[lp].units;
         __syncthreads();
       }
@@ -982,31 +982,35 @@ constexpr int kWarpKernelThreads = kThreads + 32;
 
 // What was measured of a plane of more than four blocks waits for phase 2 in the plane's own slot, when that holds it:
 // sizes, the measuring scratch and, with the Huffman stage, the code.  (Measuring a second time was half of phase 2.)
+template <bool PARTS>
 __device__ __forceinline__ uint32_t scratch_words(const Plan& pl) {
-  return (uint32_t)pl.H + 1u + 2u * (pl.nsr + 1u) + pl.nbm + (pl.entropy ? pl.nsr + 1u : 0u);
+  return (uint32_t)pl.H * (PARTS ? pl.seg : 1u) + 1u + 2u * (pl.nsr + 1u) + pl.nbm + (pl.entropy ? pl.nsr + 1u : 0u);
 }
+template <bool PARTS>
 __device__ __forceinline__ bool scratch_saved(const Plan& pl) {
-  return 32u + 4u * scratch_words(pl) + (pl.entropy ? 4u * 256u : 0u) <= pl.npay;
+  return 32u + 4u * scratch_words<PARTS>(pl) + (pl.entropy ? 4u * 256u : 0u) <= pl.npay;
 }
+template <bool PARTS>
 __device__ __forceinline__ void scratch_save(const Team& t, const Plan& pl, const Dest& d, uint64_t gp, const SalientInfo& info, uint32_t* sal) {
   uint4* slot = reinterpret_cast<uint4*>(d.dst + pl.slots_off + gp * pl.npay);
-  const HufEncode* h = sal_scratch(Geometry(pl), sal).huf;
+  const HufEncode* h = sal_scratch(Geometry(pl), sal, Split<PARTS>(pl).seg).huf;
   if (t.lane == 0) {
     slot[0] = make_uint4(info.nnz_s, info.n_dense, info.n_out_d, info.size);
     slot[1] = pl.entropy ? make_uint4(info.coded, h->nlens, h->smin, h->smax) : make_uint4(0u, 0u, 0u, 0u);
   }
   uint32_t* w = reinterpret_cast<uint32_t*>(slot + 2);
-  const uint32_t n = scratch_words(pl);
+  const uint32_t n = scratch_words<PARTS>(pl);
   for (uint32_t i = t.lane; i < n; i += t.size) w[i] = sal[i];
   if (info.coded)
     for (uint32_t i = t.lane; i < 256u; i += t.size) w[n + i] = h->code[i];
 }
+template <bool PARTS>
 __device__ __forceinline__ SalientInfo scratch_load(const Team& t, const Plan& pl, const Dest& d, uint64_t gp, uint32_t* sal) {
   const uint4* slot = reinterpret_cast<const uint4*>(d.dst + pl.slots_off + gp * pl.npay);
-  HufEncode* h = sal_scratch(Geometry(pl), sal).huf;
+  HufEncode* h = sal_scratch(Geometry(pl), sal, Split<PARTS>(pl).seg).huf;
   const uint4 v = __ldcg(slot), x = __ldcg(slot + 1);
   const uint32_t* w = reinterpret_cast<const uint32_t*>(slot + 2);
-  const uint32_t n = scratch_words(pl);
+  const uint32_t n = scratch_words<PARTS>(pl);
   for (uint32_t i = t.lane; i < n; i += t.size) sal[i] = __ldcg(w + i);
   if (x.x) {
     for (uint32_t i = t.lane; i < 256u; i += t.size) h->code[i] = __ldcg(w + n + i);
@@ -1083,14 +1087,14 @@ __device__ __noinline__ void warp_tile_measure(BlockCtl* c, WarpList* l, uint8_t
     const Team team = make_warp_team(nullptr);
     for (uint32_t m = leaders; m; m &= m - 1u) {
       const uint32_t src = (uint32_t)__ffs((int)m) - 1u, lp = lp0 + src / TT;
-      const SalientInfo info = salient_measure<DT>(team, pl, tbuf + (uint64_t)lp * pl.plane_bytes, sal);
+      const SalientInfo info = salient_measure<DT, false>(team, pl, tbuf + (uint64_t)lp * pl.plane_bytes, sal);
       bool raw;
       const uint32_t u = plane_units(pl, info, raw);
       total += u;
       nraw += raw ? 1u : 0u;
       const uint32_t mt = __shfl_sync(full, meta, (int)src);
       if (lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
-      if (c->d.fits && scratch_saved(pl)) scratch_save(team, pl, c->d, p0 + lp, info, sal);
+      if (c->d.fits && scratch_saved<false>(pl)) scratch_save<false>(team, pl, c->d, p0 + lp, info, sal);
       __syncwarp();
     }
   }
@@ -1156,9 +1160,9 @@ __device__ __noinline__ void warp_plane_write(BlockCtl* c, uint64_t gp, const ui
   const Team team = make_warp_team(nullptr);
   if (!plane) plane = fetch_plane(pl, c->a.src, gp, buf, team.lane, 32u, true);
   __syncwarp();
-  const SalientInfo info = scratch_saved(pl) ? scratch_load(team, pl, c->d, gp, sal) : salient_measure<DT>(team, pl, plane, sal);
+  const SalientInfo info = scratch_saved<false>(pl) ? scratch_load<false>(team, pl, c->d, gp, sal) : salient_measure<DT, false>(team, pl, plane, sal);
   __syncwarp();
-  write_blockwise<DT>(team, pl, c->d, gp, plane, info, sal, meta >> 2, place);
+  write_blockwise<DT, false>(team, pl, c->d, gp, plane, info, sal, meta >> 2, place);
   __syncwarp();
 }
 
@@ -1535,11 +1539,11 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
 // An outlier-rich plane is measured by the whole CTA while it lies in its stage and written in phase 2.
 // -------------------------------------------------------------------------------------------------
 // Phase 1: the plane in `plane` is measured, tile (= plane) `tile` published.  Ends with a barrier.
-template <int DT>
+template <int DT, bool PARTS>
 __device__ __noinline__ void cta_tile_measure(BlockCtl* c, double* red, const uint8_t* plane, uint32_t* sal, uint32_t tile,
                                               uint32_t meta) {
   const Team team = make_cta_team(blockDim.x, red);
-  const SalientInfo info = salient_measure<DT>(team, c->pl, plane, sal);
+  const SalientInfo info = salient_measure<DT, PARTS>(team, c->pl, plane, sal);
   if (threadIdx.x == 0) {
     bool raw;
     const uint32_t units = plane_units(c->pl, info, raw);
@@ -1547,7 +1551,7 @@ __device__ __noinline__ void cta_tile_measure(BlockCtl* c, double* red, const ui
     count_blockwise(units, raw ? 0u : 1u, raw ? 1u : 0u);
     if (c->d.fits) store_marker(c->d, tile, meta, units);
   }
-  if (c->d.fits && scratch_saved(c->pl)) scratch_save(team, c->pl, c->d, tile, info, sal);
+  if (c->d.fits && scratch_saved<PARTS>(c->pl)) scratch_save<PARTS>(team, c->pl, c->d, tile, info, sal);
   if (threadIdx.x == 0) c->own_info = info;
   __syncthreads();
 }
@@ -1632,7 +1636,7 @@ __device__ __forceinline__ void plane_load(const Plan& pl, const uint8_t* src, u
 
 // Phase 2 of the CTA-team kernels: the CTA's own plane, then planes from the queue until it is empty.  While one is written,
 // the next is claimed and fetched into the other stage.
-template <int DT>
+template <int DT, bool PARTS>
 __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal) {
   const Plan& pl = c->pl;
   const Team team = make_cta_team(blockDim.x, red);
@@ -1666,9 +1670,9 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
       }
     }
     SalientInfo info;
-    const bool saved = scratch_saved(pl);
+    const bool saved = scratch_saved<PARTS>(pl);
     if (kept) info = c->own_info;
-    else if (saved) info = scratch_load(team, pl, c->d, tile, sal);
+    else if (saved) info = scratch_load<PARTS>(team, pl, c->d, tile, sal);
     if (claims) c->ahead = queue_entry(c, mine, false);
     fetch_wait();
     __syncthreads();
@@ -1676,19 +1680,19 @@ __device__ __noinline__ void cta_phase2(BlockCtl* c, double* red, uint8_t* stage
     const uint8_t* plane = stage + plane_head(pl, tile);
     fetched = ahead < pl.ntiles;
     if (fetched) fetch_start(pl, c->a.src, ahead, stages + (uint64_t)(cur ^ 1u) * pl.stage_bytes);
-    if (!saved && !kept) info = salient_measure<DT>(team, pl, plane, sal);
+    if (!saved && !kept) info = salient_measure<DT, PARTS>(team, pl, plane, sal);
     kept = false;
-    if (c->ok) write_blockwise<DT>(team, pl, c->d, (uint64_t)tile, plane, info, sal, mk.y >> 2, c->base);
+    if (c->ok) write_blockwise<DT, PARTS>(team, pl, c->d, (uint64_t)tile, plane, info, sal, mk.y >> 2, c->base);
     if (claims) c->next = ahead == kPending ? queue_entry(c, mine, true) : ahead;
     fetch_wait();
     if (fetched) cur ^= 1u;
   }
 }
 // Behind phase 1 of a CTA-team kernel.
-template <int DT>
+template <int DT, bool PARTS>
 __device__ __forceinline__ void cta_finish(BlockCtl* c, double* red, uint8_t* stages, uint32_t* sal, bool aborted) {
   __syncthreads();
-  if (c->own != kNoTile && !aborted) cta_phase2<DT>(c, red, stages, sal);
+  if (c->own != kNoTile && !aborted) cta_phase2<DT, PARTS>(c, red, stages, sal);
   else if (threadIdx.x == 0 && has_totals(*cta_totals())) atomicAdd(&c->a.sc->done, 1ull);  // (see queue_entry)
 }
 
@@ -1911,7 +1915,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
         issue(s);  // the stage is free: next load
       }
     } else {  // (the same for every thread) phase 1 of the block-wise path
-      cta_tile_measure<DT>(&s_ctl, s_red, plane, sal, tile, cls | (n_out << 2));
+      cta_tile_measure<DT, true>(&s_ctl, s_red, plane, sal, tile, cls | (n_out << 2));
       if (tid == 0) {
         issue(s);
         queue_push(&s_ctl, tile, s, s_tiles[s] >= pl.ntiles);
@@ -1929,7 +1933,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
         mbar_wait(&s_full[k], 1u, 1u << 10);
       }
   }
-  if (scan_on) cta_finish<DT>(&s_ctl, s_red, smem + pl.sm_tile, sal, s_abort != 0u);
+  if (scan_on) cta_finish<DT, true>(&s_ctl, s_red, smem + pl.sm_tile, sal, s_abort != 0u);
   cta_exit(pl, a, d, &s_last);
 }
 
@@ -1943,11 +1947,12 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
 // 56 elements a lane, and what can wait does: the codes are computed and stored as if the plane were normal while the
 // first warp works out the three-sigma thresholds, and the count of outliers is looked at behind the NEXT plane's
 // first barrier, so that a plane costs three barriers.  A plane that turns out outlier-rich is still in its stage then;
-// it is measured at the end of that turn, and phase 2 rewrites its slot.
+// it is measured at the end of that turn, and phase 2 rewrites its slot.  PARTS: the plane has fewer rows of blocks than the CTA
+// has warps (see fh_blocks.cuh; instances of their own, as the sweep of the others loses 5 % to the registers these take).
 // -------------------------------------------------------------------------------------------------
 constexpr int kCtaThreads = kCtaMaxWarps * 32;
 
-template <int DT, int SIGMA, int K, int EDGE>
+template <int DT, int SIGMA, int K, int EDGE, bool PARTS>
 __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 5];
@@ -2025,7 +2030,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     return false;
   };
   auto measure = [&](uint32_t s) {
-    cta_tile_measure<DT>(&s_ctl, s_red, smem + (uint64_t)s * pl.stage_bytes + plane_head(pl, prev), sal, prev, prev_meta);
+    cta_tile_measure<DT, PARTS>(&s_ctl, s_red, smem + (uint64_t)s * pl.stage_bytes + plane_head(pl, prev), sal, prev, prev_meta);
     if (tid == 0) {
       issue(s);
       queue_push(&s_ctl, prev, s, s_tiles[s] >= pl.ntiles);
@@ -2115,7 +2120,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
         mbar_wait(&s_full[k], 1u, 1u << 10);
       }
   }
-  if (scan_on) cta_finish<DT>(&s_ctl, s_red, smem, sal, s_abort != 0u);
+  if (scan_on) cta_finish<DT, PARTS>(&s_ctl, s_red, smem, sal, s_abort != 0u);
   cta_exit(pl, a, d, &s_last);
 }
 

@@ -48,7 +48,8 @@ struct Plan {
   uint64_t slots_off;    // 64 + 16 P
   uint64_t ovf_off;      // slots_off + P * npay: start of the overflow region
   uint32_t nbx, nby, nblk, nbm;  // 8x8 blocks per row / column / plane, bitmap words
-  uint32_t qs, nsr;              // block-wise path: log2 of the blocks side by side in a step of four, rows of steps
+  uint32_t qs, nsr;              // block-wise path: log2 of the blocks side by side in a step of four, (parts of) rows of steps
+  uint32_t seg, segb;            // ... parts of a row of steps, block columns of a part
   // tiling
   uint32_t ppt;          // planes per tile
   uint32_t ntiles;

@@ -16,14 +16,18 @@ int launch_cta_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
              ? FH_OK : FH_ERR_CUDA;
 }
 
-template <int DT, int SIGMA, int K, int EDGE>
-int launch_cta_regs_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+template <int DT, int SIGMA, int K, int EDGE, bool PARTS>
+int launch_cta_regs_p(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int grid = 0;
-  int rc = grid_for(compress_cta_regs<DT, SIGMA, K, EDGE>, pl.sm_total, pl.ntiles, &grid, (int)pl.team);
+  int rc = grid_for(compress_cta_regs<DT, SIGMA, K, EDGE, PARTS>, pl.sm_total, pl.ntiles, &grid, (int)pl.team);
   if (rc != FH_OK) return rc;
   grid = spread_grid(grid, pl.ntiles);
-  return launch_dependent(compress_cta_regs<DT, SIGMA, K, EDGE>, grid, (int)pl.team, pl.sm_total, stream,
+  return launch_dependent(compress_cta_regs<DT, SIGMA, K, EDGE, PARTS>, grid, (int)pl.team, pl.sm_total, stream,
                           with_first_request(pl, grid, 1), a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+}
+template <int DT, int SIGMA, int K, int EDGE>
+int launch_cta_regs_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+  return pl.seg > 1u ? launch_cta_regs_p<DT, SIGMA, K, EDGE, true>(pl, a, stream) : launch_cta_regs_p<DT, SIGMA, K, EDGE, false>(pl, a, stream);
 }
 
 // Slots per lane; as the CTA has as few warps as hold the plane, a warp's share is 225 to 448 groups (8 to 14 slots).

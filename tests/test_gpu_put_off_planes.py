@@ -84,3 +84,12 @@ def test_channel_statistics_of_a_captured_call(mode, shape):
                 step()
                 assert torch.equal(dst[:want[k].numel()], want[k])
     torch.cuda.synchronize()
+
+
+# fewer rows of blocks than the team has warps: the rows are measured and written in parts
+@pytest.mark.parametrize("shape", [(2, 20, 1, 5000), (1, 12, 8, 1001), (1, 12, 17, 700), (1, 20, 3, 1100), (1, 6, 40, 880)])
+@pytest.mark.parametrize("dtype", [synth.F32, synth.BF16])
+@pytest.mark.parametrize("entropy", [0, 1])
+def test_parity_of_flat_planes(shape, dtype, entropy):
+    full_parity(synth.TensorSpec("t", shape, dtype, "spiky_relu", 46), bits=4, entropy=entropy, salient_mode=api.FH_SALIENT_ALL)
+    full_parity(synth.TensorSpec("t", shape, dtype, "spiky_normal", 47), bits=2, entropy=entropy, eps=0.25)
