@@ -181,8 +181,9 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     // (CTA-team kernels: two stages; a third buys nothing that more resident CTAs do not give)
     const uint32_t ns_max = v.cta ? 2u : (uint32_t)fh::kMaxStages;
     ns = ns < 2 ? 2 : (ns > ns_max ? ns_max : ns);
-    split_rows(v.cta ? pl.team / 32 : 1u);
-    const uint32_t sal_bytes = sal_bytes_of(v.cta ? pl.team / 32 : 1u);
+    const uint32_t warps = v.cta ? pl.team / 32 : 1u;
+    split_rows(warps);
+    uint32_t sal_bytes = sal_bytes_of(warps);
     const uint32_t areas = blockwise ? (v.cta ? 1u : (uint32_t)fh::kWarps) : 0u;
     for (;;) {
       pl.nstage = ns;
@@ -193,11 +194,15 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
       const uint32_t behind = areas * sal_bytes;
       pl.sm_total = pl.sm_sal + (behind > 32u ? behind : 32u);
       if (pl.sm_total <= kSmemLimit) break;
-      if (ns == 2) {  // the pipeline needs two stages
+      if (ns > 2) {
+        --ns;
+      } else if (pl.seg > 1) {  // rows in one part take less scratch
+        split_rows(1u);
+        sal_bytes = sal_bytes_of(warps);
+      } else {  // the pipeline needs two stages
         v.fast = false;
         break;
       }
-      --ns;
     }
   }
   if (!compress) {
@@ -234,7 +239,7 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     pl.nstage = 0;
     pl.stage_bytes = 0;
     split_rows(fh::kWarps);
-    const uint32_t sal_bytes = sal_bytes_of(fh::kWarps);
+    uint32_t sal_bytes = sal_bytes_of(fh::kWarps);
     uint64_t ppt = kTileTarget / pl.plane_bytes;
     if (ppt < 1) ppt = 1;
     if (ppt > kMaxPpt) ppt = kMaxPpt;
@@ -248,8 +253,14 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
       pl.sal_stride = sal_bytes;
       pl.sm_total = pl.sm_sal + (blockwise ? sal_bytes : 0u);
       if (pl.sm_total <= kSmemLimit) break;
-      if (ppt == 1) return FH_ERR_UNSUPPORTED;
-      ppt = ppt / 2;
+      if (ppt > 1) {
+        ppt = ppt / 2;
+      } else if (pl.seg > 1) {
+        split_rows(1u);
+        sal_bytes = sal_bytes_of(fh::kWarps);
+      } else {
+        return FH_ERR_UNSUPPORTED;
+      }
     }
   }
   const uint64_t ntiles = (pl.P + pl.ppt - 1) / pl.ppt;

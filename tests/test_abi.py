@@ -96,3 +96,14 @@ def test_missing_library_fails_loudly(tmp_path, monkeypatch):
 def test_a_schedule_takes_nothing_but_tensor_descriptions(desc):
     with pytest.raises(TypeError, match="fh_tensor_desc"):
         api.fh_run_schedule([api.SchedItem(desc, api.FH_KEEP, None, None)], api.fh_params(), None)
+
+
+@pytest.mark.parametrize("hw,dtype,entropy", [((2, 26795), 0, 0), ((6, 8943), 0, 0), ((16, 3182), 0, 1), ((50, 2023), 1, 0), ((2, 47980), 1, 1)])
+def test_the_largest_planes_are_accepted(lib, hw, dtype, entropy):
+    """Planes that leave a few hundred bytes of shared memory.  (A schedule's entries are checked in order, before any CUDA call:
+    the second one's error says that the first has passed.)"""
+    entries = (api.fh_sched_entry * 2)()
+    entries[0].desc, entries[0].action, entries[0].d_dense, entries[0].d_restored = api.desc((1, 1, *hw), dtype), api.FH_COMPRESS, 256, 256
+    entries[1].action = 99
+    rep, p = api.fh_sched_report(), api.default_params(bits=2, entropy=entropy)
+    assert lib.fh_run_schedule(entries, 2, C.byref(p), 256, 4096, C.byref(rep), None) == api.FH_ERR_ARG
