@@ -10,6 +10,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <tuple>
 #include <utility>
 #include <vector>
@@ -601,8 +602,8 @@ int fh_run_schedule(const fh_sched_entry* entries, int32_t count, const fh_param
     space.reset(s->sched);
     s->sched = nullptr;
   }
-  if (!space) space.reset(new SchedSpace);
-  if (!space->reserve(words)) return FH_ERR_CUDA;
+  if (!space) space.reset(new (std::nothrow) SchedSpace);
+  if (!space || !space->reserve(words)) return FH_ERR_CUDA;
   unsigned long long* d_off = space->words;
   unsigned long long* d_out2 = d_off + (k + 1);
   unsigned long long* d_dst = d_out2 + 2 * k;

@@ -93,3 +93,39 @@ def test_channel_statistics_of_a_captured_call(mode, shape):
 def test_parity_of_flat_planes(shape, dtype, entropy):
     full_parity(synth.TensorSpec("t", shape, dtype, "spiky_relu", 46), bits=4, entropy=entropy, salient_mode=api.FH_SALIENT_ALL)
     full_parity(synth.TensorSpec("t", shape, dtype, "spiky_normal", 47), bits=2, entropy=entropy, eps=0.25)
+
+
+def test_schedules_of_two_host_threads_on_one_stream():
+    """The workspace a stream keeps for the next schedule goes to one caller at a time; schedules of different lengths."""
+    import threading
+    import torch
+    stream, p = torch.cuda.Stream(), api.default_params(bits=4)
+    jobs = []
+    for t, count in enumerate((3, 400)):
+        shape = (2, 16, 14, 14)
+        raws = [to_dev(synth.make(synth.TensorSpec("s", shape, synth.F32, "spiky_relu", 800 + 10 * t + i % 3))) for i in range(count)]
+        items = [api.SchedItem(api.desc(shape, tensor_id=i), api.FH_COMPRESS, x, torch.empty_like(x)) for i, x in enumerate(raws)]
+        arena = torch.zeros(count * ((api.compressed_bytes(items[0].desc, p, 1) + 255) & ~255), dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        rep = api.fh_run_schedule(items, p, arena, stream=stream)
+        assert rep.status == api.FH_OK
+        jobs.append((items, arena, rep.total_packed_bytes, arena.clone(), [i.restored.clone() for i in items]))
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(items, arena, packed, want, restored):
+        for _ in range(20):
+            arena.zero_()
+            items[0].restored.zero_()
+            torch.cuda.synchronize()
+            rep = api.fh_run_schedule(items, p, arena, stream=stream)
+            if (rep.status, rep.total_packed_bytes) != (api.FH_OK, packed) or not torch.equal(arena, want) or \
+                    not all(torch.equal(i.restored, r) for i, r in zip(items, restored)):
+                bad.append(len(items))
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
