@@ -180,13 +180,13 @@ size_t fh_compressed_bytes(const fh_tensor_desc* desc, const fh_params* params, 
  * (i / 4, plane index, tensor_id low, tensor_id high), i the element's index within its plane.  The draw
  * thus depends on (seed, tensor id, element position) only and results are reproducible.  Dense-block codes
  * keep round-to-nearest (their error bound needs it).  One generator call per four elements makes this mode
- * about twice as slow as rounding = 0 (with salient_mode AUTO; other modes run on the general-purpose kernel and are
- * slower still).
+ * up to twice as slow as rounding = 0 (with salient_mode AUTO and planes of up to 35,840 elements; other modes and larger
+ * planes run on the general-purpose kernel and are slower still).
  *
  * entropy = 1 (Section 4.4.1: "a Huffman tree is constructed from the quantization array for encoding"): the
  * residual code bytes of an outlier-rich plane's dense blocks are Huffman-coded, one code per plane (see the
  * container description); the stage is lossless and is skipped for a plane it would not shrink.  The container
- * carries version 2.  This mode runs on the general-purpose kernel and is not tuned.
+ * carries version 2.
  */
 int fh_compress(const fh_tensor_desc* desc, const fh_params* params, const void* d_src, void* d_dst,
                 size_t dst_capacity, uint64_t* d_out2, void* stream);
@@ -199,7 +199,7 @@ int fh_compress(const fh_tensor_desc* desc, const fh_params* params, const void*
  *                      FH_ERR_CORRUPT (reported through d_status, the header lives on the device)
  *   d_dst              dense output, device, 16-byte aligned
  *   d_status           optional uint64 in device (or mapped pinned) memory: (uint64)(int64) status
- * Never reads past src_bytes.  Planes whose table entry is corrupt are left unwritten.
+ * Never reads past src_bytes.  What a plane holds whose table entry or payload is corrupt is unspecified.
  */
 int fh_decompress(const void* d_src, size_t src_bytes, const fh_tensor_desc* expect, void* d_dst,
                   uint64_t* d_status, void* stream);

@@ -56,7 +56,7 @@ using fh::Variant;
 
 constexpr size_t kTileTarget = 32 * 1024;         // dense bytes a tile of the generic kernel aims for
 constexpr size_t kStageTarget = 72 * 1024;        // shared memory the stages of the CTA-team kernel aim for
-constexpr size_t kWarpStageTarget = 72 * 1024;    // ... and those of the warp-team kernel (two CTAs per SM)
+constexpr size_t kWarpStageTarget = 72 * 1024;    // ... and those of the warp-team kernel (three CTAs per SM)
 constexpr uint32_t kMaxPpt = 2048;
 
 std::atomic<uint64_t> g_launches{0};
@@ -158,8 +158,8 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   Variant v;
   // ---- fast compress kernels.  Random rounding runs on the register kernels in the plane-wise three-sigma mode, on the
   // generic kernel otherwise; planes beyond the register kernels' reach on the kernel that sweeps them in shared memory
-  // when they are whole 16-byte chunks.
-  const bool whole16 = pl.HW % 4 == 0 && pl.plane_bytes % 16 == 0;
+  // when they are whole 16-byte chunks (in bf16: two stages of such a plane in fp32 do not fit).
+  const bool whole16 = pl.HW % 4 == 0 && pl.plane_bytes % 16 == 0 && pl.dtype == FH_BF16;
   const bool warp_fits = pl.groups <= 256, regs_fit = pl.groups <= (uint32_t)(fh::kCtaMaxWarps * fh::kCtaGroups);
   if (compress && (pl.rounding == 0 || pl.mode == FH_SALIENT_AUTO) && (warp_fits || regs_fit || (whole16 && pl.rounding == 0))) {
     v.fast = true;
@@ -174,8 +174,8 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
       pl.team = 32u * ((pl.groups + fh::kCtaGroups - 1u) / fh::kCtaGroups);
       pl.stage_bytes = (uint32_t)((pl.plane_bytes + 16 + 127) & ~(uint64_t)127);
     } else {
-      v.cta = true;  // CTA size by plane size: enough work per thread between barriers
-      pl.team = pl.plane_bytes <= 64 * 1024 ? 256 : 512;
+      v.cta = true;
+      pl.team = 512;
       pl.stage_bytes = (uint32_t)((pl.plane_bytes + 127) & ~(uint64_t)127);
     }
     uint32_t ns = (uint32_t)((v.cta ? kStageTarget : kWarpStageTarget) / pl.stage_bytes);

@@ -14,9 +14,9 @@
 //   compress_warp<DT, SIGMA, TT, K, EDGE>   planes of at most 256 groups: bulk-copy (TMA) pipeline, a sub-warp
 //       team per plane, groups kept in registers; a warp handles the outlier-rich planes of its slice;
 //   compress_cta_regs<DT, SIGMA, K, EDGE, PARTS>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
-//   compress_cta<DT, SIGMA, NT>            still larger ones of whole 16-byte chunks: swept in shared memory;
-//   compress_generic<DT, BITS, ROUND>      everything else (still larger ragged planes, random rounding outside the
-//       plane-wise three-sigma mode).
+//   compress_cta<SIGMA>                    still larger bf16 planes of whole 16-byte chunks: swept in shared memory;
+//   compress_generic<DT, BITS, ROUND>      everything else (still larger ragged or fp32 planes, random rounding outside
+//       the plane-wise three-sigma mode).
 // The kernel's last CTA writes the header and the result words and returns the scratch to its idle state.
 #pragma once
 
@@ -435,7 +435,7 @@ struct Rec {
 template <int DT, int BITS, bool ROUND>
 __global__ void __launch_bounds__(kThreads, ROUND ? 4 : 1) compress_generic(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ double s_red[kMaxWarps * 5];
+  __shared__ double s_red[kMaxWarps * 4];
   __shared__ uint32_t s_tile, s_last;
   __shared__ BlockCtl s_ctl;
 
@@ -706,13 +706,6 @@ __device__ __forceinline__ uint32_t max2_nan_bf16(uint32_t a, uint32_t b) {
 
 // Runs of exactly K * TT groups (EDGE 0) start on 16-byte boundaries; in bf16 a lane then takes groups in neighbouring
 // pairs, so that loads are 16 bytes wide and codes leave twice as wide (1 GiB of 32 x 32 planes: 373 -> 342 us).
-// Slot k's group within the run:
-template <int DT, int K, int TT, int EDGE>
-__device__ __forceinline__ uint32_t slot_group(uint32_t lane, int k) {
-  if (DT == kBF16 && EDGE == 0) return 2u * (lane + (uint32_t)((k >> 1) * TT)) + (uint32_t)(k & 1);
-  return lane + (uint32_t)(k * TT);
-}
-
 // Loads the run of `n` elements and takes the lane's minimum and maximum.
 template <int DT, int K, int TT, int EDGE, int GRAIN>
 __device__ __forceinline__ void run_load_as(const uint8_t* p, uint32_t lane, int32_t n, float (&x)[K][4], float& lo, float& hi) {
@@ -1530,12 +1523,10 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
 }
 
 // -------------------------------------------------------------------------------------------------
-// CTA-team kernel: planes of more than 256 groups (whole 16-byte chunks).  One plane per tile, all
-// NT threads of the CTA work on it.  The plane stays in its shared-memory stage and is swept two or
-// three times (min/max; integer moments; count + codes), so that few registers are needed and
-// shared memory alone limits how many CTAs fit an SM (two stages each).  What every warp repeats per
-// plane -- reductions, thresholds, quantiser parameters -- does not shrink with the warp's share of the
-// plane, so NT is kept small for small planes.  Thread 0 keeps the next ticket in flight while the CTA works.
+// CTA-team kernel: bf16 planes beyond the register variant's reach, of whole 16-byte chunks (of such a plane in fp32 two
+// stages do not fit).  One plane per tile, all threads of the CTA work on it.  The plane stays in its shared-memory stage
+// and is swept two or three times (min/max; integer moments; count + codes), so that few registers are needed.
+// A warp has at most 892 groups, whose integer sums fit 32 bits.  Thread 0 keeps the next ticket in flight while the CTA works.
 // An outlier-rich plane is measured by the whole CTA while it lies in its stage and written in phase 2.
 // -------------------------------------------------------------------------------------------------
 // Phase 1: the plane in `plane` is measured, tile (= plane) `tile` published.  Ends with a barrier.
@@ -1696,21 +1687,14 @@ __device__ __forceinline__ void cta_finish(BlockCtl* c, double* red, uint8_t* st
   else if (threadIdx.x == 0 && has_totals(*cta_totals())) atomicAdd(&c->a.sc->done, 1ull);  // (see queue_entry)
 }
 
-template <int DT>
 __device__ __forceinline__ void lds_group(const uint8_t* plane, uint32_t g, float (&v)[4]) {
-  if (DT == kF32) {
-    const float4 t4 = reinterpret_cast<const float4*>(plane)[g];
-    v[0] = t4.x; v[1] = t4.y; v[2] = t4.z; v[3] = t4.w;
-  } else {
-    const uint2 t2 = reinterpret_cast<const uint2*>(plane)[g];
-    v[0] = __uint_as_float(t2.x << 16); v[1] = __uint_as_float(t2.x & 0xFFFF0000u);
-    v[2] = __uint_as_float(t2.y << 16); v[3] = __uint_as_float(t2.y & 0xFFFF0000u);
-  }
+  const uint2 t2 = reinterpret_cast<const uint2*>(plane)[g];
+  v[0] = __uint_as_float(t2.x << 16); v[1] = __uint_as_float(t2.x & 0xFFFF0000u);
+  v[2] = __uint_as_float(t2.y << 16); v[3] = __uint_as_float(t2.y & 0xFFFF0000u);
 }
 // The group's distances from lo (x - lo is x + (-lo): the same rounding).
-template <int DT>
 __device__ __forceinline__ void lds_dist(const uint8_t* plane, uint32_t g, float nlo, float (&v)[4]) {
-  lds_group<DT>(plane, g, v);
+  lds_group(plane, g, v);
   const f32x2 nlo2 = pack2(nlo, nlo);
   unpack2(add2(pack2(v[0], v[1]), nlo2), v[0], v[1]);
   unpack2(add2(pack2(v[2], v[3]), nlo2), v[2], v[3]);
@@ -1722,7 +1706,7 @@ __device__ __forceinline__ void lds_dist(const uint8_t* plane, uint32_t g, float
     const f32x2 inv2 = pack2(inv, inv), mag2 = pack2(kMagicF, kMagicF);                                         \
     _Pragma("unroll 2") for (uint32_t g = tid; g < groups; g += NT) {                                         \
       float v[4];                                                                                             \
-      lds_dist<DT>(plane, g, nlo, v);                                                                         \
+      lds_dist(plane, g, nlo, v);                                                                         \
       uint32_t w0, w1, w2, w3;                                                                                \
       unpack2u(fma2(pack2(v[0], v[1]), inv2, mag2), w0, w1);                                                  \
       unpack2u(fma2(pack2(v[2], v[3]), inv2, mag2), w2, w3);                                                  \
@@ -1742,11 +1726,14 @@ __device__ __forceinline__ void lds_dist(const uint8_t* plane, uint32_t g, float
     }                                                                                                         \
   }
 
-template <int DT, bool SIGMA, int NT>
-__global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const CompressArgs a) {
+constexpr int kSweepThreads = 512;
+
+template <bool SIGMA>
+__global__ void __launch_bounds__(kSweepThreads) compress_cta(const Plan pl, const CompressArgs a) {
+  constexpr int DT = kBF16, NT = kSweepThreads;
   constexpr bool COUNT = SIGMA;
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ double s_red[kMaxWarps * 5];
+  __shared__ double s_red[kMaxWarps * 4];
   __shared__ __align__(8) uint64_t s_full[kMaxStages];
   __shared__ uint32_t s_tiles[kMaxStages];
   __shared__ uint32_t s_abort, s_last;
@@ -1818,11 +1805,11 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
 #pragma unroll 2
       for (uint32_t g = tid; g < groups; g += 2 * NT) {
         float v[4];
-        lds_group<DT>(plane, g, v);
+        lds_group(plane, g, v);
         lo = min_nan(lo, min_nan(min3_nan(v[0], v[1], v[2]), v[3]));
         hi = max_nan(hi, max_nan(max3_nan(v[0], v[1], v[2]), v[3]));
         if (g + NT < groups) {
-          lds_group<DT>(plane, g + NT, v);
+          lds_group(plane, g + NT, v);
           lo1 = min_nan(lo1, min_nan(min3_nan(v[0], v[1], v[2]), v[3]));
           hi1 = max_nan(hi1, max_nan(max3_nan(v[0], v[1], v[2]), v[3]));
         }
@@ -1845,7 +1832,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
 #pragma unroll 2
         for (uint32_t g = tid; g < groups; g += NT) {
           float v[4];
-          lds_dist<DT>(plane, g, nlo, v);
+          lds_dist(plane, g, nlo, v);
           sigma_addends4(v[0], v[1], v[2], v[3], sc, as, aq);
           ++ng;
         }
@@ -1894,7 +1881,7 @@ __global__ void __launch_bounds__(NT) compress_cta(const Plan pl, const Compress
     } else if (SIGMA && need_count) {  // nothing may be stored: count only
       for (uint32_t g = tid; g < groups; g += NT) {
         float v[4];
-        lds_dist<DT>(plane, g, nlo, v);
+        lds_dist(plane, g, nlo, v);
 #pragma unroll
         for (int e = 0; e < 4; ++e) c0 += (v[e] > dhi) || (v[e] < dlo);
       }
@@ -1955,7 +1942,7 @@ constexpr int kCtaThreads = kCtaMaxWarps * 32;
 template <int DT, int SIGMA, int K, int EDGE, bool PARTS>
 __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ double s_red[kMaxWarps * 5];
+  __shared__ double s_red[kMaxWarps * 4];
   __shared__ __align__(8) uint64_t s_full[2];
   __shared__ uint32_t s_tiles[2], s_abort, s_last, s_count[2];
   __shared__ float2 s_thr;

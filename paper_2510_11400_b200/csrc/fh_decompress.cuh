@@ -2,8 +2,8 @@
 //
 // Planes are independent and their slots sit at closed-form offsets, so the kernels need no hand-out.  Normal planes
 // are the fused unpack-and-dequantise: codes are read straight from the slot (they are 1/16 to 1/4 of the output) and
-// leave as 16-byte stores.  Raw planes are copied; outlier-rich planes are restored four blocks per warp and step
-// (decode_salient).  Every read of the container is bounds-checked against src_bytes; a plane whose table entry or
+// leave as 16-byte stores.  Raw planes are copied; outlier-rich planes are restored a lane per dense block (decode_salient),
+// small ones four blocks per warp and step (decode_few).  Every read of the container is bounds-checked against src_bytes; a plane whose table entry or
 // payload is inconsistent reports FH_ERR_CORRUPT.
 #pragma once
 
@@ -626,7 +626,7 @@ __device__ __forceinline__ void decode_chunk_shifted(const uint8_t* slot, uint32
 template <int DT>
 __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, const DecompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ double s_red[kMaxWarps * 5];
+  __shared__ double s_red[kMaxWarps * 4];
   __shared__ uint32_t s_hdr_ok, s_bits;
   __shared__ float s_eps;
   __shared__ unsigned long long s_total;

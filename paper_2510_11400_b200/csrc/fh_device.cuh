@@ -11,7 +11,7 @@
 
 namespace fh {
 
-constexpr int kThreads = 256;             // CTA size of every kernel
+constexpr int kThreads = 256;             // CTA size, but for the CTA-team kernels' and the warp-team kernel's producer warp
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxWarps = 20;            // largest CTA of any kernel: 640 threads
 constexpr int kCtaMaxWarps = 20;         // CTA-team kernel, register variant: warps of a CTA at most ...
@@ -92,14 +92,6 @@ __device__ __forceinline__ uint32_t a4(uint32_t x) { return (x + 3u) & ~3u; }
 __device__ __forceinline__ uint32_t a16(uint32_t x) { return (x + 15u) & ~15u; }
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
 __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -208,7 +200,6 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c) {
 }
 
 __device__ __forceinline__ float bf16_bits_to_f32(uint32_t h) { return __uint_as_float(h << 16); }
-// fp32 -> bf16 bits, round half to even (finite inputs).
 // fp32 -> bf16, round to nearest even (the hardware conversion; the values converted here are never NaN).
 __device__ __forceinline__ uint32_t f32_to_bf16_bits(float f) {
   uint16_t r;
@@ -389,7 +380,7 @@ struct Team {
   uint32_t mask;   // warp member mask of the team (sub-warp teams)
   bool block;      // the team is the whole CTA
   uint32_t nwarps; // warps of a CTA team
-  double* red;     // shared scratch for CTA-wide reductions: kMaxWarps * 5 doubles (see red_half, team_excl_scan)
+  double* red;     // shared scratch for CTA-wide reductions: kMaxWarps * 4 doubles (see red_half)
 };
 
 __device__ __forceinline__ Team make_team(uint32_t team_size, double* red) {
@@ -554,60 +545,6 @@ __device__ __forceinline__ uint32_t team_sum_u32(const Team& t, uint32_t v, uint
     asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(v) : "r"(0xFFFFFFFFu));
   }
   return v;
-}
-
-// In-place exclusive prefix sum of arr[0..n) (shared memory) by the team; returns the total.
-// Every lane takes a contiguous chunk; chunk sums are scanned across the team.
-__device__ __forceinline__ uint32_t team_excl_scan(const Team& t, uint32_t* arr, uint32_t n) {
-  if (!t.block && t.size == 32u && n <= 32u) {  // a warp and at most one element per lane: one shuffle scan
-    const uint32_t v = t.lane < n ? arr[t.lane] : 0u;
-    uint32_t incl = v;
-    for (uint32_t o = 1; o < 32u; o <<= 1) {
-      const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (t.lane >= o) incl += up;
-    }
-    if (t.lane < n) arr[t.lane] = incl - v;
-    __syncwarp();
-    return __shfl_sync(0xFFFFFFFFu, incl, 31);
-  }
-  const uint32_t chunk = (n + t.size - 1u) / t.size;
-  const uint32_t b = min(t.lane * chunk, n), e = min(b + chunk, n);
-  uint32_t local = 0;
-  for (uint32_t i = b; i < e; ++i) local += arr[i];
-  uint32_t incl = local, total;
-  if (!t.block) {
-    for (uint32_t o = 1; o < t.size; o <<= 1) {
-      const uint32_t up = __shfl_up_sync(t.mask, incl, o, t.size);
-      if (t.lane >= o) incl += up;
-    }
-    total = __shfl_sync(t.mask, incl, t.size - 1u, t.size);
-  } else {
-    uint32_t* r = reinterpret_cast<uint32_t*>(t.red + kMaxWarps * 4);  // region of its own, behind the two halves
-    const uint32_t wl = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    for (uint32_t o = 1; o < 32u; o <<= 1) {
-      const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (wl >= o) incl += up;
-    }
-    __syncthreads();
-    if (wl == 31u) r[warp] = incl;
-    __syncthreads();
-    uint32_t base = 0;
-    total = 0;
-    for (uint32_t k = 0; k < t.nwarps; ++k) {
-      if (k < warp) base += r[k];
-      total += r[k];
-    }
-    incl += base;
-  }
-  uint32_t run = incl - local;
-  team_sync(t);  // all chunk sums are read before anybody overwrites
-  for (uint32_t i = b; i < e; ++i) {
-    const uint32_t v = arr[i];
-    arr[i] = run;
-    run += v;
-  }
-  team_sync(t);
-  return total;
 }
 
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {

@@ -73,10 +73,6 @@ int grid_for(K kernel, size_t smem, uint32_t ntiles, int* grid, int threads = fh
   return FH_OK;
 }
 
-// Launch that may overlap the tail of the previous kernel on the stream: every kernel of this library
-// passes dep_wait() before it touches global memory, so stream order is kept.
-// Tiles a CTA requests at once when it starts: all its stages when every CTA of the grid gets that many, fewer
-// when the tensor is small, so that the tiles spread over all CTAs before any CTA takes a second one.
 // Grid of a compress kernel that hands out tiles in order: when every CTA gets several, a prime number of CTAs.  Equally
 // fast CTAs then take tiles c, c + grid, ..., and a periodic pattern of outlier-rich planes -- every eighth channel, say --
 // spreads over all of them instead of landing on the few whose index shares a factor with the period (with 296 CTAs and
@@ -85,6 +81,8 @@ inline int spread_grid(int grid, uint32_t ntiles) {
   return ntiles >= 2u * (uint32_t)grid && grid >= 2 ? (int)prime_at_most((uint64_t)grid) : grid;
 }
 
+// Tiles a CTA requests at once when it starts: all its stages when every CTA of the grid gets that many, fewer
+// when the tensor is small, so that the tiles spread over all CTAs before any CTA takes a second one.
 inline Plan with_first_request(const Plan& pl, int grid, uint32_t least) {
   Plan q = pl;
   const uint32_t each = pl.ntiles / (uint32_t)(grid > 0 ? grid : 1);
@@ -92,6 +90,8 @@ inline Plan with_first_request(const Plan& pl, int grid, uint32_t least) {
   return q;
 }
 
+// Launch that may overlap the tail of the previous kernel on the stream: every kernel of this library
+// passes dep_wait() before it touches global memory, so stream order is kept.
 template <typename K, typename A>
 cudaError_t launch_dependent(K kernel, int grid, int threads, size_t smem, cudaStream_t stream, const Plan& pl,
                              const A& a) {

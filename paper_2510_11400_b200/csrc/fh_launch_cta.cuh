@@ -6,13 +6,13 @@
 
 namespace fh {
 
-template <int DT, bool SIGMA, int NT>
+template <bool SIGMA>
 int launch_cta_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   int grid = 0;
-  int rc = grid_for(compress_cta<DT, SIGMA, NT>, pl.sm_total, pl.ntiles, &grid, NT);
+  int rc = grid_for(compress_cta<SIGMA>, pl.sm_total, pl.ntiles, &grid, kSweepThreads);
   if (rc != FH_OK) return rc;
   grid = spread_grid(grid, pl.ntiles);
-  return launch_dependent(compress_cta<DT, SIGMA, NT>, grid, NT, pl.sm_total, stream, with_first_request(pl, grid, 2), a) == cudaSuccess
+  return launch_dependent(compress_cta<SIGMA>, grid, kSweepThreads, pl.sm_total, stream, with_first_request(pl, grid, 2), a) == cudaSuccess
              ? FH_OK : FH_ERR_CUDA;
 }
 
@@ -41,19 +41,13 @@ int launch_cta_regs(const Plan& pl, const CompressArgs& a, cudaStream_t stream) 
   return launch_cta_regs_t<DT, SIGMA, 14, 1>(pl, a, stream);
 }
 
-template <int DT, bool SIGMA>
-int launch_cta_g(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
-  switch (pl.team) {
-    case 256: return launch_cta_t<DT, SIGMA, 256>(pl, a, stream);
-    case 512: return launch_cta_t<DT, SIGMA, 512>(pl, a, stream);
-  }
-  return FH_ERR_UNSUPPORTED;
-}
-
 template <int DT>
 int launch_compress_cta(const Plan& pl, const Variant& v, const CompressArgs& a, cudaStream_t stream) {
   const bool sigma = pl.mode == FH_SALIENT_AUTO;
-  if (!v.regs) return sigma ? launch_cta_g<DT, true>(pl, a, stream) : launch_cta_g<DT, false>(pl, a, stream);
+  if (!v.regs) {
+    if constexpr (DT == kBF16) return sigma ? launch_cta_t<true>(pl, a, stream) : launch_cta_t<false>(pl, a, stream);
+    return FH_ERR_UNSUPPORTED;  // (make_plan sends them elsewhere)
+  }
   if (!sigma) return launch_cta_regs<DT, 0>(pl, a, stream);
   return pl.rounding ? launch_cta_regs<DT, 2>(pl, a, stream) : launch_cta_regs<DT, 1>(pl, a, stream);
 }

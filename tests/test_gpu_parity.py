@@ -97,8 +97,8 @@ SHAPES = [
     (2, 6, 33, 17),    # ragged 8x8 blocks in both directions
     (1, 12, 32, 32),   # one warp per plane, vector loads
     (2, 8, 28, 28),
-    (1, 6, 56, 56),    # whole-CTA teams of 128 threads
-    (1, 3, 112, 112),  # whole-CTA teams of 512 threads
+    (1, 6, 56, 56),    # a CTA of two warps per plane
+    (1, 3, 112, 112),  # a CTA of seven
     (1, 2, 64, 100),
     (1, 2, 128, 120),  # 60 KB planes
     (300, 1, 4, 4),    # many tiny planes, several tiles with a ragged last tile
@@ -114,17 +114,16 @@ def test_parity_auto_mode_mixed_planes(shape, dtype, bits):
     full_parity(spec, bits=bits)
 
 
-# Planes of 257 to 4096 groups run on the CTA-team kernel that keeps a thread's groups in registers: one shape per
-# (threads, groups per thread) it is built for, each with a plane that fills the threads exactly and one that does
-# not, and one shape beyond it (the kernel that sweeps the plane in shared memory).
+# Planes of 257 to 8960 groups run on the CTA-team kernel that keeps its warps' groups in registers, as few warps as hold the
+# plane: one to fifteen of them, shares that fill the warps exactly (112 x 112) and shares that do not.
 CTA_SHAPES = [
-    (1, 4, 56, 64), (1, 4, 57, 60),      # 896 groups = 128 x 7; 855
-    (1, 4, 64, 64), (1, 4, 40, 100),     # 1024 = 128 x 8; 1000
-    (1, 4, 64, 112), (1, 4, 60, 100),    # 1792 = 256 x 7; 1500
-    (1, 4, 128, 64), (1, 4, 80, 100),    # 2048 = 256 x 8; 2000
-    (1, 4, 112, 112), (1, 4, 100, 120),  # 3136 = 448 x 7; 3000
-    (1, 4, 128, 128), (1, 4, 100, 160),  # 4096 = 512 x 8; 4000
-    (1, 3, 160, 164),                    # 6560 groups: beyond the register variant
+    (1, 4, 56, 64), (1, 4, 57, 60),      # 896 groups = 2 warps x 448; 855
+    (1, 4, 64, 64), (1, 4, 40, 100),     # 1024; 1000
+    (1, 4, 64, 112), (1, 4, 60, 100),    # 1792 = 4 x 448; 1500
+    (1, 4, 128, 64), (1, 4, 80, 100),    # 2048; 2000
+    (1, 4, 112, 112), (1, 4, 100, 120),  # 3136 = 7 x 448; 3000
+    (1, 4, 128, 128), (1, 4, 100, 160),  # 4096; 4000
+    (1, 3, 160, 164),                    # 6560: 15 warps
 ]
 
 

@@ -28,3 +28,11 @@ def test_parity_at_the_edges_of_the_sweep(hw, dtype):
 @pytest.mark.parametrize("hw", [(128, 280), (191, 187), (160, 228), (191, 191)])  # 35,840 elements and beyond: other kernels
 def test_parity_beyond_the_register_kernel(hw):
     full_parity(synth.TensorSpec("t", (1, 3, *hw), synth.BF16, "spiky_relu", 35), bits=4)
+
+
+# planes beyond the register kernel in fp32 (the general-purpose kernel), and the widest and tallest that fit
+@pytest.mark.parametrize("hw,dtype", [((160, 228), synth.F32), ((191, 187), synth.F32), ((224, 224), synth.F32), ((1, 50614), synth.F32),
+                                      ((2, 35544), synth.BF16), ((30000, 1), synth.BF16), ((300, 300), synth.BF16)])
+def test_parity_of_the_largest_planes(hw, dtype):
+    full_parity(synth.TensorSpec("t", (1, 9, *hw), dtype, "spiky_relu", 36), bits=2)
+    full_parity(synth.TensorSpec("t", (1, 9, *hw), dtype, "relu", 37), bits=2, rounding=1, seed=7)
