@@ -9,9 +9,9 @@ one (reverse order), salient_mode AUTO.  The headline workload is the ResNet-18-
 activations at batch 64 (17 fp32 tensors, 563.5 MiB dense).  `value` is dense GB/s: the dense bytes
 that went through compress plus those that came out of decompress, divided by the device time.
 
-Beside the headline the line carries `sweep` (the size sweep of configs[3]: single tensors of 64 MiB, 256 MiB and
+Beside the headline the line carries `sweep` (a size sweep: single tensors of 64 MiB, 256 MiB and
 1 GiB, fp32 and bf16, compress and decompress timed separately over copies that do not fit the L2 cache),
-`schedule` (configs[4] through fh_run_schedule) and `parity_checked` (status words re-read after the timed
+`schedule` (20 CIFAR-ResNet-shaped tensors through fh_run_schedule) and `parity_checked` (status words re-read after the timed
 region and one tensor's container per code width compared byte for byte with the CPU oracle).
 
 One JSON line goes to stdout (rank 0).  With N > 1 (launched by torchrun) every rank runs the
@@ -47,22 +47,22 @@ UNIT = "GB/s"
 
 def workload_specs(name: str):
     if name == "resnet18_b64":
-        return synth.config2(64), "configs[1]: ResNet-18-shaped saved activations, batch 64, 224x224 input, fp32, " \
+        return synth.config2(64), "ResNet-18-shaped saved activations, batch 64, 224x224 input, fp32, " \
                                   "17 tensors, 563.5 MiB dense; even tensors ReLU(N(0,1)), odd N(0,1)"
     if name == "mobilenetv2_b128":
-        return synth.config3(128), "configs[2]: MobileNetV2-shaped expanded activations, batch 128, bf16, Laplace(0,1) " \
+        return synth.config3(128), "MobileNetV2-shaped expanded activations, batch 128, bf16, Laplace(0,1) " \
                                    "with channel-clustered +-50 outliers"
     if name == "mobilenetv2_b128_iid":
-        return synth.config3(128, stress=True), "configs[2]: MobileNetV2-shaped expanded activations, batch 128, bf16, " \
+        return synth.config3(128, stress=True), "MobileNetV2-shaped expanded activations, batch 128, bf16, " \
                                                 "Laplace(0,1) with 1 % outliers at +-50, independent per element"
     if name == "cifar_schedule":
-        return synth.config5(128), "configs[4]: 20 ResNet-18/CIFAR-shaped tensors, batch 128, fp32"
+        return synth.config5(128), "20 ResNet-18/CIFAR-shaped tensors, batch 128, fp32"
     if name == "config1":
-        return synth.config1(), "configs[0]: 32x16x32x32 fp32 ReLU(N(0,1))"
+        return synth.config1(), "32x16x32x32 fp32 ReLU(N(0,1))"
     if name.startswith("sweep_"):          # sweep_<MiB>_<f32|bf16>
         _, mib, dt = name.split("_")
         return synth.config4(int(mib), synth.F32 if dt == "f32" else synth.BF16), \
-            f"configs[3]: single {mib} MiB {dt} tensor of 32x32 planes, ReLU(N(0,1))"
+            f"single {mib} MiB {dt} tensor of 32x32 planes, ReLU(N(0,1))"
     if name.startswith("shape_"):          # shape_<n>x<c>x<h>x<w>_<f32|bf16>_<kind>: one tensor, for profiling
         _, dims, dt, kind = name.split("_", 3)
         shape = tuple(int(v) for v in dims.split("x"))
@@ -246,7 +246,7 @@ def run_reference(args, specs, wl_desc):
 # ------------------------------------------------------------------------------------------------
 
 def size_sweep(api, peak, mibs=(64, 256, 1024), repeats=20):
-    """configs[3]: single tensors of 32x32 planes, ReLU(N(0,1)), 2 bits, three-sigma mode; compress and
+    """single tensors of 32x32 planes, ReLU(N(0,1)), 2 bits, three-sigma mode; compress and
     decompress timed separately with CUDA events over back-to-back calls on copies that together exceed the L2
     cache.  fraction = (dense + container bytes) / time / measured copy bandwidth."""
     import ctypes as C
@@ -298,7 +298,7 @@ def size_sweep(api, peak, mibs=(64, 256, 1024), repeats=20):
 
 
 def schedule_leg(api, mode, repeats=20):
-    """configs[4]: the 20 CIFAR-ResNet-shaped tensors at batch 128, every other one compressed, through
+    """the 20 CIFAR-ResNet-shaped tensors at batch 128, every other one compressed, through
     fh_run_schedule (forward-order compress, reverse-order decompress, one stream)."""
     import torch
     specs = synth.config5(128)
