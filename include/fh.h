@@ -28,6 +28,9 @@
  *     tensor seen: the words through which tiles tell one another where their payloads go)
  *     that it creates on first use and frees in fh_shutdown(); growing it for a tensor with more
  *     planes synchronises the device once.
+ *   - Calls may be captured once their stream's scratch exists.  A captured fh_compress is not meant to be replayed on
+ *     values with outlier-rich planes: their places are found by words that carry the call's number, which a replay
+ *     repeats.
  *   - There is no CPU fallback: without a CUDA device every entry point that does work returns
  *     FH_ERR_CUDA.
  *
