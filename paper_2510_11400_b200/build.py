@@ -11,8 +11,9 @@ from concurrent.futures import ThreadPoolExecutor
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfh_sm100a.so")
-SOURCES = [os.path.join(CSRC, f) for f in ("fh.cu", "fh_warp_f32.cu", "fh_warp_bf16.cu", "fh_cta_f32.cu", "fh_cta_bf16.cu",
-                                          "fh_generic.cu", "fh_decompress.cu", "fh_plan.cpp")]
+SOURCES = [os.path.join(CSRC, f) for f in ("fh_warp_f32.cu", "fh_warp_bf16.cu", "fh_warp_f32_plain.cu", "fh_warp_bf16_plain.cu",
+                                          "fh_warp_f32_random.cu", "fh_warp_bf16_random.cu", "fh_cta_f32.cu", "fh_cta_bf16.cu",
+                                          "fh_generic.cu", "fh_decompress.cu", "fh.cu", "fh_plan.cpp")]
 HEADERS = [os.path.join(CSRC, f) for f in ("fh_device.cuh", "fh_blocks.cuh", "fh_channel.cuh", "fh_compress.cuh",
                                           "fh_decompress.cuh", "fh_launch.cuh", "fh_launch_cta.cuh",
                                           "fh_launch_warp.cuh")] + \

@@ -433,9 +433,12 @@ int get_channel_scratch(StreamScratch* s, size_t planes, size_t channels, cudaSt
 
 int launch_compress(const Plan& pl, const Variant& v, const fh::CompressArgs& a, cudaStream_t stream) {
   const bool f32 = pl.dtype == FH_F32;
-  const int rc = !v.fast ? fh::launch_compress_generic(pl, a, stream)
-                 : v.cta ? (f32 ? fh::launch_compress_cta_f32(pl, v, a, stream) : fh::launch_compress_cta_bf16(pl, v, a, stream))
-                         : (f32 ? fh::launch_compress_warp_f32(pl, a, stream) : fh::launch_compress_warp_bf16(pl, a, stream));
+  int rc;
+  if (!v.fast) rc = fh::launch_compress_generic(pl, a, stream);
+  else if (v.cta) rc = f32 ? fh::launch_compress_cta_f32(pl, v, a, stream) : fh::launch_compress_cta_bf16(pl, v, a, stream);
+  else if (pl.mode != FH_SALIENT_AUTO) rc = f32 ? fh::launch_compress_warp_f32_plain(pl, a, stream) : fh::launch_compress_warp_bf16_plain(pl, a, stream);
+  else if (pl.rounding) rc = f32 ? fh::launch_compress_warp_f32_random(pl, a, stream) : fh::launch_compress_warp_bf16_random(pl, a, stream);
+  else rc = f32 ? fh::launch_compress_warp_f32(pl, a, stream) : fh::launch_compress_warp_bf16(pl, a, stream);
   if (rc == FH_OK) g_launches.fetch_add(1);
   return rc;
 }

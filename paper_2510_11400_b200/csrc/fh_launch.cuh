@@ -40,8 +40,13 @@ int sm_count();
 uint64_t prime_at_most(uint64_t n);
 
 // All of these enqueue on `stream` and return an fh_status; the caller holds the library's mutex.
+// (Warp-team kernels: with the plane-wise three-sigma rule, without it, and with it and random rounding.)
 int launch_compress_warp_f32(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
+int launch_compress_warp_f32_plain(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
+int launch_compress_warp_f32_random(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
 int launch_compress_warp_bf16(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
+int launch_compress_warp_bf16_plain(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
+int launch_compress_warp_bf16_random(const Plan& pl, const CompressArgs& a, cudaStream_t stream);
 int launch_compress_cta_f32(const Plan& pl, const Variant& v, const CompressArgs& a, cudaStream_t stream);
 int launch_compress_cta_bf16(const Plan& pl, const Variant& v, const CompressArgs& a, cudaStream_t stream);
 int launch_compress_generic(const Plan& pl, const CompressArgs& a, cudaStream_t stream);

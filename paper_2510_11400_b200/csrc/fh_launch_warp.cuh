@@ -17,22 +17,28 @@ int launch_warp_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   return launch_dependent(compress_warp<DT, SIGMA, TT, K, EDGE>, grid, kWarpKernelThreads, pl.sm_total, stream, q, a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
 
-// Slots per lane: the team is the smallest that holds the plane, so (teams of two and more) at least four are whole;
-// seven with three of them masked (7 x 7, 14 x 14 and 28 x 28 take seven), eight with one, or exactly eight (8 x 8,
-// 16 x 16, 32 x 32).
+// Slots per lane.  The team is the smallest that holds the plane in eight slots, so teams of two and more need five to eight: as
+// many as the plane needs, of which all but the last are whole.  (Seven slots, three of them masked, for whatever needs five to
+// seven took 112 us for 2,048 x 64 fp32 planes of 24 x 24, five take 100; 28 x 28, seven with one masked: 58.9 -> 55.8 us for
+// 1,024 x 64 planes; bf16: 97.8 -> 83.5 and 57.7 -> 54.3.)
 template <int DT, int SIGMA, int TT>
 int launch_warp_k(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   if constexpr (TT == 1) {
     if (pl.HW == 16u) return launch_warp_t<DT, SIGMA, 1, 4, 0>(pl, a, stream);
     return pl.groups <= 4u ? launch_warp_t<DT, SIGMA, 1, 4, 4>(pl, a, stream) : launch_warp_t<DT, SIGMA, 1, 8, 4>(pl, a, stream);
   } else {
-    if (pl.HW == 32u * TT) return launch_warp_t<DT, SIGMA, TT, 8, 0>(pl, a, stream);
-    return pl.groups <= 7u * TT ? launch_warp_t<DT, SIGMA, TT, 7, 3>(pl, a, stream) : launch_warp_t<DT, SIGMA, TT, 8, 1>(pl, a, stream);
+    if (pl.HW == 32u * TT) return launch_warp_t<DT, SIGMA, TT, 8, 0>(pl, a, stream);  // (8 x 8, 16 x 16, 32 x 32)
+    switch ((pl.groups + TT - 1u) / TT) {
+      case 5: return launch_warp_t<DT, SIGMA, TT, 5, 1>(pl, a, stream);
+      case 6: return launch_warp_t<DT, SIGMA, TT, 6, 1>(pl, a, stream);
+      case 7: return launch_warp_t<DT, SIGMA, TT, 7, 1>(pl, a, stream);  // (7 x 7, 14 x 14, 28 x 28)
+      default: return launch_warp_t<DT, SIGMA, TT, 8, 1>(pl, a, stream);
+    }
   }
 }
 
 template <int DT, int SIGMA>
-int launch_warp_s(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+int launch_compress_warp(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   switch (pl.team) {
     case 1: return launch_warp_k<DT, SIGMA, 1>(pl, a, stream);
     case 2: return launch_warp_k<DT, SIGMA, 2>(pl, a, stream);
@@ -42,12 +48,6 @@ int launch_warp_s(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
     case 32: return launch_warp_k<DT, SIGMA, 32>(pl, a, stream);
   }
   return FH_ERR_UNSUPPORTED;
-}
-
-template <int DT>
-int launch_compress_warp(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
-  if (pl.mode != FH_SALIENT_AUTO) return launch_warp_s<DT, 0>(pl, a, stream);
-  return pl.rounding ? launch_warp_s<DT, 2>(pl, a, stream) : launch_warp_s<DT, 1>(pl, a, stream);
 }
 
 }  // namespace fh

@@ -1,0 +1,5 @@
+#include "fh_launch_warp.cuh"
+
+int fh::launch_compress_warp_bf16_random(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+  return launch_compress_warp<kBF16, 2>(pl, a, stream);
+}

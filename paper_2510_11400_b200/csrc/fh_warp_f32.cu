@@ -1,5 +1,5 @@
 #include "fh_launch_warp.cuh"
 
 int fh::launch_compress_warp_f32(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
-  return launch_compress_warp<kF32>(pl, a, stream);
+  return launch_compress_warp<kF32, 1>(pl, a, stream);
 }

@@ -25,6 +25,20 @@ def test_parity_at_the_edges_of_the_sweep(hw, dtype):
     full_parity(synth.TensorSpec("t", shape, dtype, "relu", 34), bits=8, salient_mode=api.FH_SALIENT_OFF)
 
 
+# the first and the last plane size of five, six and seven slots to a lane, teams of 2, 8 and 32 lanes
+SLOTS = [(1, 33), (5, 8), (1, 41), (6, 8), (7, 7), (1, 56), (3, 43), (10, 16), (7, 23), (12, 16), (1, 193), (14, 16),
+         (27, 19), (20, 32), (1, 641), (24, 32), (1, 769), (28, 32)]
+
+
+@pytest.mark.parametrize("hw", SLOTS)
+@pytest.mark.parametrize("dtype", [synth.F32, synth.BF16])
+def test_parity_at_the_edges_of_the_slots(hw, dtype):
+    shape = (1, 23, *hw)
+    full_parity(synth.TensorSpec("t", shape, dtype, "normal", 41), bits=4)
+    full_parity(synth.TensorSpec("t", shape, dtype, "spiky_relu", 42), bits=2, rounding=1, seed=5)
+    full_parity(synth.TensorSpec("t", shape, dtype, "relu", 43), bits=8, salient_mode=api.FH_SALIENT_ALL)
+
+
 @pytest.mark.parametrize("hw", [(128, 280), (191, 187), (160, 228), (191, 191)])  # 35,840 elements and beyond: other kernels
 def test_parity_beyond_the_register_kernel(hw):
     full_parity(synth.TensorSpec("t", (1, 3, *hw), synth.BF16, "spiky_relu", 35), bits=4)
