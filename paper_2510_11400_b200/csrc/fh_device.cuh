@@ -357,18 +357,33 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
   out[2] = c2;
   out[3] = c3;
 }
-// Code of one element (distance d = x - lo) under random rounding: t = fp32 product d * inv, n = floor(t), and the code
-// goes up iff floor(frac(t) * 2^24) + r reaches 2^24, r = word >> 8; as r is an integer, the code is floor(t + r * 2^-24),
-// exactly.  With sums rounded down: the floor of a sum is not changed by rounding it down (every integer here is a
-// number of fp32), so r's upper 23 bits are added as 1 + a * 2^-23 by bit pattern, and 2^23 after that leaves the floor
-// in the mantissa.  The lowest bit goes in first, at 2^-24: what rounding down takes from that sum lies below its grid,
-// which is no coarser than 2^-24 for t < 1 and cannot matter to a multiple of 2^-23; for t >= 1 the bit itself cannot.
-// (Conversions between float and integer run at an eighth of the issue rate.)  64 x 64 planes of 112 x 112: 124.5 us a call
-// with the fraction compared, 117.7 so; the generator's products as 64-bit multiplications: 131.
-__device__ __forceinline__ uint32_t quant_code_random(float d, float inv, uint32_t L, uint32_t word) {
-  const float t = __fadd_rd(__fmul_rn(d, inv), __uint_as_float((word & 0x100u) * 0x338000u));  // + 2^-24 when r is odd
-  const float up = __fadd_rd(t, __uint_as_float((word >> 9) | 0x3F800000u));
-  return min(__float_as_uint(__fadd_rd(up, 8388608.0f)) - 0x4B000001u, L);
+// Codes of a group under random rounding, packed: t = fp32 product d * inv of a distance d = x - lo, n = floor(t), and the code
+// goes up iff floor(frac(t) * 2^24) + r reaches 2^24, r = word >> 8.  As n * 2^24 is an integer, floor(frac(t) * 2^24) are the low
+// 24 bits of floor(t * 2^24) -- a scaling that is exact, and at most 255 * 2^24 -- and the code is the top byte of that plus r,
+// which cannot overflow.  t may come out a little above the last code L; such a position carries L whatever the draw.
+// One conversion and about four other instructions an element (a conversion takes a scheduler eight cycles, but on another
+// pipe than the generator's products, which take it four each).
+template <int BITS>
+__device__ __forceinline__ uint32_t quant4_random(const float (&d)[4], float inv, const uint32_t (&rnd)[4]) {
+  constexpr float L = (float)((1u << BITS) - 1u);
+  const f32x2 inv2 = pack2(inv, inv), one2 = pack2(16777216.0f, 16777216.0f);
+  float t[4];
+  uint32_t u[4];
+  unpack2(mul2(pack2(d[0], d[1]), inv2), t[0], t[1]);
+  unpack2(mul2(pack2(d[2], d[3]), inv2), t[2], t[3]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) t[e] = fminf(t[e], L);
+  unpack2(mul2(pack2(t[0], t[1]), one2), t[0], t[1]);
+  unpack2(mul2(pack2(t[2], t[3]), one2), t[2], t[3]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) u[e] = __float2uint_rz(t[e]) + (rnd[e] >> 8);
+  const uint32_t q = __byte_perm(__byte_perm(u[0], u[1], 0x0073u), __byte_perm(u[2], u[3], 0x0073u), 0x5410u);  // a code to a byte
+  if (BITS == 8) return q;
+  if (BITS == 4) {
+    const uint32_t y = q | (q >> 4);
+    return (y & 0xFFu) | ((y >> 8) & 0xFF00u);
+  }
+  return ((q * 0x00041041u) >> 18) & 0xFFu;  // (the partial products' fields do not overlap)
 }
 
 // ------------------------------------------------------------------------------------------------
