@@ -56,7 +56,7 @@ __device__ __forceinline__ SalScratch sal_scratch(const Geometry& pl, uint32_t* 
   s.outl = s.dense + pl.nsr + 1u;
   s.bitmap = s.outl + pl.nsr + 1u;
   s.chunks = s.bitmap + pl.nbm;
-  s.huf = reinterpret_cast<HufEncode*>(s.chunks + pl.nsr + 1u);
+  s.huf = reinterpret_cast<HufEncode*>(sal + (((uint32_t)(s.chunks - sal) + pl.nsr + 1u + 3u) & ~3u));  // (`sal` is 16-byte aligned)
   return s;
 }
 

@@ -579,64 +579,84 @@ constexpr uint32_t kHufMaxLen = 24;
 constexpr uint32_t kHufLutBits = 10;     // decoder: with 60 symbols about one code in a hundred is longer
 constexpr uint32_t kHufStageWords = 48;  // a chunk has at most 64 * 24 / 8 = 192 bytes
 
-// Encoder scratch of one unit (shared memory).
+// Encoder scratch of one unit (shared memory, 16-byte aligned).
 struct HufEncode {
-  uint32_t hist[256];
+  uint32_t hist[256];                // once it has been read: the nodes' parents (merged nodes), 256 sorted leaves and 256 merged nodes
   uint32_t code[256];                // by symbol: length << 24 | code value; 0: does not occur
-  uint32_t key[256 + 2];             // symbols that occur, weight << 8 | symbol, sorted; two sentinels behind them
-  uint32_t mw[256];                  // weights of the merged nodes, in order of creation
-  uint16_t lpar[256], mpar[256];     // parent (a merged node) of a sorted leaf, of a merged node
+  uint32_t used[256 + 4];            // symbols that occur, ascending, weight << 8 | symbol; four sentinels behind them
+  // weights of the sorted leaves and a sentinel, then of the merged nodes in order of creation (kHufNone: not there yet)
+  uint32_t weight[2 * 260];
+  uint8_t sorted[256];               // index into `used` of the sorted leaves
   uint32_t cnt[32], first[32];       // symbols of a length, then running rank; a length's first code value
   uint32_t smin, smax, maxlen, nlens;
   uint32_t stage[1][4 * kHufStageWords];  // chunks' bits while a warp assembles four of them; one per warp of the team
 };
+constexpr uint32_t kHufNone = 0xFFFFFFu, kHufMerged = 260;
+
+// First code value of length `lane`, from the number `n` of symbols of that length (0 for length 0), for codes that do not
+// oversubscribe: the sum over the shorter lengths k of n_k 2^(length - k), by a prefix sum in units of 2^-31.
+__device__ __forceinline__ uint32_t huffman_first(uint32_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t sum = lane ? n << (31u - lane) : 0u;
+  const uint32_t own = sum;
+#pragma unroll
+  for (uint32_t o = 1; o < 32u; o <<= 1) {
+    const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, sum, o);
+    if (lane >= o) sum += up;
+  }
+  return (sum - own) >> (31u - lane);
+}
 
 // A whole warp: code lengths and canonical codes from h->hist.  Symbols are ranked by comparison with all others (a few
 // dozen occur); one lane merges the two queues with the heads of both in registers, the next elements already on
-// their way from shared memory; depths are walks up the tree, a lane per leaf; code values are first-of-length plus
-// rank among the length's symbols.  About 3 us for 60 symbols; one thread doing all of it took 220 us.
+// their way from shared memory, without a branch; depths are walks up the tree, a lane per leaf; code values are
+// first-of-length plus rank among the length's symbols, over the symbols that occur.
 static __device__ __noinline__ void huffman_build(HufEncode* h) {
   const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, lt = (1u << lane) - 1u;
+  uint16_t* parent = reinterpret_cast<uint16_t*>(h->hist);
   uint32_t n = 0;
+#pragma unroll
   for (uint32_t i = 0; i < 8u; ++i) {
     const uint32_t sym = i * 32u + lane, w = h->hist[sym], m = __ballot_sync(full, w != 0u);
-    if (w) h->mw[n + __popc(m & lt)] = w << 8 | sym;  // (weights stay below 2^24; mw serves as a buffer here)
+    if (w) h->used[n + __popc(m & lt)] = w << 8 | sym;  // (weights stay below 2^24)
     n += __popc(m);
     h->code[sym] = 0;
   }
+  if (lane < 4u) h->used[n + lane] = 0xFFFFFFFFu;
   h->cnt[lane] = 0;
   __syncwarp();
   for (uint32_t i = lane; i < n; i += 32u) {
-    const uint32_t k = h->mw[i];
+    const uint32_t k = h->used[i];
     uint32_t rank = 0;
-#pragma unroll 4
-    for (uint32_t j = 0; j < n; ++j) rank += h->mw[j] < k;
-    h->key[rank] = k;
+#pragma unroll 2
+    for (uint32_t j = 0; j < n; j += 4u) {
+      const uint4 u = *reinterpret_cast<const uint4*>(&h->used[j]);
+      rank += (u.x < k ? 1u : 0u) + (u.y < k ? 1u : 0u) + (u.z < k ? 1u : 0u) + (u.w < k ? 1u : 0u);
+    }
+    h->weight[rank] = k >> 8;
+    h->sorted[rank] = (uint8_t)i;
   }
-  if (lane < 2u) h->key[n + lane] = 0xFFFFFFFFu;
+  for (uint32_t i = lane; i < n; i += 32u) h->weight[kHufMerged + i] = kHufNone;
+  if (lane < 2u) h->weight[n + lane] = kHufNone;
   __syncwarp();
   if (lane == 0 && n > 1u) {
-    constexpr uint32_t kNone = 0xFFFFFFu;
-    uint32_t li = 0, mi = 0, a0 = h->key[0] >> 8, a1 = h->key[1] >> 8, b0 = kNone, b1 = kNone;
+    uint32_t li = 0, mi = 0, a0 = h->weight[0], a1 = h->weight[1], b0 = kHufNone, b1 = kHufNone;
     for (uint32_t mn = 0; mn + 1u < n; ++mn) {
       uint32_t sum = 0;
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        if (a0 <= b0) {  // equal weights: the leaf has the smaller id
-          sum += a0;
-          h->lpar[li] = (uint16_t)mn;
-          ++li;
-          a0 = a1;
-          a1 = h->key[li + 1u] >> 8;
-        } else {
-          sum += b0;
-          h->mpar[mi] = (uint16_t)mn;
-          ++mi;
-          b0 = b1;
-          b1 = mi + 1u < mn ? h->mw[mi + 1u] : kNone;
-        }
+        const bool leaf = a0 <= b0;  // equal weights: the leaf has the smaller id
+        sum += leaf ? a0 : b0;
+        parent[leaf ? li : 256u + mi] = (uint16_t)mn;
+        li += leaf ? 1u : 0u;
+        mi += leaf ? 0u : 1u;
+        const uint32_t next = h->weight[leaf ? li + 1u : kHufMerged + mi + 1u];
+        a0 = leaf ? a1 : a0;
+        b0 = leaf ? b0 : b1;
+        a1 = leaf ? next : a1;
+        b1 = leaf ? b1 : next;
       }
-      h->mw[mn] = sum;
+      h->weight[kHufMerged + mn] = sum;
       if (mi == mn) b0 = sum;
       else if (mi + 1u == mn) b1 = sum;
     }
@@ -646,36 +666,34 @@ static __device__ __noinline__ void huffman_build(HufEncode* h) {
   for (uint32_t i = lane; i < n; i += 32u) {
     uint32_t d = 1;
     if (n > 1u)
-      for (uint32_t v = h->lpar[i]; v + 2u != n; v = h->mpar[v]) ++d;  // (the root is merged node n - 2)
+      for (uint32_t v = parent[i]; v + 2u != n; v = parent[256u + v]) ++d;  // (the root is merged node n - 2)
     d = min(d, 31u);
-    h->code[h->key[i] & 255u] = d << 24;
+    h->code[h->used[h->sorted[i]] & 255u] = d << 24;
     atomicAdd(&h->cnt[d], 1u);
     deepest = max(deepest, d);
   }
   asm volatile("redux.sync.max.u32 %0, %0, %1;" : "+r"(deepest) : "r"(full));
   __syncwarp();
-  uint32_t first = 0;
-  for (uint32_t k = 1; k < lane; ++k) first += h->cnt[k] << (lane - k);
+  const uint32_t first = huffman_first(h->cnt[lane]);
   __syncwarp();
   h->first[lane] = first;
   h->cnt[lane] = 0;
   __syncwarp();
-  uint32_t smin = 256, smax = 0;
-  for (uint32_t i = 0; i < 8u; ++i) {
-    const uint32_t sym = i * 32u + lane, len = h->code[sym] >> 24;
-    const uint32_t same = __match_any_sync(full, len), used = h->cnt[len];
+  for (uint32_t i = 0; i < n; i += 32u) {
+    const uint32_t sym = h->used[min(i + lane, n - 1u)] & 255u, len = i + lane < n ? h->code[sym] >> 24 : 0u;
+    const uint32_t same = __match_any_sync(full, len), before = h->cnt[len];
     __syncwarp();
-    if (len) h->code[sym] = len << 24 | ((h->first[len] + used + __popc(same & lt)) & 0xFFFFFFu);
-    if ((same & lt) == 0u) h->cnt[len] = used + __popc(same);
+    if (len) h->code[sym] = len << 24 | ((h->first[len] + before + __popc(same & lt)) & 0xFFFFFFu);
+    if ((same & lt) == 0u) h->cnt[len] = before + __popc(same);
     __syncwarp();
-    const uint32_t m = __ballot_sync(full, len != 0u && sym != 0u);
-    if (m) {
-      smin = min(smin, i * 32u + (uint32_t)__ffs((int)m) - 1u);
-      smax = i * 32u + 31u - (uint32_t)__clz((int)m);
-    }
   }
-  if (smin > 255u) smin = smax = 1u;
-  if (lane == 0) {
+  if (lane == 0) {  // (symbol 0 is not among those whose lengths are stored as a run)
+    uint32_t smin = 1, smax = 1;
+    const uint32_t least = n && (h->used[0] & 255u) == 0u ? 1u : 0u;
+    if (n > least) {
+      smin = h->used[least] & 255u;
+      smax = h->used[n - 1u] & 255u;
+    }
     h->smin = smin;
     h->smax = smax;
     h->maxlen = deepest;
@@ -729,8 +747,7 @@ static __device__ __noinline__ void huffman_tables(HufDecode* t) {
   }
   const uint32_t longest = __ballot_sync(full, n != 0u);
   __syncwarp();
-  uint32_t first = 0;
-  for (uint32_t k = 1; k < lane && k <= kHufMaxLen; ++k) first += t->count[k] << (lane - k);
+  const uint32_t first = huffman_first(n);
   const uint32_t index = incl - n;
   t->base[lane] = index - first;
   const unsigned long long lim = (unsigned long long)(first + n) << (32u - min(max(lane, 1u), 31u));
