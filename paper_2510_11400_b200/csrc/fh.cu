@@ -167,6 +167,11 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     if (warp_fits) {
       pl.team = fh::team_of_groups(pl.groups);
       pl.ppt = fh::kThreads / pl.team;
+      // Huffman stage: smaller tiles, down to what one warp sweeps, while there are fewer than SMs; the warps without a plane
+      // of their own share the measuring
+      if (blockwise && pl.entropy)
+        while (pl.ppt * pl.team > 32u && (pl.P + pl.ppt - 1) / pl.ppt < (uint64_t)fh::sm_count() && pl.ppt / 2 * pl.plane_bytes % 16 == 0)
+          pl.ppt /= 2;
       if (pl.ppt > pl.P) pl.ppt = (uint32_t)pl.P;
       pl.stage_bytes = (uint32_t)((pl.ppt * pl.plane_bytes + 127) & ~(uint64_t)127);
     } else if (regs_fit) {

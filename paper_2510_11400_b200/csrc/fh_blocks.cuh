@@ -244,7 +244,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
   for (uint32_t sr = wid; sr < nsr; sr += nw) {
     const StepUnit un = step_unit(g, sp, sr);
     const uint32_t by = un.sr * (4u >> g.qs) + sl.qrow, y = by * 8u + sl.r;
-    uint32_t row = 0, n_dense = 0, n_out = 0;
+    uint32_t row = 0, n_dense = 0, n_out = 0, n_zero = 0;
     for (uint32_t bx0 = un.bx0; bx0 < un.bx1; bx0 += sl.qm + 1u) {
       const uint32_t bx = bx0 + (sl.q & sl.qm), x0 = bx * 8u;
       const bool valid = by < g.nby && bx < g.nbx;
@@ -259,9 +259,13 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
         seg_codes(v, nin, inv2e, ca, cb, vm);
         if (dense) {
           n_out += __popc(vm);
-          if (entropy) {
+          if (entropy) {  // (residuals of 0 are by far the most frequent: counted apart, their bin is not fought over)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) atomicAdd(&sc.huf->hist[((j < 4 ? ca : cb) >> (8 * (j & 3))) & 255u], 1u);
+            for (int j = 0; j < 8; ++j) {
+              const uint32_t code = ((j < 4 ? ca : cb) >> (8 * (j & 3))) & 255u;
+              if (code == 128u) ++n_zero;
+              else atomicAdd(&sc.huf->hist[code], 1u);
+            }
           }
           if (sl.r == 0) {
             const uint32_t b = by * g.nbx + bx;
@@ -276,9 +280,11 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
     if (g.qs > 1) row += __shfl_xor_sync(full, row, 2);
     if ((sl.q & sl.qm) == 0u && y < H) sc.rowp[y * sp.seg + un.part] = row;
     asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_out) : "r"(full));
+    if (entropy) asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_zero) : "r"(full));
     if (lane == 0) {
       sc.dense[sr] = n_dense;
       sc.outl[sr] = n_out;
+      if (n_zero) atomicAdd(&sc.huf->hist[128], n_zero);
     }
   }
   team_sync(t);

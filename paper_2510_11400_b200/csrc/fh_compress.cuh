@@ -7,12 +7,13 @@
 // A call is ONE kernel, one pass over the dense tensor.  Tiles (runs of consecutive planes) are handed
 // out in order by a ticket.  Per plane: statistics, three-sigma class, and
 //   normal plane:   codes and table entry, written at once (the slot's offset is closed-form);
-//   other planes:   measured at once while they lie in shared memory (block classes, CSR and code sizes,
-//                   salient versus raw); the tile publishes the overflow size of its planes, obtains the sum
-//                   over all earlier tiles from the placement scan (fh_device.cuh) and writes the payloads.
+//   other planes:   measured (block classes, CSR and code sizes, salient versus raw) while they lie in shared memory or,
+//                   larger ones of the warp-team kernel, when the CTA has run out of tiles; the tile publishes the overflow
+//                   size of its planes, obtains the sum over all earlier tiles from the placement scan (fh_device.cuh) and
+//                   the payloads are written.
 // Variants by plane size:
 //   compress_warp<DT, SIGMA, TT, K, EDGE>   planes of at most 256 groups: bulk-copy (TMA) pipeline, a sub-warp
-//       team per plane, groups kept in registers; a warp handles the outlier-rich planes of its slice;
+//       team per plane, groups kept in registers; a warp handles an outlier-rich plane;
 //   compress_cta_regs<DT, SIGMA, K, EDGE, PARTS>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
 //   compress_cta<SIGMA>                    still larger bf16 planes of whole 16-byte chunks: swept in shared memory;
 //   compress_generic<DT, BITS, ROUND>      everything else (still larger ragged or fp32 planes, random rounding outside
@@ -344,8 +345,9 @@ __device__ __forceinline__ uint2 load_marker(const Dest& d, uint64_t plane) {
 }
 
 // The block-wise path runs in two phases so that nothing in the streaming phase ever waits for another CTA.
-// Phase 1, while a tile lies in shared memory: its outlier-rich planes are measured, the tile publishes the
-// overflow size of its planes to the scan and is put off.  Phase 2, when the CTA has run out of tiles: tiles put off are
+// Phase 1, while a tile lies in shared memory: its outlier-rich planes are measured, or listed and measured when the CTA has run
+// out of tiles (see warp_measure_put_off); the tile publishes the
+// overflow size of its planes to the scan and is put off.  Phase 2, then: tiles put off are
 // taken again (they come from the L2 cache when the tensor is small), obtain their place from the scan -- every tile
 // before one has been published, or is about to be, by a CTA in phase 1 -- and the payloads are written.  Tiles put off
 // wait in `defer_next`: linked from the CTA's own list (entry [tile]: the tile listed before it), or, in the CTA-team
@@ -356,7 +358,7 @@ struct BlockCtl {
   Plan pl;
   CompressArgs a;
   Dest d;
-  uint32_t U[kMaxStages], C[kMaxStages], arr[kMaxStages];  // warp-team kernel, per stage: units, counts, warps done
+  uint32_t U[kMaxStages], C[kMaxStages], arr[kMaxStages];  // warp-team kernel, per stage: units, counts (see kRawShift), warps done
   uint32_t base, ok;
   uint32_t head;                                           // warp-team and generic kernel: the tile this CTA listed last
   uint32_t held[kMaxStages];                               // the tile each stage buffer holds
@@ -368,17 +370,22 @@ struct BlockCtl {
 // Warp-team kernel: what the tiles in the stages have gathered so far, and the tiles put off, as far as there is room (the
 // others are linked like those of the CTA-team kernels).  A slice is what one warp sweeps of a tile.
 constexpr uint32_t kListed = 32, kListedPlanes = 128;  // (static shared memory stays below what kSmemLimit leaves)
+// Planes of more than four blocks are put off before they are measured (see warp_measure_put_off), so many of a CTA; until
+// then `place` holds their tiles (kNoTile: an entry that is nobody's).
+constexpr uint32_t kPutOff = kListed;
+// A stage's counts: salient planes, raw ones, those put off (a tile has at most 256 planes).
+constexpr uint32_t kRawShift = 10, kOffShift = 20, kCountMask = (1u << kRawShift) - 1u;
 struct WarpList {
   uint32_t sum[kMaxStages][kWarps];  // overflow units of a slice (when the slice has outlier-rich planes)
   uint32_t mask[kMaxStages];         // slices that have some
   uint32_t count;                    // tiles put off
-  uint32_t handed[2];                // phase 2: items handed out in each of its passes
+  uint32_t handed;                   // phase 2: items handed out
   uint32_t tile[kListed];
   uint32_t units[kListed], base[kListed];  // the tile's overflow units and, in phase 2, its place (kNoTile: not to be had)
   uint32_t before[kListed][kWarps];  // units of the tile's slices before this one
   uint8_t stage[kListed], slices[kListed];
-  uint16_t n[kListed];               // outlier-rich planes of the tile
-  // phase 2, planes of more than four blocks: those of the listed tiles
+  uint32_t n[kListed];               // outlier-rich planes of the tile (as far as they are measured)
+  // planes of more than four blocks: those put off, then, in phase 2, those of the listed tiles
   uint32_t planes;
   uint32_t place[kListedPlanes], meta[kListedPlanes];
   uint16_t lp[kListedPlanes];
@@ -967,9 +974,13 @@ __device__ __forceinline__ uint32_t plane_sweep(const Team& team, const Plan& pl
 // Warp-team streaming kernel: planes of at most 256 groups.  Eight consumer warps and one producer
 // warp per CTA.  The producer requests tiles and streams them into a ring of shared-memory stages
 // with bulk copies.  A consumer warp sweeps its own planes of a tile (statistics, class, codes, stores)
-// and never waits for another warp.  Outlier-rich planes are rare: a warp that has some in its slice
-// measures them and adds their overflow size to the tile's sum in shared memory; the last of the tile's
-// eight warps to get there publishes the tile and puts it on the CTA's list for phase 2.
+// and never waits for another warp.  Outlier-rich planes are rare: a warp that has some in its slice encodes them (planes of at
+// most four blocks) and adds their overflow size to the tile's sum in shared memory, or lists them (larger ones); the last of the
+// tile's eight warps to get there publishes the tile or, when planes of it are only listed, puts it on the CTA's list for later.
+//
+// Registers are what this kernel is short of: 72 a thread at three CTAs to an SM.  What the compiler cannot keep goes to local
+// memory, for which the stages leave some 28 KB of L1: with 24 bytes a thread spilled in the sweep that is just enough, with 36
+// it is not (32 x 32 planes, fp32: 3 % slower, 24 x 24: 6 %).  So little is held across the calls of the outlined functions.
 // -------------------------------------------------------------------------------------------------
 constexpr int kWarpKernelThreads = kThreads + 32;
 
@@ -1049,77 +1060,116 @@ __device__ __forceinline__ void encode_small(const Plan& pl, uint32_t n, PlaneOf
   }
 }
 
-// Phase 1, a warp with outlier-rich planes in its slice (`leaders`: the first lanes of their teams; lp0: first
-// plane of the slice): they are measured, their sizes go into the sums of the tile in stage s and into their table
+// The slice of a tile that the warp sweeps: it changes from tile to tile, so that a periodic pattern of outlier-rich planes does
+// not land on the same warp every time.
+__device__ __forceinline__ uint32_t warp_slice(uint32_t tile) { return ((threadIdx.x >> 5) + tile) & ((uint32_t)kWarps - 1u); }
+
+// Phase 1, a warp with small outlier-rich planes in its slice (`leaders`: the first lanes of their teams; lp0: first
+// plane of the slice): they are encoded where they lie, their sizes go into the sums of the tile in stage s and into their table
 // markers.
 template <int DT, int TT>
-__device__ __noinline__ void warp_tile_measure(BlockCtl* c, WarpList* l, uint8_t* tbuf, uint64_t p0, uint32_t s, uint32_t slice,
-                                               uint32_t leaders, uint32_t meta, uint32_t* sal) {
+__device__ __noinline__ void warp_tile_encode(BlockCtl* c, WarpList* l, uint8_t* tbuf, uint32_t s, uint32_t leaders, uint32_t meta) {
   const Plan& pl = c->pl;
+  const uint32_t tile = c->held[s], slice = warp_slice(tile);
+  const uint64_t p0 = (uint64_t)tile * pl.ppt;
   const uint32_t lane = threadIdx.x & 31u, lp0 = slice * (32u / TT), n = __popc(leaders), full = 0xFFFFFFFFu;
+  const uint32_t fits = c->d.fits;
   uint32_t total = 0, nraw = 0;
-  if (is_small_plane(pl)) {
-    const uint32_t fits = c->d.fits;
-    encode_small<DT>(
-        pl, n, [&](uint32_t k) { return tbuf + (uint64_t)(lp0 + nth_bit(leaders, k) / TT) * pl.plane_bytes; },
-        [&](uint32_t k, uint32_t size, bool raw) {
-          const uint32_t bytes = raw ? (uint32_t)pl.plane_bytes : size, u = ovf_units(pl, bytes);
-          total += u;
-          nraw += raw ? 1u : 0u;
-          // (the leader's lane adds class and count afterwards)
-          if (fits) store_marker(c->d, p0 + lp0 + nth_bit(leaders, k) / TT, 0u, u, bytes, raw);
-        });
-    __syncwarp();
-    if (fits && ((leaders >> lane) & 1u))
-      reinterpret_cast<uint32_t*>(c->d.dst + 64)[4ull * (p0 + lp0 + lane / TT) + 1ull] = (meta & ~3u) | kClsSalient;
-    total += __shfl_xor_sync(full, total, 1);
-    total += __shfl_xor_sync(full, total, 2);
-    nraw += __shfl_xor_sync(full, nraw, 1);
-    nraw += __shfl_xor_sync(full, nraw, 2);
-  } else {
-    const Team team = make_warp_team(nullptr);
-    for (uint32_t m = leaders; m; m &= m - 1u) {
-      const uint32_t src = (uint32_t)__ffs((int)m) - 1u, lp = lp0 + src / TT;
-      const SalientInfo info = salient_measure<DT, false>(team, pl, tbuf + (uint64_t)lp * pl.plane_bytes, sal);
-      bool raw;
-      const uint32_t u = plane_units(pl, info, raw);
-      total += u;
-      nraw += raw ? 1u : 0u;
-      const uint32_t mt = __shfl_sync(full, meta, (int)src);
-      if (lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
-      if (c->d.fits && scratch_saved<false>(pl)) scratch_save<false>(team, pl, c->d, p0 + lp, info, sal);
-      __syncwarp();
-    }
-  }
+  encode_small<DT>(
+      pl, n, [&](uint32_t k) { return tbuf + (uint64_t)(lp0 + nth_bit(leaders, k) / TT) * pl.plane_bytes; },
+      [&](uint32_t k, uint32_t size, bool raw) {
+        const uint32_t bytes = raw ? (uint32_t)pl.plane_bytes : size, u = ovf_units(pl, bytes);
+        total += u;
+        nraw += raw ? 1u : 0u;
+        // (the leader's lane adds class and count afterwards)
+        if (fits) store_marker(c->d, p0 + lp0 + nth_bit(leaders, k) / TT, 0u, u, bytes, raw);
+      });
+  __syncwarp();
+  if (fits && ((leaders >> lane) & 1u))
+    reinterpret_cast<uint32_t*>(c->d.dst + 64)[4ull * (p0 + lp0 + lane / TT) + 1ull] = (meta & ~3u) | kClsSalient;
+  total += __shfl_xor_sync(full, total, 1);
+  total += __shfl_xor_sync(full, total, 2);
+  nraw += __shfl_xor_sync(full, nraw, 1);
+  nraw += __shfl_xor_sync(full, nraw, 2);
   if (lane == 0) {
     l->sum[s][slice] = total;
     atomicOr(&l->mask[s], 1u << slice);
     if (total) atomicAdd(&c->U[s], total);
-    atomicAdd(&c->C[s], (n - nraw) | (nraw << 16));
+    atomicAdd(&c->C[s], (n - nraw) | (nraw << kRawShift));
   }
 }
 
-// Phase 1, the last of a tile's eight warps (one thread): the tile's sums are complete.
+// The same for larger planes, which are listed, and measured when the CTA has run out of tiles (see warp_measure_put_off), as
+// long as the list has room, and measured at once otherwise.
+template <int DT, int TT>
+__device__ __noinline__ void warp_tile_measure(BlockCtl* c, uint8_t* tbuf, uint64_t p0, uint32_t s, uint32_t slice, uint32_t leaders,
+                                               uint32_t meta, uint32_t* sal) {
+  const Plan& pl = c->pl;
+  const uint32_t lane = threadIdx.x & 31u, lp0 = slice * (32u / TT), n = __popc(leaders), full = 0xFFFFFFFFu;
+  uint32_t total = 0, nraw = 0;
+  const Team team = make_warp_team(nullptr);
+  for (uint32_t m = leaders; m; m &= m - 1u) {
+    const uint32_t src = (uint32_t)__ffs((int)m) - 1u, lp = lp0 + src / TT;
+    const SalientInfo info = salient_measure<DT, false>(team, pl, tbuf + (uint64_t)lp * pl.plane_bytes, sal);
+    bool raw;
+    const uint32_t u = plane_units(pl, info, raw);
+    total += u;
+    nraw += raw ? 1u : 0u;
+    const uint32_t mt = __shfl_sync(full, meta, (int)src);
+    if (lane == 0 && c->d.fits) store_marker(c->d, p0 + lp, mt, u);
+    if (c->d.fits && scratch_saved<false>(pl)) scratch_save<false>(team, pl, c->d, p0 + lp, info, sal);
+    __syncwarp();
+  }
+  if (lane == 0) {
+    if (total) atomicAdd(&c->U[s], total);
+    atomicAdd(&c->C[s], (n - nraw) | (nraw << kRawShift));
+  }
+}
+template <int DT, int TT>
+__device__ __noinline__ void warp_tile_put_off(BlockCtl* c, WarpList* l, uint8_t* tbuf, uint32_t s, uint32_t leaders, uint32_t meta,
+                                               uint8_t* sal_base) {
+  const uint32_t tile = c->held[s], slice = warp_slice(tile), lane = threadIdx.x & 31u, n = __popc(leaders);
+  uint32_t at = 0;
+  if (lane == 0) at = atomicAdd(&l->planes, n);
+  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  if (at + n <= kPutOff) {
+    if ((leaders >> lane) & 1u) {
+      const uint32_t k = at + __popc(leaders & ((1u << lane) - 1u));
+      l->place[k] = tile;
+      l->lp[k] = (uint16_t)(slice * (32u / TT) + lane / TT);
+      l->meta[k] = meta;
+    }
+    if (lane == 0) atomicAdd(&c->C[s], n << kOffShift);
+    return;
+  }
+  if (at + lane < kPutOff) l->place[at + lane] = kNoTile;
+  warp_tile_measure<DT, TT>(c, tbuf, (uint64_t)tile * c->pl.ppt, s, slice, leaders, meta,
+                            reinterpret_cast<uint32_t*>(sal_base + (threadIdx.x >> 5) * c->pl.sal_stride));
+}
+
+// Phase 1, one thread: a tile with outlier-rich planes is published, or, when some of them are put off unmeasured, listed until
+// they are.
 static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, WarpList* l, uint32_t s, uint32_t tile) {
-  __threadfence_block();  // the other warps' sums after their arrivals
   const uint32_t U = c->U[s], C = c->C[s];
-  scan_publish(c->a.scan, tile, U);
-  if (C == 0u) return;
-  count_blockwise(U, C & 0xFFFFu, C >> 16);
+  if (C < (1u << kOffShift)) scan_publish(c->a.scan, tile, U);
+  const uint32_t nsal = C & kCountMask, nraw = (C >> kRawShift) & kCountMask, off = C >> kOffShift;
+  count_blockwise(U, nsal, nraw);
   const uint32_t mask = l->mask[s];
   c->U[s] = 0;
   c->C[s] = 0;
   l->mask[s] = 0;
-  if (!c->d.fits) return;
-  const uint32_t i = atomicAdd(&l->count, 1u);
+  if (!c->d.fits && off == 0u) return;
+  // (larger planes: the list is for tiles with planes that are put off, of which there are no more than such planes)
+  const uint32_t i = off || is_small_plane(c->pl) ? atomicAdd(&l->count, 1u) : kListed;
   if (i >= kListed) {
     c->a.defer_next[tile] = atomicExch(&c->head, tile);
     return;
   }
   l->tile[i] = tile;
   l->units[i] = U;
-  l->n[i] = (uint16_t)((C & 0xFFFFu) + (C >> 16));
+  l->n[i] = nsal + nraw;
   l->stage[i] = (uint8_t)s;
+  if (off) return;
   l->slices[i] = (uint8_t)mask;
   uint32_t run = 0;
 #pragma unroll
@@ -1144,6 +1194,77 @@ __device__ __forceinline__ uint8_t* fetch_plane(const Plan& pl, const uint8_t* s
   return to + (start - a0);
 }
 
+// Exclusive prefix sum over the warp, `run` going on to what follows.
+__device__ __forceinline__ uint32_t warp_excl(uint32_t v, uint32_t& run) {
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu;
+  uint32_t incl = v;
+#pragma unroll
+  for (uint32_t o = 1; o < 32u; o <<= 1) {
+    const uint32_t up = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += up;
+  }
+  const uint32_t r = run + incl - v;
+  run += __shfl_sync(full, incl, 31);
+  return r;
+}
+
+// Phase 2, a warp: the small outlier-rich planes of one slice of a tile, whose overflow parts start `at` units into the region.
+// `mk`: the table marker of the slice's plane `lane`; `staged`: where the tile still lies (null: nowhere, the planes are fetched
+// again into `buf`).  Returns the slice's units.
+template <int DT, int TT>
+__device__ __forceinline__ uint4 slice_marker(BlockCtl* c, uint32_t tile, uint32_t slice) {
+  const Plan& pl = c->pl;
+  const uint32_t lane = threadIdx.x & 31u, lp = slice * (32u / TT) + lane;
+  const uint64_t gp = (uint64_t)tile * pl.ppt + lp;
+  return lane < 32u / TT && lp < pl.ppt && gp < pl.P ? __ldcg(reinterpret_cast<const uint4*>(c->d.dst + 64) + gp) : make_uint4(0u, 0u, 0u, 0u);
+}
+template <int DT, int TT>
+__device__ __noinline__ uint32_t warp_slice_write(BlockCtl* c, uint32_t tile, uint32_t slice, const uint4 mk, uint32_t at, uint8_t* staged,
+                                                  uint8_t* buf) {
+  const Plan& pl = c->pl;
+  const Dest& d = c->d;
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, lp0 = slice * (32u / TT);
+  const uint64_t p0 = (uint64_t)tile * pl.ppt;
+  const uint32_t pb = (uint32_t)pl.plane_bytes;
+  const uint32_t planes = __ballot_sync(full, (mk.y & 3u) != kClsNormal), n = __popc(planes);
+  if (n == 0u) return 0u;
+  uint32_t end = at;
+  const uint32_t place = warp_excl((mk.y & 3u) != kClsNormal ? mk.x : 0u, end);  // (of the lane's plane)
+  // as many planes at a time as have room in the buffer (at least four: a quarter of a stage), eight lanes or all to one
+  const uint32_t lanes = pl.nblk == 1u ? 8u : 32u, step = pl.nblk == 1u ? 4u : 1u, room = a16(pb + 16u);
+  for (uint32_t k0 = 0; k0 < n; k0 += step) {
+    const uint32_t here = min(step, n - k0), k = k0 + lane / lanes, j = lane & (lanes - 1u);
+    const bool mine = lane / lanes < here;
+    const uint32_t b = nth_bit(planes, mine ? k : k0);
+    const uint64_t gp = p0 + lp0 + b;
+    uint32_t w = __shfl_sync(full, mk.w, (int)b);
+    const uint32_t bytes = __shfl_sync(full, mk.z, (int)b), meta = __shfl_sync(full, mk.y, (int)b),
+                   units = __shfl_sync(full, mk.x, (int)b), off = __shfl_sync(full, place, (int)b);
+    uint8_t* plane;
+    if (staged) {
+      plane = staged + (uint64_t)(lp0 + b) * pb;
+    } else {
+      auto at_buf = [&](uint32_t i) { return buf + i * room + ((uint32_t)((p0 + lp0 + nth_bit(planes, k0 + i)) * pb) & 15u); };
+      plane = fetch_plane(pl, c->a.src, gp, buf + (lane / lanes) * room, j, lanes, mine);
+      __syncwarp();
+      encode_small<DT>(pl, here, at_buf, [](uint32_t, uint32_t, bool) {});
+      __syncwarp();
+    }
+    const unsigned long long off16 = (pl.ovf_off >> 4) + off;
+    if (mine && (off16 + units) * 16ull <= d.capacity) {  // (never write past the capacity)
+      SplitOut out;
+      out.slot = d.dst + pl.slots_off + gp * pl.npay;
+      out.ovf = d.dst + off16 * 16ull;
+      out.npay = pl.npay;
+      payload_copy(w ? plane : small_payload(plane), bytes, out, j, lanes);
+      if (j == 0u)
+        reinterpret_cast<uint4*>(d.dst + 64)[gp] = make_uint4(units ? (uint32_t)off16 : 0u, (w ? kClsRaw : kClsSalient) | (meta & ~3u), 0u, 0u);
+    }
+    __syncwarp();
+  }
+  return end - at;
+}
+
 // Phase 2, a warp: an outlier-rich plane of more than four blocks, whose overflow part starts `place` units into the region.
 // `plane`: where it still lies, or null.
 template <int DT>
@@ -1159,172 +1280,224 @@ __device__ __noinline__ void warp_plane_write(BlockCtl* c, uint64_t gp, const ui
   __syncwarp();
 }
 
-// Phase 2, a warp: the outlier-rich planes of one slice of a tile, whose overflow parts start `at` units into the region.
-// `staged`: where the tile still lies (null: nowhere, the planes are fetched again into `buf`).  Returns the slice's
-// units.
-template <int DT, int TT>
-__device__ __noinline__ uint32_t warp_slice_write(BlockCtl* c, uint32_t tile, uint32_t slice, uint32_t at, uint8_t* staged, uint8_t* buf,
-                                                  uint32_t* sal) {
-  const Plan& pl = c->pl;
-  const Dest& d = c->d;
-  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, lp0 = slice * (32u / TT);
-  const uint64_t p0 = (uint64_t)tile * pl.ppt;
-  const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0), pb = (uint32_t)pl.plane_bytes;
-  uint4 mk = make_uint4(0u, 0u, 0u, 0u);
-  if (lane < 32u / TT && lp0 + lane < np) {
-    mk = __ldcg(reinterpret_cast<const uint4*>(d.dst + 64) + p0 + lp0 + lane);
-  }
-  const uint32_t planes = __ballot_sync(full, (mk.y & 3u) != kClsNormal), n = __popc(planes);
-  if (n == 0u) return 0u;
-  const uint32_t u = (mk.y & 3u) != kClsNormal ? mk.x : 0u;
-  uint32_t incl = u;
-#pragma unroll
-  for (uint32_t o = 1; o < 32u; o <<= 1) {
-    const uint32_t up = __shfl_up_sync(full, incl, o);
-    if (lane >= o) incl += up;
-  }
-  const uint32_t all = __shfl_sync(full, incl, 31);
-  const uint32_t place = at + incl - u;  // (of the lane's plane)
-  if (is_small_plane(pl)) {
-    // as many planes at a time as have room in the buffer (at least four: a quarter of a stage), eight lanes or all to one
-    const uint32_t lanes = pl.nblk == 1u ? 8u : 32u, step = pl.nblk == 1u ? 4u : 1u, room = a16(pb + 16u);
-    for (uint32_t k0 = 0; k0 < n; k0 += step) {
-      const uint32_t here = min(step, n - k0), k = k0 + lane / lanes, j = lane & (lanes - 1u);
-      const bool mine = lane / lanes < here;
-      const uint32_t b = nth_bit(planes, mine ? k : k0);
-      const uint64_t gp = p0 + lp0 + b;
-      uint32_t w = __shfl_sync(full, mk.w, (int)b);
-      const uint32_t bytes = __shfl_sync(full, mk.z, (int)b), meta = __shfl_sync(full, mk.y, (int)b),
-                     units = __shfl_sync(full, mk.x, (int)b), off = __shfl_sync(full, place, (int)b);
-      uint8_t* plane;
-      if (staged) {
-        plane = staged + (uint64_t)(lp0 + b) * pb;
-      } else {
-        auto at_buf = [&](uint32_t i) { return buf + i * room + ((uint32_t)((p0 + lp0 + nth_bit(planes, k0 + i)) * pb) & 15u); };
-        plane = fetch_plane(pl, c->a.src, gp, buf + (lane / lanes) * room, j, lanes, mine);
-        __syncwarp();
-        encode_small<DT>(pl, here, at_buf, [](uint32_t, uint32_t, bool) {});
-        __syncwarp();
+// Phase 2, a warp: takes one of the tiles that were not listed, and its place; kNoTile when there are none left.
+static __device__ __noinline__ uint32_t warp_take_linked(BlockCtl* c, uint32_t& place) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t tile = kNoTile;
+  if (lane == 0)
+    for (tile = *(volatile uint32_t*)&c->head; tile != kNoTile;) {
+      const uint32_t seen = atomicCAS(&c->head, tile, c->a.defer_next[tile]);
+      if (seen == tile) {
+        c->a.defer_next[tile] = 0u;
+        break;
       }
-      const unsigned long long off16 = (pl.ovf_off >> 4) + off;
-      if (mine && (off16 + units) * 16ull <= d.capacity) {  // (never write past the capacity)
-        SplitOut out;
-        out.slot = d.dst + pl.slots_off + gp * pl.npay;
-        out.ovf = d.dst + off16 * 16ull;
-        out.npay = pl.npay;
-        payload_copy(w ? plane : small_payload(plane), bytes, out, j, lanes);
-        if (j == 0u)
-          reinterpret_cast<uint4*>(d.dst + 64)[gp] = make_uint4(units ? (uint32_t)off16 : 0u, (w ? kClsRaw : kClsSalient) | (meta & ~3u), 0u, 0u);
-      }
-      __syncwarp();
+      tile = seen;
     }
-  } else {
-    for (uint32_t m = planes; m; m &= m - 1u) {
-      const uint32_t b = (uint32_t)__ffs((int)m) - 1u;
-      warp_plane_write<DT>(c, p0 + lp0 + b, nullptr, __shfl_sync(full, mk.y, (int)b), __shfl_sync(full, place, (int)b), buf, sal);
-    }
-  }
-  return all;
+  tile = __shfl_sync(0xFFFFFFFFu, tile, 0);
+  place = 0;
+  if (tile == kNoTile || scan_prefix(c->a.scan, tile, place)) return tile;
+  if (lane == 0) report_error(c->a, kErrTimeout);
+  return kNoTile;
 }
 
-// Phase 2 of the warp-team kernel.  The places of the listed tiles first, a warp to a tile (a look-up by every warp that
-// needs one had thousands of warps polling the same words: 7 x 7 planes, fp32: 25 -> 45 us).  Then the slices are handed
-// out to the warps, which need nothing of one another, in two passes: tiles that still lie in a stage (the last ones the
-// CTA streamed: all of them when the tensor is small), then the others, whose planes the warps fetch into their part of
-// the stages.  (Tile by tile with the whole CTA, a 28 x 28 bf16 tensor with every eighth channel outlier-rich had one warp
-// working and seven waiting.)
+// Phase 2, one warp: the places of the n listed tiles that have overflow (kNoTile: not to be had; units are below 2^32 - 1).
+static __device__ __noinline__ void warp_list_places(BlockCtl* c, WarpList* l, uint32_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const bool asks = lane < n && l->units[min(lane, kListed - 1u)] != 0u;
+  const uint32_t m = __ballot_sync(0xFFFFFFFFu, asks), want = __popc(m);
+  if (lane < n && !asks) l->base[lane] = 0u;
+  if (want == 0u) return;
+  const uint32_t from = lane < want ? nth_bit(m, lane) : nth_bit(m, 0u);
+  uint32_t base = 0;
+  const bool ok = want == 1u ? scan_prefix(c->a.scan, l->tile[from], base) : scan_places(c->a.scan, l->tile[from], want, base);
+  if (!ok && lane == 0) report_error(c->a, kErrTimeout);
+  if (lane < want) l->base[from] = ok ? base : kNoTile;
+}
+
+// Phase 2 of the warp-team kernel, small planes.  One warp looks up the places of the listed tiles (every warp for itself: 7 x 7
+// planes, fp32: 25 -> 45 us).  Then every warp copies the payloads of the slices it has encoded, of tiles that still lie in a
+// stage: the last ones the CTA streamed, all of them when the tensor is small.  The other tiles, if there are any, are handed out
+// slice by slice; their planes are fetched and encoded again, in the stages, a part to a warp.
 template <int DT, int TT>
-__device__ __noinline__ void warp_phase2(BlockCtl* c, WarpList* l, uint8_t* stages, uint8_t* sal_base) {
+__device__ __noinline__ void warp_phase2_small(BlockCtl* c, WarpList* l, uint8_t* stages) {
+  const Plan& pl = c->pl;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, full = 0xFFFFFFFFu, n = min(l->count, kListed);
+  uint8_t* buf = stages + min(warp, (uint32_t)kWarps - 1u) * ((pl.sm_sal / (uint32_t)kWarps) & ~15u);
+  // (the warp's slice of a tile, as in phase 1; the first one's markers are on their way while the places are looked up)
+  uint4 ahead = make_uint4(0u, 0u, 0u, 0u);
+  if (warp < (uint32_t)kWarps) ahead = slice_marker<DT, TT>(c, l->tile[0], warp_slice(l->tile[0]));
+  else warp_list_places(c, l, n);
+  const bool away = threadIdx.x < n && c->held[l->stage[min(threadIdx.x, kListed - 1u)]] != l->tile[min(threadIdx.x, kListed - 1u)];
+  const bool others = __syncthreads_or(away || c->head != kNoTile) != 0;  // (the places are known)
+  if (warp < (uint32_t)kWarps)
+    for (uint32_t i = 0; i < n; ++i) {
+      const uint32_t tile = l->tile[i], slice = warp_slice(tile), st = l->stage[i];
+      if (c->held[st] != tile || !((l->slices[i] >> slice) & 1u) || l->base[i] == kNoTile) continue;
+      const uint4 mk = i ? slice_marker<DT, TT>(c, tile, slice) : ahead;
+      warp_slice_write<DT, TT>(c, tile, slice, mk, l->base[i] + l->before[i][slice], stages + (uint64_t)st * pl.stage_bytes, buf);
+    }
+  if (!others) return;
+  __syncthreads();  // the stages are free
+  if (warp == (uint32_t)kWarps) return;
+  for (;;) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(&l->handed, 1u);
+    item = __shfl_sync(full, item, 0);
+    if (item >= n * (uint32_t)kWarps) break;
+    const uint32_t i = item / (uint32_t)kWarps, slice = item % (uint32_t)kWarps, tile = l->tile[i];
+    if (c->held[l->stage[i]] == tile || !((l->slices[i] >> slice) & 1u) || l->base[i] == kNoTile) continue;
+    warp_slice_write<DT, TT>(c, tile, slice, slice_marker<DT, TT>(c, tile, slice), l->base[i] + l->before[i][slice], nullptr, buf);
+  }
+  uint32_t at;
+  for (uint32_t tile; (tile = warp_take_linked(c, at)) != kNoTile;)
+    for (uint32_t slice = 0; slice < (uint32_t)kWarps; ++slice)
+      at += warp_slice_write<DT, TT>(c, tile, slice, slice_marker<DT, TT>(c, tile, slice), at, nullptr, buf);
+}
+
+// Measuring a plane of more than four blocks is a chain of 10,000 to 30,000 cycles in one warp.  A warp that does it where the
+// plane is found holds up its tile's stage, and with it the ring: so the planes that a CTA finds are listed, and measured by all
+// its warps side by side when it has run out of tiles; only then are their tiles published.  (A CTA that waits for a tile's
+// publication waits for one that is doing this or is still streaming; neither waits for anybody.)  Each warp keeps what it
+// measured last, and phase 2 has it write that plane without measuring it again.  Planes that still lie in their stages are taken
+// there when all do; otherwise all are fetched, into the stages, a part to a warp.  us a call, before and with scan_places: bf16,
+// 2 bits, 128 x 192 planes of 28 x 28, every eighth channel outlier-rich 92 -> 66; Huffman stage, fp32, 8 x 512 of 7 x 7, 13 % of
+// them outlier-rich, 75 -> 26, 8 x 128 of 28 x 28 48 -> 36.
+struct WarpOwn {
+  uint32_t tile, lp;  // tile: kNoTile if there is none
+  const uint8_t* plane;
+  SalientInfo info;
+};
+template <int DT>
+__device__ __noinline__ void warp_measure_put_off(BlockCtl* c, WarpList* l, uint8_t* stages, uint8_t* buf, uint32_t* sal, WarpOwn& own) {
+  const Plan& pl = c->pl;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, full = 0xFFFFFFFFu;
+  const uint32_t n = min(l->planes, kPutOff), tiles = min(l->count, kListed), mine = min(threadIdx.x, tiles - 1u);
+  const Team team = make_warp_team(nullptr);
+  const bool held = __syncthreads_and(c->held[l->stage[mine]] == l->tile[mine]) != 0;
+  while (warp < (uint32_t)kWarps) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(&l->handed, 1u);
+    item = __shfl_sync(full, item, 0);
+    if (item >= n) break;
+    const uint32_t tile = l->place[item], lp = l->lp[item];
+    const uint32_t m = __ballot_sync(full, tile != kNoTile && lane < tiles && l->tile[lane] == tile);
+    if (m == 0u) continue;
+    const uint32_t i = (uint32_t)__ffs((int)m) - 1u;
+    const uint64_t gp = (uint64_t)tile * pl.ppt + lp;
+    const uint8_t* plane = held ? stages + (uint64_t)l->stage[i] * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes
+                                : fetch_plane(pl, c->a.src, gp, buf, lane, 32u, true);
+    __syncwarp();
+    const SalientInfo info = salient_measure<DT, false>(team, pl, plane, sal);
+    bool raw;
+    const uint32_t u = plane_units(pl, info, raw);
+    if (lane == 0) {
+      if (c->d.fits) store_marker(c->d, gp, l->meta[item], u);
+      atomicAdd(&l->units[i], u);
+      atomicAdd(&l->n[i], 1u);
+      count_blockwise(u, raw ? 0u : 1u, raw ? 1u : 0u);
+    }
+    if (c->d.fits && scratch_saved<false>(pl)) scratch_save<false>(team, pl, c->d, gp, info, sal);
+    own.tile = tile;
+    own.lp = lp;
+    own.plane = plane;
+    own.info = info;
+    __syncwarp();
+  }
+  __syncthreads();
+  if (threadIdx.x < tiles) scan_publish(c->a.scan, l->tile[threadIdx.x], l->units[threadIdx.x]);
+  if (threadIdx.x < (uint32_t)kMaxStages && !held) c->held[threadIdx.x] = kNoTile;
+  if (threadIdx.x == 0) l->planes = l->handed = 0;
+  __syncthreads();
+}
+
+// Phase 2 of the warp-team kernel, planes of more than four blocks.  The places of the listed tiles first, by one warp; then their
+// planes go to the warps one by one, each warp's own first; then the tiles that were not listed, a warp each.
+template <int DT>
+__device__ __noinline__ void warp_phase2_large(BlockCtl* c, WarpList* l, uint8_t* stages, uint8_t* sal_base) {
   const Plan& pl = c->pl;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, full = 0xFFFFFFFFu;
   uint32_t* sal = reinterpret_cast<uint32_t*>(sal_base + min(warp, (uint32_t)kWarps - 1u) * pl.sal_stride);
   uint8_t* buf = stages + min(warp, (uint32_t)kWarps - 1u) * ((pl.sm_sal / (uint32_t)kWarps) & ~15u);
+  WarpOwn own;
+  own.tile = kNoTile;
+  warp_measure_put_off<DT>(c, l, stages, buf, sal, own);
+  if (!c->d.fits) return;
   const uint32_t n = min(l->count, kListed);
-  const bool small = is_small_plane(pl);
-  auto place_of = [&](uint32_t tile) {
-    uint32_t base = 0;
-    if (scan_prefix(c->a.scan, tile, base)) return base;
-    if (lane == 0) report_error(c->a, kErrTimeout);
-    return kNoTile;  // (no place: units are below 2^32 - 1)
-  };
+  if (warp == (uint32_t)kWarps) warp_list_places(c, l, n);
+  __syncthreads();
   for (uint32_t i = warp; i < n; i += (uint32_t)kWarps + 1u) {
-    const uint32_t tile = l->tile[i];
-    uint32_t base = l->units[i] ? place_of(tile) : 0u;
-    if (!small && base != kNoTile) {  // the tile's planes join the list; without room there, the tile joins the others
-      uint32_t at = 0;
-      if (lane == 0) at = atomicAdd(&l->planes, (uint32_t)l->n[i]);
-      at = __shfl_sync(full, at, 0);
-      const bool room = at + l->n[i] <= kListedPlanes;
-      if (!room) {
-        for (uint32_t k = at + lane; k < kListedPlanes; k += 32u) l->of[k] = (uint8_t)kListed;
-        if (lane == 0) c->a.defer_next[tile] = atomicExch(&c->head, tile);
-      }
-      const uint64_t p0 = (uint64_t)tile * pl.ppt;
-      const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
-      for (uint32_t lp0 = 0, run = base; room && lp0 < np; lp0 += 32u) {
-        const uint2 mk = lp0 + lane < np ? load_marker(c->d, p0 + lp0 + lane) : make_uint2(0u, 0u);
-        const bool mine = (mk.y & 3u) != kClsNormal;
-        const uint32_t m = __ballot_sync(full, mine), u = mine ? mk.x : 0u;
-        uint32_t incl = u;
-#pragma unroll
-        for (uint32_t o = 1; o < 32u; o <<= 1) {
-          const uint32_t up = __shfl_up_sync(full, incl, o);
-          if (lane >= o) incl += up;
-        }
-        if (mine) {
-          const uint32_t k = at + __popc(m & ((1u << lane) - 1u));
-          l->place[k] = run + incl - u;
-          l->meta[k] = mk.y;
-          l->lp[k] = (uint16_t)(lp0 + lane);
-          l->of[k] = (uint8_t)i;
-        }
-        at += __popc(m);
-        run += __shfl_sync(full, incl, 31);
-      }
+    const uint32_t tile = l->tile[i], base = l->base[i];
+    if (base == kNoTile) continue;
+    // the tile's planes join the list; without room there, the tile joins the others
+    uint32_t at = 0;
+    if (lane == 0) at = atomicAdd(&l->planes, l->n[i]);
+    at = __shfl_sync(full, at, 0);
+    if (at + l->n[i] > kListedPlanes) {
+      for (uint32_t k = at + lane; k < kListedPlanes; k += 32u) l->of[k] = (uint8_t)kListed;
+      if (lane == 0) c->a.defer_next[tile] = atomicExch(&c->head, tile);
+      continue;
     }
-    if (lane == 0) l->base[i] = base;
+    const uint64_t p0 = (uint64_t)tile * pl.ppt;
+    const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
+    for (uint32_t lp0 = 0, run = base; lp0 < np; lp0 += 32u) {
+      const uint2 mk = lp0 + lane < np ? load_marker(c->d, p0 + lp0 + lane) : make_uint2(0u, 0u);
+      const bool mine = (mk.y & 3u) != kClsNormal;
+      const uint32_t m = __ballot_sync(full, mine), place = warp_excl(mine ? mk.x : 0u, run);
+      if (mine) {
+        const uint32_t k = at + __popc(m & ((1u << lane) - 1u));
+        l->place[k] = place;
+        l->meta[k] = mk.y;
+        l->lp[k] = (uint16_t)(lp0 + lane);
+        l->of[k] = (uint8_t)i;
+      }
+      at += __popc(m);
+    }
   }
-  for (uint32_t pass = 0; pass < 2u; ++pass) {
-    __syncthreads();  // the places are known; the stages are free
-    if (warp == (uint32_t)kWarps) continue;
-    for (;;) {
-      uint32_t item = 0;
-      if (lane == 0) item = atomicAdd(&l->handed[pass], 1u);
-      item = __shfl_sync(full, item, 0);
-      if (!small) {
-        if (item >= min(l->planes, kListedPlanes)) break;
-        const uint32_t i = l->of[item];
-        if (i == kListed) continue;
-        const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
-        const bool held = c->held[st] == tile;
-        if (held == (pass == 0u))
-          warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, held ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr,
-                               l->meta[item], l->place[item], buf, sal);
-        continue;
+  __syncthreads();  // the list is complete
+  const uint32_t planes = min(l->planes, kListedPlanes);
+  uint32_t own_place = kNoTile, own_meta = 0;
+  for (uint32_t k0 = 0; own.tile != kNoTile && own_place == kNoTile && k0 < planes; k0 += 32u) {  // the warp's own plane leaves it
+    const uint32_t k = min(k0 + lane, planes - 1u), i = l->of[k];
+    const uint32_t m = __ballot_sync(full, i < kListed && l->tile[min(i, kListed - 1u)] == own.tile && l->lp[k] == own.lp);
+    if (m == 0u) continue;
+    const uint32_t at = k0 + (uint32_t)__ffs((int)m) - 1u;
+    own_place = l->place[at];
+    own_meta = l->meta[at];
+    __syncwarp();
+    if (lane == 0) l->of[at] = (uint8_t)kListed;
+  }
+  __syncthreads();
+  if (own_place != kNoTile) {
+    write_blockwise<DT, false>(make_warp_team(nullptr), pl, c->d, (uint64_t)own.tile * pl.ppt + own.lp, own.plane, own.info, sal, own_meta >> 2,
+                               own_place);
+    __syncwarp();
+  }
+  // (planes lie in stages when all do, and are fetched into them otherwise: then none is held)
+  while (warp < (uint32_t)kWarps) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(&l->handed, 1u);
+    item = __shfl_sync(full, item, 0);
+    if (item >= planes) break;
+    const uint32_t i = l->of[item];
+    if (i == kListed) continue;
+    const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
+    const uint8_t* plane = c->held[st] == tile ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr;
+    warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, plane, l->meta[item], l->place[item], buf, sal);
+  }
+  if (c->head == kNoTile) return;  // (the same for every thread: nothing was linked since the list was made)
+  __syncthreads();                 // the stages are free
+  if (warp == (uint32_t)kWarps) return;
+  uint32_t at;
+  for (uint32_t tile; (tile = warp_take_linked(c, at)) != kNoTile;) {
+    const uint64_t p0 = (uint64_t)tile * pl.ppt;
+    const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
+    for (uint32_t lp0 = 0; lp0 < np; lp0 += 32u) {
+      const uint2 mk = lp0 + lane < np ? load_marker(c->d, p0 + lp0 + lane) : make_uint2(0u, 0u);
+      const uint32_t place = warp_excl((mk.y & 3u) != kClsNormal ? mk.x : 0u, at);
+      for (uint32_t m = __ballot_sync(full, (mk.y & 3u) != kClsNormal); m; m &= m - 1u) {
+        const uint32_t b = (uint32_t)__ffs((int)m) - 1u;
+        warp_plane_write<DT>(c, p0 + lp0 + b, nullptr, __shfl_sync(full, mk.y, (int)b), __shfl_sync(full, place, (int)b), buf, sal);
       }
-      if (item >= n * (uint32_t)kWarps) break;
-      const uint32_t i = item / (uint32_t)kWarps, slice = item % (uint32_t)kWarps, tile = l->tile[i], st = l->stage[i];
-      const bool held = c->held[st] == tile;
-      if (held != (pass == 0u) || !((l->slices[i] >> slice) & 1u) || l->base[i] == kNoTile) continue;
-      warp_slice_write<DT, TT>(c, tile, slice, l->base[i] + l->before[i][slice],
-                               held ? stages + (uint64_t)st * pl.stage_bytes : nullptr, buf, sal);
-    }
-    while (pass) {  // the tiles that were not listed, a warp each
-      uint32_t tile = kNoTile;
-      if (lane == 0)
-        for (tile = *(volatile uint32_t*)&c->head; tile != kNoTile;) {
-          const uint32_t seen = atomicCAS(&c->head, tile, c->a.defer_next[tile]);
-          if (seen == tile) {
-            c->a.defer_next[tile] = 0u;
-            break;
-          }
-          tile = seen;
-        }
-      tile = __shfl_sync(full, tile, 0);
-      if (tile == kNoTile) break;
-      uint32_t at = place_of(tile);
-      if (at == kNoTile) break;
-      for (uint32_t slice = 0; slice < (uint32_t)kWarps; ++slice) at += warp_slice_write<DT, TT>(c, tile, slice, at, nullptr, buf, sal);
     }
   }
 }
@@ -1361,7 +1534,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
         s_ctl.held[s] = kNoTile;
         s_list.mask[s] = 0;
       }
-      s_list.count = s_list.planes = s_list.handed[0] = s_list.handed[1] = 0;
+      s_list.count = s_list.planes = s_list.handed = 0;
     }
   }
   // (the ticket counter of this call was returned to zero by the call before the previous one, which had
@@ -1481,7 +1654,6 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     }
   } else {
     // ======================= consumers =======================
-    const Team team = make_team(TT, nullptr);
     const uint32_t grain = plane_grain(pl);
     uint32_t rp = 0, s = 0, phase = 0;
     for (;;) {
@@ -1497,22 +1669,37 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
       if (tile >= pl.ntiles) break;
       const uint32_t p0 = tile * pl.ppt;
       const uint32_t np = (uint32_t)min((uint64_t)pl.ppt, pl.P - p0);
-      // (which warp takes which slice changes from tile to tile, so that a periodic pattern of outlier-rich planes does not
-      // land on the same warp every time)
-      const uint32_t slice = (warp + tile) & ((uint32_t)kWarps - 1u);
-      const uint32_t lp = slice * (32u / TT) + lane / TT, at = min(lp, np - 1u);
+      // (what follows from the lane's number is worked out anew for each tile: kept in registers, it takes those of the sweep)
+      uint32_t me = lane;
+      asm volatile("" : "+r"(me));
+      Team team;
+      team.size = TT;
+      team.lane = me & (TT - 1u);
+      team.mask = TT == 32 ? 0xFFFFFFFFu : ((1u << (TT & 31)) - 1u) << (me & ~(TT - 1u));
+      team.block = false;
+      team.nwarps = 0;
+      team.red = nullptr;
+      const uint32_t slice = warp_slice(tile);
+      const uint32_t lp = slice * (32u / TT) + me / TT, at = min(lp, np - 1u);
       const bool active = lp < np;
       uint8_t* stage = smem + pl.sm_tile + (uint64_t)s * pl.stage_bytes;
       const uint32_t meta = plane_sweep<DT, SIGMA, K, TT, EDGE>(team, pl, d, a, stage + (uint64_t)at * pl.plane_bytes,
                                                                 (uint64_t)p0 + at, grain, active, rp);
       if (scan_on) {  // phase 1 of the block-wise path
         const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, active && (meta & 3u) != kClsNormal && team.lane == 0);
-        if (leaders)
-          warp_tile_measure<DT, TT>(&s_ctl, &s_list, stage, (uint64_t)p0, s, slice, leaders, meta,
-                                    reinterpret_cast<uint32_t*>(smem + pl.sm_sal + warp * pl.sal_stride));
+        // (planes of teams of sixteen lanes and more have more than four blocks)
+        if (leaders) {
+          if (TT <= 8 && is_small_plane(pl)) warp_tile_encode<DT, (TT <= 8 ? TT : 8)>(&s_ctl, &s_list, stage, s, leaders, meta);
+          else
+            warp_tile_put_off<DT, TT>(&s_ctl, &s_list, stage, s, leaders, meta, smem + pl.sm_sal);
+        }
         if (lane == 0) {
           if (leaders) __threadfence_block();  // the warp's sums before its arrival
-          if ((atomicAdd(&s_ctl.arr[s], 1u) & 7u) == 7u) warp_tile_publish(&s_ctl, &s_list, s, tile);
+          if ((atomicAdd(&s_ctl.arr[s], 1u) & 7u) == 7u) {  // the last of the tile's eight warps: its sums are complete
+            __threadfence_block();                          // (the other warps' after their arrivals)
+            if (*(volatile uint32_t*)&s_ctl.C[s] == 0u) scan_publish(a.scan, tile, 0u);
+            else warp_tile_publish(&s_ctl, &s_list, s, tile);
+          }
         }
       }
       __syncwarp();
@@ -1523,7 +1710,10 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   }
   if (scan_on) {
     __syncthreads();
-    if (s_list.count != 0u && !s_abort) warp_phase2<DT, TT>(&s_ctl, &s_list, smem + pl.sm_tile, smem + pl.sm_sal);
+    if (s_list.count != 0u && !s_abort) {
+      if (TT <= 8 && is_small_plane(pl)) warp_phase2_small<DT, (TT <= 8 ? TT : 8)>(&s_ctl, &s_list, smem + pl.sm_tile);
+      else warp_phase2_large<DT>(&s_ctl, &s_list, smem + pl.sm_tile, smem + pl.sm_sal);
+    }
   }
   cta_exit(pl, a, s_ctl.d, &s_last);
 }

@@ -790,9 +790,8 @@ __device__ __forceinline__ void huffman_lut(HufDecode* t, uint32_t i, uint32_t n
 //                                        of that call was performed when its kernel completed, so no fence is
 //                                        needed between a tile's add and the clearing store.
 //   gpre[g] = epoch << 32 | sum of U     over all tiles of groups 0..g, published by whoever has worked it out
-// Progress: tiles are taken in ticket order by CTAs that are running, a CTA works through its tiles in
-// increasing order, and a tile publishes before it waits; so the smallest tile that has not published is
-// never waiting.  Every wait is bounded all the same and reports a time-out instead of hanging.
+// Progress: tiles are taken in ticket order by CTAs that are running, and a CTA publishes all its tiles before it waits for
+// another's; so nobody who waits holds up a tile.  Every wait is bounded all the same and reports a time-out instead of hanging.
 struct Scan {
   unsigned long long* tile;
   unsigned long long* grp;
@@ -872,6 +871,100 @@ static __device__ __noinline__ bool scan_prefix(const Scan& s, uint32_t t, uint3
   }
   if (g > 0 && lane == 0) st_relaxed(&s.gpre[g - 1u], ((unsigned long long)s.epoch << 32) | (gsum & 0xFFFFFFFFull));
   prefix = (uint32_t)(gsum + warp_sum_u64(own));
+  return true;
+}
+
+// The same for up to 32 tiles at once by one warp: lane i < n asks for tile t (with t in no particular order) and gets the sum
+// before it.  One warp to a CTA asks, and the group sums are read once for all its tiles: with a warp to a tile, 128 x 192 bf16
+// planes of 28 x 28 (3,072 tiles, every one with an outlier-rich plane) had 3,100 warps reading the same dozen lines, which held
+// up the publications they waited for: 8 to 35 us from the last publication to the last place.
+static __device__ __noinline__ bool scan_places(const Scan& s, uint32_t t, uint32_t n, uint32_t& prefix) {
+  constexpr uint32_t kAhead = 4;
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, g = t >> 5;
+  const bool asks = lane < n;
+  // tiles of the own groups: the first few tiles' words are on their way while the group prefixes are looked up
+  unsigned long long own[kAhead];
+#pragma unroll
+  for (uint32_t i = 0; i < kAhead; ++i) {
+    const uint32_t ti = __shfl_sync(full, t, (int)i);
+    own[i] = i < n && lane < (ti & 31u) ? ld_relaxed(&s.tile[(ti & ~31u) + lane]) : 0ull;
+  }
+  // prefixes of the groups: those that somebody has published, then the lowest of the others by walking back, then forward
+  bool have = !asks || g == 0u;
+  unsigned long long pre = 0;
+  uint32_t polls = 0;
+  while (!__all_sync(full, have)) {
+    uint32_t low = have ? 0xFFFFFFFFu : g, high = have ? 0u : g;
+    asm volatile("redux.sync.min.u32 %0, %0, %1;" : "+r"(low) : "r"(full));
+    asm volatile("redux.sync.max.u32 %0, %0, %1;" : "+r"(high) : "r"(full));
+    const unsigned long long v = have ? 0ull : ld_relaxed(&s.gpre[g - 1u]);
+    unsigned long long sum = 0;
+    bool found = true;
+    for (uint32_t hi = low;;) {
+      const bool act = lane < hi;
+      const uint32_t j = act ? hi - 1u - lane : 0u;
+      const unsigned long long vp = act ? ld_relaxed(&s.gpre[j]) : 0ull, vg = act ? ld_relaxed(&s.grp[j]) : 0ull;
+      const bool known = act && (uint32_t)(vp >> 32) == s.epoch;
+      const uint32_t pm = __ballot_sync(full, known), first = pm ? (uint32_t)__ffs((int)pm) - 1u : 32u;
+      // (every group before another one is a whole group of 32 tiles)
+      found = __all_sync(full, lane > first || !act || known || (vg >> 40) == 32ull);
+      if (!found) break;
+      sum += warp_sum_u64(lane > first || !act ? 0ull : (known ? vp & 0xFFFFFFFFull : vg & ((1ull << 40) - 1ull)));
+      if (first < 32u || hi <= 32u) break;
+      hi -= 32u;
+    }
+    if (!have && (uint32_t)(v >> 32) == s.epoch) {
+      have = true;
+      pre = v & 0xFFFFFFFFull;
+    }
+    if (found) {
+      // groups low - 1 (whose prefix is `sum`), low, low + 1, ... as far as they are complete and somebody here asks
+      const uint32_t j = low + lane - 1u;
+      const unsigned long long vg = lane > 0u && j < high ? ld_relaxed(&s.grp[j]) : 0ull;  // (none when one group is asked for)
+      const uint32_t not_done = ~__ballot_sync(full, lane == 0u || (vg >> 40) == 32ull);
+      const uint32_t upto = not_done ? (uint32_t)__ffs((int)not_done) - 1u : 32u;
+      unsigned long long incl = lane == 0u ? sum : (vg & ((1ull << 40) - 1ull));
+#pragma unroll
+      for (uint32_t o = 1; o < 32u; o <<= 1) {
+        const unsigned long long up = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += up;
+      }
+      if (lane < upto) st_relaxed(&s.gpre[j], ((unsigned long long)s.epoch << 32) | (incl & 0xFFFFFFFFull));
+      const uint32_t at = have ? 0u : g - low;  // (the lane that holds the prefix this one wants)
+      const unsigned long long mine = __shfl_sync(full, incl, (int)min(at, 31u));
+      if (!have && at < upto) {
+        have = true;
+        pre = mine;
+      }
+    } else {
+      if (++polls >= s.polls) return false;
+      __nanosleep(polls < 4u ? 100u : 500u);
+    }
+  }
+  // the own groups
+  for (uint32_t i0 = 0; i0 < n; i0 += kAhead) {
+    if (i0) {
+#pragma unroll
+      for (uint32_t i = 0; i < kAhead; ++i) {
+        const uint32_t ti = __shfl_sync(full, t, (int)min(i0 + i, 31u));
+        own[i] = i0 + i < n && lane < (ti & 31u) ? ld_relaxed(&s.tile[(ti & ~31u) + lane]) : 0ull;
+      }
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < kAhead; ++i) {
+      if (i0 + i >= n) break;
+      const uint32_t ti = __shfl_sync(full, t, (int)(i0 + i));
+      const bool act = lane < (ti & 31u);
+      while (!__all_sync(full, !act || (uint32_t)(own[i] >> 32) == s.epoch)) {
+        if (++polls >= s.polls) return false;
+        __nanosleep(polls < 4u ? 100u : 500u);
+        if (act) own[i] = ld_relaxed(&s.tile[(ti & ~31u) + lane]);
+      }
+      const unsigned long long sum = warp_sum_u64(act ? own[i] & 0xFFFFFFFFull : 0ull);
+      if (lane == i0 + i) pre += sum;
+    }
+  }
+  prefix = (uint32_t)pre;
   return true;
 }
 
