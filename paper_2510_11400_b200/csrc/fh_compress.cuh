@@ -1542,8 +1542,10 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   if (tid == (uint32_t)kThreads && a.early_ticket)
     first_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)pl.first_req);
   __syncthreads();
-  dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
-  dep_trigger();  // the next kernel on the stream may become resident as this one drains
+  if (warp < (uint32_t)kWarps || !a.early_load) {  // (the producer only reads the input and takes tickets)
+    dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
+    dep_trigger();  // the next kernel on the stream may become resident as this one drains
+  }
   // (the sweeps only need the first and the last of these: the others wait in shared memory, not in registers)
   Dest d = {};
   if (warp < (uint32_t)kWarps) {  // (the producer goes straight to its first loads)
@@ -2167,8 +2169,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
       s_ctl.own = kNoTile;
     }
   }
-  dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
-  dep_trigger();  // the next kernel on the stream may become resident as this one drains
   auto issue = [&](uint32_t s) {
     const uint32_t t = next_ticket;
     s_tiles[s] = t;
@@ -2178,11 +2178,15 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
       next_ticket = issued < early ? t + 1u : (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
     }
   };
+  // the previous kernel on the stream has completed; global memory may be touched from here on (the input is only read)
+  if (!a.early_load) dep_wait();
   if (tid == 0) {  // the first loads before anything else
     if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + early);
     issue(0);
     issue(1);
   }
+  if (a.early_load) dep_wait();
+  dep_trigger();  // the next kernel on the stream may become resident as this one drains
   const Dest d = make_dest(pl, a);
   if (tid == 0) {
     if (!d.fits && blockIdx.x == 0) report_error(a, kErrCapacity);

@@ -983,6 +983,7 @@ struct CompressArgs {
   uint32_t* defer_next;                 // one word per tile, zero between calls: tiles put off (see BlockCtl)
   uint32_t parity;                      // which of the two ticket counters this call uses
   uint32_t early_ticket;                // 1: tiles may be requested before the previous kernel on the stream has completed
+  uint32_t early_load;                  // 1: ... and loaded: the input was complete before that kernel started
   // channel- and tensor-wide three-sigma modes: the statistics passes' results per channel (ChanStat, four words each),
   // the words that the call's last CTA returns to zero, and outlier counts per plane
   unsigned long long* chan_stats;
@@ -990,6 +991,9 @@ struct CompressArgs {
   const uint32_t* plane_nout;
 };
 
+// Decompress kernels that follow one another in a schedule need nothing of one another: the first waits for the compress
+// kernels and then lets its successor start, which starts its own successor and waits for its predecessor only before it ends.
+constexpr uint32_t kInOrder = 0, kFirst = 1, kAfter = 2;
 struct DecompressArgs {
   const uint8_t* src_base;
   unsigned long long src_bytes;
@@ -997,6 +1001,7 @@ struct DecompressArgs {
   uint8_t* dst;
   unsigned long long* d_status;        // optional
   Scratch* sc;
+  uint32_t order;                      // kInOrder, kFirst, kAfter: see decompress_begin
   unsigned long long team_stride;      // a prime, at most the number of warps of the grid (see decompress_kernel)
   unsigned long long cta_stride;       // ... of CTAs
 };
