@@ -227,10 +227,6 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
     pl.sal_stride = (uint32_t)base + pl.pay_bytes;
     pl.sm_total = units * pl.sal_stride;
     if (pl.sm_total > kSmemLimit) return FH_ERR_UNSUPPORTED;
-    {
-      const uint64_t ctas = (pl.P * ((pl.HW + 7 + 1023) / 1024) + fh::kWarps - 1) / fh::kWarps;
-      pl.ntiles = (uint32_t)(ctas > 0x7FFFFFFFull ? 0x7FFFFFFFull : ctas);
-    }
     *out = pl;
     if (var) *var = Variant();
     return FH_OK;

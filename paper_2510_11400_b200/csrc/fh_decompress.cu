@@ -6,15 +6,17 @@
 namespace fh {
 namespace {
 
-template <int DT>
+template <int DT, bool ALIGNED>
 int launch_decompress_t(const Plan& pl, const DecompressArgs& a, cudaStream_t stream) {
   int grid = 0;
-  int rc = grid_for(decompress_kernel<DT>, pl.sm_total, pl.ntiles, &grid);
+  const uint32_t lines = chunk_lines(pl.HW, Chunk<DT>::VE, ALIGNED), chunks = (lines + Chunk<DT>::kLines - 1) / Chunk<DT>::kLines;
+  const uint64_t ctas = (pl.P * chunks + kWarps - 1) / kWarps;
+  int rc = grid_for(decompress_kernel<DT, ALIGNED>, pl.sm_total, (uint32_t)std::min<uint64_t>(ctas, 0x7FFFFFFFu), &grid);
   if (rc != FH_OK) return rc;
   DecompressArgs b = a;
   b.team_stride = prime_at_most((uint64_t)grid * kWarps);
   b.cta_stride = prime_at_most((uint64_t)grid);
-  return launch_dependent(decompress_kernel<DT>, grid, kThreads, pl.sm_total, stream, pl, b) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+  return launch_dependent(decompress_kernel<DT, ALIGNED>, grid, kThreads, pl.sm_total, stream, pl, b) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
 
 // Planes of at most 128 groups: tiles of 256 / team planes restored in shared memory, one bulk store per tile.
@@ -52,10 +54,24 @@ int launch_decompress_small(const Plan& pl0, const DecompressArgs& a, cudaStream
   return FH_OK;
 }
 
+// (see decompress_large)
+constexpr uint64_t kLargeBytes = 128ull << 20;
+int launch_decompress_large(const Plan& pl, const DecompressArgs& a, cudaStream_t stream) {
+  int grid = 0;
+  const uint64_t ctas = (pl.P * ((pl.HW + 3 + 1023) / 1024) + kWarps - 1) / kWarps;
+  int rc = grid_for(decompress_large<kF32>, pl.sm_total, (uint32_t)std::min<uint64_t>(ctas, 0x7FFFFFFFu), &grid);
+  if (rc != FH_OK) return rc;
+  DecompressArgs b = a;
+  b.team_stride = prime_at_most((uint64_t)grid * kWarps);
+  b.cta_stride = prime_at_most((uint64_t)grid);
+  return launch_dependent(decompress_large<kF32>, grid, kThreads, pl.sm_total, stream, pl, b) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+}
+
 template <int DT>
 int launch_decompress_dt(const Plan& pl, const DecompressArgs& a, cudaStream_t stream) {
   if (pl.groups <= 128 && pl.team == 32u) return launch_decompress_small<DT>(pl, a, stream);
-  return launch_decompress_t<DT>(pl, a, stream);
+  if (DT == kF32 && pl.dense_bytes > kLargeBytes) return launch_decompress_large(pl, a, stream);
+  return pl.plane_bytes % 16 == 0 ? launch_decompress_t<DT, true>(pl, a, stream) : launch_decompress_t<DT, false>(pl, a, stream);
 }
 
 }  // namespace

@@ -520,12 +520,338 @@ __device__ __forceinline__ void store_group(uint8_t* out, uint32_t g, float v0, 
   }
 }
 
+// Four codes (the low bits of `word`) as biased floats 2^23 + q; dequant2 takes the bias off again and applies scale and
+// minimum, two values an instruction.  Whole bytes are put under the exponent by one byte permutation.
+template <int BITS>
+__device__ __forceinline__ void spread4(uint32_t word, uint32_t (&q)[4]) {
+  constexpr uint32_t bias = 0x4B000000u;
+  if (BITS == 8) {
+#pragma unroll
+    for (uint32_t j = 0; j < 4u; ++j) q[j] = __byte_perm(word, bias, 0x7440u + j);
+  } else if (BITS == 4) {
+    const uint32_t even = word & 0x0F0Fu, odd = (word >> 4) & 0x0F0Fu;
+    q[0] = __byte_perm(even, bias, 0x7440u);
+    q[1] = __byte_perm(odd, bias, 0x7440u);
+    q[2] = __byte_perm(even, bias, 0x7441u);
+    q[3] = __byte_perm(odd, bias, 0x7441u);
+  } else {
+#pragma unroll
+    for (uint32_t j = 0; j < 4u; ++j) q[j] = ((word >> (2u * j)) & 3u) | bias;
+  }
+}
+__device__ __forceinline__ void dequant2(uint32_t q0, uint32_t q1, f32x2 scale2, f32x2 lo2, float& v0, float& v1) {
+  const f32x2 q = pack2(__uint_as_float(q0), __uint_as_float(q1)), back = pack2(-8388608.0f, -8388608.0f);
+  unpack2(fma2(add2(q, back), scale2, lo2), v0, v1);
+}
+
+// What a warp takes of a plane at a time: up to kLines lines of 32 16-byte vectors of the OUTPUT, 4 KB (fp32) or 2 KB (bf16).
+// Lane l restores vector l of every line.
+template <int DT>
+struct Chunk {
+  static constexpr uint32_t VE = DT == kF32 ? 4u : 8u;     // elements of a vector
+  static constexpr int kLines = DT == kF32 ? 8 : 4;
+};
+// Codes of a lane's vectors.  ALIGNED: the plane starts on a 16-byte boundary of the tensor and is whole vectors.  Codes of a
+// word and more a vector are loaded by the lane that restores it, narrower ones as whole words, lane after lane, and handed on
+// by shuffle (WORDS).  Otherwise vectors are counted from the one that holds the plane's first element, `shift`
+// of whose elements belong to the plane before, and a vector's codes are picked out of NW + 1 words by a funnel shift.
+template <int DT, int BITS, bool ALIGNED>
+struct ChunkCodes {
+  static constexpr int VE = (int)Chunk<DT>::VE, VB = VE * BITS, K = Chunk<DT>::kLines, NW = VB > 32 ? 2 : 1;
+  static constexpr bool WORDS = ALIGNED && VB < 32;
+  static constexpr int J = WORDS ? K * VB / 32 : K, N = ALIGNED ? NW : NW + 1;
+  uint32_t w[J][N];
+
+  // vectors v0 + 32 k + lane, those below v1
+  __device__ __forceinline__ void load(const uint8_t* slot, uint32_t nwords, uint32_t lane, uint32_t v0, uint32_t v1, uint32_t shift) {
+    const uint32_t* s32 = reinterpret_cast<const uint32_t*>(slot);
+#pragma unroll
+    for (int k = 0; k < J; ++k) {
+      const uint32_t v = v0 + (uint32_t)k * 32u + lane;
+#pragma unroll
+      for (int n = 0; n < N; ++n) w[k][n] = 0;
+      if (WORDS) {
+        const uint32_t i = (v0 >> 5) * VB + (uint32_t)k * 32u + lane;
+        if (i < (v1 * VB + 31u) >> 5) w[k][0] = __ldg(s32 + i);
+      } else if (ALIGNED) {
+        if (v < v1) {
+          if (VB == 32) {
+            w[k][0] = __ldg(s32 + v);
+          } else {
+            const uint2 t = __ldg(reinterpret_cast<const uint2*>(slot) + v);
+            w[k][0] = t.x;
+            w[k][N - 1] = t.y;
+          }
+        }
+      } else {
+        const int32_t i0 = (int32_t)(v * VE) - (int32_t)shift, w0 = (i0 * BITS) >> 5;
+#pragma unroll
+        for (int n = 0; n < N; ++n)
+          if (v < v1 && (uint32_t)(w0 + n) < nwords) w[k][n] = __ldg(s32 + w0 + n);
+      }
+    }
+  }
+
+  // restores them to the plane at `out`
+  __device__ __forceinline__ void restore(uint32_t lane, uint32_t v0, uint32_t v1, uint32_t HW, uint32_t shift, float scale, float lo, uint8_t* out) const {
+    const f32x2 scale2 = pack2(scale, scale), lo2 = pack2(lo, lo);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const uint32_t v = v0 + (uint32_t)k * 32u + lane;
+      uint32_t mine = 0;
+      if (WORDS) {  // the vector's bits are bits (32 k + lane) * VB ... of the chunk's
+        constexpr uint32_t per = 32 / VB;  // vectors of a word
+        mine = __shfl_sync(0xFFFFFFFFu, w[k * VB / 32][0], (uint32_t)(k * VB) % 32u + lane / per) >> (lane % per * VB);
+      }
+      if (v >= v1) continue;
+      const int32_t i0 = (int32_t)(v * VE) - (int32_t)shift;
+      float x[VE];
+#pragma unroll
+      for (int h = 0; h < VE; h += 4) {
+        constexpr int per = 32 / BITS;  // codes of a word
+        const int n = h / per;
+        uint32_t word = WORDS ? mine : w[WORDS ? 0 : k][n], q[4];
+        if (!ALIGNED) word = __funnelshift_r(word, w[WORDS ? 0 : k][n + 1 < N ? n + 1 : N - 1], (uint32_t)(i0 * BITS) & 31u);
+        spread4<BITS>(word >> ((h % per) * BITS), q);
+        dequant2(q[0], q[1], scale2, lo2, x[h], x[h + 1]);
+        dequant2(q[2], q[3], scale2, lo2, x[h + 2], x[h + 3]);
+      }
+      if (ALIGNED || (i0 >= 0 && i0 + VE <= (int32_t)HW)) {
+        uint4 t;
+        if (DT == kF32) {
+          t = make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
+        } else {
+          t.x = f32x2_to_bf16x2(x[0], x[1]);
+          t.y = f32x2_to_bf16x2(x[2], x[3]);
+          t.z = f32x2_to_bf16x2(x[VE - 4], x[VE - 3]);
+          t.w = f32x2_to_bf16x2(x[VE - 2], x[VE - 1]);
+        }
+        *reinterpret_cast<uint4*>(out + (int64_t)i0 * (DT == kF32 ? 4 : 2)) = t;
+      } else {  // the plane's first and last vectors, which it may share with its neighbours
+#pragma unroll
+        for (int j = 0; j < VE; ++j)
+          if (i0 + j >= 0 && i0 + j < (int32_t)HW) store_elem<DT>(out, (uint32_t)(i0 + j), x[j]);
+      }
+    }
+  }
+};
+
+// What the streaming part of decompress_kernel needs to know of the container.
+struct StreamIn {
+  const uint8_t* src;
+  uint8_t* dst;
+  unsigned long long total, slots_off, ovf_off, plane_bytes;
+  uint32_t P, HW, npay, nsal;
+};
+
+// The normal and the raw planes: warp `w` takes items w, w + stride, ...; item = plane * chunks + chunk.  (Chunks of equal size
+// instead of whole ones and a rest: bf16 planes of 56 x 56 31.0 -> 33.7 us.)  What bounds it is latency: the next item's codes and
+// table entry are requested before the present one is worked on.
+// us a call, chunk by chunk before and now: bf16, 2 bits, 128 x 96 planes of 112 x 112 84.5 -> 67.1, 128 x 144 of 56 x 56 41.9 ->
+// 31.0, 128 x 192 of 28 x 28 17.1 -> 14.1; fp32, 4 bits, 64 x 128 of 28 x 28 9.3 -> 8.3.  `first`: the first item's entry,
+// which was asked for along with the header.  False when the container is inconsistent.
+template <int DT, int BITS, bool ALIGNED>
+__device__ __forceinline__ bool stream_planes(const StreamIn& in, uint32_t w, uint32_t stride, uint4 first) {
+  constexpr uint32_t VE = Chunk<DT>::VE, LINES = Chunk<DT>::kLines;
+  const uint32_t lane = threadIdx.x & 31u, HW = in.HW;
+  const uint32_t lines = chunk_lines(HW, VE, ALIGNED), chunks = (lines + LINES - 1u) / LINES;
+  const uint32_t dp = stride / chunks, dc = stride - dp * chunks;
+  const uint64_t pb = in.plane_bytes;
+  uint32_t gp = w / chunks, ch = w - gp * chunks;
+  bool good = true;
+  if (gp >= in.P) return true;
+  ChunkCodes<DT, BITS, ALIGNED> cur, nxt;
+  uint4 e = first, en;
+  // first vector of chunk c; `shift`: elements of the plane's first vector that belong to the plane before
+  auto from = [&](uint32_t c) { return min(c * LINES, lines) * 32u; };
+  auto shift_of = [&](uint32_t p) { return ALIGNED ? 0u : ((uint32_t)(p * pb) & 15u) / (DT == kF32 ? 4u : 2u); };
+  auto last = [&](uint32_t p, uint32_t c) { return min(from(c + 1u), (HW + shift_of(p) + VE - 1u) / VE); };
+  auto load = [&](uint32_t p, uint32_t c, ChunkCodes<DT, BITS, ALIGNED>& to) {
+    // (the slot sits at a closed-form offset; what a plane of another class keeps there is read and dropped)
+    to.load(in.src + in.slots_off + (uint64_t)p * in.npay, in.npay >> 2, lane, from(c), last(p, c), shift_of(p));
+  };
+  load(gp, ch, cur);
+  for (;;) {
+    uint32_t gn = gp + dp, cn = ch + dc;
+    if (cn >= chunks) {
+      cn -= chunks;
+      ++gn;
+    }
+    const bool more = gn < in.P;
+    if (more) {
+      load(gn, cn, nxt);
+      en = __ldg(reinterpret_cast<const uint4*>(in.src + 64) + gn);
+    }
+    const uint32_t cls = e.y & 3u;
+    const unsigned long long off = (unsigned long long)e.x * 16ull;
+    uint8_t* out = in.dst + gp * pb;
+    if (cls == kClsNormal) {
+      if (off == in.slots_off + (uint64_t)gp * in.npay)
+        cur.restore(lane, from(ch), last(gp, ch), HW, shift_of(gp), __uint_as_float(e.w), __uint_as_float(e.z), out);
+      else good = false;
+    } else if (cls == kClsRaw) {
+      // the continuation, when there is one, lies in the overflow region
+      const unsigned long long ovf_avail = off ? in.total - off : 0ull;
+      if ((off != 0 && (off < in.ovf_off || off > in.total)) || (pb > in.npay && pb - in.npay > ovf_avail)) {
+        good = false;
+      } else {
+        SplitIn raw;
+        raw.slot = in.src + in.slots_off + (uint64_t)gp * in.npay;
+        raw.ovf = in.src + off;
+        raw.npay = in.npay;
+        constexpr uint32_t unit = ALIGNED ? 16u : (DT == kF32 ? 4u : 2u);
+        const uint32_t n = (uint32_t)pb / unit, i1 = (uint32_t)((uint64_t)n * (ch + 1u) / chunks);
+#pragma unroll 4
+        for (uint32_t i = (uint32_t)((uint64_t)n * ch / chunks) + lane; i < i1; i += 32u) {
+          if (ALIGNED) reinterpret_cast<uint4*>(out)[i] = __ldg(reinterpret_cast<const uint4*>(raw.at(16u * i)));
+          else if (DT == kF32) reinterpret_cast<uint32_t*>(out)[i] = raw.ld32(4u * i);
+          else reinterpret_cast<uint16_t*>(out)[i] = (uint16_t)raw.ld16(2u * i);
+        }
+      }
+    } else if (cls != kClsSalient || in.nsal == 0u) {
+      good = false;
+    }
+    if (!more) return good;
+    gp = gn;
+    ch = cn;
+    cur = nxt;
+    e = en;
+  }
+}
+
+// Outlier-rich planes of the streaming kernels, from up to 256 table entries at a time: CTA c looks at those of planes c, c + hop,
+// ..., gathers those that are outlier-rich and restores them, a warp each (pl.team = 32) or, when they have many blocks, the whole
+// CTA one after the other.  (A macro: as a function, inlined or not, it costs the streaming loops registers, 28 x 28 planes 5 %.)
+#define FH_RESTORE_OUTLIER_RICH(DT) \
+  if (s_nsal) { \
+    const uint32_t hop = (uint32_t)a.cta_stride, most = blockIdx.x < hop ? ((uint32_t)pl.P + hop - 1u) / hop : 0u; \
+    const Team unit = pl.team == 32u ? make_warp_team(s_red) : make_team(kThreads, s_red); \
+    uint32_t* scr = reinterpret_cast<uint32_t*>(smem + (pl.team == 32u ? (uint64_t)warp * pl.sal_stride : 0ull)); \
+    HufDecode* hd = reinterpret_cast<HufDecode*>(reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes) - 1; \
+    for (uint32_t base = 0; base < most; base += kThreads) { \
+      const uint64_t gp = blockIdx.x + (uint64_t)(base + tid) * hop; \
+      if (gp < pl.P && (__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp) + 1) & 3u) == kClsSalient) \
+        s_list[atomicAdd(&s_nlist, 1u)] = (uint32_t)gp; \
+      __syncthreads(); \
+      const uint32_t n = s_nlist; \
+      for (uint32_t q = pl.team == 32u ? warp : 0u; q < n; q += pl.team == 32u ? (uint32_t)kWarps : 1u) { \
+        const uint32_t gp = s_list[q]; \
+        const unsigned long long off = (unsigned long long)__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp)) * 16ull; \
+        if (off != 0 && (off < ovf_off || off > total)) {  /* (the same for every thread of the unit) */ \
+          bad = true; \
+          continue; \
+        } \
+        SplitIn in; \
+        in.slot = src + slots_off + (uint64_t)gp * npay; \
+        in.ovf = src + off; \
+        in.npay = npay; \
+        /* the payload comes to shared memory first when it fits there */ \
+        const unsigned long long ovf_avail = off ? total - off : 0ull; \
+        const uint32_t got = (uint32_t)min((unsigned long long)pl.pay_bytes, npay + (ovf_avail & ~15ull)); \
+        const uint32_t nnz_s = in.ld32(0), n_dense = in.ld32(4), n_out_d = in.ld32(8), coded = in.ld32(12), es = (uint32_t)pl.esize; \
+        const uint64_t size = 16ull + 4ull * pl.nbm + 4ull * ((uint64_t)pl.H + 1) + a4(2u * nnz_s) + a4(es * nnz_s) + \
+                              (coded ? (uint64_t)coded : 64ull * n_dense) + a4(es * n_out_d); \
+        uint8_t* pay = reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes; \
+        bool good; \
+        if (nnz_s <= pl.HW && n_dense <= pl.nblk && n_out_d <= pl.HW && size <= got) { \
+          for (uint32_t o = 16u * unit.lane; o < (uint32_t)size; o += 16u * unit.size) \
+            *reinterpret_cast<uint4*>(pay + o) = __ldg(reinterpret_cast<const uint4*>(in.at(o))); \
+          team_sync(unit); \
+          FlatIn flat; \
+          flat.p = pay; \
+          flat.npay = got; \
+          good = decode_salient<DT>(unit, s_pl, flat, 0ull, s_eps, a.dst + gp * pl.plane_bytes, scr, hd, s_hdr_ok); \
+        } else { \
+          good = decode_salient<DT>(unit, s_pl, in, ovf_avail, s_eps, a.dst + gp * pl.plane_bytes, scr, hd, s_hdr_ok); \
+        } \
+        if (!good) bad = true; \
+        team_sync(unit);  /* the scratch is reused */ \
+      } \
+      __syncthreads(); \
+      if (tid == 0) s_nlist = 0; \
+      __syncthreads(); \
+    } \
+  }
+
+// Planes of more than 128 groups.  Work items are (plane, chunk) pairs, a warp each (stream_planes), so that large
+// planes spread over many warps; no barrier in the streaming part.  The items' stride is
+// a prime (warps beyond it stay idle), so that a periodic pattern of expensive planes -- every eighth channel
+// outlier-rich, say -- spreads over all warps instead of landing on the few whose index shares a factor with the period.
+// ALIGNED: planes are whole 16-byte vectors (and so lie on 16-byte boundaries).
+// Outlier-rich planes are left for the end (when the header says that there are any): CTA c then looks at the table
+// entries of planes c, c + stride, ... -- the stride a prime again -- gathers those that are outlier-rich and restores
+// them, a warp each (pl.team = 32) or, when they have many blocks, the whole CTA one after the other.
+template <int DT, bool ALIGNED>
+__global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, const DecompressArgs a) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ double s_red[kMaxWarps * 4];
+  __shared__ uint32_t s_hdr_ok, s_bits;
+  __shared__ float s_eps;
+  __shared__ unsigned long long s_total;
+  __shared__ Plan s_pl;  // copy for the outlined slow path, which takes it by address
+  __shared__ uint32_t s_nsal, s_list[kThreads], s_nlist;
+  const uint32_t tid = threadIdx.x, warp = tid >> 5;
+  if (tid == 0) {
+    s_pl = pl;
+    s_nlist = 0;
+  }
+  decompress_begin(a);
+  const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
+  const uint8_t* src = a.src_base + off_in;
+  const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;
+
+  const uint32_t stride = (uint32_t)a.team_stride, wid = blockIdx.x * kWarps + warp;
+  // the first item's table entry along with the header (every CTA checks it, it is 64 bytes)
+  constexpr uint32_t VE = Chunk<DT>::VE, LINES = Chunk<DT>::kLines;
+  const uint32_t gp0 = wid / ((chunk_lines(pl.HW, VE, ALIGNED) + LINES - 1u) / LINES);
+  uint4 first = make_uint4(0u, 0u, 0u, 0u);
+  if (gp0 < pl.P && src_bytes >= 64ull + 16ull * pl.P) first = __ldg(reinterpret_cast<const uint4*>(src + 64) + gp0);
+  if (tid == 0) {
+    uint32_t bits = 0;
+    float eps = 0.0f;
+    unsigned long long total = 0;
+    uint32_t nsal = 0;
+    s_hdr_ok = check_header(pl, src, src_bytes, bits, eps, total, nsal);
+    s_nsal = nsal;
+    s_bits = bits;
+    s_eps = eps;
+    s_total = total;
+  }
+  __syncthreads();
+  const bool hdr_ok = s_hdr_ok != 0;
+  bool bad = !hdr_ok;
+  if (hdr_ok) {
+    const uint32_t bits = s_bits;
+    const unsigned long long total = s_total;
+    const uint32_t npay = a16(4u * ((pl.HW * bits + 31u) / 32u));
+    const unsigned long long slots_off = 64ull + 16ull * pl.P, ovf_off = slots_off + pl.P * (unsigned long long)npay;
+    StreamIn in;
+    in.src = src;
+    in.dst = a.dst;
+    in.total = total;
+    in.slots_off = slots_off;
+    in.ovf_off = ovf_off;
+    in.plane_bytes = pl.plane_bytes;
+    in.P = (uint32_t)pl.P;
+    in.HW = pl.HW;
+    in.npay = npay;
+    in.nsal = s_nsal;
+    if (wid < stride) {
+      if (bits == 2u) bad = !stream_planes<DT, 2, ALIGNED>(in, wid, stride, first);
+      else if (bits == 4u) bad = !stream_planes<DT, 4, ALIGNED>(in, wid, stride, first);
+      else bad = !stream_planes<DT, 8, ALIGNED>(in, wid, stride, first);
+    }
+    FH_RESTORE_OUTLIER_RICH(DT)
+  }
+  decompress_exit(a, bad);
+}
+
 // Normal plane, whole-warp team, one chunk of up to 256 groups starting at group g0 (a multiple of
 // 256).  The chunk's code bytes are fetched as 32-bit words, one or more coalesced loads per lane
 // issued before anything else, and handed to the lanes that need them by shuffle: lane l restores
 // groups g0 + l, g0 + 32 + l, ...  `w` holds the lane's words: word j*32 + l of the chunk's codes.
-template <int DT, int BITS>
-__device__ __forceinline__ void decode_chunk32(const uint32_t (&w)[8], uint32_t lane, uint32_t g0, uint32_t g1,
+template <int BITS>
+__device__ __forceinline__ void decode_chunk_large(const uint32_t (&w)[8], uint32_t lane, uint32_t g0, uint32_t g1,
                                                float scale, float lo, uint8_t* out) {
   constexpr uint32_t L = (1u << BITS) - 1u;
 #pragma unroll
@@ -542,44 +868,8 @@ __device__ __forceinline__ void decode_chunk32(const uint32_t (&w)[8], uint32_t 
       word = w[k];
     }
     if (g < g1)
-      store_group<DT>(out, g, dequant(word & L, scale, lo), dequant((word >> BITS) & L, scale, lo),
+      store_group<kF32>(out, g, dequant(word & L, scale, lo), dequant((word >> BITS) & L, scale, lo),
                       dequant((word >> (2 * BITS)) & L, scale, lo), dequant((word >> (3 * BITS)) & L, scale, lo));
-  }
-}
-
-// The same for bf16 planes of whole 16-byte chunks: a lane restores two neighbouring groups at a time -- groups
-// g0 + 64 k + 2 l and the one after it -- so that eight values leave as one 16-byte store (four stores of 512
-// contiguous bytes per warp and chunk instead of eight of 256).
-template <int BITS>
-__device__ __forceinline__ void decode_chunk32_bf16_pairs(const uint32_t (&w)[8], uint32_t lane, uint32_t g0, uint32_t g1,
-                                                          float scale, float lo, uint8_t* out) {
-  constexpr uint32_t L = (1u << BITS) - 1u, full = 0xFFFFFFFFu;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint32_t g = g0 + (uint32_t)k * 64u + 2u * lane;
-    uint32_t wa, wb;  // code words of groups g and g + 1
-    if (BITS == 2) {         // a byte per group: halfword 32 k + l of the chunk = word 16 k + (l >> 1)
-      const uint32_t src = __shfl_sync(full, w[k >> 1], (uint32_t)(k & 1) * 16u + (lane >> 1));
-      const uint32_t h = src >> ((lane & 1u) * 16u);
-      wa = h & 0xFFu;
-      wb = (h >> 8) & 0xFFu;
-    } else if (BITS == 4) {  // two bytes per group: word 32 k + l, the lane's own
-      wa = w[k] & 0xFFFFu;
-      wb = w[k] >> 16;
-    } else {                 // a word per group: words 64 k + 2 l and the next, held by lanes 2 l mod 32 and the next
-      const uint32_t sl = (2u * lane) & 31u;
-      const uint32_t a0 = __shfl_sync(full, w[2 * k], sl), a1 = __shfl_sync(full, w[2 * k + 1], sl);
-      const uint32_t b0 = __shfl_sync(full, w[2 * k], sl + 1u), b1 = __shfl_sync(full, w[2 * k + 1], sl + 1u);
-      wa = lane < 16u ? a0 : a1;
-      wb = lane < 16u ? b0 : b1;
-    }
-    uint4 v;
-    v.x = f32x2_to_bf16x2(dequant(wa & L, scale, lo), dequant((wa >> BITS) & L, scale, lo));
-    v.y = f32x2_to_bf16x2(dequant((wa >> (2 * BITS)) & L, scale, lo), dequant((wa >> (3 * BITS)) & L, scale, lo));
-    v.z = f32x2_to_bf16x2(dequant(wb & L, scale, lo), dequant((wb >> BITS) & L, scale, lo));
-    v.w = f32x2_to_bf16x2(dequant((wb >> (2 * BITS)) & L, scale, lo), dequant((wb >> (3 * BITS)) & L, scale, lo));
-    if (g + 1u < g1) reinterpret_cast<uint4*>(out)[g >> 1] = v;
-    else if (g < g1) reinterpret_cast<uint2*>(out)[g] = make_uint2(v.x, v.y);
   }
 }
 
@@ -588,10 +878,10 @@ __device__ __forceinline__ void decode_chunk32_bf16_pairs(const uint32_t (&w)[8]
 // elements' codes out of the bit stream with a funnel shift.  The plane's first and last vectors, which it may share
 // with its neighbours, leave as element stores.  `v0`: first vector of the chunk, counted from the one that holds the
 // plane's first element; `shift`: elements of that vector that belong to the plane before.
-template <int DT, int BITS>
-__device__ __forceinline__ void decode_chunk_shifted(const uint8_t* slot, uint32_t nwords, uint32_t lane, uint32_t v0, uint32_t HW,
+template <int BITS>
+__device__ __forceinline__ void decode_chunk_large_shifted(const uint8_t* slot, uint32_t nwords, uint32_t lane, uint32_t v0, uint32_t HW,
                                                      uint32_t shift, float scale, float lo, uint8_t* out) {
-  constexpr int VE = DT == kF32 ? 4 : 8, K = DT == kF32 ? 8 : 4;  // elements of a vector, vectors per lane
+  constexpr int VE = 4, K = 8;  // elements of a vector, vectors per lane
   constexpr uint32_t L = (1u << BITS) - 1u;
   constexpr int NW = VE * BITS > 32 ? 2 : 1;                      // words of codes of a vector
   const uint32_t* s32 = reinterpret_cast<const uint32_t*>(slot);
@@ -613,33 +903,22 @@ __device__ __forceinline__ void decode_chunk_shifted(const uint8_t* slot, uint32
 #pragma unroll
     for (int j = 0; j < VE; ++j) v[j] = dequant((cw[k][(j * BITS) >> 5] >> ((j * BITS) & 31)) & L, scale, lo);
     if (i0 >= 0 && i0 + VE <= (int32_t)HW) {
-      if (DT == kF32) {
-        *reinterpret_cast<float4*>(out + 4ll * i0) = make_float4(v[0], v[1], v[2], v[3]);
-      } else {
-        uint4 q;
-        q.x = f32x2_to_bf16x2(v[0], v[1]);
-        q.y = f32x2_to_bf16x2(v[2], v[3]);
-        q.z = f32x2_to_bf16x2(v[VE - 4], v[VE - 3]);
-        q.w = f32x2_to_bf16x2(v[VE - 2], v[VE - 1]);
-        *reinterpret_cast<uint4*>(out + 2ll * i0) = q;
-      }
+      *reinterpret_cast<float4*>(out + 4ll * i0) = make_float4(v[0], v[1], v[2], v[3]);
     } else {
 #pragma unroll
       for (int j = 0; j < VE; ++j)
-        if (i0 + j >= 0 && i0 + j < (int32_t)HW) store_elem<DT>(out, (uint32_t)(i0 + j), v[j]);
+        if (i0 + j >= 0 && i0 + j < (int32_t)HW) store_elem<kF32>(out, (uint32_t)(i0 + j), v[j]);
     }
   }
 }
 
-// Planes of more than 128 groups.  Work items are (plane, chunk of 1024 elements) pairs, a warp each, so that large
-// planes spread over many warps; no barrier in the streaming part.  Warp w takes items w, w + stride, ...; the stride is
-// a prime (warps beyond it stay idle), so that a periodic pattern of expensive planes -- every eighth channel
-// outlier-rich, say -- spreads over all warps instead of landing on the few whose index shares a factor with the period.
-// Outlier-rich planes are left for the end (when the header says that there are any): CTA c then looks at the table
-// entries of planes c, c + stride, ... -- the stride a prime again -- gathers those that are outlier-rich and restores
-// them, a warp each (pl.team = 32) or, when they have many blocks, the whole CTA one after the other.
+// fp32 tensors that are larger than the L2 cache: the same in chunks of 1,024 elements, one at a time, nothing requested ahead.
+// Their restored elements go to memory while they are written, and requests ahead of the stores cost such a tensor more than
+// their latency: 400 MB restored from 4 bits, 40 x 40 planes 80 us so and 86 with stream_planes, 28 x 28 76 and 84, 62 x 24 76 and
+// 83, 32 x 32 (1 GiB) 213 and 217; 25 MB of 28 x 28 9.2 and 8.3.  (bf16 tensors have twice the elements to work on per byte and
+// gain from requests ahead at any size.)
 template <int DT>
-__global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, const DecompressArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) decompress_large(const Plan pl, const DecompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 4];
   __shared__ uint32_t s_hdr_ok, s_bits;
@@ -677,7 +956,7 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
     const unsigned long long total = s_total;
     const uint32_t npay = a16(4u * ((pl.HW * bits + 31u) / 32u));
     const unsigned long long slots_off = 64ull + 16ull * pl.P, ovf_off = slots_off + pl.P * (unsigned long long)npay;
-    constexpr uint32_t VE = DT == kF32 ? 4u : 8u;
+    constexpr uint32_t VE = 4u;
     const bool aligned = (pl.plane_bytes & 15u) == 0u;  // (dst is 16-byte aligned)
     const uint32_t chunks = (pl.HW + (aligned ? 0u : VE - 1u) + 1023u) >> 10;
     const uint32_t items = (uint32_t)pl.P * chunks, stride = (uint32_t)a.team_stride;
@@ -709,18 +988,14 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
         }
         const float lo = __uint_as_float(e.z), scale = __uint_as_float(e.w);
         if (!aligned) {
-          const uint32_t shift = ((uint32_t)(gp * pl.plane_bytes) & 15u) / (DT == kF32 ? 4u : 2u), v0 = ch * (1024u / VE);
-          if (bits == 2u) decode_chunk_shifted<DT, 2>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
-          else if (bits == 4u) decode_chunk_shifted<DT, 4>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
-          else decode_chunk_shifted<DT, 8>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
-        } else if (DT == kBF16) {
-          if (bits == 2u) decode_chunk32_bf16_pairs<2>(cw, lane, g0, g1, scale, lo, out);
-          else if (bits == 4u) decode_chunk32_bf16_pairs<4>(cw, lane, g0, g1, scale, lo, out);
-          else decode_chunk32_bf16_pairs<8>(cw, lane, g0, g1, scale, lo, out);
+          const uint32_t shift = ((uint32_t)(gp * pl.plane_bytes) & 15u) / 4u, v0 = ch * (1024u / VE);
+          if (bits == 2u) decode_chunk_large_shifted<2>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
+          else if (bits == 4u) decode_chunk_large_shifted<4>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
+          else decode_chunk_large_shifted<8>(slot, npay >> 2, lane, v0, pl.HW, shift, scale, lo, out);
         } else {
-          if (bits == 2u) decode_chunk32<DT, 2>(cw, lane, g0, g1, scale, lo, out);
-          else if (bits == 4u) decode_chunk32<DT, 4>(cw, lane, g0, g1, scale, lo, out);
-          else decode_chunk32<DT, 8>(cw, lane, g0, g1, scale, lo, out);
+          if (bits == 2u) decode_chunk_large<2>(cw, lane, g0, g1, scale, lo, out);
+          else if (bits == 4u) decode_chunk_large<4>(cw, lane, g0, g1, scale, lo, out);
+          else decode_chunk_large<8>(cw, lane, g0, g1, scale, lo, out);
         }
       } else if (cls == kClsRaw) {
         // the continuation, when there is one, lies in the overflow region
@@ -733,63 +1008,13 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
         in.slot = slot;
         in.ovf = src + off;
         in.npay = npay;
-        const uint32_t i1 = min(pl.HW * (DT == kF32 ? 2u : 1u), (ch + 1u) * (DT == kF32 ? 2048u : 1024u));
-        for (uint32_t i = ch * (DT == kF32 ? 2048u : 1024u) + lane; i < i1; i += 32u)
-          reinterpret_cast<uint16_t*>(out)[i] = (uint16_t)in.ld16(2u * i);
+        const uint32_t i1 = min(pl.HW, (ch + 1u) * 1024u);
+        for (uint32_t i = ch * 1024u + lane; i < i1; i += 32u) reinterpret_cast<uint32_t*>(out)[i] = in.ld32(4u * i);
       } else if (cls != kClsSalient || s_nsal == 0u) {
         bad = true;
       }
     }
-    // the outlier-rich planes, from up to 256 table entries at a time
-    if (s_nsal) {
-      const uint32_t hop = (uint32_t)a.cta_stride, most = blockIdx.x < hop ? ((uint32_t)pl.P + hop - 1u) / hop : 0u;
-      const Team unit = pl.team == 32u ? make_warp_team(s_red) : make_team(kThreads, s_red);
-      uint32_t* scr = reinterpret_cast<uint32_t*>(smem + (pl.team == 32u ? (uint64_t)warp * pl.sal_stride : 0ull));
-      HufDecode* hd = reinterpret_cast<HufDecode*>(reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes) - 1;
-      for (uint32_t base = 0; base < most; base += kThreads) {
-        const uint64_t gp = blockIdx.x + (uint64_t)(base + tid) * hop;
-        if (gp < pl.P && (__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp) + 1) & 3u) == kClsSalient)
-          s_list[atomicAdd(&s_nlist, 1u)] = (uint32_t)gp;
-        __syncthreads();
-        const uint32_t n = s_nlist;
-        for (uint32_t q = pl.team == 32u ? warp : 0u; q < n; q += pl.team == 32u ? (uint32_t)kWarps : 1u) {
-          const uint32_t gp = s_list[q];
-          const unsigned long long off = (unsigned long long)__ldg(reinterpret_cast<const uint32_t*>(src + 64 + 16ull * gp)) * 16ull;
-          if (off != 0 && (off < ovf_off || off > total)) {  // (the same for every thread of the unit)
-            bad = true;
-            continue;
-          }
-          SplitIn in;
-          in.slot = src + slots_off + (uint64_t)gp * npay;
-          in.ovf = src + off;
-          in.npay = npay;
-          // the payload comes to shared memory first when it fits there
-          const unsigned long long ovf_avail = off ? total - off : 0ull;
-          const uint32_t got = (uint32_t)min((unsigned long long)pl.pay_bytes, npay + (ovf_avail & ~15ull));
-          const uint32_t nnz_s = in.ld32(0), n_dense = in.ld32(4), n_out_d = in.ld32(8), coded = in.ld32(12), es = (uint32_t)pl.esize;
-          const uint64_t size = 16ull + 4ull * pl.nbm + 4ull * ((uint64_t)pl.H + 1) + a4(2u * nnz_s) + a4(es * nnz_s) +
-                                (coded ? (uint64_t)coded : 64ull * n_dense) + a4(es * n_out_d);
-          uint8_t* pay = reinterpret_cast<uint8_t*>(scr) + pl.sal_stride - pl.pay_bytes;
-          bool good;
-          if (nnz_s <= pl.HW && n_dense <= pl.nblk && n_out_d <= pl.HW && size <= got) {
-            for (uint32_t o = 16u * unit.lane; o < (uint32_t)size; o += 16u * unit.size)
-              *reinterpret_cast<uint4*>(pay + o) = __ldg(reinterpret_cast<const uint4*>(in.at(o)));
-            team_sync(unit);
-            FlatIn flat;
-            flat.p = pay;
-            flat.npay = got;
-            good = decode_salient<DT>(unit, s_pl, flat, 0ull, s_eps, a.dst + gp * pl.plane_bytes, scr, hd, s_hdr_ok);
-          } else {
-            good = decode_salient<DT>(unit, s_pl, in, ovf_avail, s_eps, a.dst + gp * pl.plane_bytes, scr, hd, s_hdr_ok);
-          }
-          if (!good) bad = true;
-          team_sync(unit);  // the scratch is reused
-        }
-        __syncthreads();
-        if (tid == 0) s_nlist = 0;
-        __syncthreads();
-      }
-    }
+    FH_RESTORE_OUTLIER_RICH(DT)
   }
   decompress_exit(a, bad);
 }

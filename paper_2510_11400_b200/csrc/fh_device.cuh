@@ -88,6 +88,11 @@ __device__ __forceinline__ unsigned long long status_word(uint32_t code) {
   return (unsigned long long)st;
 }
 
+// Lines of 32 output vectors (of `ve` elements) that a plane spans; off the 16-byte grid it may begin anywhere in its first.
+__host__ __device__ __forceinline__ uint32_t chunk_lines(uint32_t HW, uint32_t ve, bool aligned) {
+  return ((HW + (aligned ? 0u : ve - 1u) + ve - 1u) / ve + 31u) / 32u;
+}
+
 __device__ __forceinline__ uint32_t a4(uint32_t x) { return (x + 3u) & ~3u; }
 __device__ __forceinline__ uint32_t a16(uint32_t x) { return (x + 15u) & ~15u; }
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
