@@ -151,7 +151,7 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
   // one more sum and the encoder's tables
   auto sal_bytes_of = [&](uint32_t warps) {
     const size_t words = (size_t)pl.H * pl.seg + 1 + 2 * ((size_t)pl.nsr + 1) + pl.nbm +
-                         (pl.entropy ? (size_t)pl.nsr + 1 + 3 + sizeof(fh::HufEncode) / 4 + (warps - 1) * 4 * fh::kHufStageWords : 0);
+                         (pl.entropy ? (size_t)pl.nsr + 1 + fh::kHufEncodeWords + (warps - 1) * 4 * fh::kHufStageWords : 0);
     return (uint32_t)A16(4 * words + 16);
   };
   const bool blockwise = compress && pl.mode != FH_SALIENT_OFF;

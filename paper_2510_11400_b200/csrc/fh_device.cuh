@@ -589,14 +589,21 @@ struct HufEncode {
   uint32_t hist[256];                // once it has been read: the nodes' parents (merged nodes), 256 sorted leaves and 256 merged nodes
   uint32_t code[256];                // by symbol: length << 24 | code value; 0: does not occur
   uint32_t used[256 + 4];            // symbols that occur, ascending, weight << 8 | symbol; four sentinels behind them
-  // weights of the sorted leaves and a sentinel, then of the merged nodes in order of creation (kHufNone: not there yet)
-  uint32_t weight[2 * 260];
   uint8_t sorted[256];               // index into `used` of the sorted leaves
   uint32_t cnt[32], first[32];       // symbols of a length, then running rank; a length's first code value
   uint32_t smin, smax, maxlen, nlens;
-  uint32_t stage[1][4 * kHufStageWords];  // chunks' bits while a warp assembles four of them; one per warp of the team
+  union {
+    // weights of the sorted leaves and a sentinel, then of the merged nodes in order of creation (kHufNone: not there yet);
+    // done with once the code is built
+    uint32_t weight[2 * 260];
+    uint32_t stage[1][4 * kHufStageWords];  // chunks' bits while a warp assembles four of them; one per warp of the team
+  };
 };
 constexpr uint32_t kHufNone = 0xFFFFFFu, kHufMerged = 260;
+// Words set aside for it and for its alignment: a fixed figure, since which planes are too large for the Huffman stage follows
+// from it and must not move with the tables.
+constexpr uint32_t kHufEncodeWords = 1542;
+static_assert(sizeof(HufEncode) / 4 + 3 <= kHufEncodeWords, "the encoder's tables do not fit");
 
 // First code value of length `lane`, from the number `n` of symbols of that length (0 for length 0), for codes that do not
 // oversubscribe: the sum over the shorter lengths k of n_k 2^(length - k), by a prefix sum in units of 2^-31.
