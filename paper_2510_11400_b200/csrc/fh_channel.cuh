@@ -12,7 +12,7 @@
 // the L2 cache comes from there from the second time on.  A lane has 64 bytes in flight; the
 // passes follow one another by programmatic launch; no memset between them (the streaming kernel's last CTA returns the
 // statistics to zero).  Element by element with a warp per plane the three took 162 us for 32 x 96 bf16 planes of
-// 112 x 112 (77 MB) and 27 us for 32 x 960 of 7 x 7; now 67 and 17.
+// 112 x 112 (77 MB) and 27 us for 32 x 960 of 7 x 7; now 61 and 17.
 #pragma once
 
 #include "fh_device.cuh"
@@ -61,11 +61,46 @@ __device__ __forceinline__ void load_group_raw(const uint8_t* plane, uint32_t g,
 
 constexpr uint32_t kChanPiece = 512;  // groups of a piece: their integer sums fit 32 bits
 
+// Tensor-wide statistics have a single destination: the CTA's threads are combined in shared memory, and one of them issues the
+// atomics.
+template <int PASS>
+__device__ __forceinline__ void channel_pass_whole(const ChannelArgs& a, float wlo, float whi, unsigned long long ws, unsigned long long wq,
+                                                   float* s_lo, float* s_hi, unsigned long long* s_s, unsigned long long* s_q) {
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu;
+  for (uint32_t o = 16; o > 0; o >>= 1) {
+    wlo = fminf(wlo, __shfl_xor_sync(full, wlo, o));
+    whi = fmaxf(whi, __shfl_xor_sync(full, whi, o));
+  }
+  ws = warp_sum_u64(ws);
+  wq = warp_sum_u64(wq);
+  const uint32_t warp = threadIdx.x >> 5;
+  if (lane == 0) {
+    s_lo[warp] = wlo;
+    s_hi[warp] = whi;
+    s_s[warp] = ws;
+    s_q[warp] = wq;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (uint32_t k = 1; k < (uint32_t)kWarps; ++k) {
+      wlo = fminf(wlo, s_lo[k]);
+      whi = fmaxf(whi, s_hi[k]);
+      ws += s_s[k];
+      wq += s_q[k];
+    }
+    if (PASS == 0) {  // (every CTA of the grid owns at least one plane, so both values are numbers of the input)
+      atomicMax(&a.chan->lo_inv, ~float_key(wlo));
+      atomicMax(&a.chan->hi_key, float_key(whi));
+    } else {
+      atomicAdd(&a.chan->Is, ws);
+      atomicAdd(&a.chan->Iq, wq);
+    }
+  }
+}
+
 template <int DT, int PASS, bool VEC>
 __global__ void __launch_bounds__(kThreads, 4) channel_pass(const Plan pl, const ChannelArgs a) {
   const uint32_t tt = a.team, lane = threadIdx.x & 31u, tl = lane & (tt - 1u), full = 0xFFFFFFFFu;
-  // Tensor-wide statistics have a single destination: a team gathers over its planes, the CTA's teams are
-  // combined in shared memory, and one thread per CTA issues the atomics.
   const bool whole = pl.mode == kModeTensor;
   __shared__ float s_lo[kWarps], s_hi[kWarps];
   __shared__ unsigned long long s_s[kWarps], s_q[kWarps];
@@ -164,37 +199,163 @@ __global__ void __launch_bounds__(kThreads, 4) channel_pass(const Plan pl, const
       }
     }
   }
-  if (whole && PASS < 2) {
-    for (uint32_t o = 16; o > 0; o >>= 1) {
-      wlo = fminf(wlo, __shfl_xor_sync(full, wlo, o));
-      whi = fmaxf(whi, __shfl_xor_sync(full, whi, o));
-    }
-    ws = warp_sum_u64(ws);
-    wq = warp_sum_u64(wq);
-    const uint32_t warp = threadIdx.x >> 5;
-    if (lane == 0) {
-      s_lo[warp] = wlo;
-      s_hi[warp] = whi;
-      s_s[warp] = ws;
-      s_q[warp] = wq;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (uint32_t k = 1; k < (uint32_t)kWarps; ++k) {
-        wlo = fminf(wlo, s_lo[k]);
-        whi = fmaxf(whi, s_hi[k]);
-        ws += s_s[k];
-        wq += s_q[k];
-      }
-      if (PASS == 0) {  // (every CTA of the grid owns at least one plane, so both values are numbers of the input)
-        atomicMax(&a.chan->lo_inv, ~float_key(wlo));
-        atomicMax(&a.chan->hi_key, float_key(whi));
-      } else {
-        atomicAdd(&a.chan->Is, ws);
-        atomicAdd(&a.chan->Iq, wq);
-      }
-    }
+  if (whole && PASS < 2) channel_pass_whole<PASS>(a, wlo, whi, ws, wq, s_lo, s_hi, s_s, s_q);
+}
+
+// The same for planes of more than 64 groups (a team is a whole warp then) that are whole groups: a warp takes a run of pieces in
+// channel order, so that it works out a channel's scale and thresholds (a chain of loads, 64-bit arithmetic and a square
+// root) once or twice and not once a piece, and sends its sums off at the channel's end.  The next loads are asked for before the
+// present ones' elements are worked on.  What bounds it is the L2 cache's latency and rate.  A whole call, a piece at a time and
+// now, us: bf16, 32 x 96 of 112 x 112 136.6 -> 131.4, 32 x 144 of 56 x 56 78.7 -> 76.7, 32 x 192 of 28 x 28 46.9 -> 43.9; fp32, 32 x 96
+// of 112 x 112 172.5 -> 161.3.  (Planes that are not whole groups, loaded element by element, have no registers to load ahead:
+// 47 x 33 66.9 -> 70.7; they stay with the kernel above.)
+template <int DT, int PASS>
+__global__ void __launch_bounds__(kThreads, 4) channel_pass_runs(const Plan pl, const ChannelArgs a) {
+  constexpr uint32_t U = DT == kF32 ? 4u : 8u;  // groups a lane loads at a time: 64 bytes
+  const uint32_t lane = threadIdx.x & 31u, full = 0xFFFFFFFFu, warp = threadIdx.x >> 5;
+  const bool whole = pl.mode == kModeTensor;
+  __shared__ float s_lo[kWarps], s_hi[kWarps];
+  __shared__ unsigned long long s_s[kWarps], s_q[kWarps];
+  const uint32_t pieces = (pl.groups + kChanPiece - 1u) / kChanPiece, part = ((pl.groups + pieces - 1u) / pieces + 31u) & ~31u;
+  const uint32_t planes = whole ? (uint32_t)pl.P : pl.N;  // of a channel
+  const uint64_t nw = (uint64_t)gridDim.x * kWarps, w0 = (uint64_t)blockIdx.x * kWarps + warp, items = pl.P * pieces;
+  uint32_t left = (uint32_t)(items * (w0 + 1u) / nw - items * w0 / nw);  // pieces of the run
+  uint32_t c, n, piece;
+  {
+    const uint32_t i = (uint32_t)(items * w0 / nw), q = i / pieces;
+    piece = i - q * pieces;
+    c = q / planes;
+    n = q - c * planes;
   }
+  float lo = __int_as_float(0x7F800000), hi = __int_as_float(0xFF800000);
+  unsigned long long ws = 0, wq = 0;
+  uint32_t nout = 0;
+  uint32_t g = piece * part + lane, end = min(pl.groups, (piece + 1u) * part);
+  uint64_t p = (uint64_t)n * (whole ? 1u : pl.C) + c;
+  uint32_t buf[U][DT == kF32 ? 4 : 2], nxt[U][DT == kF32 ? 4 : 2];
+  auto load = [&](uint32_t (&to)[U][DT == kF32 ? 4 : 2]) {
+    const uint8_t* plane = a.src + p * pl.plane_bytes;
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      uint32_t t[4];
+      load_group_raw<DT, true>(plane, min(g + u * 32u, end - 1u), pl.HW, t);
+#pragma unroll
+      for (int k = 0; k < (DT == kF32 ? 4 : 2); ++k) to[u][k] = t[k];
+    }
+  };
+  dep_trigger();
+  dep_wait();
+  if (left) load(buf);
+  float clo = 0.0f, dlo = 0.0f, dhi = 0.0f;
+  SigmaScale sc = {};
+  bool fresh = true;
+  uint32_t as = 0, aq = 0, cnt = 0;
+  while (left) {
+    ChanStat* cs = a.chan + (whole ? 0u : c);
+    const uint32_t g_now = g, end_now = end;
+    const uint64_t p_now = p;
+    const bool last = g - lane + U * 32u >= end;  // (of the piece)
+    bool flush = false;
+    if (PASS == 0 && g == 0u) a.plane_nout[p] = 0;  // (lane 0, ahead of the plane's first group)
+    g += U * 32u;
+    if (last) {
+      --left;
+      if (++piece == pieces) {
+        piece = 0;
+        if (++n == planes) {
+          n = 0;
+          ++c;
+          flush = true;
+        }
+        p = (uint64_t)n * (whole ? 1u : pl.C) + c;
+      }
+      g = piece * part + lane;
+      end = min(pl.groups, (piece + 1u) * part);
+      flush |= left == 0u;
+    }
+    if (left) load(nxt);
+    if (PASS > 0 && fresh) {
+      clo = key_float(~cs->lo_inv);
+      sc = sigma_scale(__fsub_rn(key_float(cs->hi_key), clo));  // (not `applies`: a constant channel, or a range outside the rule's domain)
+      if (PASS == 2) sigma_thresholds((long long)cs->Is, (long long)cs->Iq, sc, a.inv_nhw, dlo, dhi);
+      fresh = false;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      float v[4];
+      if (DT == kF32) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __uint_as_float(buf[u][k]);
+      } else {
+        v[0] = __uint_as_float(buf[u][0] << 16); v[1] = __uint_as_float(buf[u][0] & 0xFFFF0000u);
+        v[2] = __uint_as_float(buf[u][1] << 16); v[3] = __uint_as_float(buf[u][1] & 0xFFFF0000u);
+      }
+      if (PASS == 0) {  // (an element read twice changes nothing; non-finite input is reported by the streaming kernel)
+        lo = fminf(lo, fminf(fminf(v[0], v[1]), fminf(v[2], v[3])));
+        hi = fmaxf(hi, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+      } else {
+        const bool in = g_now + u * 32u < end_now;
+        float d[4];
+#pragma unroll
+        for (uint32_t k = 0; k < 4u; ++k) d[k] = __fsub_rn(v[k], clo);
+        if (PASS == 1) {
+          if (in) {
+            sigma_addends(d, sc, as, aq);
+            ++cnt;
+          }
+        } else {
+#pragma unroll
+          for (uint32_t k = 0; k < 4u; ++k) cnt += in && (d[k] > dhi || d[k] < dlo);
+        }
+      }
+    }
+    if (last) {
+      if (PASS == 1) {  // (a lane's sums of a piece fit 32 bits)
+        if (sc.applies) {
+          ws += as - cnt * kMagicBits;
+          wq += aq - cnt * kMagicBits;
+        }
+        as = aq = cnt = 0;
+      } else if (PASS == 2) {
+        asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(cnt) : "r"(full));
+        if (!sc.applies) cnt = 0;
+        if (lane == 0 && cnt) {
+          if (pieces == 1u) a.plane_nout[p_now] = cnt;
+          else atomicAdd(&a.plane_nout[p_now], cnt);
+        }
+        nout += cnt;
+        cnt = 0;
+      }
+    }
+    if (flush && !whole) {
+      if (PASS == 0) {
+        const uint32_t kl = __reduce_max_sync(full, ~float_key(lo)), kh = __reduce_max_sync(full, float_key(hi));
+        if (lane == 0) {
+          atomicMax(&cs->lo_inv, kl);
+          atomicMax(&cs->hi_key, kh);
+        }
+        lo = __int_as_float(0x7F800000);
+        hi = __int_as_float(0xFF800000);
+      } else if (PASS == 1) {
+        ws = warp_sum_u64(ws);
+        wq = warp_sum_u64(wq);
+        if (lane == 0 && sc.applies) {
+          atomicAdd(&cs->Is, ws);
+          atomicAdd(&cs->Iq, wq);
+        }
+        ws = wq = 0;
+      } else {
+        if (lane == 0 && nout) atomicAdd(&cs->nout, (unsigned long long)nout);
+        nout = 0;
+      }
+      fresh = true;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u)
+#pragma unroll
+      for (int k = 0; k < (DT == kF32 ? 4 : 2); ++k) buf[u][k] = nxt[u][k];
+  }
+  if (whole && PASS < 2) channel_pass_whole<PASS>(a, lo, hi, ws, wq, s_lo, s_hi, s_s, s_q);
 }
 
 }  // namespace fh

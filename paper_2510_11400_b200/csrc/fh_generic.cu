@@ -25,9 +25,10 @@ template <int DT, int PASS, bool VEC>
 int launch_channel_pass(const Plan& pl, const ChannelArgs& ca, cudaStream_t stream) {
   int grid = 0;
   const uint64_t items = pl.P * ((pl.groups + kChanPiece - 1) / kChanPiece), per = kThreads / ca.team, want = (items + per - 1) / per;
-  const int rc = grid_for(channel_pass<DT, PASS, VEC>, 0, (uint32_t)(want < 0x7FFFFFFFull ? want : 0x7FFFFFFFull), &grid);
+  const auto kernel = VEC && ca.team == 32u ? channel_pass_runs<DT, PASS> : channel_pass<DT, PASS, VEC>;
+  const int rc = grid_for(kernel, 0, (uint32_t)(want < 0x7FFFFFFFull ? want : 0x7FFFFFFFull), &grid);
   if (rc != FH_OK) return rc;
-  return launch_dependent(channel_pass<DT, PASS, VEC>, grid, kThreads, 0, stream, pl, ca) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+  return launch_dependent(kernel, grid, kThreads, 0, stream, pl, ca) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
 
 template <int DT, bool VEC>
