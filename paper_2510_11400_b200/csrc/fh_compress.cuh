@@ -14,7 +14,7 @@
 // Variants by plane size:
 //   compress_warp<DT, SIGMA, TT, K, EDGE>   planes of at most 256 groups: bulk-copy (TMA) pipeline, a sub-warp
 //       team per plane, groups kept in registers; a warp handles an outlier-rich plane;
-//   compress_cta_regs<DT, SIGMA, K, EDGE, PARTS>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
+//   compress_cta_regs<DT, SIGMA, K, EDGE, PARTS, WORDS>   planes of up to 8,960 groups: one plane per CTA and tile, in registers;
 //   compress_cta<SIGMA>                    still larger bf16 planes of whole 16-byte chunks: swept in shared memory;
 //   compress_generic<DT, BITS, ROUND>      everything else (still larger ragged or fp32 planes, random rounding outside
 //       the plane-wise three-sigma mode).
@@ -713,6 +713,46 @@ __device__ __forceinline__ uint32_t max2_nan_bf16(uint32_t a, uint32_t b) {
 
 // Runs of exactly K * TT groups (EDGE 0) start on 16-byte boundaries; in bf16 a lane then takes groups in neighbouring
 // pairs, so that loads are 16 bytes wide and codes leave twice as wide (1 GiB of 32 x 32 planes: 373 -> 342 us).
+// Loads a bf16 run of `n` elements as it lies there, two words a group, and takes the lane's minimum and maximum.
+template <int K, int TT, int EDGE, int GRAIN>
+__device__ __forceinline__ void run_load_words(const uint8_t* p, uint32_t lane, int32_t n, uint32_t (&x)[K][2], float& lo, float& hi) {
+  static_assert(EDGE > 0 || K % 2 == 0, "pairs");
+  const uint32_t last = (uint32_t)(n - 1) >> 2;
+  uint32_t l0 = 0, h0 = 0, l1 = 0, h1 = 0, safe = 0;
+  uint4 pair = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t v = lane + (uint32_t)(k * TT);
+    uint32_t w[4];
+    if (EDGE == 0) {
+      if (k & 1) {
+        w[0] = pair.z; w[1] = pair.w;
+      } else {
+        pair = (reinterpret_cast<const uint4*>(p) + lane)[(k >> 1) * TT];
+        w[0] = pair.x; w[1] = pair.y;
+      }
+    } else {
+      group_load<kBF16>(p, k >= K - EDGE ? min(v, last) : v, GRAIN, w);
+    }
+    if (k == 0) safe = __byte_perm(w[0], 0u, 0x1010);
+    if (k >= K - EDGE) {
+      const int32_t in = n - 4 * (int32_t)v;
+      w[0] = in >= 2 ? w[0] : (in == 1 ? __byte_perm(w[0], safe, 0x5410) : safe);
+      w[1] = in >= 4 ? w[1] : (in == 3 ? __byte_perm(w[1], safe, 0x5410) : safe);
+    }
+    if (k == 0) l0 = h0 = w[0], l1 = h1 = w[1];
+    else {
+      l0 = min2_nan_bf16(l0, w[0]); l1 = min2_nan_bf16(l1, w[1]);
+      h0 = max2_nan_bf16(h0, w[0]); h1 = max2_nan_bf16(h1, w[1]);
+    }
+    x[k][0] = w[0];
+    x[k][1] = w[1];
+  }
+  l0 = min2_nan_bf16(l0, l1);
+  h0 = max2_nan_bf16(h0, h1);
+  lo = min_nan(__uint_as_float(l0 << 16), __uint_as_float(l0 & 0xFFFF0000u));
+  hi = max_nan(__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xFFFF0000u));
+}
 // Loads the run of `n` elements and takes the lane's minimum and maximum.
 template <int DT, int K, int TT, int EDGE, int GRAIN>
 __device__ __forceinline__ void run_load_as(const uint8_t* p, uint32_t lane, int32_t n, float (&x)[K][4], float& lo, float& hi) {
@@ -745,41 +785,13 @@ __device__ __forceinline__ void run_load_as(const uint8_t* p, uint32_t lane, int
     lo = min_nan(lo, lo1);
     hi = max_nan(hi, hi1);
   } else {
-    static_assert(EDGE > 0 || K % 2 == 0, "pairs");
-    uint32_t l0 = 0, h0 = 0, l1 = 0, h1 = 0, safe = 0;
-    uint4 pair = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t w[K][2];
+    run_load_words<K, TT, EDGE, GRAIN>(p, lane, n, w, lo, hi);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      const uint32_t v = lane + (uint32_t)(k * TT);
-      uint32_t w[4];
-      if (EDGE == 0) {
-        if (k & 1) {
-          w[0] = pair.z; w[1] = pair.w;
-        } else {
-          pair = (reinterpret_cast<const uint4*>(p) + lane)[(k >> 1) * TT];
-          w[0] = pair.x; w[1] = pair.y;
-        }
-      } else {
-        group_load<DT>(p, k >= K - EDGE ? min(v, last) : v, GRAIN, w);
-      }
-      if (k == 0) safe = __byte_perm(w[0], 0u, 0x1010);
-      if (k >= K - EDGE) {
-        const int32_t in = n - 4 * (int32_t)v;
-        w[0] = in >= 2 ? w[0] : (in == 1 ? __byte_perm(w[0], safe, 0x5410) : safe);
-        w[1] = in >= 4 ? w[1] : (in == 3 ? __byte_perm(w[1], safe, 0x5410) : safe);
-      }
-      if (k == 0) l0 = h0 = w[0], l1 = h1 = w[1];
-      else {
-        l0 = min2_nan_bf16(l0, w[0]); l1 = min2_nan_bf16(l1, w[1]);
-        h0 = max2_nan_bf16(h0, w[0]); h1 = max2_nan_bf16(h1, w[1]);
-      }
-      x[k][0] = __uint_as_float(w[0] << 16); x[k][1] = __uint_as_float(w[0] & 0xFFFF0000u);
-      x[k][2] = __uint_as_float(w[1] << 16); x[k][3] = __uint_as_float(w[1] & 0xFFFF0000u);
+      x[k][0] = __uint_as_float(w[k][0] << 16); x[k][1] = __uint_as_float(w[k][0] & 0xFFFF0000u);
+      x[k][2] = __uint_as_float(w[k][1] << 16); x[k][3] = __uint_as_float(w[k][1] & 0xFFFF0000u);
     }
-    l0 = min2_nan_bf16(l0, l1);
-    h0 = max2_nan_bf16(h0, h1);
-    lo = min_nan(__uint_as_float(l0 << 16), __uint_as_float(l0 & 0xFFFF0000u));
-    hi = max_nan(__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xFFFF0000u));
   }
 }
 template <int DT, int K, int TT, int EDGE>
@@ -787,6 +799,11 @@ __device__ __forceinline__ void run_load(const uint8_t* p, uint32_t lane, int32_
   if (EDGE == 0 || grain == 2u) run_load_as<DT, K, TT, EDGE, 2>(p, lane, n, x, lo, hi);
   else if (DT == kF32 && grain == 1u) run_load_as<DT, K, TT, EDGE, 1>(p, lane, n, x, lo, hi);
   else run_load_as<DT, K, TT, EDGE, 0>(p, lane, n, x, lo, hi);
+}
+template <int DT, int K, int TT, int EDGE>
+__device__ __forceinline__ void run_load(const uint8_t* p, uint32_t lane, int32_t n, uint32_t grain, uint32_t (&x)[K][2], float& lo, float& hi) {
+  if (EDGE == 0 || grain >= 1u) run_load_words<K, TT, EDGE, 2>(p, lane, n, x, lo, hi);
+  else run_load_words<K, TT, EDGE, 0>(p, lane, n, x, lo, hi);
 }
 // The grain of planes that follow one another from a 16-byte boundary on (for bf16 an 8-byte boundary is as good).
 __device__ __forceinline__ uint32_t plane_grain(const Plan& pl) {
@@ -914,6 +931,152 @@ __device__ __forceinline__ void run_codes_any(const Plan& pl, const uint8_t* p, 
   } else if (pl.bits == 2) run_codes<DT, K, TT, EDGE, 2>(lane, n, inv, at, x);
   else if (pl.bits == 4) run_codes<DT, K, TT, EDGE, 4>(lane, n, inv, at, x);
   else run_codes<DT, K, TT, EDGE, 8>(lane, n, inv, at, x);
+}
+
+// ---- The same for bf16 runs that stay in registers as they lie in memory, two words a group: half the registers, so that more
+// warps are resident, for six more instructions a group where distances are needed once more.
+// Distances of a group's elements from the minimum.
+__device__ __forceinline__ void word_distances(uint32_t w0, uint32_t w1, f32x2 nlo2, f32x2& p, f32x2& q) {
+  p = add2(pack2(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xFFFF0000u)), nlo2);
+  q = add2(pack2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xFFFF0000u)), nlo2);
+}
+// Masked positions are set to the minimum, which is distance 0; then the moments.
+template <int DT, int K, int TT, int EDGE, bool SIGMA>
+__device__ __forceinline__ void run_distances(uint32_t lane, int32_t n, float lo, const SigmaScale& sc, uint32_t (&x)[K][2], uint32_t& as,
+                                              uint32_t& aq) {
+  const uint32_t lo2 = __byte_perm(__float_as_uint(lo), 0u, 0x3232);  // (the minimum is one of the elements)
+  const f32x2 nlo2 = pack2(-lo, -lo);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (k >= K - EDGE) {
+      const int32_t in = n - 4 * (int32_t)(lane + (uint32_t)(k * TT));
+      x[k][0] = in >= 2 ? x[k][0] : (in == 1 ? __byte_perm(x[k][0], lo2, 0x5410) : lo2);
+      x[k][1] = in >= 4 ? x[k][1] : (in == 3 ? __byte_perm(x[k][1], lo2, 0x5410) : lo2);
+    }
+    if (SIGMA) {
+      f32x2 p, q;
+      word_distances(x[k][0], x[k][1], nlo2, p, q);
+      sigma_addends2(p, q, sc, as, aq);
+      // (or the compiler keeps the distances for what follows, in local memory)
+      asm volatile("" : "+r"(x[k][0]), "+r"(x[k][1]));
+    }
+  }
+}
+// The element that comes right above or below in the order of bf16 values.
+__device__ __forceinline__ uint32_t bf16_above(uint32_t c) { return c & 0x8000u ? (c == 0x8000u ? 1u : c - 1u) : c + 1u; }
+__device__ __forceinline__ uint32_t bf16_below(uint32_t c) { return c & 0x8000u ? c + 1u : (c == 0u ? 0x8001u : c - 1u); }
+// A threshold on distances as one on elements: the largest element whose distance from `lo` does not exceed `t` (EQUAL: is less
+// than `t`), twice in a word.  Distances, rounded as they are, grow with the element, so the neighbours of lo + t are looked at; false when
+// none of three is it (the sum cancels), which leaves the comparison of distances.
+template <bool EQUAL>
+__device__ __forceinline__ bool element_cut(float lo, float t, uint32_t& cut) {
+  const uint32_t b = __float_as_uint(__fadd_rn(lo, t));
+  uint32_t c = (b >> 16) + ((b >> 31) && (b & 0xFFFFu) ? 1u : 0u);
+  auto beyond = [&](uint32_t e) {
+    const float d = __fsub_rn(__uint_as_float(e << 16), lo);
+    return EQUAL ? !(d < t) : d > t;
+  };
+  if (beyond(c)) c = bf16_below(c);
+  else if (!beyond(bf16_above(c))) c = bf16_above(c);
+  cut = c | c << 16;
+  return !beyond(c) && beyond(bf16_above(c));
+}
+struct Cuts {  // outliers are the elements above `above` and, when `low`, those up to `below`; !exact: compare distances
+  uint32_t above, below, low, exact;
+};
+__device__ __forceinline__ Cuts element_cuts(float lo, float dlo, float dhi) {
+  Cuts c;
+  c.low = 0.0f < dlo;
+  c.below = 0;
+  bool exact = element_cut<false>(lo, dhi, c.above);
+  if (c.low) exact &= element_cut<true>(lo, dlo, c.below);
+  c.exact = exact;
+  return c;
+}
+template <int DT, int K, int TT, int EDGE>
+__device__ __forceinline__ uint32_t run_count(uint32_t lane, int32_t n, float lo, float dlo, float dhi, const Cuts& c, const uint32_t (&x)[K][2]) {
+  uint32_t all = 0;
+  if (c.exact) {  // one comparison and one addition for two elements; counts of at most 4 K are exact in bf16
+    static_assert(2 * K <= 256, "counts in bf16");
+    auto pair = [](uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); };
+    const __nv_bfloat162 above = pair(c.above), below = pair(c.below);
+    __nv_bfloat162 c0 = pair(0u), c1 = pair(0u);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      c0 = __hadd2(c0, __hgt2(pair(x[k][0]), above));
+      c1 = __hadd2(c1, __hgt2(pair(x[k][1]), above));
+    }
+    if (c.low) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        c0 = __hadd2(c0, __hle2(pair(x[k][0]), below));
+        c1 = __hadd2(c1, __hle2(pair(x[k][1]), below));
+      }
+    }
+    c0 = __hadd2(c0, c1);
+    all = (uint32_t)(__low2float(c0) + __high2float(c0));
+  } else {
+    const f32x2 nlo2 = pack2(-lo, -lo);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      f32x2 p, q;
+      uint32_t w0 = x[k][0], w1 = x[k][1];
+      asm volatile("" : "+r"(w0), "+r"(w1));
+      word_distances(w0, w1, nlo2, p, q);
+      float d[4];
+      unpack2(p, d[0], d[1]);
+      unpack2(q, d[2], d[3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) all += (d[e] > dhi) || (d[e] < dlo);
+    }
+  }
+#pragma unroll
+  for (int k = K - EDGE; k < K && EDGE > 0; ++k)  // masked positions (distance 0) are no elements
+    if (0.0f < dlo) all -= (uint32_t)(4 - min(max(n - 4 * (int32_t)(lane + (uint32_t)(k * TT)), 0), 4));
+  return all;
+}
+template <int DT, int K, int TT, int EDGE, int BITS>
+__device__ __forceinline__ void run_codes(uint32_t lane, int32_t n, float lo, float inv, uint8_t* slot, const uint32_t (&x)[K][2]) {
+  constexpr uint32_t bias = kMagicBits * (1u + (1u << BITS) + (1u << (2 * BITS)) + (1u << (3 * BITS)));
+  constexpr bool PAIR = EDGE == 0;
+  const f32x2 inv2 = pack2(inv, inv), mag2 = pack2(kMagicF, kMagicF), nlo2 = pack2(-lo, -lo);
+  uint8_t* out = slot + lane * (PAIR ? BITS : BITS / 2);
+  uint32_t before = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    f32x2 p, q;
+    uint32_t a = x[k][0], b = x[k][1], w0, w1, w2, w3;
+    // (or the compiler works out all groups' distances ahead of the branch on the width, and has no registers for them)
+    asm volatile("// %2" : "+r"(a), "+r"(b) : "n"(BITS));
+    word_distances(a, b, nlo2, p, q);
+    unpack2u(fma2(p, inv2, mag2), w0, w1);
+    unpack2u(fma2(q, inv2, mag2), w2, w3);
+    const uint32_t word = w0 + (w1 << BITS) + (w2 << (2 * BITS)) + (w3 << (3 * BITS)) - bias;
+    if (PAIR) {
+      const int o = (k >> 1) * TT * BITS;
+      if (!(k & 1)) before = word;
+      else if (BITS == 2) *reinterpret_cast<uint16_t*>(out + o) = (uint16_t)(before | (word << 8));
+      else if (BITS == 4) *reinterpret_cast<uint32_t*>(out + o) = before | (word << 16);
+      else *reinterpret_cast<uint2*>(out + o) = make_uint2(before, word);
+    } else if (k < K - EDGE || n > 4 * (int32_t)(lane + (uint32_t)(k * TT))) {
+      if (BITS == 2) out[k * TT] = (uint8_t)word;
+      else if (BITS == 4) *reinterpret_cast<uint16_t*>(out + 2 * k * TT) = (uint16_t)word;
+      else *reinterpret_cast<uint32_t*>(out + 4 * k * TT) = word;
+    }
+  }
+}
+template <int DT, int SIGMA, int K, int TT, int EDGE>
+__device__ __forceinline__ void run_codes_any(const Plan& pl, const uint8_t* p, uint32_t grain, uint32_t lane, int32_t n, float lo,
+                                              float inv, uint32_t g0, uint64_t gp, uint8_t* slot, const uint32_t (&x)[K][2]) {
+  uint8_t* at = slot + g0 * (uint32_t)pl.bits / 2u;
+  constexpr int GRAIN = EDGE == 0 ? 2 : -1;
+  if (SIGMA == 2) {
+    if (pl.bits == 2) run_codes_random<DT, 2, GRAIN>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+    else if (pl.bits == 4) run_codes_random<DT, 4, GRAIN>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+    else run_codes_random<DT, 8, GRAIN>(pl, p, grain, lane, TT, n, lo, inv, g0, gp, at);
+  } else if (pl.bits == 2) run_codes<DT, K, TT, EDGE, 2>(lane, n, lo, inv, at, x);
+  else if (pl.bits == 4) run_codes<DT, K, TT, EDGE, 4>(lane, n, lo, inv, at, x);
+  else run_codes<DT, K, TT, EDGE, 8>(lane, n, lo, inv, at, x);
 }
 // Zero padding of a slot behind the codes, by `n` threads of which this is number `i`.
 __device__ __forceinline__ void pad_slot(const Plan& pl, uint8_t* slot, uint32_t i, uint32_t n) {
@@ -2137,14 +2300,48 @@ __global__ void __launch_bounds__(kSweepThreads) compress_cta(const Plan pl, con
 // -------------------------------------------------------------------------------------------------
 constexpr int kCtaThreads = kCtaMaxWarps * 32;
 
-template <int DT, int SIGMA, int K, int EDGE, bool PARTS>
-__global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan pl, const CompressArgs a) {
+// What the sweep only looks at now and then: the destination and, of thread 0, the next ticket, the number of loads issued and
+// the last plane's minimum and scale, for its table entry.
+struct CtaOwn {
+  Dest d;
+  uint32_t next_ticket, issued;
+  float lo, scale;
+};
+// WORDS: bf16 runs are held as they lie in memory, with which 24 warps fit on an SM instead of 20 (28 without the plane's own
+// statistics).  That is taken for CTAs of 7, 11 and 12 warps, which come to three, two and two on an SM then and not to
+// two, one and one: with few warps resident, the three barriers a plane are what such planes wait for.  us a call, 2 bits, before
+// and now: 128 x 96 planes of 112 x 112 118.1 -> 108.0, with every eighth channel outlier-rich 250.2 -> 220.4, without statistics
+// 73.2 -> 61.7, random rounding 249.3 -> 214.5; 64 x 32 of 140 x 140 46.3 -> 36.6, of 146 x 146 47.4 -> 39.9; 100 x 61 of
+// 127 x 93 72.0 -> 68.1.  Elsewhere it is as many CTAs or little more, and the six instructions a group cost more than it gives:
+// 56 x 56 (2 warps) 50.2 -> 55.6, 120 x 119 (8 warps) 50.2 -> 50.9.
+// What is not needed in every step is kept in shared memory then, since what does not fit the registers goes to local memory, for
+// which the stages leave little L1.
+template <bool WORDS>
+struct Held {
+  using T = float;
+  static constexpr int N = 4;
+};
+template <>
+struct Held<true> {
+  using T = uint32_t;
+  static constexpr int N = 2;
+};
+// (registers are dealt out by the threads that a CTA may have: 96, 80 or 72)
+constexpr int cta_threads(bool words, int sigma) { return !words ? kCtaThreads : (sigma == 1 ? 768 : 896); }
+
+template <int DT, int SIGMA, int K, int EDGE, bool PARTS, bool WORDS>
+__global__ void __launch_bounds__(cta_threads(WORDS, SIGMA), 1) compress_cta_regs(const Plan pl, const CompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 4];
   __shared__ __align__(8) uint64_t s_full[2];
   __shared__ uint32_t s_tiles[2], s_abort, s_last, s_count[2];
   __shared__ float2 s_thr;
+  __shared__ Cuts s_cut;
+  __shared__ bool s_look;
   __shared__ BlockCtl s_ctl;
+  __shared__ CtaOwn s_own;
+  CtaOwn r_own;
+  CtaOwn& own = WORDS ? s_own : r_own;
 
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const Team team = make_cta_team(blockDim.x, s_red);
@@ -2153,8 +2350,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
   uint32_t rp = 0;
   // Thread 0 requests the tiles and issues the loads: the first two in one request (one, when there are too few for every
   // CTA to get two), later ones one at a time, the request running one tile ahead of its use.  Tiles come in ticket order.
-  uint32_t next_ticket = 0, issued = 0;
-  const uint32_t early = pl.nstage;
   if (tid == 0) {
     mbar_init(&s_full[0], 1);
     mbar_init(&s_full[1], 1);
@@ -2162,7 +2357,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     s_abort = 0;
     s_count[0] = s_count[1] = 0;
     *cta_totals() = CtaTotals{0u, 0u, 0u, 0u};
-    if (a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + early);
+    own.issued = 0;
+    if (a.early_ticket) own.next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + pl.nstage);
     if (scan_on) {  // (before the wait for the previous kernel, whose tail hides it)
       s_ctl.pl = pl;
       s_ctl.a = a;
@@ -2170,25 +2366,25 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     }
   }
   auto issue = [&](uint32_t s) {
-    const uint32_t t = next_ticket;
+    const uint32_t t = own.next_ticket;
     s_tiles[s] = t;
     if (t < pl.ntiles) {
       plane_load(pl, a.src, t, smem + (uint64_t)s * pl.stage_bytes, &s_full[s]);
-      ++issued;
-      next_ticket = issued < early ? t + 1u : (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
+      own.next_ticket = ++own.issued < pl.nstage ? t + 1u : (uint32_t)atomicAdd(&a.sc->ticket[a.parity], 1ull);
     }
   };
   // the previous kernel on the stream has completed; global memory may be touched from here on (the input is only read)
   if (!a.early_load) dep_wait();
   if (tid == 0) {  // the first loads before anything else
-    if (!a.early_ticket) next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + early);
+    if (!a.early_ticket) own.next_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], kStarted + pl.nstage);
     issue(0);
     issue(1);
   }
   if (a.early_load) dep_wait();
   dep_trigger();  // the next kernel on the stream may become resident as this one drains
-  const Dest d = make_dest(pl, a);
+  if (!WORDS || tid == 0) own.d = make_dest(pl, a);
   if (tid == 0) {
+    const Dest d = own.d;
     if (!d.fits && blockIdx.x == 0) report_error(a, kErrCapacity);
     if (scan_on) s_ctl.d = d;
   }
@@ -2199,7 +2395,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
   const int32_t n = (int32_t)(min(4u * g1, pl.HW) - 4u * g0);
   // the plane before, whose class is still open: its tile (kNoTile: none), and for its table entry minimum, scale
   uint32_t prev = kNoTile, prev_meta = 0;
-  float prev_lo = 0.0f, prev_scale = 0.0f;
   // Class of the plane before, behind a barrier that all its counts precede (every thread gets the same answer): a
   // normal plane is complete -- table entry, publication, its stage takes the next load --, another is to be measured.
   auto settle = [&](uint32_t s) -> bool {
@@ -2210,7 +2405,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     }
     if ((prev_meta & 3u) != kClsNormal) return true;
     if (tid == 0) {
-      if (d.fits) store_table_entry(d, prev, (uint32_t)((pl.slots_off + (uint64_t)prev * pl.npay) >> 4), prev_meta, prev_lo, prev_scale);
+      if (own.d.fits) store_table_entry(own.d, prev, (uint32_t)((pl.slots_off + (uint64_t)prev * pl.npay) >> 4), prev_meta, own.lo, own.scale);
       if (scan_on) scan_publish(a.scan, prev, 0u);
       issue(s);
     }
@@ -2230,7 +2425,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     if (tile >= pl.ntiles) break;
     const bool ready = mbar_wait(&s_full[s], (phase >> s) & 1u, 1u << 20);
     phase ^= 1u << s;
-    float x[K][4], lo, hi;
+    typename Held<WORDS>::T x[K][Held<WORDS>::N];
+    float lo, hi;
     const uint8_t* run = smem + (uint64_t)s * pl.stage_bytes + plane_head(pl, tile) + (uint64_t)g0 * (DT == kF32 ? 16u : 8u);
     run_load<DT, K, 32, EDGE>(run, lane, n, grain, x, lo, hi);
     if (!ready) s_abort = 1;
@@ -2255,20 +2451,30 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
         const long long Is = warp_sum_s32_wide(pr.x), Iq = warp_sum_s32_wide(pr.y);
         float tl, th;
         sigma_thresholds(Is, Iq, sc, pl.inv_hw, tl, th);
-        if (lane == 0) s_thr = make_float2(tl, th);
+        if (lane == 0) {
+          s_thr = make_float2(tl, th);
+          if (WORDS) {
+            s_look = range > th || 0.0f < tl;
+            if (s_look) s_cut = element_cuts(lo, tl, th);
+          }
+        }
       }
       if (tid == 0) s_count[s ^ 1u] = 0;  // (settled by every thread before the barrier just passed)
     }
     float inv, scale;
     quant_params(range, (1u << pl.bits) - 1u, inv, scale);
+    if (!WORDS || tid == 0) {  // (the plane before is settled, or is not a normal one)
+      own.lo = lo;
+      own.scale = scale;
+    }
     uint32_t n_out = 0, cls = kClsNormal;
     if (!SIGMA) {
       if (pl.mode == kModeAll) cls = kClsSalient;
       if (pl.mode >= kModeChannel) cls = channel_class(pl, a, tile, n_out);
     }
     auto codes = [&]() {
-      if (!d.fits || cls != kClsNormal) return;
-      uint8_t* slot = d.dst + pl.slots_off + (uint64_t)tile * pl.npay;
+      if (!own.d.fits || cls != kClsNormal) return;
+      uint8_t* slot = own.d.dst + pl.slots_off + (uint64_t)tile * pl.npay;
       run_codes_any<DT, SIGMA, K, 32, EDGE>(pl, run, grain, lane, n, lo, inv, g0, tile, slot, x);
       pad_slot(pl, slot, tid, blockDim.x);
     };
@@ -2276,8 +2482,10 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
       if (!rule) return;
       __syncthreads();  // the third barrier: the thresholds
       const float dlo = s_thr.x, dhi = s_thr.y;
-      if (range > dhi || 0.0f < dlo) {  // otherwise no element can lie outside
-        uint32_t cnt = run_count<DT, K, 32, EDGE>(lane, n, dlo, dhi, x);
+      if (WORDS ? s_look : range > dhi || 0.0f < dlo) {  // otherwise no element can lie outside
+        uint32_t cnt;
+        if constexpr (!WORDS) cnt = run_count<DT, K, 32, EDGE>(lane, n, dlo, dhi, x);
+        else cnt = run_count<DT, K, 32, EDGE>(lane, n, own.lo, dlo, dhi, s_cut, x);
         asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(cnt) : "r"(0xFFFFFFFFu));
         if (lane == 0 && cnt) atomicAdd(&s_count[s], cnt);
       }
@@ -2298,8 +2506,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
     }
     prev = tile;
     prev_meta = cls | (n_out << 2);
-    prev_lo = lo;
-    prev_scale = scale;
     s ^= 1u;
     // (s_tiles of the next turn was written when the plane before was settled, behind the first barrier: a later one --
     // the second, with three-sigma statistics, or this one -- makes it known)
@@ -2320,7 +2526,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) compress_cta_regs(const Plan p
       }
   }
   if (scan_on) cta_finish<DT, PARTS>(&s_ctl, s_red, smem, sal, s_abort != 0u);
-  cta_exit(pl, a, d, &s_last);
+  cta_exit(pl, a, own.d, &s_last);
 }
 
 }  // namespace fh

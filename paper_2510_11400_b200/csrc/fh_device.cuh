@@ -6,6 +6,7 @@
 // planes, the whole CTA for large ones.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
