@@ -968,6 +968,8 @@ __device__ __forceinline__ uint32_t bf16_below(uint32_t c) { return c & 0x8000u 
 // A threshold on distances as one on elements: the largest element whose distance from `lo` does not exceed `t` (EQUAL: is less
 // than `t`), twice in a word.  Distances, rounded as they are, grow with the element, so the neighbours of lo + t are looked at; false when
 // none of three is it (the sum cancels), which leaves the comparison of distances.
+// (Comparing distances always, 128 x 96 planes of 112 x 112: 109.1 -> 127.5 us.  Runs held as fp32 do better to compare their distances
+// than to read the words again for this: 56 x 56 50.2 -> 57.0.)
 template <bool EQUAL>
 __device__ __forceinline__ bool element_cut(float lo, float t, uint32_t& cut) {
   const uint32_t b = __float_as_uint(__fadd_rn(lo, t));
