@@ -224,20 +224,19 @@ __device__ __forceinline__ void warp_excl_scan(uint32_t* arr, uint32_t n) {
 
 // Measuring part: block classes, CSR row lengths, sizes.  The team is a whole warp or a whole CTA.  Leaves rowp, dense
 // and outl (and chunks) as exclusive prefix sums with the total behind the last entry, the bitmap and the code.
-template <int DT, bool PARTS>
-__device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
+template <int DT, bool PARTS, bool ENTROPY>
+__device__ __noinline__ SalientInfo salient_measure_as(const Team t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
   const Geometry g(pl);
   const Split<PARTS> sp(pl);
   const SalScratch sc = sal_scratch(g, sal, sp.seg);
   const uint32_t H = g.H, W = g.W, nsr = g.nsr, tau_den = pl.tau_den, full = 0xFFFFFFFFu;
-  const bool entropy = pl.entropy != 0;
   const uint32_t nw = t.block ? t.nwarps : 1u, wid = t.block ? threadIdx.x >> 5 : 0u, lane = threadIdx.x & 31u;
   const float inv2e = __fdiv_rn(1.0f, __fmul_rn(2.0f, pl.eps));
   const StepLane sl = step_lane(g);
   const bool vec = seg_vec<DT>(plane, W);
   const uint32_t least = pl.tau_num * 64u;  // (at most 2^22)
   for (uint32_t i = t.lane; i < g.nbm; i += t.size) sc.bitmap[i] = 0;
-  if (entropy)
+  if (ENTROPY)
     for (uint32_t i = t.lane; i < 256u; i += t.size) sc.huf->hist[i] = 0;
   if (t.lane == 0) sc.rowp[H * sp.seg] = sc.dense[nsr] = sc.outl[nsr] = 0;
   team_sync(t);
@@ -259,7 +258,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
         seg_codes(v, nin, inv2e, ca, cb, vm);
         if (dense) {
           n_out += __popc(vm);
-          if (entropy) {  // (residuals of 0 are by far the most frequent: counted apart, their bin is not fought over)
+          if (ENTROPY) {  // (residuals of 0 are by far the most frequent: counted apart, their bin is not fought over)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const uint32_t code = ((j < 4 ? ca : cb) >> (8 * (j & 3))) & 255u;
@@ -280,7 +279,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
     if (g.qs > 1) row += __shfl_xor_sync(full, row, 2);
     if ((sl.q & sl.qm) == 0u && y < H) sc.rowp[y * sp.seg + un.part] = row;
     asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_out) : "r"(full));
-    if (entropy) asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_zero) : "r"(full));
+    if (ENTROPY) asm volatile("redux.sync.add.u32 %0, %0, %1;" : "+r"(n_zero) : "r"(full));
     if (lane == 0) {
       sc.dense[sr] = n_dense;
       sc.outl[sr] = n_out;
@@ -299,7 +298,7 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
   info.nnz_s = sc.rowp[H * sp.seg];
   info.n_out_d = sc.outl[nsr];
   info.coded = 0;
-  if (entropy && info.n_dense) {
+  if (ENTROPY && info.n_dense) {
     // Huffman stage (Section 4.4.1): the code from the histogram, then the size of every dense block's chunk
     HufEncode* h = sc.huf;
     if (wid == 0) huffman_build(h);
@@ -339,6 +338,11 @@ __device__ __noinline__ SalientInfo salient_measure(const Team t, const Plan& pl
   info.size = 16u + 4u * g.nbm + 4u * (H + 1u) + a4(2u * info.nnz_s) + a4(e * info.nnz_s) +
               (info.coded ? info.coded : 64u * info.n_dense) + a4(e * info.n_out_d);
   return info;
+}
+// With the Huffman stage and without: its counts take registers that the others' loop lacks.
+template <int DT, bool PARTS>
+__device__ __forceinline__ SalientInfo salient_measure(const Team& t, const Plan& pl, const uint8_t* plane, uint32_t* sal) {
+  return pl.entropy ? salient_measure_as<DT, PARTS, true>(t, pl, plane, sal) : salient_measure_as<DT, PARTS, false>(t, pl, plane, sal);
 }
 
 // Writing part; `sal` holds what salient_measure left.  Every lane recomputes the codes of its block rows and stores
