@@ -370,20 +370,22 @@ struct BlockCtl {
 // Warp-team kernel: what the tiles in the stages have gathered so far, and the tiles put off, as far as there is room (the
 // others are linked like those of the CTA-team kernels).  A slice is what one warp sweeps of a tile.
 constexpr uint32_t kListed = 32, kListedPlanes = 128;  // (static shared memory stays below what kSmemLimit leaves)
-// Planes of more than four blocks are put off before they are measured (see warp_measure_put_off), so many of a CTA; until
-// then `place` holds their tiles (kNoTile: an entry that is nobody's).
-constexpr uint32_t kPutOff = kListed;
+// Planes of more than four blocks are put off before they are measured (see warp_measure_put_off), so many of a CTA, as long as they
+// are few in their slice; until then `place` holds their tiles (kNoTile: an entry that is nobody's).  A tile with such a plane has
+// to be listed, so the list keeps an entry for each of them.
+constexpr uint32_t kPutOff = kListed / 2;
 // A stage's counts: salient planes, raw ones, those put off (a tile has at most 256 planes).
 constexpr uint32_t kRawShift = 10, kOffShift = 20, kCountMask = (1u << kRawShift) - 1u;
 struct WarpList {
   uint32_t sum[kMaxStages][kWarps];  // overflow units of a slice (when the slice has outlier-rich planes)
   uint32_t mask[kMaxStages];         // slices that have some
   uint32_t count;                    // tiles put off
-  uint32_t handed;                   // phase 2: items handed out
+  uint32_t measured;                 // ... of larger planes, those that were published when they were found
+  uint32_t handed[2];                // phase 2: items handed out, in each of two passes
   uint32_t tile[kListed];
   uint32_t units[kListed], base[kListed];  // the tile's overflow units and, in phase 2, its place (kNoTile: not to be had)
   uint32_t before[kListed][kWarps];  // units of the tile's slices before this one
-  uint8_t stage[kListed], slices[kListed];
+  uint8_t stage[kListed], slices[kListed];  // slices: those with such planes; larger planes: 0 for a tile that is published
   uint32_t n[kListed];               // outlier-rich planes of the tile (as far as they are measured)
   // planes of more than four blocks: those put off, then, in phase 2, those of the listed tiles
   uint32_t planes;
@@ -1294,9 +1296,15 @@ template <int DT, int TT>
 __device__ __noinline__ void warp_tile_put_off(BlockCtl* c, WarpList* l, uint8_t* tbuf, uint32_t s, uint32_t leaders, uint32_t meta,
                                                uint8_t* sal_base) {
   const uint32_t tile = c->held[s], slice = warp_slice(tile), lane = threadIdx.x & 31u, n = __popc(leaders);
-  uint32_t at = 0;
-  if (lane == 0) at = atomicAdd(&l->planes, n);
-  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  // No more of a slice than its part of the room and half of its planes: planes that are many everywhere keep every warp as busy as any
+  // order would.  (Whole slices until 32 planes were listed, and tiles measured after that with a warp each, us a call: bf16, 66,666 x 3
+  // planes of 54 x 1, 13 % outlier-rich, 210, now 123; fp32, every plane, 2,358 x 16 of 172 x 2 442 -> 297, 512 x 64 of 20 x 20 271 -> 190.)
+  const uint32_t slices = (c->pl.ppt * TT + 31u) / 32u, share = max(min(kPutOff / slices, 16u / TT), 1u);
+  uint32_t at = kPutOff;
+  if (n <= share) {
+    if (lane == 0) at = atomicAdd(&l->planes, n);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  }
   if (at + n <= kPutOff) {
     if ((leaders >> lane) & 1u) {
       const uint32_t k = at + __popc(leaders & ((1u << lane) - 1u));
@@ -1324,8 +1332,9 @@ static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, WarpList* l, 
   c->C[s] = 0;
   l->mask[s] = 0;
   if (!c->d.fits && off == 0u) return;
-  // (larger planes: the list is for tiles with planes that are put off, of which there are no more than such planes)
-  const uint32_t i = off || is_small_plane(c->pl) ? atomicAdd(&l->count, 1u) : kListed;
+  // (larger planes: as many entries are kept for tiles with planes that are put off as there are such planes)
+  const bool room = off || is_small_plane(c->pl) || atomicAdd(&l->measured, 1u) < kListed - kPutOff;
+  const uint32_t i = room ? atomicAdd(&l->count, 1u) : kListed;
   if (i >= kListed) {
     c->a.defer_next[tile] = atomicExch(&c->head, tile);
     return;
@@ -1334,8 +1343,8 @@ static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, WarpList* l, 
   l->units[i] = U;
   l->n[i] = nsal + nraw;
   l->stage[i] = (uint8_t)s;
+  l->slices[i] = off ? 0xFFu : (uint8_t)mask;  // (larger planes' warps set no mask)
   if (off) return;
-  l->slices[i] = (uint8_t)mask;
   uint32_t run = 0;
 #pragma unroll
   for (uint32_t k = 0; k < (uint32_t)kWarps; ++k) {
@@ -1506,7 +1515,7 @@ __device__ __noinline__ void warp_phase2_small(BlockCtl* c, WarpList* l, uint8_t
   if (warp == (uint32_t)kWarps) return;
   for (;;) {
     uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(&l->handed, 1u);
+    if (lane == 0) item = atomicAdd(&l->handed[0], 1u);
     item = __shfl_sync(full, item, 0);
     if (item >= n * (uint32_t)kWarps) break;
     const uint32_t i = item / (uint32_t)kWarps, slice = item % (uint32_t)kWarps, tile = l->tile[i];
@@ -1538,10 +1547,11 @@ __device__ __noinline__ void warp_measure_put_off(BlockCtl* c, WarpList* l, uint
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, full = 0xFFFFFFFFu;
   const uint32_t n = min(l->planes, kPutOff), tiles = min(l->count, kListed), mine = min(threadIdx.x, tiles - 1u);
   const Team team = make_warp_team(nullptr);
+  if (n == 0u) return;
   const bool held = __syncthreads_and(c->held[l->stage[mine]] == l->tile[mine]) != 0;
   while (warp < (uint32_t)kWarps) {
     uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(&l->handed, 1u);
+    if (lane == 0) item = atomicAdd(&l->handed[0], 1u);
     item = __shfl_sync(full, item, 0);
     if (item >= n) break;
     const uint32_t tile = l->place[item], lp = l->lp[item];
@@ -1569,9 +1579,9 @@ __device__ __noinline__ void warp_measure_put_off(BlockCtl* c, WarpList* l, uint
     __syncwarp();
   }
   __syncthreads();
-  if (threadIdx.x < tiles) scan_publish(c->a.scan, l->tile[threadIdx.x], l->units[threadIdx.x]);
+  if (threadIdx.x < tiles && l->slices[threadIdx.x]) scan_publish(c->a.scan, l->tile[threadIdx.x], l->units[threadIdx.x]);
   if (threadIdx.x < (uint32_t)kMaxStages && !held) c->held[threadIdx.x] = kNoTile;
-  if (threadIdx.x == 0) l->planes = l->handed = 0;
+  if (threadIdx.x == 0) l->planes = l->handed[0] = 0;
   __syncthreads();
 }
 
@@ -1631,27 +1641,31 @@ __device__ __noinline__ void warp_phase2_large(BlockCtl* c, WarpList* l, uint8_t
     __syncwarp();
     if (lane == 0) l->of[at] = (uint8_t)kListed;
   }
-  __syncthreads();
+  const bool away = threadIdx.x < n && c->held[l->stage[min(threadIdx.x, kListed - 1u)]] != l->tile[min(threadIdx.x, kListed - 1u)];
+  const bool others = __syncthreads_or(away || c->head != kNoTile) != 0;
   if (own_place != kNoTile) {
     write_blockwise<DT, false>(make_warp_team(nullptr), pl, c->d, (uint64_t)own.tile * pl.ppt + own.lp, own.plane, own.info, sal, own_meta >> 2,
                                own_place);
     __syncwarp();
   }
-  // (planes lie in stages when all do, and are fetched into them otherwise: then none is held)
-  while (warp < (uint32_t)kWarps) {
-    uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(&l->handed, 1u);
-    item = __shfl_sync(full, item, 0);
-    if (item >= planes) break;
-    const uint32_t i = l->of[item];
-    if (i == kListed) continue;
-    const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
-    const uint8_t* plane = c->held[st] == tile ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr;
-    warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, plane, l->meta[item], l->place[item], buf, sal);
+  // planes that lie in stages, then those that are fetched into them (where planes have been put off, one or the other: see above)
+  for (uint32_t pass = 0; pass < (others ? 2u : 1u); ++pass) {
+    if (pass) __syncthreads();  // the stages are free
+    while (warp < (uint32_t)kWarps) {
+      uint32_t item = 0;
+      if (lane == 0) item = atomicAdd(&l->handed[pass], 1u);
+      item = __shfl_sync(full, item, 0);
+      if (item >= planes) break;
+      const uint32_t i = l->of[item];
+      if (i == kListed) continue;
+      const uint32_t tile = l->tile[i], st = l->stage[i], lp = l->lp[item];
+      const bool held = c->held[st] == tile;
+      if (held != (pass == 0u)) continue;
+      warp_plane_write<DT>(c, (uint64_t)tile * pl.ppt + lp, held ? stages + (uint64_t)st * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes : nullptr,
+                           l->meta[item], l->place[item], buf, sal);
+    }
   }
-  if (c->head == kNoTile) return;  // (the same for every thread: nothing was linked since the list was made)
-  __syncthreads();                 // the stages are free
-  if (warp == (uint32_t)kWarps) return;
+  if (!others || warp == (uint32_t)kWarps) return;
   uint32_t at;
   for (uint32_t tile; (tile = warp_take_linked(c, at)) != kNoTile;) {
     const uint64_t p0 = (uint64_t)tile * pl.ppt;
@@ -1699,7 +1713,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
         s_ctl.held[s] = kNoTile;
         s_list.mask[s] = 0;
       }
-      s_list.count = s_list.planes = s_list.handed = 0;
+      s_list.count = s_list.measured = s_list.planes = s_list.handed[0] = s_list.handed[1] = 0;
     }
   }
   // (the ticket counter of this call was returned to zero by the call before the previous one, which had

@@ -38,3 +38,19 @@ def test_parity_with_planes_measured_late(shape, dtype, kind, kw):
 def test_parity_of_small_planes_in_many_tiles(shape, dtype):
     full_parity(synth.TensorSpec("t", shape, dtype, "relu", 49), bits=2)
     full_parity(synth.TensorSpec("t", shape, dtype, "spiky_relu", 50), bits=4)
+
+
+# planes that are many in their slice of a tile, which are measured where they are found: tiles with only such planes, in their stages
+# and fetched again; more of them than are listed; tiles of both kinds
+@pytest.mark.parametrize("shape,dtype,kind,kw", [
+    ((3333, 3, 54, 1), synth.BF16, "relu", dict(bits=2)),
+    ((250, 128, 2, 43), synth.F32, "laplace_ch", dict(bits=4)),
+    ((61, 24, 1, 89), synth.F32, "spiky_relu", dict(bits=8, **ALL)),
+    ((300, 16, 172, 2), synth.F32, "spiky_relu", dict(bits=8, **ALL)),
+    ((64, 64, 20, 20), synth.BF16, "spiky_relu", dict(bits=4, **ALL)),
+    ((300, 999, 1, 40), synth.F32, "relu", dict(bits=4, **ALL)),
+    ((300, 999, 1, 40), synth.BF16, "spiky_relu", dict(bits=2)),
+    ((400, 61, 8, 3), synth.F32, "normal", dict(bits=4, entropy=1)),
+])
+def test_parity_with_many_planes_in_a_slice(shape, dtype, kind, kw):
+    full_parity(synth.TensorSpec("t", shape, dtype, kind, 51), **kw)
