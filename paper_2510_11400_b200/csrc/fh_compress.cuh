@@ -1488,8 +1488,12 @@ static __device__ __noinline__ void warp_list_places(BlockCtl* c, WarpList* l, u
   if (lane < want) l->base[from] = ok ? base : kNoTile;
 }
 
-// Phase 2 of the warp-team kernel, small planes.  One warp looks up the places of the listed tiles (every warp for itself: 7 x 7
-// planes, fp32: 25 -> 45 us).  Then every warp copies the payloads of the slices it has encoded, of tiles that still lie in a
+// Phase 2 of the warp-team kernel, small planes.  The places of the listed tiles are looked up first: by one warp for all of them or,
+// when a CTA has at most two tiles, a warp to a tile.  (us a call, by one / a warp to a tile / as they are.  By one the last place
+// comes later: fp32, 170 x 513 planes of 22 x 2 45 / 41 / 40, 200 x 512 of 7 x 7 40 / 35 / 34, 64 x 256 of 14 x 14 18.1 / 17.1 / 17.0.  When there
+// are many, more warps that poll hold up the publications they wait for: bf16, every eighth channel outlier-rich, 128 x 960 of 7 x 7 39 /
+// 44 / 38, 128 x 384 of 14 x 14 45 / 53 / 47.  Every warp for itself: 7 x 7 planes, fp32: 25 -> 45.)
+// Then every warp copies the payloads of the slices it has encoded, of tiles that still lie in a
 // stage: the last ones the CTA streamed, all of them when the tensor is small.  The other tiles, if there are any, are handed out
 // slice by slice; their planes are fetched and encoded again, in the stages, a part to a warp.
 template <int DT, int TT>
@@ -1500,7 +1504,16 @@ __device__ __noinline__ void warp_phase2_small(BlockCtl* c, WarpList* l, uint8_t
   // (the warp's slice of a tile, as in phase 1; the first one's markers are on their way while the places are looked up)
   uint4 ahead = make_uint4(0u, 0u, 0u, 0u);
   if (warp < (uint32_t)kWarps) ahead = slice_marker<DT, TT>(c, l->tile[0], warp_slice(l->tile[0]));
-  else warp_list_places(c, l, n);
+  if (pl.ntiles > 2u * gridDim.x) {
+    if (warp == (uint32_t)kWarps) warp_list_places(c, l, n);
+  } else {
+    for (uint32_t i = (uint32_t)kWarps - warp; i < n; i += (uint32_t)kWarps + 1u) {
+      uint32_t base = 0;
+      const bool ok = l->units[i] == 0u || scan_prefix(c->a.scan, l->tile[i], base);
+      if (!ok && lane == 0) report_error(c->a, kErrTimeout);
+      if (lane == 0) l->base[i] = ok ? base : kNoTile;  // (units are below 2^32 - 1)
+    }
+  }
   const bool away = threadIdx.x < n && c->held[l->stage[min(threadIdx.x, kListed - 1u)]] != l->tile[min(threadIdx.x, kListed - 1u)];
   const bool others = __syncthreads_or(away || c->head != kNoTile) != 0;  // (the places are known)
   if (warp < (uint32_t)kWarps)
