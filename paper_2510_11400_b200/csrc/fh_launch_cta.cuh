@@ -31,13 +31,26 @@ int launch_cta_regs_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream
                      : launch_cta_regs_p<DT, SIGMA, K, EDGE, false, WORDS>(pl, a, stream);
 }
 
+// Whether the planes of a bf16 tensor are held as words (see Held): CTAs of 7, 11 and 12 warps, by how many planes there are.  A plane
+// alone takes longer so, by 0.3 us; it pays where more CTAs have one at once than could otherwise, and where there are so many that it
+// makes no difference how full the last ones are.  us a call, 4 bits, 112 x 112, as fp32 / as words: 296 planes 8.0 / 9.4, 444
+// 10.2 / 9.8, 480 10.4 / 13.0, 960 15.0 / 18.4, 1,480 20.4 / 20.0, 2,000 25.5 / 24.8, 6,000 61.9 / 57.8; 134 x 134 (11 warps): 148 7.0 / 7.3,
+// 296 11.9 / 9.6, 400 12.6 / 13.9, 592 17.1 / 18.1, 740 19.7 / 19.2, 2,000 44.5 / 36.3; 146 x 146 (12): 400 13.4 / 15.3, 740 20.9 / 22.0, 900
+// 24.1 / 23.0.  With random rounding they gain wherever there are more of them: 112 x 112, 296 12.0 / 11.9, 592 24.4 / 17.5, 2,000 56.3 / 48.1
+// (but 700 26.1 / 28.9).
+inline bool word_runs(uint32_t nw, int sigma, uint32_t planes) {
+  if (nw != 7u && nw != 11u && nw != 12u) return false;
+  const uint32_t sms = (uint32_t)sm_count(), at_once = sms * (20u / nw), as_words = sms * ((sigma == 1 ? 24u : 28u) / nw);
+  return planes > at_once && (sigma == 2 || planes <= as_words || planes > 5u * at_once);
+}
+
 // Slots per lane; as the CTA has as few warps as hold the plane, a warp's share is 225 to 448 groups (8 to 14 slots).
 template <int DT, int SIGMA>
 int launch_cta_regs(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   const uint32_t nw = pl.team / 32u, slots = ((pl.groups + nw - 1u) / nw + 31u) / 32u;
   const bool whole = pl.HW == nw * 4u * kCtaGroups;  // (112 x 112)
   if constexpr (DT == kBF16) {
-    if (nw == 7u || nw == 11u || nw == 12u) {  // (see Held; a warp's share is at least 385 groups)
+    if (word_runs(nw, SIGMA, pl.ntiles)) {
       if (whole) return launch_cta_regs_t<DT, SIGMA, 14, 0, true>(pl, a, stream);
       if (slots <= 13u) return launch_cta_regs_t<DT, SIGMA, 13, 1, true>(pl, a, stream);
       return launch_cta_regs_t<DT, SIGMA, 14, 1, true>(pl, a, stream);

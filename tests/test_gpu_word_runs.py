@@ -50,3 +50,38 @@ def test_parity_of_hard_thresholds(bits):
     st_g, packed, total_g = gpu_compress(raw, shape, synth.BF16, bits=bits)
     assert st_o == st_g == api.FH_OK and total_o == total_g
     assert np.array_equal(packed[:total_g].cpu().numpy(), buf_o)
+
+
+def room(hw):
+    """Planes that are worked on at once, held as fp32 and as words (with three-sigma statistics): 20 and 24 warps to an SM."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    warps = -(-(-(-hw[0] * hw[1] // 4)) // 448)
+    return sms * (20 // warps), sms * (24 // warps)
+
+
+@pytest.mark.parametrize("hw", [hw for hw in PLANES if 10753 <= hw[0] * hw[1] <= 12544 or 17921 <= hw[0] * hw[1] <= 21504])
+def test_parity_of_as_many_planes_as_are_held_as_words(hw):
+    n = room(hw)[0] + 1
+    full_parity(synth.TensorSpec("t", (1, n, *hw), synth.BF16, "laplace_ch", 95), bits=4)
+    full_parity(synth.TensorSpec("t", (1, n, *hw), synth.BF16, "spiky_relu", 96), bits=2)
+    full_parity(synth.TensorSpec("t", (1, n, *hw), synth.BF16, "normal", 97), bits=8, salient_mode=api.FH_SALIENT_OFF)
+    full_parity(synth.TensorSpec("t", (1, n, *hw), synth.BF16, "spiky_normal", 98), bits=2, rounding=1)
+
+
+@pytest.mark.parametrize("hw", [(112, 112), (134, 134), (146, 146)])
+def test_parity_where_the_numbers_of_planes_change_how_they_are_held(hw):
+    fp32, words = room(hw)
+    for n in (1, fp32, words, words + 1, 5 * fp32, 5 * fp32 + 1):
+        full_parity(synth.TensorSpec("t", (1, n, *hw), synth.BF16, "laplace_ch", 99), bits=2)
+
+
+def test_parity_of_hard_thresholds_in_planes_held_as_words():
+    x = np.tile(values(), (12, 1))
+    raw = synth.to_bf16_bits(x.reshape(-1))
+    shape = (1, x.shape[0], 112, 112)
+    assert room((112, 112))[0] < x.shape[0] <= room((112, 112))[1]
+    st_o, buf_o, total_o, _ = oracle_compress(raw, shape, synth.BF16, bits=4)
+    st_g, packed, total_g = gpu_compress(raw, shape, synth.BF16, bits=4)
+    assert st_o == st_g == api.FH_OK and total_o == total_g
+    assert np.array_equal(packed[:total_g].cpu().numpy(), buf_o)
