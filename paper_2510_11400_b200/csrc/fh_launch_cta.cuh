@@ -27,6 +27,8 @@ int launch_cta_regs_p(const Plan& pl, const CompressArgs& a, cudaStream_t stream
 }
 template <int DT, int SIGMA, int K, int EDGE, bool WORDS = false>
 int launch_cta_regs_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+  // (the first K - EDGE slots are not masked: a warp that has fewer groups would read past its run)
+  if (pl.groups / (pl.team / 32u) < 32u * (K - EDGE)) return FH_ERR_UNSUPPORTED;
   return pl.seg > 1u ? launch_cta_regs_p<DT, SIGMA, K, EDGE, true, WORDS>(pl, a, stream)
                      : launch_cta_regs_p<DT, SIGMA, K, EDGE, false, WORDS>(pl, a, stream);
 }
@@ -44,7 +46,9 @@ inline bool word_runs(uint32_t nw, int sigma, uint32_t planes) {
   return planes > at_once && (sigma == 2 || planes <= as_words || planes > 5u * at_once);
 }
 
-// Slots per lane; as the CTA has as few warps as hold the plane, a warp's share is 225 to 448 groups (8 to 14 slots).
+// Slots per lane; as the CTA has as few warps as hold the plane, a warp's share is 224 to 448 groups (7 to 14 slots).  Shares differ by
+// one group at most, so that with `slots` slots in the largest the smallest fills all but the last (224, 320, 384 and 416 groups at
+// least: just what the instances below leave unmasked).
 template <int DT, int SIGMA>
 int launch_cta_regs(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
   const uint32_t nw = pl.team / 32u, slots = ((pl.groups + nw - 1u) / nw + 31u) / 32u;

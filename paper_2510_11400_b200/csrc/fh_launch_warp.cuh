@@ -8,10 +8,17 @@ namespace fh {
 
 template <int DT, int SIGMA, int TT, int K, int EDGE>
 int launch_warp_t(const Plan& pl, const CompressArgs& a, cudaStream_t stream) {
+  // (the first K - EDGE slots are not masked: a smaller plane's team would read past it)
+  if (pl.groups < (uint32_t)(TT * (K - EDGE)) || pl.groups > (uint32_t)(TT * K)) return FH_ERR_UNSUPPORTED;
   int grid = 0;
   int rc = grid_for(compress_warp<DT, SIGMA, TT, K, EDGE>, pl.sm_total, pl.ntiles, &grid, kWarpKernelThreads);
   if (rc != FH_OK) return rc;
   grid = spread_grid(grid, pl.ntiles);
+  // Outlier-rich planes of tiles that are no longer in a stage are fetched again, into a warp's part of the stages, which has to hold
+  // them: four planes of a block each, or one.  Where tiles have been made small for the Huffman stage it does not, but then a CTA gets no
+  // more tiles than it has stages, and nothing is fetched.
+  const size_t part = (pl.sm_sal / (uint32_t)kWarps) & ~15u, fetched = (pl.nblk == 1u ? 4u : 1u) * A16(pl.plane_bytes + 16);
+  if (pl.mode != kModeOff && part < fetched && pl.ntiles > (uint64_t)pl.nstage * (uint32_t)grid) return FH_ERR_UNSUPPORTED;
   Plan q = with_first_request(pl, grid, 1);
   q.nstage = pl.nstage;  // (the ring has all its stages, however many tiles the first request is for)
   return launch_dependent(compress_warp<DT, SIGMA, TT, K, EDGE>, grid, kWarpKernelThreads, pl.sm_total, stream, q, a) == cudaSuccess ? FH_OK : FH_ERR_CUDA;

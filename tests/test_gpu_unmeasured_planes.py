@@ -54,3 +54,11 @@ def test_parity_of_small_planes_in_many_tiles(shape, dtype):
 ])
 def test_parity_with_many_planes_in_a_slice(shape, dtype, kind, kw):
     full_parity(synth.TensorSpec("t", shape, dtype, kind, 51), **kw)
+
+
+# Huffman stage, fewer tiles than SMs: tiles of eight, four, two planes and one, so that a warp's part of the stages holds less than a
+# plane; on either side of each change
+@pytest.mark.parametrize("planes", [147, 148, 294, 296, 297, 588, 592, 1176, 1184, 1185])
+def test_parity_of_small_tiles(planes):
+    full_parity(synth.TensorSpec("t", (1, planes, 32, 32), synth.F32, "spiky_relu", 52), bits=4, entropy=1, **ALL)
+    full_parity(synth.TensorSpec("t", (1, planes, 31, 29), synth.BF16, "spiky_relu", 53), bits=2, entropy=1)
