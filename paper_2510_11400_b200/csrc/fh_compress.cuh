@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, ROUND ? 4 : 1) compress_generic(cons
       uint32_t U = 0, nsal = 0, nraw = 0;  // (every thread keeps the same figures)
       for (uint32_t lp = 0; lp < np; ++lp) {
         if ((rec[lp].meta & 3u) == kClsNormal) continue;
-        const SalientInfo info = salient_measure<DT, true>(cta, s_ctl.pl, tile_buf + head + (uint64_t)lp * pl.plane_bytes, sal);
+        const SalientInfo info = salient_measure_outlined<DT, true>(cta, s_ctl.pl, tile_buf + head + (uint64_t)lp * pl.plane_bytes, sal);
         bool raw;
         const uint32_t u = plane_units(pl, info, raw);
         if (tid == 0 && d.fits) store_marker(d, p0 + lp, rec[lp].meta, u);
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, ROUND ? 4 : 1) compress_generic(cons
       for (uint32_t lp = 0; lp < np; ++lp) {
         if ((rec[lp].meta & 3u) == kClsNormal) continue;
         const uint8_t* plane = tile_buf + head + (uint64_t)lp * pl.plane_bytes;
-        const SalientInfo info = salient_measure<DT, true>(cta, s_ctl.pl, plane, sal);
+        const SalientInfo info = salient_measure_outlined<DT, true>(cta, s_ctl.pl, plane, sal);
         write_blockwise<DT, true>(cta, s_ctl.pl, d, p0 + lp, plane, info, sal, rec[lp].meta >> 2, at);
         at += rec[lp].units;
         __syncthreads();
