@@ -370,22 +370,21 @@ struct BlockCtl {
 // Warp-team kernel: what the tiles in the stages have gathered so far, and the tiles put off, as far as there is room (the
 // others are linked like those of the CTA-team kernels).  A slice is what one warp sweeps of a tile.
 constexpr uint32_t kListed = 32, kListedPlanes = 128;  // (static shared memory stays below what kSmemLimit leaves)
-// Planes of more than four blocks are put off before they are measured (see warp_measure_put_off), so many of a CTA, as long as they
-// are few in their slice; until then `place` holds their tiles (kNoTile: an entry that is nobody's).  A tile with such a plane has
-// to be listed, so the list keeps an entry for each of them.
-constexpr uint32_t kPutOff = kListed / 2;
+// Planes of more than four blocks are put off before they are measured (see warp_measure_put_off), as many of a CTA as are listed.  A
+// tile with such a plane has to be listed too: the first warp that finds one asks for the entry.
+constexpr uint32_t kNoEntry = 0xFFFFFFFFu, kEntryAsked = 0xFFFFFFFEu, kEntryFull = 0xFFFFFFFDu;
 // A stage's counts: salient planes, raw ones, those put off (a tile has at most 256 planes).
 constexpr uint32_t kRawShift = 10, kOffShift = 20, kCountMask = (1u << kRawShift) - 1u;
 struct WarpList {
   uint32_t sum[kMaxStages][kWarps];  // overflow units of a slice (when the slice has outlier-rich planes)
   uint32_t mask[kMaxStages];         // slices that have some
   uint32_t count;                    // tiles put off
-  uint32_t measured;                 // ... of larger planes, those that were published when they were found
+  uint32_t entry[kMaxStages];        // larger planes: the list entry of the tile in a stage
   uint32_t handed[2];                // phase 2: items handed out, in each of two passes
   uint32_t tile[kListed];
   uint32_t units[kListed], base[kListed];  // the tile's overflow units and, in phase 2, its place (kNoTile: not to be had)
   uint32_t before[kListed][kWarps];  // units of the tile's slices before this one
-  uint8_t stage[kListed], slices[kListed];  // slices: those with such planes; larger planes: 0 for a tile that is published
+  uint8_t stage[kListed], slices[kListed];  // slices: those with such planes; larger planes: 0 for a tile that has been published
   uint32_t n[kListed];               // outlier-rich planes of the tile (as far as they are measured)
   // planes of more than four blocks: those put off, then, in phase 2, those of the listed tiles
   uint32_t planes;
@@ -1296,26 +1295,43 @@ template <int DT, int TT>
 __device__ __noinline__ void warp_tile_put_off(BlockCtl* c, WarpList* l, uint8_t* tbuf, uint32_t s, uint32_t leaders, uint32_t meta,
                                                uint8_t* sal_base) {
   const uint32_t tile = c->held[s], slice = warp_slice(tile), lane = threadIdx.x & 31u, n = __popc(leaders);
-  // No more of a slice than its part of the room and half of its planes: planes that are many everywhere keep every warp as busy as any
-  // order would.  (Whole slices until 32 planes were listed, and tiles measured after that with a warp each, us a call: bf16, 66,666 x 3
-  // planes of 54 x 1, 13 % outlier-rich, 210, now 123; fp32, every plane, 2,358 x 16 of 172 x 2 442 -> 297, 512 x 64 of 20 x 20 271 -> 190.)
-  const uint32_t slices = (c->pl.ppt * TT + 31u) / 32u, share = max(min(kPutOff / slices, 16u / TT), 1u);
-  uint32_t at = kPutOff;
-  if (n <= share) {
-    if (lane == 0) at = atomicAdd(&l->planes, n);
-    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  // (Not when every plane is outlier-rich and a CTA has several tiles: every warp has as many of them then, and measures its own while
+  // the next tile is on its way.  us a call, put off / at once: fp32, 512 x 64 planes of 20 x 20 212 / 188, 2,358 x 16 of 172 x 2
+  // 322 / 295; with one tile to a CTA the plane measured last need not be measured again: bf16, 4 x 513 of 23 x 23 26 / 33.)
+  const bool even = c->pl.mode == kModeAll && !c->pl.entropy && c->pl.ntiles > gridDim.x;
+  uint32_t at = kListedPlanes, e = kEntryFull;
+  if (lane == 0 && !even) {
+    at = atomicAdd(&l->planes, n);
+    if (at + n <= kListedPlanes) {
+      e = atomicCAS(&l->entry[s], kNoEntry, kEntryAsked);
+      if (e == kNoEntry) {
+        e = atomicAdd(&l->count, 1u);
+        if (e < kListed) {
+          l->tile[e] = tile;
+          l->stage[e] = (uint8_t)s;
+          l->slices[e] = 0xFFu;
+        } else {
+          e = kEntryFull;
+        }
+        atomicExch(&l->entry[s], e);
+      }
+      // (another warp is about to store it; without it the planes are measured here)
+      for (uint32_t k = 0; e == kEntryAsked && k < (1u << 16); ++k) e = *(volatile uint32_t*)&l->entry[s];
+    }
   }
-  if (at + n <= kPutOff) {
+  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  e = __shfl_sync(0xFFFFFFFFu, e, 0);
+  if (e < kListed) {
     if ((leaders >> lane) & 1u) {
       const uint32_t k = at + __popc(leaders & ((1u << lane) - 1u));
-      l->place[k] = tile;
+      l->of[k] = (uint8_t)e;
       l->lp[k] = (uint16_t)(slice * (32u / TT) + lane / TT);
       l->meta[k] = meta;
     }
     if (lane == 0) atomicAdd(&c->C[s], n << kOffShift);
     return;
   }
-  if (at + lane < kPutOff) l->place[at + lane] = kNoTile;
+  if (lane < n && at + lane < kListedPlanes) l->of[at + lane] = (uint8_t)kListed;  // (nobody's)
   warp_tile_measure<DT, TT>(c, tbuf, (uint64_t)tile * c->pl.ppt, s, slice, leaders, meta,
                             reinterpret_cast<uint32_t*>(sal_base + (threadIdx.x >> 5) * c->pl.sal_stride));
 }
@@ -1328,13 +1344,18 @@ static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, WarpList* l, 
   const uint32_t nsal = C & kCountMask, nraw = (C >> kRawShift) & kCountMask, off = C >> kOffShift;
   count_blockwise(U, nsal, nraw);
   const uint32_t mask = l->mask[s];
+  const uint32_t entry = l->entry[s];
   c->U[s] = 0;
   c->C[s] = 0;
   l->mask[s] = 0;
-  if (!c->d.fits && off == 0u) return;
-  // (larger planes: as many entries are kept for tiles with planes that are put off as there are such planes)
-  const bool room = off || is_small_plane(c->pl) || atomicAdd(&l->measured, 1u) < kListed - kPutOff;
-  const uint32_t i = room ? atomicAdd(&l->count, 1u) : kListed;
+  l->entry[s] = kNoEntry;
+  if (off) {
+    l->units[entry] = U;
+    l->n[entry] = nsal + nraw;
+    return;
+  }
+  if (!c->d.fits) return;
+  const uint32_t i = atomicAdd(&l->count, 1u);
   if (i >= kListed) {
     c->a.defer_next[tile] = atomicExch(&c->head, tile);
     return;
@@ -1343,8 +1364,7 @@ static __device__ __noinline__ void warp_tile_publish(BlockCtl* c, WarpList* l, 
   l->units[i] = U;
   l->n[i] = nsal + nraw;
   l->stage[i] = (uint8_t)s;
-  l->slices[i] = off ? 0xFFu : (uint8_t)mask;  // (larger planes' warps set no mask)
-  if (off) return;
+  l->slices[i] = (uint8_t)mask;  // (larger planes' warps set none)
   uint32_t run = 0;
 #pragma unroll
   for (uint32_t k = 0; k < (uint32_t)kWarps; ++k) {
@@ -1546,9 +1566,9 @@ __device__ __noinline__ void warp_phase2_small(BlockCtl* c, WarpList* l, uint8_t
 // its warps side by side when it has run out of tiles; only then are their tiles published.  (A CTA that waits for a tile's
 // publication waits for one that is doing this or is still streaming; neither waits for anybody.)  Each warp keeps what it
 // measured last, and phase 2 has it write that plane without measuring it again.  Planes that still lie in their stages are taken
-// there when all do; otherwise all are fetched, into the stages, a part to a warp.  us a call, before and with scan_places: bf16,
-// 2 bits, 128 x 192 planes of 28 x 28, every eighth channel outlier-rich 92 -> 66; Huffman stage, fp32, 8 x 512 of 7 x 7, 13 % of
-// them outlier-rich, 75 -> 26, 8 x 128 of 28 x 28 48 -> 36.
+// there when all do; otherwise all are fetched, into the stages, a part to a warp.  us a call, measured where they are found / so: bf16,
+// 2 bits, 128 x 192 planes of 28 x 28, every eighth channel outlier-rich 91 / 71, 66,666 x 3 of 54 x 1, 13 % outlier-rich, 136 / 102; Huffman
+// stage, fp32, 8 x 512 of 7 x 7, 14 % outlier-rich, 95 / 26, 8 x 128 of 28 x 28 55 / 36.
 struct WarpOwn {
   uint32_t tile, lp;  // tile: kNoTile if there is none
   const uint8_t* plane;
@@ -1558,7 +1578,7 @@ template <int DT>
 __device__ __noinline__ void warp_measure_put_off(BlockCtl* c, WarpList* l, uint8_t* stages, uint8_t* buf, uint32_t* sal, WarpOwn& own) {
   const Plan& pl = c->pl;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, full = 0xFFFFFFFFu;
-  const uint32_t n = min(l->planes, kPutOff), tiles = min(l->count, kListed), mine = min(threadIdx.x, tiles - 1u);
+  const uint32_t n = min(l->planes, kListedPlanes), tiles = min(l->count, kListed), mine = min(threadIdx.x, tiles - 1u);
   const Team team = make_warp_team(nullptr);
   if (n == 0u) return;
   const bool held = __syncthreads_and(c->held[l->stage[mine]] == l->tile[mine]) != 0;
@@ -1567,10 +1587,9 @@ __device__ __noinline__ void warp_measure_put_off(BlockCtl* c, WarpList* l, uint
     if (lane == 0) item = atomicAdd(&l->handed[0], 1u);
     item = __shfl_sync(full, item, 0);
     if (item >= n) break;
-    const uint32_t tile = l->place[item], lp = l->lp[item];
-    const uint32_t m = __ballot_sync(full, tile != kNoTile && lane < tiles && l->tile[lane] == tile);
-    if (m == 0u) continue;
-    const uint32_t i = (uint32_t)__ffs((int)m) - 1u;
+    const uint32_t i = l->of[item];
+    if (i == kListed) continue;
+    const uint32_t tile = l->tile[i], lp = l->lp[item];
     const uint64_t gp = (uint64_t)tile * pl.ppt + lp;
     const uint8_t* plane = held ? stages + (uint64_t)l->stage[i] * pl.stage_bytes + (uint64_t)lp * pl.plane_bytes
                                 : fetch_plane(pl, c->a.src, gp, buf, lane, 32u, true);
@@ -1725,8 +1744,9 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
         s_ctl.U[s] = s_ctl.C[s] = s_ctl.arr[s] = 0;
         s_ctl.held[s] = kNoTile;
         s_list.mask[s] = 0;
+        s_list.entry[s] = kNoEntry;
       }
-      s_list.count = s_list.measured = s_list.planes = s_list.handed[0] = s_list.handed[1] = 0;
+      s_list.count = s_list.planes = s_list.handed[0] = s_list.handed[1] = 0;
     }
   }
   // (the ticket counter of this call was returned to zero by the call before the previous one, which had
@@ -1734,7 +1754,7 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
   if (tid == (uint32_t)kThreads && a.early_ticket)
     first_ticket = (uint32_t)atomicAdd(&a.sc->ticket[a.parity], (unsigned long long)pl.first_req);
   __syncthreads();
-  if (warp < (uint32_t)kWarps || !a.early_load) {  // (the producer only reads the input and takes tickets)
+  if (warp < (uint32_t)kWarps || !a.early_load) {  // (the producer only reads the input and takes tickets: see dep_wait)
     dep_wait();     // the previous kernel on the stream has completed; global memory may be touched from here on
     dep_trigger();  // the next kernel on the stream may become resident as this one drains
   }

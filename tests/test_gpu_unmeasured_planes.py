@@ -51,6 +51,8 @@ def test_parity_of_small_planes_in_many_tiles(shape, dtype):
     ((300, 999, 1, 40), synth.F32, "relu", dict(bits=4, **ALL)),
     ((300, 999, 1, 40), synth.BF16, "spiky_relu", dict(bits=2)),
     ((400, 61, 8, 3), synth.F32, "normal", dict(bits=4, entropy=1)),
+    ((100000, 1, 1, 40), synth.F32, "spiky_relu", dict(bits=4)),            # all of them, two tiles to a CTA: more planes than are listed
+    ((15000, 8, 1, 520), synth.BF16, "spiky_relu", dict(bits=2)),           # one in a tile, more tiles to a CTA than are listed
 ])
 def test_parity_with_many_planes_in_a_slice(shape, dtype, kind, kw):
     full_parity(synth.TensorSpec("t", shape, dtype, kind, 51), **kw)
