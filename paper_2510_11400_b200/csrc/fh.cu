@@ -276,13 +276,20 @@ int make_plan(const fh_tensor_desc* d, const fh_params* p, bool compress, Plan* 
 
 // ---- per-stream scratch ---------------------------------------------------------------------
 // What one call of the schedule runner needs: offsets, sizes and statuses on the device, where they are read back to
-// (pinned), and its events.  A stream's scratch keeps one for the next call (allocating all of it anew took 20 us of a
-// 400 us schedule); calls that overlap on a stream get their own, freed when they end.
+// (pinned), its events and its side streams.  A stream's scratch keeps one for the next call (allocating all of it anew took
+// 20 us of a 400 us schedule); calls that overlap on a stream get their own, freed when they end.
+constexpr size_t kSideStreams = 3;
 struct SchedSpace {
   unsigned long long *words = nullptr, *host = nullptr;
   size_t cap = 0;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+  cudaStream_t side[kSideStreams] = {};
+  cudaEvent_t side_done[kSideStreams] = {};
   ~SchedSpace() {
+    for (cudaEvent_t e : side_done)
+      if (e) cudaEventDestroy(e);
+    for (cudaStream_t t : side)
+      if (t) cudaStreamDestroy(t);
     if (words) cudaFree(words);
     if (host) cudaFreeHost(host);
     for (cudaEvent_t e : ev)
@@ -301,6 +308,10 @@ struct SchedSpace {
     if (cudaMallocHost(&host, want * sizeof(unsigned long long)) != cudaSuccess) return false;
     cap = want;
     return true;
+  }
+  bool have_side(size_t i) {
+    if (!side[i] && cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking) != cudaSuccess) return false;
+    return side_done[i] || cudaEventCreateWithFlags(&side_done[i], cudaEventDisableTiming) == cudaSuccess;
   }
 };
 
@@ -465,7 +476,7 @@ int enqueue_compress(const fh_tensor_desc* desc, const fh_params* params, const 
   a.out2 = d_out2;
   a.sc = s->sc;
   a.early_ticket = 1;
-  a.early_load = after_compress && pl.mode < fh::kModeChannel ? 1 : 0;
+  a.early_load = after_compress && pl.mode < fh::kModeChannel && pl.dense_bytes % 16 == 0 ? 1 : 0;  // (by bulk copies alone)
   rc = next_call(&s->calls, pl.mode == FH_SALIENT_OFF ? nullptr : s->scan, s->tile_cap, s, (pl.ntiles + 31u) / 32u, stream, &a);
   if (rc != FH_OK) return rc;
   if (pl.mode >= fh::kModeChannel) {  // statistics per channel over the batch, or over the tensor: three passes ahead of the streaming kernel
@@ -490,25 +501,27 @@ int enqueue_compress(const fh_tensor_desc* desc, const fh_params* params, const 
   return rc;
 }
 
-// `order`, `words`: see decompress_begin; kernels that may run side by side have counters of their own (zero before the call).
+// `words`: counters of a stream that has no scratch of its own (zero before the call, and again when the kernel has completed).
 int enqueue_decompress(const void* d_src, size_t src_bytes, const fh_tensor_desc* expect, void* d_dst,
                        const unsigned long long* d_off_in, unsigned long long* d_status, cudaStream_t stream,
-                       uint32_t order = fh::kInOrder, fh::Scratch* words = nullptr) {
+                       fh::Scratch* words = nullptr) {
   Plan pl;
   int rc = make_plan(expect, nullptr, false, &pl, nullptr);
   if (rc != FH_OK) return rc;
   std::lock_guard<std::mutex> lock(g_mu);
-  StreamScratch* s = nullptr;
-  rc = get_scratch(stream, 0, &s);
-  if (rc != FH_OK) return rc;
+  if (!words) {
+    StreamScratch* s = nullptr;
+    rc = get_scratch(stream, 0, &s);
+    if (rc != FH_OK) return rc;
+    words = s->sc;
+  }
   fh::DecompressArgs a = {};
   a.src_base = (const uint8_t*)d_src;
   a.src_bytes = src_bytes;
   a.d_off_in = d_off_in;
   a.dst = (uint8_t*)d_dst;
   a.d_status = d_status;
-  a.sc = words ? words : s->sc;
-  a.order = order;
+  a.sc = words;
   rc = fh::launch_decompress(pl, a, stream);
   if (rc == FH_OK) g_launches.fetch_add(1);
   return rc;
@@ -601,11 +614,13 @@ int fh_run_schedule(const fh_sched_entry* entries, int32_t count, const fh_param
   const size_t k = idx.size();
   if (k == 0) return FH_OK;
   // device words: offsets[k+1] | out2[2k] | decode status[k]; cleared, so that a call that ends early reports nothing stale; then
-  // the decompress kernels' counters, which are not read back
+  // the side streams' counters, which are not read back
   const size_t words = (k + 1) + 2 * k + k, counters = (sizeof(fh::Scratch) + 7) / 8;
   // The inputs of all compress kernels are complete before the first of them starts, so the others need not wait to load
-  // them; nor do the decompress kernels wait for one another: unless buffers overlap, whose results depend on the order.
-  // (Twenty CIFAR-ResNet-shaped tensors at batch 128, ten of them compressed: 340 us a call in order, 309 so.)
+  // them; nor do the decompress kernels wait for one another, so they are dealt out to this stream and two or three more, which wait
+  // for the last compress kernel and which this one waits for: unless buffers overlap, whose results depend on the order.  (Every
+  // other of twenty CIFAR-ResNet-shaped fp32 tensors, us a call strictly in order, with early loads, with side streams too: batch 128
+  // 317, 308, 277, batch 1 178, 180, 146.)
   bool inputs_apart = false, outputs_apart = false;
   try {
     using Range = std::pair<uintptr_t, uintptr_t>;
@@ -634,12 +649,11 @@ int fh_run_schedule(const fh_sched_entry* entries, int32_t count, const fh_param
     s->sched = nullptr;
   }
   if (!space) space.reset(new (std::nothrow) SchedSpace);
-  if (!space || !space->reserve(words + k * counters)) return FH_ERR_CUDA;
+  if (!space || !space->reserve(words + kSideStreams * counters)) return FH_ERR_CUDA;
   unsigned long long* d_off = space->words;
   unsigned long long* d_out2 = d_off + (k + 1);
   unsigned long long* d_dst = d_out2 + 2 * k;
-  fh::Scratch* d_counters = reinterpret_cast<fh::Scratch*>(space->words + words);
-  if (cudaMemsetAsync(space->words, 0, (words + k * counters) * sizeof(unsigned long long), stream) != cudaSuccess) rc = FH_ERR_CUDA;
+  if (cudaMemsetAsync(space->words, 0, (words + kSideStreams * counters) * sizeof(unsigned long long), stream) != cudaSuccess) rc = FH_ERR_CUDA;
   cudaEventRecord(space->ev[0], stream);
   for (size_t j = 0; j < k && rc == FH_OK; ++j) {  // forward order
     const fh_sched_entry& en = entries[idx[j]];
@@ -647,11 +661,29 @@ int fh_run_schedule(const fh_sched_entry* entries, int32_t count, const fh_param
                           d_out2 + 2 * j, stream, j > 0 && inputs_apart);
   }
   cudaEventRecord(space->ev[1], stream);
+  // Small tensors only wait for memory, so that more of them side by side take less time: in all 1 MB on two side streams 154 us, on
+  // three 146; larger ones take room from one another: 126 MB 277 and 284.  (Between 4 and 16 MB they are the same.)
+  const size_t most = report->total_dense_bytes < (8ull << 20) ? 3 : 2;
+  size_t sides = 0;  // side streams that wait for the compress kernels
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (outputs_apart && rc == FH_OK && cudaStreamIsCapturing(stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+    while (sides < most && sides + 1 < k && space->have_side(sides) &&
+           cudaStreamWaitEvent(space->side[sides], space->ev[1], 0) == cudaSuccess)
+      ++sides;
+  uint64_t given[1 + kSideStreams] = {};  // dense bytes of this stream, of the side streams
   for (size_t j = k; j-- > 0 && rc == FH_OK;) {  // reverse order
     const fh_sched_entry& en = entries[idx[j]];
-    rc = enqueue_decompress(d_arena, arena_bytes, &en.desc, en.d_restored, d_off + j, d_dst + j, stream,
-                            !outputs_apart ? fh::kInOrder : (j + 1 == k ? fh::kFirst : fh::kAfter), outputs_apart ? d_counters + j : nullptr);
+    const size_t to = std::min_element(given, given + 1 + sides) - given;
+    given[to] += (uint64_t)en.desc.n * en.desc.c * en.desc.h * en.desc.w * esize_of(en.desc.dtype);
+    rc = enqueue_decompress(d_arena, arena_bytes, &en.desc, en.d_restored, d_off + j, d_dst + j, to ? space->side[to - 1] : stream,
+                            to ? reinterpret_cast<fh::Scratch*>(space->words + words + (to - 1) * counters) : nullptr);
   }
+  for (size_t i = 0; i < sides; ++i)
+    if (cudaEventRecord(space->side_done[i], space->side[i]) != cudaSuccess ||
+        cudaStreamWaitEvent(stream, space->side_done[i], 0) != cudaSuccess) {
+      cudaStreamSynchronize(space->side[i]);
+      rc = rc == FH_OK ? FH_ERR_CUDA : rc;
+    }
   cudaEventRecord(space->ev[2], stream);
   // (read back behind the last kernel on the stream: one wait for everything)
   if (rc == FH_OK && cudaMemcpyAsync(space->host, space->words, words * sizeof(unsigned long long), cudaMemcpyDeviceToHost,

@@ -466,20 +466,6 @@ __device__ __forceinline__ uint32_t check_header(const Plan& pl, const uint8_t* 
   return ok ? version : 0u;
 }
 
-// First step of every thread that touches global memory.
-__device__ __forceinline__ void decompress_begin(const DecompressArgs& a) {
-  if (a.order == kInOrder) {
-    dep_trigger();  // the next kernel on the stream may become resident as this one drains
-    dep_wait();     // the previous kernel on the stream (the one that wrote the container) has completed
-  } else if (a.order == kFirst) {
-    dep_wait();
-    dep_trigger();  // (what starts from here on may rely on the containers)
-  } else {
-    dep_trigger();
-    __threadfence();  // the containers were complete before this kernel could start: nothing older is to be read
-  }
-}
-
 // Last step of every CTA.  The exit counter carries the CTAs that have left in its low half and, in its high half,
 // how many of them had found something wrong; only such a CTA reports and fences, and the last CTA reads the
 // status back only when there was one: a clean call ends with one atomic per CTA.  (The restored tensor needs no
@@ -500,7 +486,6 @@ __device__ __forceinline__ void decompress_exit(const DecompressArgs& a, bool ba
         code = (uint32_t)ld_relaxed(&a.sc->status);
         st_relaxed(&a.sc->status, 0ull);
       }
-      if (a.order == kAfter) dep_wait();  // (this kernel must not be seen to end before the one before it)
       if (a.d_status) *a.d_status = status_word(code);
       st_relaxed(&a.sc->exited, 0ull);
     }
@@ -795,7 +780,8 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_kernel(const Plan pl, 
     s_pl = pl;
     s_nlist = 0;
   }
-  decompress_begin(a);
+  dep_trigger();  // the next kernel on the stream may become resident as this one drains
+  dep_wait();     // the previous kernel on the stream (the one that wrote the container) has completed
   const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
   const uint8_t* src = a.src_base + off_in;
   const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;
@@ -931,7 +917,8 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_large(const Plan pl, c
     s_pl = pl;
     s_nlist = 0;
   }
-  decompress_begin(a);
+  dep_trigger();  // the next kernel on the stream may become resident as this one drains
+  dep_wait();     // the previous kernel on the stream (the one that wrote the container) has completed
   const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
   const uint8_t* src = a.src_base + off_in;
   const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;
@@ -1051,7 +1038,8 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_small(const Plan pl, c
   __shared__ Plan s_pl;  // copy for the outlined slow path, which takes it by address
   const uint32_t tid = threadIdx.x, wlane = tid & 31u;
   if (tid == 0) s_pl = pl;
-  decompress_begin(a);
+  dep_trigger();  // the next kernel on the stream may become resident as this one drains
+  dep_wait();     // the previous kernel on the stream (the one that wrote the container) has completed
   const unsigned long long off_in = a.d_off_in ? *a.d_off_in : 0ull;
   const uint8_t* src = a.src_base + off_in;
   const unsigned long long src_bytes = a.src_bytes > off_in ? a.src_bytes - off_in : 0ull;

@@ -116,9 +116,17 @@ __device__ __forceinline__ void st_relaxed32(uint32_t* p, uint32_t v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// ---- programmatic dependent launch: a kernel launched with the programmatic-serialisation attribute may
-// become resident while its predecessor on the stream is still running; it must pass dep_wait() before it
-// touches anything the predecessor reads or writes.  dep_trigger() in the predecessor allows that early start.
+// ---- programmatic dependent launch: a kernel launched with the programmatic-serialisation attribute may become resident when
+// every CTA of its predecessor on the stream has called dep_trigger() or ended.  What the library's kernels rely on:
+//  - None has completed before all earlier ones on the stream have: dep_wait() returns when they have, and in every kernel threads
+//    that write pass it.  So whatever passes dep_wait() sees all that the stream's earlier kernels have written.
+//  - Compress kernels trigger behind their wait.  So when a kernel behind a compress kernel starts, everything before that compress
+//    kernel has completed.  The others trigger first: any number of them may be resident and waiting.
+//  - Ahead of its wait a kernel touches global memory in two cases.  A compress kernel's first request for tiles (early_ticket):
+//    its ticket counter was returned to zero by the compress call before the last one on the stream, which had completed when the
+//    last one let anything start.  Loads of the input and further requests (early_load): the schedule runner's second and later
+//    compress kernels, whose inputs were complete before its first one started and are written by none of them; they are whole
+//    16-byte pieces, so that all these loads are bulk copies, which go to the L2 cache, where completed kernels' writes are.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -1004,9 +1012,6 @@ struct CompressArgs {
   const uint32_t* plane_nout;
 };
 
-// Decompress kernels that follow one another in a schedule need nothing of one another: the first waits for the compress
-// kernels and then lets its successor start, which starts its own successor and waits for its predecessor only before it ends.
-constexpr uint32_t kInOrder = 0, kFirst = 1, kAfter = 2;
 struct DecompressArgs {
   const uint8_t* src_base;
   unsigned long long src_bytes;
@@ -1014,7 +1019,6 @@ struct DecompressArgs {
   uint8_t* dst;
   unsigned long long* d_status;        // optional
   Scratch* sc;
-  uint32_t order;                      // kInOrder, kFirst, kAfter: see decompress_begin
   unsigned long long team_stride;      // a prime, at most the number of warps of the grid (see decompress_kernel)
   unsigned long long cta_stride;       // ... of CTAs
 };

@@ -95,8 +95,7 @@ inline Plan with_first_request(const Plan& pl, int grid, uint32_t least) {
   return q;
 }
 
-// Launch that may overlap the tail of the previous kernel on the stream: every kernel of this library
-// passes dep_wait() before it touches global memory, so stream order is kept.
+// Launch that may overlap the tail of the previous kernel on the stream (see dep_wait for what keeps the order).
 template <typename K, typename A>
 cudaError_t launch_dependent(K kernel, int grid, int threads, size_t smem, cudaStream_t stream, const Plan& pl,
                              const A& a) {
