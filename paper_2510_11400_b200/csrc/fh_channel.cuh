@@ -12,7 +12,7 @@
 // the L2 cache comes from there from the second time on.  A lane has 64 bytes in flight; the
 // passes follow one another by programmatic launch; no memset between them (the streaming kernel's last CTA returns the
 // statistics to zero).  Element by element with a warp per plane the three took 162 us for 32 x 96 bf16 planes of
-// 112 x 112 (77 MB) and 27 us for 32 x 960 of 7 x 7; now 61 and 17.
+// 112 x 112 (77 MB) and 27 us for 32 x 960 of 7 x 7; now 64 (16, 20 and 28) and 17 (5, 6 and 6), each kernel timed by itself.
 #pragma once
 
 #include "fh_device.cuh"

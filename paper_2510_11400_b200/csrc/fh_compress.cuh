@@ -1145,8 +1145,10 @@ __device__ __forceinline__ uint32_t plane_sweep(const Team& team, const Plan& pl
 // tile's eight warps to get there publishes the tile or, when planes of it are only listed, puts it on the CTA's list for later.
 //
 // Registers are what this kernel is short of: 72 a thread at three CTAs to an SM.  What the compiler cannot keep goes to local
-// memory, for which the stages leave some 28 KB of L1: with 24 bytes a thread spilled in the sweep that is just enough, with 36
-// it is not (32 x 32 planes, fp32: 3 % slower, 24 x 24: 6 %).  So little is held across the calls of the outlined functions.
+// memory, for which the stages leave some 28 KB of L1, so little is held across the calls of the outlined functions: a version of the
+// sweep with 36 bytes a thread spilled instead of 24 took 3 % longer on 32 x 32 fp32 planes, 6 % on 24 x 24.  Stored bytes as the
+// compiler reports them now, three-sigma rule, fp32: 8 to 20 in teams of a warp (32 x 32: 8), 8 to 32 in smaller ones (14 x 14: 28, 7 x 7:
+// 32), up to 72 in those of one lane; bf16 8 to 24 and up to 64; without the rule 28 to 84, with random rounding 20 to 92.
 // -------------------------------------------------------------------------------------------------
 constexpr int kWarpKernelThreads = kThreads + 32;
 
@@ -1787,7 +1789,8 @@ __global__ void __launch_bounds__(kWarpKernelThreads, 3) compress_warp(const Pla
     };
     // Tensors of no more tiles than the grid has stages: every CTA takes as many as its first request is for, those of the lowest
     // numbers -- one to an SM -- one more, and nobody asks whether there is another: the answer took a microsecond that the
-    // CTA's last sweep did not hide (fp32, us a call: 32 x 16 planes of 32 x 32 5.5 -> 5.1, 128 of 28 x 28 5.3 -> 4.6).
+    // CTA's last sweep did not hide (fp32, us a call among others, with the question / without: 32 x 16 planes of 32 x 32 5.6 / 5.2,
+    // 128 of 28 x 28 5.0 / 4.4, 16 x 64 of 14 x 14 5.5 / 5.0; nothing where the host takes longer to call).
     // (Tickets are still handed out in order: the tiles before a CTA's are with CTAs that run.)
     const uint32_t rest = pl.ntiles - min(pl.ntiles, pl.first_req * gridDim.x);
     const uint32_t most = pl.ntiles <= nstage * gridDim.x ? pl.first_req + (blockIdx.x < rest ? 1u : 0u) : 0xFFFFFFFFu;
@@ -2357,12 +2360,15 @@ struct CtaOwn {
   float lo, scale;
 };
 // WORDS: bf16 runs are held as they lie in memory, with which 24 warps fit on an SM instead of 20 (28 without the plane's own
-// statistics).  That is taken for CTAs of 7, 11 and 12 warps, which come to three, two and two on an SM then and not to
-// two, one and one: with few warps resident, the three barriers a plane are what such planes wait for.  us a call, 2 bits, before
+// statistics, and with random rounding, which reads the run again and takes 72 registers too).  That is taken for CTAs of 7, 11 and
+// 12 warps, which come to three, two and two on an SM then and not to two, one and one, when there are planes for them (see
+// word_runs): with few warps resident, the three barriers a plane are what such planes wait for.  us a call, 2 bits, before
 // and now: 128 x 96 planes of 112 x 112 118.1 -> 108.0, with every eighth channel outlier-rich 250.2 -> 220.4, without statistics
 // 73.2 -> 61.7, random rounding 249.3 -> 214.5; 64 x 32 of 140 x 140 46.3 -> 36.6, of 146 x 146 47.4 -> 39.9; 100 x 61 of
-// 127 x 93 72.0 -> 68.1.  Elsewhere it is as many CTAs or little more, and the six instructions a group cost more than it gives:
-// 56 x 56 (2 warps) 50.2 -> 55.6, 120 x 119 (8 warps) 50.2 -> 50.9.
+// 127 x 93 72.0 -> 68.1.  Elsewhere it is as many CTAs or little more, and with statistics the six instructions a group cost more than
+// it gives: 56 x 56 (2 warps) 50.2 -> 55.6; 125 MB of 104 x 103 (6 warps) 53.8 -> 55.6, 119 x 120 (8) 55.8 -> 56.8, 126 x 128 (9)
+// 52.7 -> 57.8, 152 x 153 (13) 69.1 -> 77.2, 158 x 158 (14) 64.0 -> 72.1.  (Not taken so far: without statistics and with random
+// rounding it would pay at more widths, 13 warps 46.4 -> 35.2 and 148 -> 122.)
 // What is not needed in every step is kept in shared memory then, since what does not fit the registers goes to local memory, for
 // which the stages leave little L1.
 template <bool WORDS>

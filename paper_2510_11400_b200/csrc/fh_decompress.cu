@@ -54,23 +54,25 @@ int launch_decompress_small(const Plan& pl0, const DecompressArgs& a, cudaStream
   return FH_OK;
 }
 
-// (see decompress_large)
+// (see decompress_large, where both sides of the line are measured)
 constexpr uint64_t kLargeBytes = 128ull << 20;
 int launch_decompress_large(const Plan& pl, const DecompressArgs& a, cudaStream_t stream) {
   int grid = 0;
   const uint64_t ctas = (pl.P * ((pl.HW + 3 + 1023) / 1024) + kWarps - 1) / kWarps;
-  int rc = grid_for(decompress_large<kF32>, pl.sm_total, (uint32_t)std::min<uint64_t>(ctas, 0x7FFFFFFFu), &grid);
+  int rc = grid_for(decompress_large, pl.sm_total, (uint32_t)std::min<uint64_t>(ctas, 0x7FFFFFFFu), &grid);
   if (rc != FH_OK) return rc;
   DecompressArgs b = a;
   b.team_stride = prime_at_most((uint64_t)grid * kWarps);
   b.cta_stride = prime_at_most((uint64_t)grid);
-  return launch_dependent(decompress_large<kF32>, grid, kThreads, pl.sm_total, stream, pl, b) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
+  return launch_dependent(decompress_large, grid, kThreads, pl.sm_total, stream, pl, b) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
 
 template <int DT>
 int launch_decompress_dt(const Plan& pl, const DecompressArgs& a, cudaStream_t stream) {
   if (pl.groups <= 128 && pl.team == 32u) return launch_decompress_small<DT>(pl, a, stream);
-  if (DT == kF32 && pl.dense_bytes > kLargeBytes) return launch_decompress_large(pl, a, stream);
+  if constexpr (DT == kF32) {
+    if (pl.dense_bytes > kLargeBytes) return launch_decompress_large(pl, a, stream);
+  }
   return pl.plane_bytes % 16 == 0 ? launch_decompress_t<DT, true>(pl, a, stream) : launch_decompress_t<DT, false>(pl, a, stream);
 }
 

@@ -899,12 +899,13 @@ __device__ __forceinline__ void decode_chunk_large_shifted(const uint8_t* slot, 
 }
 
 // fp32 tensors that are larger than the L2 cache: the same in chunks of 1,024 elements, one at a time, nothing requested ahead.
-// Their restored elements go to memory while they are written, and requests ahead of the stores cost such a tensor more than
-// their latency: 400 MB restored from 4 bits, 40 x 40 planes 80 us so and 86 with stream_planes, 28 x 28 76 and 84, 62 x 24 76 and
-// 83, 32 x 32 (1 GiB) 213 and 217; 25 MB of 28 x 28 9.2 and 8.3.  (bf16 tensors have twice the elements to work on per byte and
-// gain from requests ahead at any size.)
-template <int DT>
-__global__ void __launch_bounds__(kThreads, 4) decompress_large(const Plan pl, const DecompressArgs a) {
+// Requests ahead pay while the restored elements stay in that cache and cost once they go to memory as they are written.  us a call,
+// 4 bits, 28 x 28 / 56 x 56 / 112 x 112 planes, in this kernel and with stream_planes: 64 MiB 17.7 / 16.6 / 16.1 and 16.1 / 16.1 / 15.4, 96
+// 24.2 / 22.9 / 22.9 and 23.4 / 22.9 / 22.1, 128 30.1 / 29.2 / 30.2 and 30.0 / 30.2 / 29.2, 160 36.2 / 35.2 / 37.3 and 36.1 / 36.2 / 36.4, 196
+// 42.5 / 42.4 / 44.4 and 44.5 / 44.4 / 44.4, 256 53.8 / 54.8 / 55.8 and 56.7 / 56.8 / 55.8, 400 80.4 / 83.5 / 86.4 and 87.5 / 86.5 / 85.5.  (Neither
+// is bound by HBM alone: DRAM is busy about half of the time, and waits for code words lead the stalls.  bf16 tensors have twice the
+// elements to work on per byte and gain from requests ahead at any size.)
+static __global__ void __launch_bounds__(kThreads, 4) decompress_large(const Plan pl, const DecompressArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ double s_red[kMaxWarps * 4];
   __shared__ uint32_t s_hdr_ok, s_bits;
@@ -1001,7 +1002,7 @@ __global__ void __launch_bounds__(kThreads, 4) decompress_large(const Plan pl, c
         bad = true;
       }
     }
-    FH_RESTORE_OUTLIER_RICH(DT)
+    FH_RESTORE_OUTLIER_RICH(kF32)
   }
   decompress_exit(a, bad);
 }
