@@ -211,7 +211,9 @@ int fh_decompress(const void* d_src, size_t src_bytes, const fh_tensor_desc* exp
  * One training step's worth of codec work on one stream (Section 3.2; Algorithm 1): entries with
  * action FH_COMPRESS are compressed in forward order into d_arena (bump allocation with a
  * device-side cursor, 256-byte aligned containers, because sizes are only known on the device), then
- * restored in reverse order into their d_restored buffers.  Forward and backward phases are timed
+ * restored in reverse order into their d_restored buffers.  Where no two of the d_restored buffers and
+ * the arena overlap, tensors are restored side by side on the stream and on streams of the library that are joined to it.
+ * Forward and backward phases are timed
  * with CUDA events.  This call synchronises the stream before it returns and fills *report.
  * An arena too small gives report->status = FH_ERR_CAPACITY (later tensors are skipped, nothing is
  * written outside the arena).
