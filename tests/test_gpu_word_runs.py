@@ -1,6 +1,7 @@
 """Parity of bf16 planes that are held in registers as they lie in memory (planes of 2,689 to 3,136 and of 4,481 to 5,376 groups of
 four) with the oracle: at the edges of those ranges, on and off the 16-byte grid, and with values for which a threshold on distances is
-hard to turn into one on elements."""
+hard to turn into one on elements.  How planes are held depends on how many there are: the first tests' few are held as fp32, the same
+sizes and values come again in tests with as many as are held as words."""
 import numpy as np
 import pytest
 
